@@ -362,7 +362,7 @@ extern "C" spsyrk_status_t spsyrk_column_panel(int64_t m, int64_t nnz, spsyrk_dt
             panel_count_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(m, d_rowptr, d_colidx, c0, c1, w.cnt);
             note_launches(1);
         }
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.cnt, m, d_p_rowptr, w.partials, st));
+        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.cnt, m, d_p_rowptr, w.partials, w.err, st));
         return read_err_and_total(w, d_p_rowptr, m, nnz_out, st);
     }
     if (!d_p_vals || (nnz > 0 && !d_vals)) return SPSYRK_ERR_INVALID_ARG;
@@ -411,7 +411,7 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
 #undef COUNT
             note_launches(1);
         }
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.cnt, m, d_z_rowptr, w.partials, st));
+        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.cnt, m, d_z_rowptr, w.partials, w.err, st));
         return read_err_and_total(w, d_z_rowptr, m, nnz_out, st);
     }
     if (!d_z_vals || (nnz_x > 0 && !d_x_vals) || (nnz_y > 0 && !d_y_vals)) return SPSYRK_ERR_INVALID_ARG;

@@ -326,7 +326,7 @@ spsyrk_status_t bin_view(spsyrk_plan_s* pl, cudaStream_t st) {
             default: launch_row_work<32>(pl, st); break;
         }
     }
-    SPSYRK_CUDA_TRY(bin_items(pl->cls, rows, pl->perm, pl->class_start_dev, pl->blockhist, pl->offsets, pl->partials, st));
+    SPSYRK_CUDA_TRY(bin_items(pl->cls, rows, pl->perm, pl->class_start_dev, pl->blockhist, pl->offsets, pl->partials, P.err, st));
     if (rows > 0) {
         row_header_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(P, pl->perm, rows, pl->hdr);
         note_launches(1);
@@ -338,7 +338,7 @@ spsyrk_status_t bin_view(spsyrk_plan_s* pl, cudaStream_t st) {
         uint32_t* items8 = reinterpret_cast<uint32_t*>(pl->cnt);  // free until the symbolic pass
         row_items_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(P, pl->hdr, pl->cls, rows, pl->diag, items8);
         note_launches(1);
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(items8, rows, pl->itemoff, pl->partials, st));
+        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(items8, rows, pl->itemoff, pl->partials, P.err, st));
         SPSYRK_CUDA_TRY(cudaMemcpyAsync(&map_items, pl->itemoff + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     }
     unsigned long long wt = 0;
@@ -800,7 +800,7 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
             default: launch_row_expand<32>(pl, st); break;
         }
     }
-    PLAN_TRY(exclusive_scan_i64<uint32_t>(pl->colcnt, n, P.colptr, pl->partials, st));
+    PLAN_TRY(exclusive_scan_i64<uint32_t>(pl->colcnt, n, P.colptr, pl->partials, P.err, st));
     s = read_err(pl, st);  // synchronises; column ids are known to be in range and rows sorted from here on
     if (s != SPSYRK_OK) return fail(s);
     s = sv == 8 ? sort_by_column<uint64_t>(pl, st) : sort_by_column<uint32_t>(pl, st);
@@ -865,7 +865,7 @@ spsyrk_status_t spsyrk_plan_partition(spsyrk_plan_t plan, int64_t parts, int64_t
     if (work_all > 0 && work_all > INT64_MAX / parts) return SPSYRK_ERR_OVERFLOW;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int64_t>(pl->upper_active ? pl->work_sum : pl->dev.work, rows, pl->work_prefix, pl->partials, st));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<int64_t>(pl->upper_active ? pl->work_sum : pl->dev.work, rows, pl->work_prefix, pl->partials, pl->dev.err, st));
     partition_kernel<<<(unsigned)((parts + 1 + 255) / 256), 256, 0, st>>>(pl->work_prefix, rows, parts, pl->dev.r0, pl->part_bounds);
     note_launches(1);
     SPSYRK_CUDA_TRY(cudaGetLastError());
@@ -895,7 +895,7 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t
         }
         counts = pl->cnt_tot;
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(counts, rows, d_c_rowptr, pl->partials, st));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(counts, rows, d_c_rowptr, pl->partials, pl->dev.err, st));
     if (pl->upper_active && rows > 0) {
         // the upper part of row r starts after its lower part
         upper_begin_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(d_c_rowptr, pl->cnt, rows, pl->hi_begin);
@@ -1027,7 +1027,7 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
         onepass_slots_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev, pl->cls, pl->cnt, pl->diag, rows, pl->ub);
         note_launches(1);
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(pl->ub, rows, pl->ub_off, pl->partials, st));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(pl->ub, rows, pl->ub_off, pl->partials, pl->dev.err, st));
     int64_t total = 0;
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&total, pl->ub_off + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     s = read_err(pl, st);
@@ -1061,7 +1061,7 @@ spsyrk_status_t spsyrk_onepass_numeric(spsyrk_plan_t plan, int32_t* d_slot_colid
     pl->cnt_out = nullptr;
     pl->map_filled = map_was;
     if (s != SPSYRK_OK) return s;
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(pl->cnt, rows, d_c_rowptr, pl->partials, st));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(pl->cnt, rows, d_c_rowptr, pl->partials, pl->dev.err, st));
     int64_t nnz = 0;
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&nnz, d_c_rowptr + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     s = read_err(pl, st);

@@ -199,7 +199,7 @@ extern "C" spsyrk_status_t spsyrk_permute(int64_t m, int64_t n, int64_t nnz, sps
         permuted_lengths_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(d_rowptr, d_rperm, m, nnz, w.len, w.err);
         note_launches(1);
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.len, m, d_b_rowptr, w.partials, st));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.len, m, d_b_rowptr, w.partials, w.err, st));
     // a bad map or row pointer must be known before entries are moved by it
     uint32_t e = 0;
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, w.err, 4, cudaMemcpyDeviceToHost, st));

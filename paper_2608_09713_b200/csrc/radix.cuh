@@ -247,7 +247,7 @@ inline cudaError_t radix_pass_impl(const uint32_t* keys, const uint32_t* pa, con
     const int64_t nt = radix_tiles(n);
     if (nt == 0) return cudaSuccess;
     radix_hist_kernel<BITS><<<(unsigned)nt, RX_THREADS, 0, st>>>(keys, n, shift, hist, nt);
-    cudaError_t e = exclusive_scan_i64<uint32_t>(hist, (int64_t)NB * nt, offsets, partials, st);
+    cudaError_t e = exclusive_scan_i64<uint32_t>(hist, (int64_t)NB * nt, offsets, partials, err, st);
     if (e != cudaSuccess) return e;
     auto kern = radix_scatter_kernel<BITS, PB, Emit, HAS_PC>;
     const size_t smem = RadixSmem<BITS, PB, HAS_PC>::bytes();
