@@ -461,13 +461,15 @@ def roofline_and_variants(a, args, line, ctx, headline):
         pms = [r["mirror_pass_ms"] for r in results if r["mirror_pass_ms"]]
         if pms:
             pm = np.mean(np.array(pms), axis=0)
-            # one sorting pass moves a 16-byte record in and out plus the digit byte it writes and the next histogram reads
-            pass_bytes = nnz_c * (16 + 16 + 2)
-            mid = int(np.argmax(pm))
             line["mirror_pass"]["sort_passes_ms"] = [float(x) for x in pm]
-            line["mirror_pass"]["sort_pass_roofline"] = {"bound": "hbm", "kernel": "mirror_pass_kernel (histogram + scan + scatter of one pass)",
-                                                         "bytes_per_pass": int(pass_bytes), "achieved": pass_bytes / (float(pm[mid]) / 1e3) / 1e9,
-                                                         "peak": peak, "unit": "GB/s", "frac": pass_bytes / (float(pm[mid]) / 1e3) / 1e9 / peak}
+            if sv == 8 and a.m > 65536:
+                # a record pass moves a 16-byte record in and out plus the digit byte it writes and the next histogram reads
+                pass_bytes = nnz_c * (16 + 16 + 2)
+                mid = int(np.argmax(pm))
+                ms = float(pm[mid])
+                line["mirror_pass"]["sort_pass_roofline"] = {"bound": "hbm", "kernel": "mirror_pass_kernel (histogram + scan + scatter of one pass)",
+                                                             "bytes_per_pass": int(pass_bytes), "achieved": pass_bytes / (ms / 1e3) / 1e9,
+                                                             "peak": peak, "unit": "GB/s", "frac": pass_bytes / (ms / 1e3) / 1e9 / peak}
     if not headline:
         del keep
         full_variant(a, args, line, ctx)

@@ -214,7 +214,7 @@ spsyrk_status_t spsyrk_onepass_compact(spsyrk_plan_t plan, const int64_t *d_c_ro
  *      ascending) is left out of the reflection; it never indexes outside the arrays.
  *      Until this step's work on the stream has completed, d_f_colidx and d_f_vals (the sizes step 2
  *      gave: nnz_full entries each) also serve as scratch of the sort, which is why the workspace is about
- *      1.5 (8-byte values) to 2.2 (4-byte values) times the bytes of C_L and not 3 times; both arrays must
+ *      1.3 (4-byte values) to 1.5 (8-byte values) times the bytes of C_L and not 3 times; both arrays must
  *      be 16-byte aligned and must not overlap each other, the workspace or C_L (INVALID_ARG if misaligned).
  * nnz_l = d_l_rowptr[m].  Errors: INVALID_ARG, WORKSPACE, BAD_CSR (an entry above the diagonal), CUDA.
  */
@@ -407,10 +407,10 @@ spsyrk_status_t spsyrk_plan_buffers(spsyrk_plan_t plan, const int64_t **d_colptr
  * spsyrk_launch_count       : kernels launched by this library in this process so far.
  */
 spsyrk_status_t spsyrk_plan_enable_timing(spsyrk_plan_t plan);
-/* spsyrk_mirror_enable_timing(1): from now on the fill step of spsyrk_mirror on 8-byte values records
+/* spsyrk_mirror_enable_timing(1): from now on the fill step of spsyrk_mirror records
  *     CUDA events around each of its sorting passes (process-wide switch, not thread-safe; 0 turns it off).
  * spsyrk_mirror_timings: *passes = sorting passes of the last such fill (at most 4) and their device
- *     milliseconds (histogram, scan and scatter of the pass); waits for those events. */
+ *     milliseconds (counts, scan and placement of the pass); waits for those events. */
 spsyrk_status_t spsyrk_mirror_enable_timing(int on);
 spsyrk_status_t spsyrk_mirror_timings(int *passes, float pass_ms[4]);
 spsyrk_status_t spsyrk_plan_timings(spsyrk_plan_t plan, float symbolic_ms[8], float numeric_ms[8]);

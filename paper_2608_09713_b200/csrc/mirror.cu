@@ -2,23 +2,19 @@
 //
 // Row j of F = row j of C_L (columns <= j) followed by the reflected entries (r, c_rj) of the
 // later rows r > j that store column j, ascending in r.  That second part is a transpose of the
-// strictly lower triangle, done as a stable radix sort of the entries by column id:
+// strictly lower triangle, done as a stable sort of the entries by column id:
 //   sizes   : rows are ascending, so a row stores its diagonal iff its last entry is the diagonal and
 //             holds an entry above the diagonal iff its last entry is one:
 //             nnz(F) = 2 nnz(C_L) - #diagonals.
-//   expand  : an explicit (key, row) pair per entry, the key being the column id, or m for a
-//             diagonal entry (and for an entry that should not be there) so that it sorts past the end.
-//   sort    : stable LSD radix passes over (key, row, value); entries enter in ascending row order,
-//             so every column's segment comes out ascending in r.  The last pass writes straight
-//             into F: the s-th strictly lower entry in sorted order, of column j, lands at
-//             s + l_rowptr[j + 1].  It also records where each column's segment starts and ends
-//             (equal keys are adjacent in the last pass: one atomic at each end of a run), which is
-//             the number of reflected entries of row j.
-//   rows    : row lengths of F, scan -> f_rowptr, then the lower parts are copied into place.
+//   sort    : 4-byte values and small matrices go to buckets of columns and from there to their places
+//             (mirror_sort.cuh); 8-byte values of more than 65536 rows go through radix passes of 16-byte
+//             records, the last of which writes F (mirror_rec.cuh);
+//   rows    : row lengths of F, scan -> f_rowptr (in the bucket sort before the last pass), lower parts copied.
 #include <algorithm>
 #include <mutex>
 
 #include "mirror_rec.cuh"
+#include "mirror_sort.cuh"
 
 using namespace spsyrk;
 
@@ -26,39 +22,88 @@ namespace {
 
 constexpr size_t ALIGN = 256;
 
-constexpr int MIRROR_RADIX_BITS = 8;
+constexpr int MIRROR_RADIX_BITS = 8;  // digits of the record passes
+
+// 8-byte values: the record passes move 16-byte records in runs that the cut into buckets does not reach (three
+// passes over 5.4e8 records: 14.7 ms and 1.6 for histograms and scans, against 15.9 and 1.1), but the bucket sort takes half
+// the launches: it is used where both take two passes.  (Product and mirror of 4096 rows: 465 -> 415 us.)
+constexpr int64_t MIRROR_BUCKET_ROWS_8 = 65536;
+bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCKET_ROWS_8; }
 
 struct MirrorWs {
-    uint32_t* diagf;   // m: 1 where the row stores its diagonal entry
-    uint32_t* rowtot;  // m
-    int64_t* dcount;   // m + 1: diagonal entries of the rows before (exclusive prefix sums of diagf)
-    int64_t* fbase;    // m: l_rowptr[j + 1] - dcount[j + 1]
-    // 8-byte values: the record buffer the last pass reads (nnz_l records), the tail of the buffer that lives in
-    // F's value array, and digit bytes for inputs too small to keep them in F's column array
-    MirrorRec *rec_keep, *rec_tail;
-    uint8_t* dig_small;
+    int64_t* partials;
+    uint32_t* err;       // [0] error word, [1] number of diagonal entries
+    uint32_t* hist;      // counts of the passes and their prefix sums
+    int64_t *offsets, *mid_off;
+    // bucket sort
+    uint8_t* diagf;      // m: 1 where the row stores its diagonal entry
+    uint32_t* cnt;       // m: entries of C_L per column
+    int64_t* fstart;     // m: where the entries of column j go in F
+    int32_t* step_row;   // row of every 32nd entry
+    void* rec;           // the records the place pass reads (nnz_l)
+    void* rec_tail;      // three passes: what of the first buffer does not fit F's value array
+    uint16_t* high;      // 4-byte values: the rests of the columns beside the records
+    // record passes
+    uint32_t* diagf32;   // m
+    uint32_t* rowtot;    // m
+    int64_t* dcount;     // m + 1: diagonal entries of the rows before (exclusive prefix sums of diagf32)
+    int64_t* fbase;      // m: l_rowptr[j + 1] - dcount[j + 1]
+    // the record buffer the last pass reads (nnz_l records) and the tail of the buffer that lives in F's value array
+    MirrorRec *rec_keep, *rec_keep_tail;
     int32_t* tile_rows;  // 2 per tile
     unsigned long long* seg_start;  // m: first sorted position of column j's strictly lower entries
     unsigned long long* seg_end;    // m: one past the last
-    int64_t* partials;
-    uint32_t* err;
-    // radix sort buffers (nnz_l entries each); buffer B's key and row arrays double as the expanded input
-    uint32_t *key_a, *row_a, *key_b, *row_b;
-    void *val_a, *val_b;
-    uint32_t* hist;
-    int64_t* offsets;
+    uint8_t* dig_small;  // digit bytes of inputs too small to keep them in F's column array
 };
 
-// Scratch inside the output.  Until the last pass writes it, F's memory is free, and the sort needs two record
-// buffers of 16 nnz_l bytes each.  The buffer the last pass reads must lie outside F; the other one lives in F's
-// value array, which holds 8 (2 nnz_l - D) bytes with D <= min(m, nnz_l) diagonal entries: the first
-// nnz_l - ceil(min(m, nnz_l) / 2) records always fit, the few remaining ones go to a tail in the workspace.
-// The digit bytes (two buffers of nnz_l bytes) live in F's column array (4 (2 nnz_l - D) bytes), which is free
-// whenever a histogram reads them: the last pass, the first to write that array, starts after its histogram.
-inline int mirror_passes_4byte(int64_t m) { return (bits_for((uint64_t)m) + MIRROR_RADIX_BITS - 1) / MIRROR_RADIX_BITS; }  // keys run from 0 to m
-inline int64_t mirror_tail_records(int64_t m, int64_t nnz_l) { return (std::min(m, nnz_l) + 1) / 2; }
-constexpr int64_t MIRROR_DIG_SMALL = 32;  // inputs of fewer entries than this keep their digit bytes in the workspace
+// How the sort is cut (see mirror_sort.cuh)
+struct MirrorSplit {
+    int lbits, mbits, hbits, pieces;
+    int64_t rounds, chunk, nchunks;
+    int64_t split_hist() const { return (rounds << lbits) * nchunks; }
+    int64_t mid_hist() const { return mbits ? (rounds << (lbits + mbits)) * pieces : 0; }
+};
 
+// Column ids of at most so many bits take two passes: parts of nine bits leave runs of eight entries in a tile.  (Two parts of
+// ten bits against three of six to eight on 1.35e8 entries: 5.6 ms against 4.6.)
+constexpr int MIRROR_TWO_PASS_BITS = 18;
+
+MirrorSplit mirror_split_for(int64_t m, int64_t nnz_l, size_t sv) {
+    MirrorSplit s;
+    int bits = 1;
+    while (bits < MS_ROUND_BITS && ((m - 1) >> bits) > 0) ++bits;
+    s.rounds = (std::max<int64_t>(m - 1, 0) >> MS_ROUND_BITS) + 1;
+    if (bits <= MIRROR_TWO_PASS_BITS) {
+        s.lbits = std::max(8, (bits + 1) / 2);  // at least 256 buckets: a bucket is one CTA of the last pass
+        s.mbits = 0;
+        s.hbits = std::max(2, bits - s.lbits);
+    } else {
+        s.lbits = 8;  // what is left fits 16 bits
+        s.mbits = (bits - s.lbits + 1) / 2;
+        s.hbits = bits - s.lbits - s.mbits;
+    }
+    const int64_t tile = sv == 8 ? mirror_tile<uint64_t>() : mirror_tile<uint32_t>();
+    // Chunks of the split and pieces of the mid pass, one CTA each.  Below two tiles per SM the entries are shared out
+    // evenly; above, a chunk is whole tiles, few enough that neighbouring CTAs write neighbouring runs (148 * 24 chunks
+    // 6.6 ms for the split of 5.4e8 records, 148 * 150 to 300 6.0) and enough that the counts, one per bin and chunk, stay small.
+    constexpr int64_t FEW = 148 * 2, MANY = 148 * 150;
+    if (nnz_l <= FEW * tile) s.chunk = std::max<int64_t>((nnz_l + FEW - 1) / FEW, 256);
+    else s.chunk = std::max<int64_t>(nnz_l / (MANY * tile), 1) * tile;
+    s.chunk = (s.chunk + 31) / 32 * 32;
+    s.nchunks = std::max<int64_t>((nnz_l + s.chunk - 1) / s.chunk, 1);
+    s.pieces = (int)std::min<int64_t>(std::max<int64_t>((nnz_l / s.rounds >> s.lbits) / (4 * tile), 1), 64);
+    return s;
+}
+
+int64_t mirror_tail_records(int64_t m, int64_t nnz_l) { return (std::min(m, nnz_l) + 1) / 2; }
+
+// Scratch inside the output.  Until the last pass writes it, F's memory is free.  Three passes need two record buffers
+// of R nnz_l bytes each (R = 16 or 8, twice the size of a value).  The one the last pass reads must lie outside F; the
+// other one lives in F's value array, which holds R / 2 * (2 nnz_l - D) bytes with D <= min(m, nnz_l) diagonal entries: the
+// first nnz_l - ceil(min(m, nnz_l) / 2) records always fit, the few remaining ones go to a tail in the workspace.
+// The digit bytes of the record passes (two buffers of nnz_l bytes) and the two-byte rests of the columns live in F's column
+// array (4 (2 nnz_l - D) >= 4 nnz_l bytes) where the last pass does not read them.
+constexpr int64_t MIRROR_DIG_SMALL = 32;  // inputs of fewer entries than this keep their digit bytes in the workspace
 size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
     char* base = static_cast<char*>(ws);
     size_t off = 0;
@@ -70,43 +115,38 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
     };
     const int64_t items = std::max<int64_t>(m, 1);
     const int64_t ne = std::max<int64_t>(nnz_l, 1);
-    const int64_t hist_n = (int64_t)(1 << MIRROR_RADIX_BITS) * std::max<int64_t>(sv == 8 ? mirror_groups(nnz_l) : radix_tiles(nnz_l), 1);
-    MirrorWs t;
-    t.diagf = (uint32_t*)take(items * 4);
-    t.rowtot = (uint32_t*)take(items * 4);
-    t.dcount = (int64_t*)take((items + 1) * 8);
-    t.fbase = (int64_t*)take(items * 8);
-    t.seg_start = (unsigned long long*)take(items * 8);
-    t.seg_end = (unsigned long long*)take(items * 8);
-    t.partials = (int64_t*)take(scan_partials_count(std::max<int64_t>(items + 1, hist_n)) * 8);
-    t.err = (uint32_t*)take(8);  // [0] error word, [1] number of diagonal entries
-    t.key_a = t.row_a = t.key_b = t.row_b = nullptr;
-    t.val_a = t.val_b = nullptr;
-    t.rec_keep = t.rec_tail = nullptr;
-    t.dig_small = nullptr;
-    t.tile_rows = nullptr;
-    if (sv == 8) {
+    MirrorWs t{};
+    t.err = (uint32_t*)take(8);
+    if (mirror_by_records(m, sv)) {
+        const int64_t hist_n = (int64_t)(1 << MIRROR_RADIX_BITS) * std::max<int64_t>(mirror_groups(nnz_l), 1);
+        t.diagf32 = (uint32_t*)take(items * 4);
+        t.rowtot = (uint32_t*)take(items * 4);
+        t.dcount = (int64_t*)take((items + 1) * 8);
+        t.fbase = (int64_t*)take(items * 8);
+        t.seg_start = (unsigned long long*)take(items * 8);
+        t.seg_end = (unsigned long long*)take(items * 8);
+        t.partials = (int64_t*)take(scan_partials_count(std::max<int64_t>(items + 1, hist_n)) * 8);
         t.rec_keep = (MirrorRec*)take(ne * sizeof(MirrorRec));
-        t.rec_tail = (MirrorRec*)take((mirror_tail_records(m, nnz_l) + 1) * sizeof(MirrorRec));
+        t.rec_keep_tail = (MirrorRec*)take((mirror_tail_records(m, nnz_l) + 1) * sizeof(MirrorRec));
         t.dig_small = (uint8_t*)take(2 * MIRROR_DIG_SMALL);
         t.tile_rows = (int32_t*)take(2 * std::max<int64_t>(mirror_tiles(nnz_l), 1) * 4);
+        t.hist = (uint32_t*)take(hist_n * 4);
+        t.offsets = (int64_t*)take((hist_n + 1) * 8);
     } else {
-        // The buffer set the last pass does not read keeps its keys in F's column array and its values in F's
-        // value array (4 (2 nnz_l - D) >= 4 nnz_l bytes each, free until the last pass); only its row ids need
-        // workspace.  Passes alternate A, B, A, ...: the last one reads B when the number of passes is odd.
-        const bool a_in_f = (mirror_passes_4byte(m) % 2) == 1;
-        t.row_a = (uint32_t*)take(ne * 4);
-        t.row_b = (uint32_t*)take(ne * 4);
-        if (a_in_f) {
-            t.key_b = (uint32_t*)take(ne * 4);
-            t.val_b = take(ne * sv);
-        } else {
-            t.key_a = (uint32_t*)take(ne * 4);
-            t.val_a = take(ne * sv);
-        }
+        const MirrorSplit sp = mirror_split_for(m, nnz_l, sv);
+        const int64_t hist_n = std::max(sp.split_hist(), sp.mid_hist());
+        t.diagf = (uint8_t*)take(items);
+        t.cnt = (uint32_t*)take(items * 4);
+        t.fstart = (int64_t*)take(items * 8);
+        t.partials = (int64_t*)take(scan_partials_count(std::max<int64_t>(items, hist_n)) * 8);
+        t.hist = (uint32_t*)take(hist_n * 4);
+        t.offsets = (int64_t*)take((sp.split_hist() + 1) * 8);
+        t.mid_off = (int64_t*)take((sp.mid_hist() + 1) * 8);
+        t.step_row = (int32_t*)take((ne + 31) / 32 * 4);
+        t.rec = take(ne * 2 * sv);
+        t.rec_tail = take(sp.mbits ? (mirror_tail_records(m, nnz_l) + 1) * 2 * sv : 0);
+        t.high = (uint16_t*)take(sv == 8 ? 0 : ne * 2);
     }
-    t.hist = (uint32_t*)take(hist_n * 4);
-    t.offsets = (int64_t*)take((hist_n + 1) * 8);
     if (w) *w = t;
     return (off + ALIGN - 1) / ALIGN * ALIGN;
 }
@@ -159,34 +199,6 @@ __global__ void mirror_last_entry_kernel(const int64_t* __restrict__ l_rowptr, c
     if (lane_id() == 0 && votes) atomicAdd(err + 1, (uint32_t)__popc(votes));
 }
 
-// G lanes per row: the explicit (key, row) pair of every entry
-template <int G>
-__global__ void __launch_bounds__(256) mirror_expand_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx,
-                                                            int64_t m, uint32_t* __restrict__ key0, uint32_t* __restrict__ row0,
-                                                            uint32_t* err) {
-    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int gl = threadIdx.x & (G - 1);
-    if (r >= m) return;
-    const int64_t p0 = l_rowptr[r], p1 = l_rowptr[r + 1];
-    constexpr int UNR = 4;  // loads of several steps are issued before the first store
-    for (int64_t p = p0 + gl; p < p1; p += UNR * G) {
-        int64_t j[UNR];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) j[u] = p + u * G < p1 ? (int64_t)l_colidx[p + u * G] : r;
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const int64_t pp = p + u * G;
-            if (pp < p1) {
-                // an entry outside the lower triangle (rows that are not ascending can hide one from the size
-                // step) is keyed like a diagonal: it takes no part in the reflection
-                if (j[u] > r || j[u] < 0) atomicOr(err, ERRW_UPPER);
-                key0[pp] = (j[u] >= r || j[u] < 0) ? (uint32_t)m : (uint32_t)j[u];
-                row0[pp] = (uint32_t)r;
-            }
-        }
-    }
-}
-
 // G lanes per row: the lower part of row r of F is row r of C_L
 template <typename V, int G>
 __global__ void __launch_bounds__(256) mirror_copy_lower_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx,
@@ -221,105 +233,116 @@ __global__ void __launch_bounds__(256) mirror_copy_lower_kernel(const int64_t* _
     }
 }
 
-// row lengths of F: the row's own entries plus the length of its column's sorted segment
-__global__ void mirror_rowlen_kernel(const int64_t* __restrict__ l_rowptr, const unsigned long long* __restrict__ seg_start,
-                                     const unsigned long long* __restrict__ seg_end, int64_t m, uint32_t* __restrict__ rowtot) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= m) return;
-    const unsigned long long s = seg_start[r], e = seg_end[r];
-    rowtot[r] = (uint32_t)(l_rowptr[r + 1] - l_rowptr[r]) + (e > s ? (uint32_t)(e - s) : 0u);
-}
-
-template <typename V>
-struct EmitMirrorFinal {
-    static constexpr bool NEIGHBOURS = true;
-    const int64_t* l_rowptr;
-    int32_t* f_colidx;
-    V* f_vals;
-    unsigned long long* seg_start;
-    unsigned long long* seg_end;
-    uint32_t m;
-    __device__ __forceinline__ void operator()(int64_t dest, uint32_t key, uint32_t row, V val, uint32_t prev, uint32_t next) const {
-        if (key < m) {  // diagonal entries were keyed m and are dropped here
-            const int64_t pos = dest + l_rowptr[key + 1];
-            f_colidx[pos] = (int32_t)row;
-            f_vals[pos] = val;
-            // ends of a run of one key inside the tile; a segment that spans tiles settles through min / max
-            if (prev != key) atomicMin(&seg_start[key], (unsigned long long)dest);
-            if (next != key) atomicMax(&seg_end[key], (unsigned long long)dest + 1ull);
-        }
-    }
-};
-
 int group_width(int64_t nnz, int64_t m) {
     const double avg = m > 0 ? (double)nnz / (double)m : 0.0;
     return avg <= 4 ? 4 : avg <= 8 ? 8 : avg <= 16 ? 16 : 32;
 }
 
-template <typename V>
-spsyrk_status_t mirror_fill(const MirrorWs& ws, int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx,
+// row lengths of F: the row's own entries and those of its column, the diagonal once
+struct MirrorRowLength {
+    const int64_t* l_rowptr;
+    const uint32_t* cnt;
+    const uint8_t* diagf;
+    __device__ __forceinline__ int64_t operator()(int64_t r) const { return l_rowptr[r + 1] - l_rowptr[r] + (int64_t)cnt[r] - (int64_t)diagf[r]; }
+};
+struct MirrorRowStart {
+    const int64_t* l_rowptr;
+    const uint8_t* diagf;
+    int64_t* f_rowptr;
+    int64_t* fstart;
+    int64_t m;
+    __device__ __forceinline__ void operator()(int64_t r, int64_t ex) const {
+        f_rowptr[r] = ex;
+        fstart[r] = ex + (l_rowptr[r + 1] - l_rowptr[r]) - (int64_t)diagf[r];
+    }
+    __device__ __forceinline__ void total(int64_t t) const { f_rowptr[m] = t; }
+};
+
+// Measurement aid: CUDA events around the sorting passes (each with its counts and scan).
+bool g_mirror_timing = false;
+constexpr int MIRROR_MAX_PASSES = 4;
+cudaEvent_t g_mirror_ev[MIRROR_MAX_PASSES + 1];
+int g_mirror_passes = 0;
+
+void mirror_mark(int i, cudaStream_t st) {
+    if (g_mirror_timing) cudaEventRecord(g_mirror_ev[i], st);
+}
+
+template <typename VB>
+spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx,
                             const void* l_vals, int64_t* f_rowptr, int32_t* f_colidx, void* f_vals, cudaStream_t st) {
-    constexpr int BITS = MIRROR_RADIX_BITS;
-    MirrorWs w = ws;
-    // the buffer set without keys and values of its own keeps them in F's arrays (see carve)
-    if (!w.key_a) { w.key_a = reinterpret_cast<uint32_t*>(f_colidx); w.val_a = f_vals; }
-    if (!w.key_b) { w.key_b = reinterpret_cast<uint32_t*>(f_colidx); w.val_b = f_vals; }
-    const V* lv = static_cast<const V*>(l_vals);
-    V* fv = static_cast<V*>(f_vals);
+    // F's arrays hold records and rests during the sort: both must take 16-byte accesses
+    if (nnz_l > 0 && ((reinterpret_cast<uintptr_t>(f_vals) | reinterpret_cast<uintptr_t>(f_colidx)) & 15u)) return SPSYRK_ERR_INVALID_ARG;
+    if (m == 0 || nnz_l == 0) {
+        SPSYRK_CUDA_TRY(cudaMemsetAsync(f_rowptr, 0, (size_t)(m + 1) * sizeof(int64_t), st));
+        return SPSYRK_OK;
+    }
+    const MirrorSplit sp = mirror_split_for(m, nnz_l, sizeof(VB));
+    const int64_t nbuckets = sp.rounds << (sp.lbits + sp.mbits);  // of the place pass
+    const bool three = sp.mbits > 0;
     const int g = group_width(nnz_l, m);
-    if (m > 0) {
-        SPSYRK_CUDA_TRY(cudaMemsetAsync(w.seg_start, 0xff, (size_t)m * 8, st));
-        SPSYRK_CUDA_TRY(cudaMemsetAsync(w.seg_end, 0, (size_t)m * 8, st));
+    uint16_t* const f_high = reinterpret_cast<uint16_t*>(f_colidx);
+    MirrorSortArgs a{};
+    a.l_rowptr = l_rowptr; a.l_colidx = l_colidx; a.l_vals = l_vals; a.m = m; a.n = nnz_l; a.chunk = sp.chunk; a.nchunks = sp.nchunks;
+    a.lbits = sp.lbits; a.mbits = sp.mbits; a.hbits = sp.hbits; a.pieces = sp.pieces; a.step_row = w.step_row;
+    a.split_off = w.offsets; a.mid_off = w.mid_off;
+    a.rec_a = three ? f_vals : w.rec;
+    a.rec_a_tail = w.rec_tail;
+    a.a_split = three ? nnz_l - mirror_tail_records(m, nnz_l) : nnz_l;
+    a.rec_b = w.rec;
+    // the rests: the last pass reads them only for 4-byte values, and then not from F's memory
+    uint16_t* const last_high = sizeof(VB) == 4 ? w.high : f_high;
+    a.high_b = last_high;
+    a.high_a = !three ? last_high : sizeof(VB) == 4 ? f_high : f_high + nnz_l;  // (only the last pass's rests are read 16 bytes at a time)
+    a.place_off = three ? w.mid_off : w.offsets;
+    a.place_stride = three ? sp.pieces : sp.nchunks;
+    a.cnt = w.cnt; a.fstart = w.fstart; a.f_colidx = f_colidx; a.f_vals = f_vals; a.err = w.err;
+    const size_t split_smem = MirrorSplitSmem<VB>::bytes(1 << sp.lbits), place_smem = MirrorPlaceSmem<VB>::bytes(1 << sp.hbits);
+    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(mirror_split_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem));
+    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(mirror_place_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)place_smem));
+    mirror_mark(0, st);
+#define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf)
+    if (g <= 16) ROWS(4); else ROWS(16);
+#undef ROWS
+    for (int64_t q = 0; q < sp.rounds; ++q) {
+        a.round = (uint32_t)q;
+        mirror_split_count_kernel<<<(unsigned)sp.nchunks, MS_THREADS, 0, st>>>(a, w.hist);
     }
-    if (m > 0 && nnz_l > 0) {
-#define EXPAND(G) mirror_expand_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, w.key_b, w.row_b, w.err)
-        switch (g) {
-            case 4: EXPAND(4); break;
-            case 8: EXPAND(8); break;
-            case 16: EXPAND(16); break;
-            default: EXPAND(32); break;
-        }
-#undef EXPAND
-        note_launches(1);
-        const int npass = mirror_passes_4byte(m);
-        const uint32_t* src_key = w.key_b;
-        const uint32_t* src_row = w.row_b;
-        const V* src_val = lv;
-        for (int p = 0; p < npass; ++p) {
-            const bool to_a = (p % 2) == 0;
-            uint32_t* dst_key = to_a ? w.key_a : w.key_b;
-            uint32_t* dst_row = to_a ? w.row_a : w.row_b;
-            V* dst_val = static_cast<V*>(to_a ? w.val_a : w.val_b);
-            if (p == npass - 1) {
-                EmitMirrorFinal<V> emit{l_rowptr, f_colidx, fv, w.seg_start, w.seg_end, (uint32_t)m};
-                SPSYRK_CUDA_TRY((radix_pass<BITS, V>(src_key, src_row, src_val, nnz_l, p * BITS, w.hist, w.offsets, w.partials, emit, w.err, st)));
-            } else {
-                EmitArrays<V> emit{dst_key, dst_row, dst_val};
-                SPSYRK_CUDA_TRY((radix_pass<BITS, V>(src_key, src_row, src_val, nnz_l, p * BITS, w.hist, w.offsets, w.partials, emit, w.err, st)));
-            }
-            src_key = dst_key;
-            src_row = dst_row;
-            src_val = dst_val;
-        }
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.split_hist(), w.offsets, w.partials, w.err, st));
+    for (int64_t q = 0; q < sp.rounds; ++q) {
+        a.round = (uint32_t)q;
+        mirror_split_kernel<VB><<<(unsigned)sp.nchunks, MS_THREADS, split_smem, st>>>(a);
     }
-    // row pointers of F, then the lower parts
-    if (m > 0) {
-        mirror_rowlen_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, w.seg_start, w.seg_end, m, w.rowtot);
-        note_launches(1);
+    note_launches(1 + 2 * (int)sp.rounds);
+    mirror_mark(1, st);
+    int pass = 2;
+    if constexpr (sizeof(VB) == 4) if (three) {
+        const unsigned units = (unsigned)((sp.rounds << sp.lbits) * sp.pieces);
+        mirror_mid_count_kernel<<<units, MS_THREADS, 0, st>>>(a, w.hist);
+        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.partials, w.err, st));
+        const size_t mid_smem = MirrorMidSmem<VB>::bytes(1 << sp.mbits);
+        SPSYRK_CUDA_TRY(cudaFuncSetAttribute(mirror_mid_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
+        mirror_mid_kernel<VB><<<units, MS_THREADS, mid_smem, st>>>(a);
+        note_launches(2);
+        mirror_mark(pass++, st);
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.rowtot, m, f_rowptr, w.partials, w.err, st));
-    if (m > 0 && nnz_l > 0) {
+    mirror_column_count_kernel<<<(unsigned)nbuckets, MS_THREADS, 0, st>>>(a, last_high);
+    SPSYRK_CUDA_TRY(scan_launch(MirrorRowLength{l_rowptr, w.cnt, w.diagf}, m, MirrorRowStart{l_rowptr, w.diagf, f_rowptr, w.fstart, m}, w.partials, w.err, st));
+    mirror_place_kernel<VB><<<(unsigned)nbuckets, MS_THREADS, place_smem, st>>>(a);
+    mirror_mark(pass, st);
+    g_mirror_passes = pass;
+    const VB* lv = static_cast<const VB*>(l_vals);
+    VB* fv = static_cast<VB*>(f_vals);
 #define COPY(G) \
-    mirror_copy_lower_kernel<V, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, lv, m, f_rowptr, f_colidx, fv)
-        switch (g) {
-            case 4: COPY(4); break;
-            case 8: COPY(8); break;
-            case 16: COPY(16); break;
-            default: COPY(32); break;
-        }
-#undef COPY
-        note_launches(1);
+    mirror_copy_lower_kernel<VB, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, lv, m, f_rowptr, f_colidx, fv)
+    switch (g) {
+        case 4: COPY(4); break;
+        case 8: COPY(8); break;
+        case 16: COPY(16); break;
+        default: COPY(32); break;
     }
+#undef COPY
+    note_launches(3);
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
     {
@@ -370,12 +393,6 @@ cudaError_t launch_mirror_pass(const MirrorPassArgs& a, int64_t n, int shift, co
     return cudaGetLastError();
 }
 
-// Measurement aid: CUDA events around every radix pass (histogram + scan + scatter) of the last record-based fill.
-constexpr int MIRROR_MAX_PASSES = 4;
-bool g_mirror_timing = false;
-cudaEvent_t g_mirror_ev[MIRROR_MAX_PASSES + 1];
-int g_mirror_passes = 0;
-
 // 8-byte values: records, the first pass straight from C_L
 spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx,
                                 const void* l_vals, int64_t* f_rowptr, int32_t* f_colidx, void* f_vals, cudaStream_t st) {
@@ -389,10 +406,10 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
     if (m > 0) {
         SPSYRK_CUDA_TRY(cudaMemsetAsync(w.seg_start, 0xff, (size_t)m * 8, st));
         SPSYRK_CUDA_TRY(cudaMemsetAsync(w.seg_end, 0, (size_t)m * 8, st));
-        mirror_diag_flag_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, w.diagf);
+        mirror_diag_flag_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, w.diagf32);
         note_launches(1);
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.diagf, m, w.dcount, w.partials, w.err, st));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.diagf32, m, w.dcount, w.partials, w.err, st));
     if (m > 0 && nnz_l > 0) {
         mirror_fbase_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, w.dcount, m, w.fbase);
         note_launches(1);
@@ -415,7 +432,7 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
         auto in_keep = [&](int p) { return ((npass - 2 - p) % 2) == 0; };  // does pass p write the workspace buffer?
         for (int p = 0; p < npass; ++p) {
             const bool first = p == 0, last = p == npass - 1;
-            if (g_mirror_timing && p < MIRROR_MAX_PASSES) cudaEventRecord(g_mirror_ev[p], st);
+            if (first) mirror_mark(0, st);
             const unsigned hb = (unsigned)((nt + MR_HIST_TILES - 1) / MR_HIST_TILES);
             if (first) mirror_hist_key_kernel<BITS><<<hb, MR_THREADS, 0, st>>>(reinterpret_cast<const uint32_t*>(l_colidx), nnz_l, 0, w.hist, nt);
             else radix_hist_u8_kernel<BITS><<<hb, MR_THREADS, 0, st>>>(((p - 1) % 2) == 0 ? dig0 : dig1, nnz_l, w.hist, nt);
@@ -423,10 +440,10 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
             SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, (int64_t)NB * nt, w.offsets, w.partials, w.err, st));
             const bool src_keep = !first && in_keep(p - 1), dst_keep = in_keep(p);
             a.src = src_keep ? w.rec_keep : alias;
-            a.src_tail = w.rec_tail;
+            a.src_tail = w.rec_keep_tail;
             a.src_split = src_keep ? nnz_l : alias_split;
             a.dst = dst_keep ? w.rec_keep : alias;
-            a.dst_tail = w.rec_tail;
+            a.dst_tail = w.rec_keep_tail;
             a.dst_split = dst_keep ? nnz_l : alias_split;
             a.next_digit = (p % 2) == 0 ? dig0 : dig1;
             cudaError_t e;
@@ -435,14 +452,12 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
             else if (last) e = launch_mirror_pass<false, true>(a, nnz_l, p * BITS, w.offsets, nt, st);
             else e = launch_mirror_pass<false, false>(a, nnz_l, p * BITS, w.offsets, nt, st);
             SPSYRK_CUDA_TRY(e);
-            if (g_mirror_timing && p < MIRROR_MAX_PASSES) {
-                cudaEventRecord(g_mirror_ev[p + 1], st);
-                g_mirror_passes = p + 1;
-            }
+            mirror_mark(p + 1, st);
+            g_mirror_passes = p + 1;
         }
     }
     if (m > 0) {
-        mirror_rowlen_diag_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, w.seg_start, w.seg_end, w.diagf, m, w.rowtot);
+        mirror_rowlen_diag_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, w.seg_start, w.seg_end, w.diagf32, m, w.rowtot);
         note_launches(1);
     }
     SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.rowtot, m, f_rowptr, w.partials, w.err, st));
@@ -509,7 +524,9 @@ extern "C" spsyrk_status_t spsyrk_mirror(int64_t m, int64_t nnz_l, spsyrk_dtype_
     // step 3: fill
     if (!d_f_vals || (nnz_l > 0 && !d_l_vals)) return SPSYRK_ERR_INVALID_ARG;
     switch (dtype) {
-        case SPSYRK_F64: return mirror_fill_rec(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
+        case SPSYRK_F64:
+            if (mirror_by_records(m, sv)) return mirror_fill_rec(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
+            return mirror_fill<uint64_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
         default: return mirror_fill<uint32_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
     }
 }
