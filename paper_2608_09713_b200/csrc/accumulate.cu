@@ -285,14 +285,19 @@ __global__ void __launch_bounds__(256) add_fill_kernel(int64_t m, const int64_t*
     });
 }
 
-spsyrk_status_t read_err_and_total(const RowWs& w, const int64_t* d_rowptr_out, int64_t m, int64_t* total, cudaStream_t st) {
-    int64_t nnz = 0;
-    uint32_t e = 0;
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&nnz, d_rowptr_out + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, w.err, 4, cudaMemcpyDeviceToHost, st));
+// row pointers from the per-row counts; the total and the error word travel to the host (synchronises)
+spsyrk_status_t scan_and_total(const RowWs& w, int64_t m, int64_t* d_rowptr_out, int64_t* total, cudaStream_t st) {
+    ScopedHostBlock h;
+    SPSYRK_CUDA_TRY(h.acquire());
+    if (m == 0) {
+        SPSYRK_CUDA_TRY(cudaMemsetAsync(d_rowptr_out, 0, sizeof(int64_t), st));
+        h.host[0] = h.host[1] = 0;
+    } else {
+        SPSYRK_CUDA_TRY(scan_launch(ScanArray<uint32_t>{w.cnt}, m, ScanIntoHost{d_rowptr_out, m, w.err, h.dev}, w.partials, w.err, st));
+    }
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    if (e) return SPSYRK_ERR_BAD_CSR;
-    *total = nnz;
+    if (h.host[1]) return SPSYRK_ERR_BAD_CSR;
+    *total = h.host[0];
     return SPSYRK_OK;
 }
 
@@ -362,8 +367,7 @@ extern "C" spsyrk_status_t spsyrk_column_panel(int64_t m, int64_t nnz, spsyrk_dt
             panel_count_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(m, d_rowptr, d_colidx, c0, c1, w.cnt);
             note_launches(1);
         }
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.cnt, m, d_p_rowptr, w.partials, w.err, st));
-        return read_err_and_total(w, d_p_rowptr, m, nnz_out, st);
+        return scan_and_total(w, m, d_p_rowptr, nnz_out, st);
     }
     if (!d_p_vals || (nnz > 0 && !d_vals)) return SPSYRK_ERR_INVALID_ARG;
     if (m == 0) return SPSYRK_OK;
@@ -411,8 +415,7 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
 #undef COUNT
             note_launches(1);
         }
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.cnt, m, d_z_rowptr, w.partials, w.err, st));
-        return read_err_and_total(w, d_z_rowptr, m, nnz_out, st);
+        return scan_and_total(w, m, d_z_rowptr, nnz_out, st);
     }
     if (!d_z_vals || (nnz_x > 0 && !d_x_vals) || (nnz_y > 0 && !d_y_vals)) return SPSYRK_ERR_INVALID_ARG;
     if (m == 0) return SPSYRK_OK;

@@ -16,6 +16,38 @@ using namespace spsyrk;
 namespace spsyrk {
 static std::atomic<long long> g_launches{0};
 void note_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+
+// Allocating pinned memory takes a millisecond or more, so blocks given back are kept for the next user, up to
+// HOST_POOL_MAX of 512 bytes each.  Blocks are portable: any device's kernels may write them.
+static std::mutex g_host_mutex;
+static std::vector<int64_t*> g_host_pool;
+constexpr size_t HOST_POOL_MAX = 64;
+cudaError_t HostBlock::acquire() {
+    {
+        std::lock_guard<std::mutex> lock(g_host_mutex);
+        if (!g_host_pool.empty()) {
+            host = g_host_pool.back();
+            g_host_pool.pop_back();
+        }
+    }
+    if (!host) {
+        const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&host), HOST_WORDS * sizeof(int64_t), cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e != cudaSuccess) { host = nullptr; return e; }
+    }
+    return cudaHostGetDevicePointer(reinterpret_cast<void**>(&dev), host, 0);
+}
+void HostBlock::release() {
+    if (!host) return;
+    {
+        std::lock_guard<std::mutex> lock(g_host_mutex);
+        if (g_host_pool.size() < HOST_POOL_MAX) {
+            g_host_pool.push_back(host);
+            host = nullptr;
+        }
+    }
+    if (host) cudaFreeHost(host);
+    host = dev = nullptr;
+}
 }  // namespace spsyrk
 
 namespace {
@@ -79,7 +111,7 @@ struct spsyrk_plan_s {
     int64_t* ub_off;
     int32_t* cnt_out;
     bool have_onepass;
-    int64_t* host_pos;  // pinned, device-visible host memory the position search of spsyrk_numeric_rows writes into (4 * NCLASS)
+    HostBlock host;  // words 0..31: facts of the two views; 32..63: the position search of spsyrk_numeric_rows (upper view: unused)
     int64_t rows_cap;
     // workspace views
     int32_t* perm;
@@ -98,6 +130,11 @@ struct spsyrk_plan_s {
     int32_t* blockhist;
     int64_t* offsets;
     int64_t* partials;
+    int64_t *state_bin, *state_items;  // status words of the scans of the binning, cleared with the counters
+    uint32_t* items8;                  // rows: map words per row in class order
+    void *zero_all, *zero_bin;         // the counters every plan starts from zero; those every binning does
+    size_t zero_all_bytes, zero_bin_bytes;
+    int64_t* state_col;
     int64_t* class_start_dev;  // NCLASS + 1
     unsigned long long* work_total_dev;
     uint32_t* row_counter;  // row dispenser of the persistent heavy-row kernel
@@ -132,7 +169,7 @@ namespace {
 size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t n, int64_t nnz, size_t sv, bool full) {
     Carver c(ws);
     const int64_t items = std::max<int64_t>(std::max(m, n), 1);
-    const int64_t nb = bin_blocks(items);
+    const int64_t nb = bin_blocks_max(items);
     auto colptr = c.take<int64_t>(n + 1);
     auto desc = c.take<uint2>(nnz);
     auto work = c.take<int64_t>(m);
@@ -140,7 +177,22 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto hdr = c.take<uint4>(m);
     auto cnt = c.take<int32_t>(m);
     auto cls = c.take<uint8_t>(items);
-    auto colcnt = c.take<uint32_t>(n);
+    // counters in one piece, so that one memset clears them: the binning's, then the plan's, then the column counts
+    const int views = full ? 2 : 1;
+    const size_t bin_words = views * (1 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(items));
+    auto zero = c.take<int64_t>(bin_words + 64 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2);
+    Carver cz(zero);
+    auto take_words = [&](size_t words) { int64_t* q = zero ? zero + cz.off : nullptr; cz.off += words; return q; };
+    auto work_total_dev = reinterpret_cast<unsigned long long*>(take_words(1));
+    auto state_bin = take_words(scan_partials_count(NCLASS * nb)), state_items = take_words(scan_partials_count(items));
+    unsigned long long* u_work_total_dev = full ? reinterpret_cast<unsigned long long*>(take_words(1)) : nullptr;
+    int64_t* u_state_bin = full ? take_words(scan_partials_count(NCLASS * nb)) : nullptr;
+    int64_t* u_state_items = full ? take_words(scan_partials_count(items)) : nullptr;
+    auto err = reinterpret_cast<uint32_t*>(take_words(32));
+    auto facts = reinterpret_cast<uint32_t*>(take_words(32));  // [0..1] binary analysis, [32..63] its histogram
+    auto state_col = take_words(scan_partials_count(std::max<int64_t>(n, 1)));
+    auto colcnt = reinterpret_cast<uint32_t*>(take_words((size_t)(n + 1) / 2));
+    const size_t zero_words = cz.off;
     const int64_t rx_hist_n = (int64_t)(1 << TRANSPOSE_RADIX_BITS) * std::max<int64_t>(radix_tiles(nnz), 1);
     // The two buffer sets of the radix sort (key, row, position, value per nonzero) are reused: the set that
     // the last pass does not read receives the column lists that pass writes (row ids and records), and the
@@ -172,14 +224,12 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto offsets = c.take<int64_t>(NCLASS * nb + 1);
     auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(std::max<int64_t>(items + 1, NCLASS * nb), rx_hist_n)));
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
-    auto work_total_dev = c.take<unsigned long long>(1);
-    auto err = c.take<uint32_t>(1);
     auto row_counter = c.take<uint32_t>(1);
     auto work_prefix = c.take<int64_t>(items + 1);
     auto itemoff = c.take<int64_t>(items + 1);
     auto heavy_id = c.take<uint8_t>(std::max<int64_t>(n, 1));
     auto heavy_mask = c.take<uint64_t>(std::max<int64_t>(m, 1));
-    auto facts = c.take<uint32_t>(64);  // [0..2] binary analysis, [32..63] its histogram
+    auto items8 = c.take<uint32_t>(items);
     auto adeg = c.take<int32_t>(std::max<int64_t>(m, 1));
     auto part_bounds = c.take<int64_t>(MAX_PARTS + 1);
     auto ub = c.take<int32_t>(std::max<int64_t>(m, 1));
@@ -190,7 +240,6 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     int32_t *u_perm = nullptr, *u_cnt = nullptr, *cnt_tot = nullptr;
     uint4* u_hdr = nullptr;
     uint8_t* u_cls = nullptr;
-    unsigned long long* u_work_total_dev = nullptr;
     if (full) {
         desc_hi = c.take<uint2>(nnz);
         u_work = c.take<int64_t>(m);
@@ -200,7 +249,6 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         u_cls = c.take<uint8_t>(items);
         u_itemoff = c.take<int64_t>(items + 1);
         u_class_start_dev = c.take<int64_t>(NCLASS + 1);
-        u_work_total_dev = c.take<unsigned long long>(1);
         cnt_tot = c.take<int32_t>(m);
         hi_begin = c.take<int64_t>(items + 1);
         work_sum = c.take<int64_t>(m);
@@ -220,6 +268,10 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         pl->rx_pos_b = rx_pos_b; pl->rx_val_a = rx_val_a; pl->rx_val_b = rx_val_b; pl->rx_hist = rx_hist; pl->rx_offsets = rx_offsets;
         pl->blockhist = blockhist; pl->offsets = offsets; pl->partials = partials;
         pl->class_start_dev = class_start_dev; pl->work_total_dev = work_total_dev;
+        pl->state_bin = state_bin; pl->state_items = state_items; pl->state_col = state_col; pl->items8 = items8;
+        pl->zero_all = zero; pl->zero_all_bytes = zero_words * sizeof(int64_t);
+        pl->zero_bin = zero; pl->zero_bin_bytes = bin_words * sizeof(int64_t);
+        pl->dev.nheavy = facts + 1;
         if (up) {
             // the upper view shares everything that describes A and the scratch space; its rows are its own
             *up = *pl;
@@ -227,26 +279,38 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
             up->dev.desc = desc_hi; up->dev.work = u_work;
             up->perm = u_perm; up->hdr = u_hdr; up->cnt = u_cnt; up->cls = u_cls; up->itemoff = u_itemoff;
             up->class_start_dev = u_class_start_dev; up->work_total_dev = u_work_total_dev;
+            up->state_bin = u_state_bin; up->state_items = u_state_items;
         }
     }
     return (c.off + ALIGN - 1) / ALIGN * ALIGN;
 }
 
-spsyrk_status_t read_err(spsyrk_plan_s* pl, cudaStream_t st) {
-    uint32_t e = 0;
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, pl->dev.err, sizeof(e), cudaMemcpyDeviceToHost, st));
-    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+spsyrk_status_t status_of(uint32_t e) {
     if (e & (ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED)) return SPSYRK_ERR_BAD_CSR;
     if (e) return SPSYRK_ERR_INTERNAL;
     return SPSYRK_OK;
 }
 
+[[maybe_unused]] spsyrk_status_t read_err(spsyrk_plan_s* pl, cudaStream_t st) {
+    uint32_t e = 0;
+    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, pl->dev.err, sizeof(e), cudaMemcpyDeviceToHost, st));
+    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+    return status_of(e);
+}
+
+template <int G, typename V>
+void launch_row_expand_v(spsyrk_plan_s* pl, cudaStream_t st) {
+    const PlanDev& P = pl->dev;
+    const int64_t threads = std::max<int64_t>(P.m, 1) * G;
+    row_expand_kernel<G, V><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(P.rowptr, P.colidx, static_cast<const V*>(P.vals), P.m, P.n, P.nnz,
+                                                                               pl->colcnt, pl->rx_row_b, pl->adeg, pl->facts, P.err);
+    note_launches(1);
+}
 template <int G>
 void launch_row_expand(spsyrk_plan_s* pl, cudaStream_t st) {
-    const PlanDev& P = pl->dev;
-    const int64_t threads = (int64_t)P.m * G;
-    row_expand_kernel<G><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(P.rowptr, P.colidx, P.m, P.n, pl->colcnt, pl->rx_row_b, P.err);
-    note_launches(1);
+    if (pl->dtype == SPSYRK_F64) launch_row_expand_v<G, double>(pl, st);
+    else if (pl->dtype == SPSYRK_F32) launch_row_expand_v<G, float>(pl, st);
+    else launch_row_expand_v<G, int32_t>(pl, st);
 }
 
 template <int G>
@@ -259,10 +323,9 @@ void launch_block_desc(spsyrk_plan_s* pl, cudaStream_t st) {
 
 template <int G>
 void launch_row_work(spsyrk_plan_s* pl, cudaStream_t st) {
-    const PlanDev& P = pl->dev;
-    const int64_t threads = (int64_t)(P.r1 - P.r0) * G;
-    const int64_t ctas = std::min<int64_t>((threads + 255) / 256, (int64_t)pl->sm_count * 16);
-    row_work_kernel<G><<<(unsigned)ctas, 256, 0, st>>>(P, pl->cls, BLOCK_CLASS_MAX_WORK, pl->diag, pl->work_total_dev);
+    const int64_t rows = pl->dev.r1 - pl->dev.r0, nb = bin_blocks(rows);
+    row_work_kernel<G><<<(unsigned)nb, BIN_THREADS, 0, st>>>(pl->dev, pl->cls, BLOCK_CLASS_MAX_WORK, pl->diag, bin_tile(rows), pl->blockhist, nb,
+                                                             pl->work_total_dev);
     note_launches(1);
 }
 
@@ -311,95 +374,95 @@ __global__ void add_work_kernel(const int64_t* __restrict__ a, const int64_t* __
     if (r < rows) out[r] = a[r] + b[r];
 }
 
-// work estimate + binning of one view's current row range (dev.desc, dev.mode and diag are set); reads class sizes back (one sync)
-spsyrk_status_t bin_view(spsyrk_plan_s* pl, cudaStream_t st) {
-    const int64_t rows = pl->dev.r1 - pl->dev.r0;
+__global__ void plan_facts_kernel(PlanFacts f) { f.publish(0); }
+
+// Work estimate + binning of one view's current row range (dev.desc, dev.mode and diag are set).  The facts the host
+// needs are on their way to `host` when this returns.
+spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, cudaStream_t st) {
+    const int64_t rows = pl->dev.r1 - pl->dev.r0, nb = bin_blocks(rows);
     pl->have_symbolic = false;
     pl->have_onepass = false;
-    const PlanDev& P = pl->dev;
-    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->work_total_dev, 0, sizeof(unsigned long long), st));
-    if (rows > 0) {
-        switch (group_width(P.nnz, P.m)) {
-            case 4: launch_row_work<4>(pl, st); break;
-            case 8: launch_row_work<8>(pl, st); break;
-            case 16: launch_row_work<16>(pl, st); break;
-            default: launch_row_work<32>(pl, st); break;
-        }
-    }
-    SPSYRK_CUDA_TRY(bin_items(pl->cls, rows, pl->perm, pl->class_start_dev, pl->blockhist, pl->offsets, pl->partials, P.err, st));
-    if (rows > 0) {
-        row_header_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(P, pl->perm, rows, pl->hdr);
-        note_launches(1);
-    }
-    // where the item-map words of every light row start (rows in class order)
-    int64_t map_items = 0;
     pl->map_filled = false;
-    if (rows > 0) {
-        uint32_t* items8 = reinterpret_cast<uint32_t*>(pl->cnt);  // free until the symbolic pass
-        row_items_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(P, pl->hdr, pl->cls, rows, pl->diag, items8);
+    const PlanDev& P = pl->dev;
+    const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->facts, P.err, host};
+    if (rows == 0) {
+        SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->class_start_dev, 0, (NCLASS + 1) * sizeof(int64_t), st));
+        plan_facts_kernel<<<1, 1, 0, st>>>(facts);
         note_launches(1);
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(items8, rows, pl->itemoff, pl->partials, P.err, st));
-        SPSYRK_CUDA_TRY(cudaMemcpyAsync(&map_items, pl->itemoff + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        SPSYRK_CUDA_TRY(cudaGetLastError());
+        return SPSYRK_OK;
     }
-    unsigned long long wt = 0;
-    uint32_t facts[3] = {1u, 0u, 0u};
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(facts, pl->facts, sizeof(facts), cudaMemcpyDeviceToHost, st));
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(pl->class_start, pl->class_start_dev, sizeof(pl->class_start), cudaMemcpyDeviceToHost, st));
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&wt, pl->work_total_dev, sizeof(wt), cudaMemcpyDeviceToHost, st));
-    spsyrk_status_t s = read_err(pl, st);
-    pl->work_total = (int64_t)wt;
-    pl->map_items = map_items;
-    pl->dev.binary = (pl->dev.nnz > 0 && facts[0] == 0) ? 1 : 0;
-    pl->dev.nheavy = pl->dev.binary ? (int32_t)std::min<uint32_t>(facts[1], 64u) : 0;
-    return s;
+    switch (group_width(P.nnz, P.m)) {
+        case 4: launch_row_work<4>(pl, st); break;
+        case 8: launch_row_work<8>(pl, st); break;
+        case 16: launch_row_work<16>(pl, st); break;
+        default: launch_row_work<32>(pl, st); break;
+    }
+    SPSYRK_CUDA_TRY(scan_launch(ScanArray<int32_t>{pl->blockhist}, NCLASS * nb, BinStarts{pl->offsets, (uint32_t)nb, pl->class_start_dev}, pl->state_bin, P.err, st, true));
+    row_scatter_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(P, pl->cls, bin_tile(rows), pl->offsets, nb, pl->diag, pl->perm, pl->hdr, pl->items8, pl->cnt);
+    note_launches(1);
+    SPSYRK_CUDA_TRY(scan_launch(ScanArray<uint32_t>{pl->items8}, rows, ItemStarts{pl->itemoff, rows, facts}, pl->state_items, P.err, st, true));
+    return SPSYRK_OK;
 }
 
-// descriptors, work estimate and binning of the plan's current block of output rows and columns
-spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, cudaStream_t st) {
+// after the synchronisation
+spsyrk_status_t bin_collect(spsyrk_plan_s* pl, const int64_t* host) {
+    std::memcpy(pl->class_start, host + PF_CLASS_START, sizeof(pl->class_start));
+    pl->map_items = host[PF_MAP_ITEMS];
+    pl->work_total = host[PF_WORK];
+    pl->dev.binary = (pl->dev.nnz > 0 && host[PF_OTHER_THAN_ONE] == 0) ? 1 : 0;
+    return status_of((uint32_t)host[PF_ERR]);
+}
+
+// Descriptors, work estimate and binning of the plan's current block of output rows and columns; synchronises once.
+// fresh: the counters of the binning are zero already.
+spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st) {
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     const bool whole = pl->s0 <= 0 && pl->s1 >= pl->dev.m;
     pl->upper_active = false;
+    if (!fresh) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->zero_bin, 0, pl->zero_bin_bytes, st));
     if (whole) {
         pl->dev.desc = pl->desc_full;
-        if (pl->user_mode == SPSYRK_FULL && pl->upper) {
-            // two parts per row: this view does the lower parts like the lower-triangle mode, the upper view the rest
-            pl->upper_active = true;
-            pl->dev.mode = SPSYRK_TRIL;
-            pl->diag = true;
-            spsyrk_status_t s = bin_view(pl, st);
-            if (s != SPSYRK_OK) return s;
-            spsyrk_plan_s* up = pl->upper;
-            up->dev.r0 = pl->dev.r0; up->dev.r1 = pl->dev.r1;
-            up->dev.mode = SPSYRK_FULL;  // the upper part of row i lies in (i, m): the kernels work on the range [0, m)
-            up->dev.desc = pl->desc_hi;
-            up->dev.jaccard = pl->dev.jaccard;
-            up->diag = false;
-            s = bin_view(up, st);
-            if (s != SPSYRK_OK) return s;
-            if (rows > 0) {
-                add_work_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev.work, up->dev.work, rows, pl->work_sum);
-                note_launches(1);
-            }
-            return SPSYRK_OK;
-        }
+        // two parts per row in full-output mode: this view does the lower parts like the lower-triangle mode
+        pl->upper_active = pl->user_mode == SPSYRK_FULL && pl->upper;
+        pl->dev.mode = pl->upper_active ? SPSYRK_TRIL : (int32_t)pl->user_mode;
+        pl->diag = pl->dev.mode == SPSYRK_TRIL;
+    } else {
+        // a column range: descriptors narrowed to [s0, s1) (cut out of the whole column lists in full-output mode)
+        pl->dev.desc = pl->desc_blk;
         pl->dev.mode = (int32_t)pl->user_mode;
-        pl->diag = pl->user_mode == SPSYRK_TRIL;
-        return bin_view(pl, st);
-    }
-    // a column range: descriptors narrowed to [s0, s1) (cut out of the whole column lists in full-output mode)
-    pl->dev.desc = pl->desc_blk;
-    pl->dev.mode = (int32_t)pl->user_mode;
-    pl->diag = false;
-    if (rows > 0 && pl->dev.nnz > 0) {
-        switch (group_width(pl->dev.nnz, pl->dev.m)) {
-            case 4: launch_block_desc<4>(pl, st); break;
-            case 8: launch_block_desc<8>(pl, st); break;
-            case 16: launch_block_desc<16>(pl, st); break;
-            default: launch_block_desc<32>(pl, st); break;
+        pl->diag = false;
+        if (rows > 0 && pl->dev.nnz > 0) {
+            switch (group_width(pl->dev.nnz, pl->dev.m)) {
+                case 4: launch_block_desc<4>(pl, st); break;
+                case 8: launch_block_desc<8>(pl, st); break;
+                case 16: launch_block_desc<16>(pl, st); break;
+                default: launch_block_desc<32>(pl, st); break;
+            }
         }
     }
-    return bin_view(pl, st);
+    spsyrk_status_t s = bin_launch(pl, pl->host.dev, st);
+    if (s != SPSYRK_OK) return s;
+    spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
+    if (up) {
+        up->dev.r0 = pl->dev.r0; up->dev.r1 = pl->dev.r1;
+        up->dev.mode = SPSYRK_FULL;  // the upper part of row i lies in (i, m): the kernels work on the range [0, m)
+        up->dev.desc = pl->desc_hi;
+        up->dev.jaccard = pl->dev.jaccard;
+        up->diag = false;
+        s = bin_launch(up, pl->host.dev + 16, st);
+        if (s != SPSYRK_OK) return s;
+        if (rows > 0) {
+            add_work_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev.work, up->dev.work, rows, pl->work_sum);
+            note_launches(1);
+        }
+    }
+    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+    s = bin_collect(pl, pl->host.host);
+    if (s == SPSYRK_OK && up) s = bin_collect(up, pl->host.host + 16);
+    return s;
 }
+static_assert(PF_WORDS <= 16, "a view's facts take sixteen words of the host block");
 
 int64_t map_items_total(const spsyrk_plan_s* pl) { return pl->map_items + (pl->upper_active ? pl->upper->map_items : 0); }
 
@@ -650,10 +713,22 @@ __global__ void upper_begin_kernel(const int64_t* __restrict__ c_rowptr, const i
     if (r < rows) hi_begin[r] = c_rowptr[r] + cnt_lo[r];
 }
 
+// prefix sums of per-row counts into out[rows + 1]; the total and the error word are on their way to the host
+cudaError_t scan_counts(spsyrk_plan_s* pl, const int32_t* counts, int64_t rows, int64_t* out, cudaStream_t st) {
+    if (rows == 0) return cudaMemsetAsync(out, 0, sizeof(int64_t), st);
+    return scan_launch(ScanArray<int32_t>{counts}, rows, ScanIntoHost{out, rows, pl->dev.err, pl->host.dev}, pl->partials, pl->dev.err, st);
+}
+// waits for them
+spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, int64_t* total, cudaStream_t st) {
+    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+    if (rows == 0) { *total = 0; return SPSYRK_OK; }
+    const spsyrk_status_t s = status_of((uint32_t)pl->host.host[1]);
+    if (s == SPSYRK_OK) *total = pl->host.host[0];
+    return s;
+}
+
 // the per-class count kernels of one view (entries per row into its cnt array)
 spsyrk_status_t symbolic_view(spsyrk_plan_s* pl, bool with_map, cudaStream_t st) {
-    const int64_t rows = pl->dev.r1 - pl->dev.r0;
-    if (rows > 0) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->cnt, 0, (size_t)rows * sizeof(int32_t), st));
     pl->map_filled = false;
     mark(pl, pl->ev_sym, 1, st);
     if (with_map) launch_symbolic_sort<32>(pl, 1, st); else launch_symbolic_warp<32>(pl, 1, st);
@@ -780,62 +855,39 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
     carve(pl, up, d_workspace, m, n, nnz, sv, full);
     pl->upper = up;  // (the copy into the upper view happened with a null link)
 
-    auto fail = [&](spsyrk_status_t s) { delete up; delete pl; return s; };
+    auto fail = [&](spsyrk_status_t s) { pl->host.release(); delete up; delete pl; return s; };
 #define PLAN_TRY(expr) do { if ((expr) != cudaSuccess) return fail(SPSYRK_ERR_CUDA); } while (0)
-    PLAN_TRY(cudaMemsetAsync(P.err, 0, sizeof(uint32_t), st));
-    if (n > 0) PLAN_TRY(cudaMemsetAsync(pl->colcnt, 0, (size_t)n * sizeof(uint32_t), st));
-    // 1. row pointers must be sane before anything indexes with them
-    validate_rowptr_kernel<<<(unsigned)((m + 1 + 255) / 256), 256, 0, st>>>(d_rowptr, m, nnz, P.err);
-    note_launches(1);
-    PLAN_TRY(cudaGetLastError());
-    spsyrk_status_t s = read_err(pl, st);
-    if (s != SPSYRK_OK) return fail(s);
-    // 2. transpose: one sweep over A for the column histogram, the explicit row ids and the checks of the column
-    // ids; the histogram's scan gives colptr; stable radix sort by column
-    if (nnz > 0) {
-        switch (group_width(nnz, m)) {
-            case 4: launch_row_expand<4>(pl, st); break;
-            case 8: launch_row_expand<8>(pl, st); break;
-            case 16: launch_row_expand<16>(pl, st); break;
-            default: launch_row_expand<32>(pl, st); break;
-        }
+    PLAN_TRY(pl->host.acquire());
+    PLAN_TRY(cudaMemsetAsync(pl->zero_all, 0, pl->zero_all_bytes, st));
+    // 1. one sweep over A (checks, column histogram, row ids, row lengths, values all one?); 2. transpose: the histogram's
+    // scan gives colptr; stable radix sort by column; 3. work estimate and row binning.  One synchronisation at the end.
+    const int g = group_width(nnz, m);
+    switch (g) {
+        case 4: launch_row_expand<4>(pl, st); break;
+        case 8: launch_row_expand<8>(pl, st); break;
+        case 16: launch_row_expand<16>(pl, st); break;
+        default: launch_row_expand<32>(pl, st); break;
     }
-    PLAN_TRY(exclusive_scan_i64<uint32_t>(pl->colcnt, n, P.colptr, pl->partials, P.err, st));
-    s = read_err(pl, st);  // synchronises; column ids are known to be in range and rows sorted from here on
+    PLAN_TRY(exclusive_scan_i64<uint32_t>(pl->colcnt, n, P.colptr, pl->state_col, P.err, st, true));
+    spsyrk_status_t s = sv == 8 ? sort_by_column<uint64_t>(pl, st) : sort_by_column<uint32_t>(pl, st);
     if (s != SPSYRK_OK) return fail(s);
-    s = sv == 8 ? sort_by_column<uint64_t>(pl, st) : sort_by_column<uint32_t>(pl, st);
+    s = estimate_and_bin(pl, true, st);
     if (s != SPSYRK_OK) return fail(s);
-    // 3. binary input: value check, heavy columns as bit masks per row
-    P.binary = 0; P.nheavy = 0; P.jaccard = nullptr;
-    PLAN_TRY(cudaMemsetAsync(pl->facts, 0, 64 * sizeof(uint32_t), st));
-    if (m > 0) {
-        row_degree_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(d_rowptr, P.m, pl->adeg);
-        note_launches(1);
-    }
-    if (nnz > 0) {
-        const unsigned cb = (unsigned)std::min<int64_t>((nnz + 255) / 256, (int64_t)pl->sm_count * 16);
-        switch (dtype) {
-            case SPSYRK_F64: binary_check_kernel<double><<<cb, 256, 0, st>>>(static_cast<const double*>(d_vals), nnz, pl->facts); break;
-            case SPSYRK_F32: binary_check_kernel<float><<<cb, 256, 0, st>>>(static_cast<const float*>(d_vals), nnz, pl->facts); break;
-            default: binary_check_kernel<int32_t><<<cb, 256, 0, st>>>(static_cast<const int32_t*>(d_vals), nnz, pl->facts); break;
-        }
+    // 4. binary input: heavy columns as bit masks per row
+    if (P.binary) {
         const unsigned hb = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)pl->sm_count * 16);
         heavy_hist_kernel<<<hb, 256, 0, st>>>(pl->colcnt, n, pl->facts + 32);
-        heavy_threshold_kernel<<<1, 32, 0, st>>>(pl->facts + 32, pl->facts);
-        heavy_assign_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pl->colcnt, n, pl->facts, pl->heavy_id);
+        heavy_assign_kernel<<<hb, 256, 0, st>>>(pl->colcnt, n, pl->facts, pl->heavy_id);
         const unsigned mb = (unsigned)std::min<int64_t>((m * 32 + 255) / 256, (int64_t)pl->sm_count * 8);
-        switch (group_width(nnz, m)) {
+        switch (g) {
             case 4: heavy_mask_kernel<4><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
             case 8: heavy_mask_kernel<8><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
             case 16: heavy_mask_kernel<16><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
             default: heavy_mask_kernel<32><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
         }
-        note_launches(5);
+        note_launches(3);
         PLAN_TRY(cudaGetLastError());
     }
-    // 4. work estimate and row binning (its read-back also brings the facts above)
-    s = estimate_and_bin(pl, st);
-    if (s != SPSYRK_OK) return fail(s);
 #undef PLAN_TRY
     *plan = pl;
     return SPSYRK_OK;
@@ -850,7 +902,7 @@ spsyrk_status_t spsyrk_plan_set_block(spsyrk_plan_t plan, int64_t row_begin, int
     plan->s0 = (int32_t)col_begin;
     plan->s1 = (int32_t)col_end;
     plan->have_symbolic = false;
-    return estimate_and_bin(plan, static_cast<cudaStream_t>(cuda_stream));
+    return estimate_and_bin(plan, false, static_cast<cudaStream_t>(cuda_stream));
 }
 
 spsyrk_status_t spsyrk_plan_set_rows(spsyrk_plan_t plan, int64_t row_begin, int64_t row_end, void* cuda_stream) {
@@ -895,17 +947,14 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t
         }
         counts = pl->cnt_tot;
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(counts, rows, d_c_rowptr, pl->partials, pl->dev.err, st));
+    SPSYRK_CUDA_TRY(scan_counts(pl, counts, rows, d_c_rowptr, st));
     if (pl->upper_active && rows > 0) {
         // the upper part of row r starts after its lower part
         upper_begin_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(d_c_rowptr, pl->cnt, rows, pl->hi_begin);
         note_launches(1);
     }
-    int64_t nnz = 0;
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&nnz, d_c_rowptr + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    s = read_err(pl, st);
+    s = collect_total(pl, rows, nnz_out, st);
     if (s != SPSYRK_OK) return s;
-    *nnz_out = nnz;
     pl->have_symbolic = true;
     pl->map_filled = with_map;
     if (pl->upper_active) { pl->upper->have_symbolic = true; pl->upper->map_filled = with_map; }
@@ -939,26 +988,6 @@ spsyrk_status_t spsyrk_numeric(spsyrk_plan_t plan, const int64_t* d_c_rowptr, in
 }
 
 namespace {
-// Pinned host blocks for the read-back of spsyrk_numeric_rows.  Allocating pinned memory takes a millisecond or
-// more, so blocks of destroyed plans are kept for the next plan (a few hundred bytes each, never freed).
-std::mutex g_host_pos_mutex;
-std::vector<int64_t*> g_host_pos_pool;
-cudaError_t host_pos_acquire(int64_t** out) {
-    {
-        std::lock_guard<std::mutex> lock(g_host_pos_mutex);
-        if (!g_host_pos_pool.empty()) {
-            *out = g_host_pos_pool.back();
-            g_host_pos_pool.pop_back();
-            return cudaSuccess;
-        }
-    }
-    return cudaHostAlloc(reinterpret_cast<void**>(out), 4 * NCLASS * sizeof(int64_t), cudaHostAllocMapped | cudaHostAllocPortable);
-}
-void host_pos_release(int64_t* p) {
-    std::lock_guard<std::mutex> lock(g_host_pos_mutex);
-    g_host_pos_pool.push_back(p);
-}
-
 // out[(2 * c) + e] = first position of class c's row list (ascending local row ids) whose row is >= bound[e]
 __global__ void class_positions_kernel(const int32_t* __restrict__ perm, const int64_t* __restrict__ class_start_dev, int64_t lo_row,
                                        int64_t hi_row, int64_t* __restrict__ out) {
@@ -986,9 +1015,7 @@ spsyrk_status_t spsyrk_numeric_rows(spsyrk_plan_t plan, int64_t row_begin, int64
     // where the rows of the range sit in every class's list: one small kernel per view and one read-back
     // The kernel writes straight into pinned host memory: a device-to-host copy would queue behind whatever the
     // caller is downloading at the moment (the point of this call is to overlap with such copies).
-    if (!pl->host_pos) SPSYRK_CUDA_TRY(host_pos_acquire(&pl->host_pos));
-    int64_t* dev_pos = nullptr;
-    SPSYRK_CUDA_TRY(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dev_pos), pl->host_pos, 0));
+    int64_t* const dev_pos = pl->host.dev + 32;
     spsyrk_plan_s* views[2] = {pl, pl->upper_active ? pl->upper : nullptr};
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
@@ -998,7 +1025,7 @@ spsyrk_status_t spsyrk_numeric_rows(spsyrk_plan_t plan, int64_t row_begin, int64
     }
     SPSYRK_CUDA_TRY(cudaGetLastError());
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    const int64_t(*pos)[2 * NCLASS] = reinterpret_cast<const int64_t(*)[2 * NCLASS]>(pl->host_pos);
+    const int64_t(*pos)[2 * NCLASS] = reinterpret_cast<const int64_t(*)[2 * NCLASS]>(pl->host.host + 32);
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
         views[v]->sub_active = true;
@@ -1017,7 +1044,6 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     pl->have_onepass = false;
-    if (rows > 0) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->cnt, 0, (size_t)rows * sizeof(int32_t), st));
     // heavy rows: their counts come from their own kernels (bitmaps), as in the symbolic pass
     spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, st);
     if (s != SPSYRK_OK) return s;
@@ -1027,12 +1053,9 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
         onepass_slots_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev, pl->cls, pl->cnt, pl->diag, rows, pl->ub);
         note_launches(1);
     }
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(pl->ub, rows, pl->ub_off, pl->partials, pl->dev.err, st));
-    int64_t total = 0;
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&total, pl->ub_off + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    s = read_err(pl, st);
+    SPSYRK_CUDA_TRY(scan_counts(pl, pl->ub, rows, pl->ub_off, st));
+    s = collect_total(pl, rows, slot_entries, st);
     if (s != SPSYRK_OK) return s;
-    *slot_entries = total;
     pl->have_onepass = true;
     return SPSYRK_OK;
 }
@@ -1061,13 +1084,8 @@ spsyrk_status_t spsyrk_onepass_numeric(spsyrk_plan_t plan, int32_t* d_slot_colid
     pl->cnt_out = nullptr;
     pl->map_filled = map_was;
     if (s != SPSYRK_OK) return s;
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<int32_t>(pl->cnt, rows, d_c_rowptr, pl->partials, pl->dev.err, st));
-    int64_t nnz = 0;
-    SPSYRK_CUDA_TRY(cudaMemcpyAsync(&nnz, d_c_rowptr + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    s = read_err(pl, st);
-    if (s != SPSYRK_OK) return s;
-    *nnz_out = nnz;
-    return SPSYRK_OK;
+    SPSYRK_CUDA_TRY(scan_counts(pl, pl->cnt, rows, d_c_rowptr, st));
+    return collect_total(pl, rows, nnz_out, st);
 }
 
 spsyrk_status_t spsyrk_onepass_row_begin(spsyrk_plan_t plan, int64_t* d_row_begin, void* cuda_stream) {
@@ -1141,7 +1159,7 @@ void spsyrk_destroy(spsyrk_plan_t plan) {
     if (!plan) return;
     if (plan->timing)
         for (int i = 0; i <= NCLASS; ++i) { cudaEventDestroy(plan->ev_sym[i]); cudaEventDestroy(plan->ev_num[i]); }
-    if (plan->host_pos) host_pos_release(plan->host_pos);
+    plan->host.release();
     delete plan->upper;
     delete plan;
 }

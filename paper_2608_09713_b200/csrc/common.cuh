@@ -35,6 +35,20 @@ constexpr int NCLASS = 8;  // row / column classes produced by the binning pass
 // kernel-launch bookkeeping behind spsyrk_launch_count (defined in api.cu)
 void note_launches(int n);
 
+// Pinned host memory that kernels write the facts the host waits for into (class sizes, entry counts, the error word):
+// one synchronisation and no copy, where a copy into ordinary memory took 3 us of device time and as much again
+// on the host, up to five in a row.  Blocks of HOST_WORDS words come from a pool (defined in api.cu).
+constexpr int HOST_WORDS = 64;
+struct HostBlock {
+    int64_t* host = nullptr;
+    int64_t* dev = nullptr;  // the same memory as kernels see it
+    cudaError_t acquire();
+    void release();
+};
+struct ScopedHostBlock : HostBlock {
+    ~ScopedHostBlock() { release(); }
+};
+
 #define SPSYRK_CUDA_TRY(expr)                                  \
     do {                                                       \
         cudaError_t _e = (expr);                               \
@@ -177,17 +191,18 @@ __device__ __forceinline__ uint32_t lower_bound_i32(const int32_t* __restrict__ 
 // A CTA takes its tile's number from a counter, so a tile only ever waits for tiles that running CTAs
 // hold; it publishes its own sum, adds up what the tiles before it have published and publishes its
 // inclusive prefix.  A status word is value << 2 | kind, so value and kind arrive together.
-// `state` needs scan_partials_count(n) 64-bit words; one tile (n <= SCAN_TILE) uses none of them.
+// `state` needs scan_partials_count(n) 64-bit words; a single tile uses none of them.
 // (Three launches - tile sums, their scan, the tiles again - before: 2.5 us of device time and as much
 // host time each, ten scans per product and mirror, and the input read twice.)
 // ---------------------------------------------------------------------------------------
 constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_ITEMS = 8;
-constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+constexpr int scan_items(size_t value_bytes) { return value_bytes == 8 ? 8 : 16; }
+constexpr int SCAN_MIN_TILE = SCAN_THREADS * 8;
 constexpr unsigned long long SCAN_PARTIAL = 1, SCAN_PREFIX = 2;  // kinds of a status word (0: nothing yet)
+constexpr int SCAN_WINDOW = 256;
 constexpr int SPIN_LIMIT = 1 << 24;  // polls before a wait gives up with ERRW_INTERNAL
 
-inline int64_t scan_partials_count(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
+inline int64_t scan_partials_count(int64_t n) { return (n + SCAN_MIN_TILE - 1) / SCAN_MIN_TILE + 1; }
 
 __device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
     unsigned long long v;
@@ -206,31 +221,49 @@ __device__ __forceinline__ int64_t scan_look_back(unsigned long long* state, int
         return 0;
     }
     if (lane == 0) st_status(state + tile, ((unsigned long long)sum << 2) | SCAN_PARTIAL);
+    // SCAN_WINDOW tiles per step: when all tiles in flight start together the first of them is a thousand tiles away, and
+    // every step is a round trip to L2 (34 million counters: 0.4 ms with 32 tiles per step).
     int64_t before = 0;
-    for (int64_t last = tile - 1;; last -= 32) {  // lane l looks at tile last - l
-        const int64_t t = last - lane;
-        unsigned long long v = t >= 0 ? ld_status(state + t) : SCAN_PREFIX;
-        for (int polls = 0; __any_sync(FULL_MASK, (v & 3u) == 0); ++polls) {
-            if (polls == SPIN_LIMIT) {  // the host sees ERRW_INTERNAL; the prefix is wrong but harmless up to then
-                if (lane == 0 && err) atomicOr(err, ERRW_INTERNAL);
-                v |= SCAN_PREFIX;
-                break;
-            }
-            if ((v & 3u) == 0) v = ld_status(state + t);
+    for (int64_t last = tile - 1;; last -= SCAN_WINDOW) {  // lane l looks at tiles last - l, last - 32 - l, ...
+        unsigned long long v[SCAN_WINDOW / 32];
+#pragma unroll
+        for (int k = 0; k < SCAN_WINDOW / 32; ++k) {
+            const int64_t t = last - 32 * k - lane;
+            v[k] = t >= 0 ? ld_status(state + t) : SCAN_PREFIX;
         }
-        const unsigned full = __ballot_sync(FULL_MASK, (v & 3u) == SCAN_PREFIX);
-        const int stop = full ? __ffs(full) - 1 : 31;  // the nearest tile whose inclusive prefix is known ends the walk
-        before += warp_reduce_sum<int64_t>(lane <= stop ? (int64_t)(v >> 2) : 0);
-        if (full) break;
+        bool done = false;
+#pragma unroll
+        for (int k = 0; k < SCAN_WINDOW / 32; ++k) {
+            if (done) continue;  // (the same for all lanes)
+            const int64_t t = last - 32 * k - lane;
+            for (int polls = 0; __any_sync(FULL_MASK, (v[k] & 3u) == 0); ++polls) {
+                if (polls == SPIN_LIMIT) {  // the host sees ERRW_INTERNAL; the prefix is too small, so nothing is indexed out of range
+                    if (lane == 0 && err) atomicOr(err, ERRW_INTERNAL);
+                    v[k] |= SCAN_PREFIX;
+                    break;
+                }
+                if ((v[k] & 3u) == 0) v[k] = ld_status(state + t);
+            }
+            const unsigned full = __ballot_sync(FULL_MASK, (v[k] & 3u) == SCAN_PREFIX);
+            const int stop = full ? __ffs(full) - 1 : 31;  // the nearest tile whose inclusive prefix is known ends the walk
+            before += warp_reduce_sum<int64_t>(lane <= stop ? (int64_t)(v[k] >> 2) : 0);
+            done = full != 0;
+        }
+        if (done) break;
     }
     if (lane == 0) st_status(state + tile, ((unsigned long long)(before + sum) << 2) | SCAN_PREFIX);
     return before;
 }
 
+// In::Value is what an element is held as.  The tile's sum is published before the prefixes inside the tile are computed, and
+// those are computed as they are stored: 40 registers, six CTAs per SM (with 64-bit prefixes in registers two CTAs:
+// 0.46 ms for 34 million counters, 0.9 ms more for the large Erdos-Renyi product and mirror).
 template <typename In, typename Out>
-static __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(In in, int64_t n, Out out, unsigned long long* __restrict__ state,
-                                                                   int64_t ntiles, uint32_t* __restrict__ err) {
-    __shared__ int64_t scratch[33];
+static __global__ void __launch_bounds__(SCAN_THREADS, 6) scan_kernel(In in, int64_t n, Out out, unsigned long long* __restrict__ state,
+                                                                      int64_t ntiles, uint32_t* __restrict__ err) {
+    using Value = typename In::Value;
+    constexpr int ITEMS = scan_items(sizeof(Value));
+    __shared__ int64_t s_warp[SCAN_THREADS / 32];
     __shared__ int64_t s_before;
     __shared__ uint32_t s_tile;
     int64_t tile = 0;
@@ -239,38 +272,49 @@ static __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(In in, int64_
         __syncthreads();
         tile = s_tile;
     }
-    const int64_t base = tile * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    int64_t v[SCAN_ITEMS], s = 0;
+    // a warp owns consecutive elements, 32 per step: loads and stores are whole lines
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int64_t base = tile * (SCAN_THREADS * ITEMS) + warp * (32 * ITEMS) + lane;
+    const int left = (int)min(max(n - base, (int64_t)0), (int64_t)(32 * ITEMS));
+    Value v[ITEMS];
 #pragma unroll
-    for (int it = 0; it < SCAN_ITEMS; ++it) {
-        const int64_t idx = base + it;
-        v[it] = idx < n ? (int64_t)in(idx) : 0;
-        s += v[it];
+    for (int it = 0; it < ITEMS; ++it) v[it] = it * 32 < left ? in(base + it * 32) : Value(0);
+    int64_t s = 0;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) s += (int64_t)v[it];
+    s = warp_reduce_sum<int64_t>(s);
+    if (lane == 0) s_warp[warp] = s;
+    __syncthreads();
+    int64_t run = 0, tot = 0;
+#pragma unroll
+    for (int w = 0; w < SCAN_THREADS / 32; ++w) {
+        if (w < warp) run += s_warp[w];
+        tot += s_warp[w];
     }
-    int64_t tot;
-    int64_t ex = block_exclusive_scan<int64_t, SCAN_THREADS>(s, scratch, &tot);
     if (ntiles > 1) {
-        if (threadIdx.x < 32) {
-            const int64_t before = scan_look_back(state, tile, tot, err);
-            if (threadIdx.x == 0) s_before = before;
+        if (warp == 0) {
+            const int64_t b = scan_look_back(state, tile, tot, err);
+            if (lane == 0) s_before = b;
         }
         __syncthreads();
-        ex += s_before;
+        run += s_before;
+        tot += s_before;
     }
+    if (tile == ntiles - 1 && threadIdx.x == 0) out.total(tot);
 #pragma unroll
-    for (int it = 0; it < SCAN_ITEMS; ++it) {
-        const int64_t idx = base + it;
-        if (idx < n) out(idx, ex);
-        ex += v[it];
-        if (idx == n - 1) out.total(ex);
+    for (int it = 0; it < ITEMS; ++it) {
+        const int64_t incl = warp_inclusive_scan<int64_t>((int64_t)v[it]);
+        if (it * 32 < left) out(base + it * 32, run + incl - (int64_t)v[it]);
+        run += __shfl_sync(FULL_MASK, incl, 31);
     }
 }
 
 // reads an array; stores the prefixes and, behind the last one, the total
 template <typename T>
 struct ScanArray {
+    using Value = T;
     const T* p;
-    __device__ __forceinline__ int64_t operator()(int64_t i) const { return (int64_t)p[i]; }
+    __device__ __forceinline__ T operator()(int64_t i) const { return p[i]; }
 };
 struct ScanInto {
     int64_t* out;
@@ -279,10 +323,26 @@ struct ScanInto {
     __device__ __forceinline__ void total(int64_t t) const { out[n] = t; }
 };
 
+// the same, and the total and the error word go to the host (words 0 and 1)
+struct ScanIntoHost {
+    int64_t* out;
+    int64_t n;
+    const uint32_t* err;
+    int64_t* host;
+    __device__ __forceinline__ void operator()(int64_t i, int64_t ex) const { out[i] = ex; }
+    __device__ __forceinline__ void total(int64_t t) const {
+        const int64_t e = (int64_t)*err;
+        out[n] = t;
+        host[0] = t;
+        host[1] = e;
+    }
+};
+
 // n >= 1.  The status words are cleared here unless the caller has done so (`cleared`).
 template <typename In, typename Out>
 inline cudaError_t scan_launch(In in, int64_t n, Out out, int64_t* partials, uint32_t* err, cudaStream_t st, bool cleared = false) {
-    const int64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+    constexpr int64_t tile = SCAN_THREADS * scan_items(sizeof(typename In::Value));
+    const int64_t ntiles = (n + tile - 1) / tile;
     if (ntiles > 1 && !cleared) {
         const cudaError_t e = cudaMemsetAsync(partials, 0, (size_t)(ntiles + 1) * sizeof(int64_t), st);
         if (e != cudaSuccess) return e;
@@ -300,86 +360,16 @@ inline cudaError_t exclusive_scan_i64(const InT* in, int64_t n, int64_t* out, in
     return scan_launch(ScanArray<InT>{in}, n, ScanInto{out, n}, partials, err, st, cleared);
 }
 
-// ---------------------------------------------------------------------------------------
-// Stable binning of items 0..n-1 into NCLASS classes (a counting sort on the class id):
-// perm lists the items of class 0, then class 1, ..., each in ascending item order;
-// class_start[c] (c = 0..NCLASS) are the offsets.  cls[i] is a byte per item.
-//   blockhist : NCLASS * nblocks int32      offsets : NCLASS * nblocks + 1 int64
-// ---------------------------------------------------------------------------------------
+// Rows per CTA of the binning kernels: about four CTAs per SM for small inputs, at most BIN_MAX_TILE rows.
 constexpr int BIN_THREADS = 256;
-constexpr int BIN_ROUNDS = 8;
-constexpr int BIN_TILE = BIN_THREADS * BIN_ROUNDS;
-
-inline int64_t bin_blocks(int64_t n) { return n > 0 ? (n + BIN_TILE - 1) / BIN_TILE : 1; }
-
-static __global__ void __launch_bounds__(BIN_THREADS) bin_count_kernel(const uint8_t* __restrict__ cls, int64_t n,
-                                                                 int32_t* __restrict__ blockhist, int64_t nblocks) {
-    __shared__ int32_t hist[NCLASS];
-    if (threadIdx.x < NCLASS) hist[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * BIN_TILE;
-#pragma unroll
-    for (int r = 0; r < BIN_ROUNDS; ++r) {
-        int64_t idx = base + r * BIN_THREADS + threadIdx.x;
-        if (idx < n) atomicAdd(&hist[cls[idx]], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x < NCLASS) blockhist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = hist[threadIdx.x];
+constexpr int BIN_MAX_TILE = 2048;
+constexpr int BIN_FEW_BLOCKS = 148 * 4;
+inline int64_t bin_tile(int64_t n) {
+    const int64_t t = (n + BIN_FEW_BLOCKS - 1) / BIN_FEW_BLOCKS;
+    return t >= BIN_MAX_TILE ? BIN_MAX_TILE : t <= 32 ? 32 : (t + 31) / 32 * 32;
 }
-
-static __global__ void __launch_bounds__(BIN_THREADS) bin_scatter_kernel(const uint8_t* __restrict__ cls, int64_t n,
-                                                                   const int64_t* __restrict__ offsets, int64_t nblocks,
-                                                                   int32_t* __restrict__ perm) {
-    constexpr int NW = BIN_THREADS / 32;
-    __shared__ int64_t running[NCLASS];
-    __shared__ int32_t wcount[NW][NCLASS];
-    const int lane = lane_id(), warp = threadIdx.x >> 5;
-    if (threadIdx.x < NCLASS) running[threadIdx.x] = offsets[(int64_t)threadIdx.x * nblocks + blockIdx.x];
-    const int64_t base = (int64_t)blockIdx.x * BIN_TILE;
-    for (int r = 0; r < BIN_ROUNDS; ++r) {
-        int64_t idx = base + r * BIN_THREADS + threadIdx.x;
-        int c = idx < n ? (int)cls[idx] : -1;
-        int myrank = 0;
-#pragma unroll
-        for (int k = 0; k < NCLASS; ++k) {
-            unsigned b = __ballot_sync(FULL_MASK, c == k);
-            if (c == k) myrank = __popc(b & ((1u << lane) - 1u));
-            if (lane == 0) wcount[warp][k] = __popc(b);
-        }
-        __syncthreads();
-        if (c >= 0) {
-            int64_t pos = running[c] + myrank;
-            for (int w = 0; w < warp; ++w) pos += wcount[w][c];
-            perm[pos] = (int32_t)idx;
-        }
-        __syncthreads();
-        if (threadIdx.x < NCLASS) {
-            int t = 0;
-            for (int w = 0; w < NW; ++w) t += wcount[w][threadIdx.x];
-            running[threadIdx.x] += t;
-        }
-        __syncthreads();
-    }
-}
-
-static __global__ void bin_class_starts_kernel(const int64_t* __restrict__ offsets, int64_t nblocks, int64_t* __restrict__ class_start) {
-    int c = threadIdx.x;
-    if (c < NCLASS) class_start[c] = offsets[(int64_t)c * nblocks];
-    if (c == NCLASS) class_start[c] = offsets[(int64_t)NCLASS * nblocks];
-}
-
-// scratch sizes (in elements) for bin_items: blockhist int32, offsets int64, partials int64
-inline cudaError_t bin_items(const uint8_t* cls, int64_t n, int32_t* perm, int64_t* class_start /*device, NCLASS+1*/,
-                             int32_t* blockhist, int64_t* offsets, int64_t* partials, uint32_t* err, cudaStream_t st) {
-    const int64_t nb = bin_blocks(n);
-    bin_count_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(cls, n, blockhist, nb);
-    cudaError_t e = exclusive_scan_i64<int32_t>(blockhist, NCLASS * nb, offsets, partials, err, st);
-    if (e != cudaSuccess) return e;
-    bin_scatter_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(cls, n, offsets, nb, perm);
-    bin_class_starts_kernel<<<1, 32, 0, st>>>(offsets, nb, class_start);
-    note_launches(3);
-    return cudaGetLastError();
-}
+inline int64_t bin_blocks(int64_t n) { return n > 0 ? (n + bin_tile(n) - 1) / bin_tile(n) : 0; }
+inline int64_t bin_blocks_max(int64_t n) { return n / BIN_MAX_TILE + BIN_FEW_BLOCKS + 1; }  // over every number of rows up to n
 
 // value-type traits: accumulator type and exact conversions
 template <typename V> struct AccOf { using type = double; };

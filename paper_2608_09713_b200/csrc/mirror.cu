@@ -32,7 +32,7 @@ bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCK
 
 struct MirrorWs {
     int64_t* partials;
-    uint32_t* err;       // [0] error word, [1] number of diagonal entries
+    uint32_t* err;       // [0] error word, [1] number of diagonal entries, [2] finished CTAs
     uint32_t* hist;      // counts of the passes and their prefix sums
     int64_t *offsets, *mid_off;
     // bucket sort
@@ -116,7 +116,7 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
     const int64_t items = std::max<int64_t>(m, 1);
     const int64_t ne = std::max<int64_t>(nnz_l, 1);
     MirrorWs t{};
-    t.err = (uint32_t*)take(8);
+    t.err = (uint32_t*)take(12);
     if (mirror_by_records(m, sv)) {
         const int64_t hist_n = (int64_t)(1 << MIRROR_RADIX_BITS) * std::max<int64_t>(mirror_groups(nnz_l), 1);
         t.diagf32 = (uint32_t*)take(items * 4);
@@ -179,9 +179,9 @@ __global__ void mirror_rowtot_kernel(const int64_t* __restrict__ l_rowptr, const
 }
 
 // one thread per row: the last entry tells whether the row stores its diagonal and whether it reaches above it
-// (rows are ascending); err[1] counts the diagonals
-__global__ void mirror_last_entry_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx, int64_t m,
-                                         uint32_t* err) {
+// (rows are ascending); err[1] counts the diagonals; the last CTA to finish (err[2] counts them) sends both to the host
+__global__ void __launch_bounds__(256) mirror_last_entry_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx, int64_t m,
+                                                                uint32_t* err, int64_t* host) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool diag = false;
     if (r < m) {
@@ -194,9 +194,16 @@ __global__ void mirror_last_entry_kernel(const int64_t* __restrict__ l_rowptr, c
             else diag = last == r;
         }
     }
-    // one atomic per warp: nearly every row of a product stores its diagonal
-    const unsigned votes = __ballot_sync(FULL_MASK, diag);
-    if (lane_id() == 0 && votes) atomicAdd(err + 1, (uint32_t)__popc(votes));
+    const int diags = __syncthreads_count(diag);
+    if (threadIdx.x == 0) {
+        if (diags) atomicAdd(err + 1, (uint32_t)diags);
+        __threadfence();
+        if (atomicAdd(err + 2, 1u) == gridDim.x - 1) {
+            __threadfence();
+            host[0] = (int64_t)atomicAdd(err + 1, 0u);
+            host[1] = (int64_t)atomicOr(err, 0u);
+        }
+    }
 }
 
 // G lanes per row: the lower part of row r of F is row r of C_L
@@ -240,6 +247,7 @@ int group_width(int64_t nnz, int64_t m) {
 
 // row lengths of F: the row's own entries and those of its column, the diagonal once
 struct MirrorRowLength {
+    using Value = int64_t;
     const int64_t* l_rowptr;
     const uint32_t* cnt;
     const uint8_t* diagf;
@@ -509,16 +517,18 @@ extern "C" spsyrk_status_t spsyrk_mirror(int64_t m, int64_t nnz_l, spsyrk_dtype_
 
     if (!d_f_colidx) {  // step 2: checks and nnz(F)
         if (!nnz_full_out) return SPSYRK_ERR_INVALID_ARG;
-        SPSYRK_CUDA_TRY(cudaMemsetAsync(w.err, 0, 8, st));
+        *nnz_full_out = 0;
+        SPSYRK_CUDA_TRY(cudaMemsetAsync(w.err, 0, 12, st));
         if (m > 0) {
-            mirror_last_entry_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(d_l_rowptr, d_l_colidx, m, w.err);
+            ScopedHostBlock h;
+            SPSYRK_CUDA_TRY(h.acquire());
+            mirror_last_entry_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(d_l_rowptr, d_l_colidx, m, w.err, h.dev);
             note_launches(1);
+            SPSYRK_CUDA_TRY(cudaGetLastError());
+            SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+            if (h.host[1]) return SPSYRK_ERR_BAD_CSR;
+            *nnz_full_out = 2 * nnz_l - h.host[0];
         }
-        uint32_t e[2] = {0, 0};
-        SPSYRK_CUDA_TRY(cudaMemcpyAsync(e, w.err, 8, cudaMemcpyDeviceToHost, st));
-        SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-        if (e[0]) return SPSYRK_ERR_BAD_CSR;
-        *nnz_full_out = 2 * nnz_l - (int64_t)e[1];
         return SPSYRK_OK;
     }
     // step 3: fill
@@ -572,7 +582,7 @@ constexpr int64_t NOALLOC_MAX_ROWS = SPSYRK_NOALLOC_MAX_ROWS;
 constexpr size_t NOALLOC_UCNT_OFF = 0;
 constexpr size_t NOALLOC_ROWTOT_OFF = NOALLOC_UCNT_OFF + (size_t)NOALLOC_MAX_ROWS * 4;
 constexpr size_t NOALLOC_PARTIALS_OFF = NOALLOC_ROWTOT_OFF + (size_t)NOALLOC_MAX_ROWS * 4;
-constexpr size_t NOALLOC_PARTIALS_BYTES = ((size_t)(NOALLOC_MAX_ROWS / SCAN_TILE) + 2) * 8;
+constexpr size_t NOALLOC_PARTIALS_BYTES = ((size_t)(NOALLOC_MAX_ROWS / SCAN_MIN_TILE) + 2) * 8;
 constexpr size_t NOALLOC_ERR_OFF = (NOALLOC_PARTIALS_OFF + NOALLOC_PARTIALS_BYTES + 255) / 256 * 256;
 constexpr size_t NOALLOC_BYTES = NOALLOC_ERR_OFF + 256;
 

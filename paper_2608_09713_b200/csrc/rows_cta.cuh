@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     // Binary input: a partial product is 1.  In a dense row the heavy columns' share of every count comes
     // from the per-row bit masks (one population count per entry), and their lists are not walked.
     const bool binary = P.binary != 0;
-    const bool use_masks = NUMERIC && dense && binary && P.nheavy > 0;
+    const bool use_masks = NUMERIC && dense && binary && *P.nheavy > 0;
     const unsigned long long mask_i = use_masks ? P.heavy_mask[i] : 0ull;
     // Binary input, dense row of at most 255 nonzeros: every count is at most the row's own length, so four
     // 8-bit counters share a 32-bit word of the accumulator tile and a tile holds four times the columns

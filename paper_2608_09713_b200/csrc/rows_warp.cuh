@@ -59,18 +59,6 @@ __device__ __forceinline__ uint32_t group_inclusive_scan(uint32_t v, int gl) {
     return v;
 }
 
-// Per-row header in class order, written by the plan: the row's index inside the plan's range, the
-// position of its first nonzero in A and its number of nonzeros.
-__global__ void __launch_bounds__(256) row_header_kernel(PlanDev P, const int32_t* __restrict__ perm, int64_t rows,
-                                                         uint4* __restrict__ hdr) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= rows) return;
-    const int32_t rloc = perm[n];
-    const int64_t i = (int64_t)P.r0 + rloc;
-    const int64_t p0 = P.rowptr[i], p1 = P.rowptr[i + 1];
-    hdr[n] = make_uint4((uint32_t)rloc, (uint32_t)p0, (uint32_t)(p1 - p0), 0u);
-}
-
 // last s in [0, 32) with tab[s] <= c; tab is non-decreasing and tab[0] = 0
 __device__ __forceinline__ uint32_t last_not_above(const uint32_t* tab, uint32_t c) {
     uint32_t s = 0;
@@ -520,18 +508,6 @@ __global__ void __launch_bounds__(symbolic_warps(N) * 32) symbolic_warp_kernel(P
 // The items of a row occupy a multiple of eight words in the map (16-byte pieces).
 // =============================================================================================
 constexpr int MAP_SLOT_BITS = 9;
-
-// items of the light rows in class order, rounded up to eight: the scan of these is where a row's map words start
-static __global__ void __launch_bounds__(256) row_items_kernel(PlanDev P, const uint4* __restrict__ hdr, const uint8_t* __restrict__ cls,
-                                                               int64_t rows, bool diag, uint32_t* __restrict__ items8) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= rows) return;
-    const uint4 h = hdr[n];
-    const uint8_t c = cls[h.x];
-    uint32_t it = 0;
-    if (c >= 1 && c <= 5) it = (uint32_t)(P.work[h.x] - (diag ? (int64_t)h.z : 0));
-    items8[n] = (it + 7u) & ~7u;
-}
 
 template <int N>
 struct SymbolicSortSmem {

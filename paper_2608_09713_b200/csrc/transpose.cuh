@@ -40,31 +40,18 @@ struct PlanDev {
     // of entries) are also kept as one bit per row, heavy_mask[i] bit b = row i stores heavy column b, so
     // that their share of a count is popcount(heavy_mask[i] & heavy_mask[j]) instead of one list walk each.
     int32_t binary;               // 0 / 1, valid after the plan's analysis
-    int32_t nheavy;               // heavy columns in use (0: none)
+    const uint32_t* nheavy;       // heavy columns in use (0: none), device memory, written when the matrix is binary
     const uint8_t* heavy_id;      // [n] bit number of a heavy column, 0xff otherwise
     const uint64_t* heavy_mask;   // [m]
     float* jaccard;               // optional: the numeric pass also writes c / (|a_i| + |a_j| - c) here (int32 values)
     const int32_t* adeg;          // [m] stored entries per row of A (|a_i| of the Jaccard formula)
 };
 
-static __global__ void __launch_bounds__(256) row_degree_kernel(const int64_t* __restrict__ rowptr, int32_t m, int32_t* __restrict__ adeg) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) adeg[i] = (int32_t)(rowptr[i + 1] - rowptr[i]);
-}
-
 // ---------------------------------------------------------------------------------------------
-// Analysis of a binary matrix: value check, choice of the heavy columns, the per-row bit masks.
-// facts[0] = 1 if some stored value differs from one; facts[1] = heavy columns; facts[2] = threshold.
+// Analysis of a binary matrix (every stored value is one, see row_expand_kernel): choice of the heavy columns, the
+// per-row bit masks.  Launched for binary matrices only.
+// facts[0] = 1 if some stored value differs from one; facts[1] = heavy columns; facts[32..] histogram.
 // ---------------------------------------------------------------------------------------------
-template <typename V>
-static __global__ void __launch_bounds__(256) binary_check_kernel(const V* __restrict__ vals, int64_t nnz, uint32_t* __restrict__ facts) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    bool other = false;
-    for (; p < nnz; p += stride) other |= !(vals[p] == V(1));
-    if (__any_sync(FULL_MASK, other) && lane_id() == 0) atomicOr(&facts[0], 1u);
-}
-
 // histogram of floor(log2(column length)) over the columns
 static __global__ void __launch_bounds__(256) heavy_hist_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ hist32) {
     __shared__ uint32_t h[32];
@@ -80,29 +67,30 @@ static __global__ void __launch_bounds__(256) heavy_hist_kernel(const uint32_t* 
     if (threadIdx.x < 32 && h[threadIdx.x]) atomicAdd(&hist32[threadIdx.x], h[threadIdx.x]);
 }
 
-// threshold = the smallest power of two such that at most 64 columns have that many entries or more
-static __global__ void heavy_threshold_kernel(const uint32_t* __restrict__ hist32, uint32_t* __restrict__ facts) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    uint32_t total = 0, thr = 0xffffffffu;
-    for (int b = 31; b >= 8; --b) {
-        if (total + hist32[b] > 64u) break;
-        total += hist32[b];
-        if (hist32[b]) thr = 1u << b;
-    }
-    facts[1] = 0;
-    facts[2] = facts[0] ? 0xffffffffu : thr;  // no heavy columns unless the matrix is binary
-}
-
+// Columns of at least the threshold get a bit number; the threshold is the smallest power of two such that at most 64
+// columns have that many entries or more.
 static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ facts,
                                                                  uint8_t* __restrict__ heavy_id) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    uint8_t id = 0xff;
-    if (colcnt[k] >= facts[2]) {
-        const uint32_t b = atomicAdd(&facts[1], 1u);
-        if (b < 64u) id = (uint8_t)b;
+    __shared__ uint32_t s_thr;
+    if (threadIdx.x < 32) {
+        const int b = 31 - (int)threadIdx.x;  // lane l looks at lengths of 2^(31 - l) and more
+        const uint32_t c = facts[32 + b];
+        const uint32_t upto = warp_inclusive_scan<uint32_t>(c);
+        const unsigned fits = __ballot_sync(FULL_MASK, b >= 8 && upto <= 64u);
+        const unsigned used = __ballot_sync(FULL_MASK, c > 0) & (fits == FULL_MASK ? FULL_MASK : ((1u << __popc(fits)) - 1u));
+        if (threadIdx.x == 0) s_thr = used ? 1u << (31 - (31 - __clz(used))) : 0xffffffffu;
     }
-    heavy_id[k] = id;
+    __syncthreads();
+    const uint32_t thr = s_thr;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
+        uint8_t id = 0xff;
+        if (colcnt[k] >= thr) {
+            const uint32_t b = atomicAdd(&facts[1], 1u);
+            if (b < 64u) id = (uint8_t)b;
+        }
+        heavy_id[k] = id;
+    }
 }
 
 template <int G>
@@ -135,33 +123,41 @@ template <> struct alignas(16) ColRec<double> { int32_t j; int32_t pad; double v
 template <> struct alignas(8) ColRec<float> { int32_t j; float v; };
 template <> struct alignas(8) ColRec<int32_t> { int32_t j; int32_t v; };
 
-static __global__ void validate_rowptr_kernel(const int64_t* __restrict__ rowptr, int64_t m, int64_t nnz, uint32_t* err) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) {
-        int64_t a = rowptr[i], b = rowptr[i + 1];
-        if (a > b || a < 0 || b > nnz) atomicOr(err, ERRW_BAD_ROWPTR);
-    }
-    if (i == 0 && (rowptr[0] != 0 || rowptr[m] != nnz)) atomicOr(err, ERRW_BAD_ROWPTR);
-}
-
-// G lanes per row, one sweep over the nonzeros of A: the column histogram (its scan gives colptr), the explicit
-// row id of every nonzero (the radix sort's first payload), and the checks that column ids are in range and
-// strictly ascending inside the row.  The row pointers have been validated before.
-template <int G>
+// G lanes per row, one sweep over the nonzeros of A: the checks of the row pointers (a row indexes nothing unless its own
+// two are sane) and of the column ids (in range, strictly ascending inside the row), the column histogram (its scan gives
+// colptr), the explicit row id of every nonzero (the radix sort's first payload), the row lengths, and whether
+// every stored value is one.  Nothing waits for the checks: the kernels up to the plan's one synchronisation index
+// nothing by what they would have found wrong.
+template <int G, typename V>
 static __global__ void __launch_bounds__(256) row_expand_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                                                                int32_t m, int32_t n, uint32_t* __restrict__ colcnt,
-                                                                uint32_t* __restrict__ rowid, uint32_t* err) {
+                                                                const V* __restrict__ vals, int32_t m, int32_t n, int64_t nnz,
+                                                                uint32_t* __restrict__ colcnt, uint32_t* __restrict__ rowid,
+                                                                int32_t* __restrict__ adeg, uint32_t* facts, uint32_t* err) {
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
-    if (gid >= m) return;
-    const int64_t p0 = rowptr[gid], p1 = rowptr[gid + 1];
-    for (int64_t p = p0 + gl; p < p1; p += G) {
-        const int32_t k = colidx[p];
-        if ((uint32_t)k >= (uint32_t)n) atomicOr(err, ERRW_BAD_COL);
-        else atomicAdd(&colcnt[k], 1u);
-        if (p > p0 && colidx[p - 1] >= k) atomicOr(err, ERRW_UNSORTED);
-        rowid[p] = (uint32_t)gid;
+    bool look = __ldca(facts) == 0;  // values are looked at until one differs from one (an old zero only costs a look)
+    bool other = false;
+    if (gid < m) {
+        const int64_t p0 = rowptr[gid], p1 = rowptr[gid + 1];
+        if (gl == 0) adeg[gid] = (int32_t)(p1 - p0);
+        if (p0 > p1 || p0 < 0 || p1 > nnz) {
+            atomicOr(err, ERRW_BAD_ROWPTR);
+        } else {
+            for (int64_t p = p0 + gl; p < p1; p += G) {
+                const int32_t k = colidx[p];
+                if (look) {
+                    other = !(vals[p] == V(1));
+                    look = !other;
+                }
+                if ((uint32_t)k >= (uint32_t)n) atomicOr(err, ERRW_BAD_COL);
+                else atomicAdd(&colcnt[k], 1u);
+                if (p > p0 && colidx[p - 1] >= k) atomicOr(err, ERRW_UNSORTED);
+                rowid[p] = (uint32_t)gid;
+            }
+        }
     }
+    if (gid == 0 && gl == 0 && (rowptr[0] != 0 || rowptr[m] != nnz)) atomicOr(err, ERRW_BAD_ROWPTR);
+    if (__any_sync(FULL_MASK, other) && lane_id() == 0) atomicOr(facts, 1u);  // (few: only the CTAs that started before the first)
 }
 
 // last radix pass of the transpose: the element at sorted position s is entry s of the column lists
@@ -170,6 +166,7 @@ struct EmitTransposeFinal {
     PlanDev P;
     uint2* desc_hi;  // null in lower-triangle mode
     __device__ __forceinline__ void operator()(int64_t s, uint32_t k, uint32_t row, VB val, uint32_t p) const {
+        if (k >= (uint32_t)P.n) return;  // not a canonical matrix: reported when the plan synchronises
         const int64_t cs = P.colptr[k];
         P.at_row[s] = (int32_t)row;
         if constexpr (sizeof(VB) == 8) static_cast<uint4*>(P.at_rec)[s] = make_uint4(row, 0u, (uint32_t)val, (uint32_t)(val >> 32));
@@ -204,49 +201,165 @@ static __global__ void __launch_bounds__(256) block_desc_kernel(PlanDev P, const
     }
 }
 
-// Step a2: per-row work w[i] = sum of the descriptor lengths of row i (G lanes per row), and the
-// class of the row.  Rows of the range [r0, r1) only.
+// Step a2: per-row work w[i] = sum of the descriptor lengths of row i (G lanes per row), the class of the row and
+// the number of rows of every class in every CTA's tile (the first half of a stable counting sort by class).
 //   class 0: no work; 1..5: w <= 32, 64, 128, 256, 512 and at most 32 nonzeros (one warp, register sort)
-//   6: w <= block_max (one 256-thread CTA, bitmap accumulator); 7: larger (one 1024-thread CTA)
-template <int G>
+//   6: w <= block_max (block class, bitmap accumulator); 7: larger (one 1024-thread CTA)
 //   diag: the light-row kernels leave the diagonal products out of their item lists (lower-triangle mode
 //   over the whole column range), so a light row is classed by w minus its number of nonzeros
-static __global__ void __launch_bounds__(256) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, bool diag,
-                                                        unsigned long long* __restrict__ work_total) {
-    const int gl = threadIdx.x & (G - 1);
-    const int64_t rows = P.r1 - P.r0;
-    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
-    unsigned long long mine = 0;  // work of the rows this thread owned
-    // a fixed grid walks the rows: one atomic per CTA for the total, however many rows there are
-    for (int64_t gbase = ((int64_t)blockIdx.x * blockDim.x) / G; gbase < rows; gbase += groups) {  // uniform per CTA
-        const int64_t gid = gbase + threadIdx.x / G;
-        int64_t w = 0, deg = 0;
-        if (gid < rows) {
-            const int64_t i = P.r0 + gid;
-            const int64_t p0 = P.rowptr[i], p1 = P.rowptr[i + 1];
-            deg = p1 - p0;
-            for (int64_t p = p0 + gl; p < p1; p += G) w += P.desc[p].y;
-        }
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) w += __shfl_xor_sync(FULL_MASK, w, o);
-        if (gid < rows && gl == 0) {
-            P.work[gid] = w;
-            uint8_t c;
-            const int64_t wl = diag ? w - deg : w;  // items of a light row
-            if (w == 0) c = 0;
-            else if (deg <= 32 && wl <= 512) c = wl <= 32 ? 1 : wl <= 64 ? 2 : wl <= 128 ? 3 : wl <= 256 ? 4 : 5;
-            else c = w <= block_max ? 6 : 7;
-            cls[gid] = c;
-            mine += (unsigned long long)w;
-        }
-    }
+// A group takes UNR rows at a time, so that the loads of one row do not wait for those of the row before (one at a time:
+// 438 us for 4.2e6 rows of 16 nonzeros).
+template <int G>
+static __global__ void __launch_bounds__(BIN_THREADS) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, bool diag, int64_t tile,
+                                                                      int32_t* __restrict__ blockhist, int64_t nblocks,
+                                                                      unsigned long long* __restrict__ work_total) {
+    constexpr int GROUPS = BIN_THREADS / G;
+    constexpr int UNR = 4;
+    __shared__ int32_t hist[NCLASS];
     __shared__ unsigned long long cta_sum;
+    if (threadIdx.x < NCLASS) hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) cta_sum = 0;
     __syncthreads();
+    const int gl = threadIdx.x & (G - 1), group = threadIdx.x / G;
+    const int64_t rows = P.r1 - P.r0;
+    const int64_t t0 = (int64_t)blockIdx.x * tile, t1 = min(t0 + tile, rows);
+    const bool sane = (*P.err & (ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED)) == 0;  // a matrix that failed its checks has no descriptors
+    unsigned long long mine = 0;    // work of the rows this thread owned
+    for (int64_t base = t0; base < t1; base += GROUPS * UNR) {
+        int64_t p0[UNR], w[UNR];
+        int32_t deg[UNR];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            const int64_t r = base + u * GROUPS + group;
+            p0[u] = 0; deg[u] = 0;
+            if (r < t1 && sane) {
+                p0[u] = P.rowptr[P.r0 + r];
+                deg[u] = (int32_t)(P.rowptr[P.r0 + r + 1] - p0[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) w[u] = gl < deg[u] ? P.desc[p0[u] + gl].y : 0;
+#pragma unroll
+        for (int u = 0; u < UNR; ++u)
+            for (int32_t q = gl + G; q < deg[u]; q += G) w[u] += P.desc[p0[u] + q].y;
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            const int64_t r = base + u * GROUPS + group;
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) w[u] += __shfl_xor_sync(FULL_MASK, w[u], o);
+            if (r < t1 && gl == 0) {
+                P.work[r] = w[u];
+                int c;
+                const int64_t wl = diag ? w[u] - deg[u] : w[u];  // items of a light row
+                if (w[u] == 0) c = 0;
+                else if (deg[u] <= 32 && wl <= 512) c = wl <= 32 ? 1 : wl <= 64 ? 2 : wl <= 128 ? 3 : wl <= 256 ? 4 : 5;
+                else c = w[u] <= block_max ? 6 : 7;
+                cls[r] = (uint8_t)c;
+                atomicAdd(&hist[c], 1);
+                mine += (unsigned long long)w[u];
+            }
+        }
+    }
     const unsigned long long ws = warp_reduce_sum<unsigned long long>(mine);
     if (lane_id() == 0 && ws) atomicAdd(&cta_sum, ws);
     __syncthreads();
     if (threadIdx.x == 0 && cta_sum) atomicAdd(work_total, cta_sum);
+    if (threadIdx.x < NCLASS) blockhist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = hist[threadIdx.x];
 }
+
+// prefix sums of the class-major counts, and where every class starts
+struct BinStarts {
+    int64_t* offsets;
+    uint32_t nblocks;
+    int64_t* class_start;  // NCLASS + 1
+    __device__ __forceinline__ void operator()(int64_t i, int64_t ex) const {
+        offsets[i] = ex;
+        const uint32_t c = (uint32_t)i / nblocks;
+        if (c * nblocks == (uint32_t)i) class_start[c] = ex;
+    }
+    __device__ __forceinline__ void total(int64_t t) const { class_start[NCLASS] = t; }
+};
+
+// Second half of the counting sort: the rows in class order (ascending inside a class), for each of them the header
+// (row inside the plan's range, position of its first nonzero in A, number of nonzeros) and the words of the item map
+// it needs (its items rounded up to eight; light rows only).  An empty row's count is settled here.
+static __global__ void __launch_bounds__(BIN_THREADS) row_scatter_kernel(PlanDev P, const uint8_t* __restrict__ cls, int64_t tile,
+                                                                         const int64_t* __restrict__ offsets, int64_t nblocks, bool diag,
+                                                                         int32_t* __restrict__ perm, uint4* __restrict__ hdr,
+                                                                         uint32_t* __restrict__ items8, int32_t* __restrict__ cnt) {
+    constexpr int NW = BIN_THREADS / 32;
+    __shared__ int64_t running[NCLASS];
+    __shared__ int32_t wcount[NW][NCLASS];
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    if (threadIdx.x < NCLASS) running[threadIdx.x] = offsets[(int64_t)threadIdx.x * nblocks + blockIdx.x];
+    const int64_t rows = P.r1 - P.r0;
+    const int64_t t0 = (int64_t)blockIdx.x * tile, t1 = min(t0 + tile, rows);
+    for (int64_t base = t0; base < t1; base += BIN_THREADS) {
+        const int64_t r = base + threadIdx.x;
+        int c = -1;
+        int64_t p0 = 0, deg = 0, w = 0;
+        if (r < t1) {
+            c = cls[r];
+            p0 = P.rowptr[P.r0 + r];
+            deg = P.rowptr[P.r0 + r + 1] - p0;
+            w = P.work[r];
+        }
+        int myrank = 0;
+#pragma unroll
+        for (int k = 0; k < NCLASS; ++k) {
+            const unsigned b = __ballot_sync(FULL_MASK, c == k);
+            if (c == k) myrank = __popc(b & ((1u << lane) - 1u));
+            if (lane == 0) wcount[warp][k] = __popc(b);
+        }
+        __syncthreads();
+        if (c >= 0) {
+            int64_t pos = running[c] + myrank;
+            for (int v = 0; v < warp; ++v) pos += wcount[v][c];
+            perm[pos] = (int32_t)r;
+            hdr[pos] = make_uint4((uint32_t)r, (uint32_t)p0, (uint32_t)deg, 0u);
+            items8[pos] = c >= 1 && c <= 5 ? ((uint32_t)(diag ? w - deg : w) + 7u) & ~7u : 0u;
+            if (c == 0) cnt[r] = 0;
+        }
+        __syncthreads();
+        if (threadIdx.x < NCLASS) {
+            int t = 0;
+            for (int v = 0; v < NW; ++v) t += wcount[v][threadIdx.x];
+            running[threadIdx.x] += t;
+        }
+        __syncthreads();
+    }
+}
+
+// What the host needs to know about a view of the plan, in the order in which it is written for the host
+enum : int { PF_CLASS_START = 0, PF_MAP_ITEMS = NCLASS + 1, PF_WORK, PF_OTHER_THAN_ONE, PF_ERR, PF_WORDS };
+struct PlanFacts {
+    const int64_t* class_start;
+    const unsigned long long* work_total;
+    const uint32_t* facts;
+    const uint32_t* err;
+    int64_t* host;
+    __device__ __forceinline__ void publish(int64_t map_items) const {
+        int64_t w[PF_WORDS];  // all loads before the first store: one round trip, not thirteen
+#pragma unroll
+        for (int c = 0; c <= NCLASS; ++c) w[PF_CLASS_START + c] = class_start[c];
+        w[PF_MAP_ITEMS] = map_items;
+        w[PF_WORK] = (int64_t)*work_total;
+        w[PF_OTHER_THAN_ONE] = (int64_t)facts[0];
+        w[PF_ERR] = (int64_t)*err;
+#pragma unroll
+        for (int c = 0; c < PF_WORDS; ++c) host[c] = w[c];
+    }
+};
+// prefix sums of the map words; the last kernel before the plan's synchronisation
+struct ItemStarts {
+    int64_t* itemoff;
+    int64_t n;
+    PlanFacts facts;
+    __device__ __forceinline__ void operator()(int64_t i, int64_t ex) const { itemoff[i] = ex; }
+    __device__ __forceinline__ void total(int64_t t) const {
+        itemoff[n] = t;
+        facts.publish(t);
+    }
+};
 
 }  // namespace spsyrk
