@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "rows_cta.cuh"
+#include "rows_heavy.cuh"
 #include "rows_warp.cuh"
 
 #include <atomic>
@@ -58,8 +59,6 @@ constexpr uint32_t ROW_CHUNK_BITS_MAX_NUMERIC = 1u << 18;
 constexpr uint32_t ROW_CHUNK_BITS_MAX_SYMBOLIC = 1u << 20;
 constexpr int TRANSPOSE_RADIX_BITS = 8;
 constexpr size_t LARGE_SMEM_BUDGET = 200 * 1024;
-constexpr int GLOBAL_ACC_CTAS = 160;  // upper bound of the persistent heavy-row grid (one CTA per SM)
-constexpr uint32_t BLOCK_ACC_SLOTS = 4096;
 constexpr int64_t MAX_PARTS = 65536;
 
 size_t dtype_size(spsyrk_dtype_t t) { return t == SPSYRK_F64 ? 8 : 4; }
@@ -137,12 +136,19 @@ struct spsyrk_plan_s {
     int64_t* state_col;
     int64_t* class_start_dev;  // NCLASS + 1
     unsigned long long* work_total_dev;
-    uint32_t* row_counter;  // row dispenser of the persistent heavy-row kernel
-    double* gacc;           // its global accumulator slices (GLOBAL_ACC_CTAS x gslots, 8 bytes per slot)
-    uint32_t gslots;
+    // heavy rows by the kernel that computes them (rows_heavy.cuh)
+    int32_t* route_list;    // NROUTE lists of rows_cap each
+    uint32_t* route_count;  // NROUTE list lengths (device) ...
+    uint32_t route_n[NROUTE];  // ... and as the host knows them after the symbolic pass
+    uint32_t* bounds;       // scratch of the direct kernel
+    int2* parts_list;       // parts of the longest rows
+    uint32_t* block_base;   // entries of a heavy row before every block of columns, [row][blocks_per_row]
+    uint32_t blocks_per_row;
+    uint32_t* dispensers;   // NROUTE counters the persistent kernels take their rows from
+    int64_t sub_row_lo, sub_row_hi;  // with sub_active: the rows (of the plan's range) to compute
     uint32_t* facts;       // binary analysis (device): differs-from-one flag, heavy columns, threshold, histogram
     uint8_t* heavy_id;
-    uint64_t* heavy_mask;
+    uint32_t* heavy_mask;
     int32_t* adeg;
     int64_t* itemoff;      // rows + 1, class order: where the map words of a light row start
     int64_t map_items;     // map words the current row range needs
@@ -180,7 +186,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     // counters in one piece, so that one memset clears them: the binning's, then the plan's, then the column counts
     const int views = full ? 2 : 1;
     const size_t bin_words = views * (1 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(items));
-    auto zero = c.take<int64_t>(bin_words + 64 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2);
+    auto zero = c.take<int64_t>(bin_words + 32 + (32 + HEAVY_BINS) / 2 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2);
     Carver cz(zero);
     auto take_words = [&](size_t words) { int64_t* q = zero ? zero + cz.off : nullptr; cz.off += words; return q; };
     auto work_total_dev = reinterpret_cast<unsigned long long*>(take_words(1));
@@ -189,7 +195,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     int64_t* u_state_bin = full ? take_words(scan_partials_count(NCLASS * nb)) : nullptr;
     int64_t* u_state_items = full ? take_words(scan_partials_count(items)) : nullptr;
     auto err = reinterpret_cast<uint32_t*>(take_words(32));
-    auto facts = reinterpret_cast<uint32_t*>(take_words(32));  // [0..1] binary analysis, [32..63] its histogram
+    auto facts = reinterpret_cast<uint32_t*>(take_words((32 + HEAVY_BINS) / 2));  // [0..1] binary analysis, [32..] its histogram
     auto state_col = take_words(scan_partials_count(std::max<int64_t>(n, 1)));
     auto colcnt = reinterpret_cast<uint32_t*>(take_words((size_t)(n + 1) / 2));
     const size_t zero_words = cz.off;
@@ -197,9 +203,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     // The two buffer sets of the radix sort (key, row, position, value per nonzero) are reused: the set that
     // the last pass does not read receives the column lists that pass writes (row ids and records), and the
     // set it does read holds, once the sort is over, the block descriptors and the heavy-row accumulator slices.
-    const uint32_t gslots = pow2_at_least((uint64_t)std::max<int64_t>(m, 1), 1024u, ROW_CHUNK_BITS_MAX_NUMERIC);
-    const size_t gacc_bytes = (size_t)GLOBAL_ACC_CTAS * gslots * sizeof(double);
-    const size_t set_bytes = std::max((size_t)nnz * (12 + sv) + 4 * ALIGN, (size_t)nnz * 8 + gacc_bytes + 2 * ALIGN);
+    const size_t set_bytes = (size_t)nnz * (12 + sv) + 4 * ALIGN;
     auto set_a = c.take<char>(set_bytes);
     auto set_b = c.take<char>(set_bytes);
     Carver ca(set_a), cb(set_b);
@@ -217,18 +221,26 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto at_row = c_free.take<int32_t>(nnz + 4);  // the symbolic gathers read aligned 16-byte pieces: up to 3 entries past the end
     auto at_rec = c_free.take<char>(nnz * (sv == 8 ? 16 : 8));
     auto desc_blk = c_src.take<uint2>(nnz);
-    auto gacc = c_src.take<double>((size_t)GLOBAL_ACC_CTAS * gslots);
     auto rx_hist = c.take<uint32_t>(rx_hist_n);
     auto rx_offsets = c.take<int64_t>(rx_hist_n + 1);
     auto blockhist = c.take<int32_t>(NCLASS * nb);
     auto offsets = c.take<int64_t>(NCLASS * nb + 1);
     auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(std::max<int64_t>(items + 1, NCLASS * nb), rx_hist_n)));
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
-    auto row_counter = c.take<uint32_t>(1);
+    auto route_count = c.take<uint32_t>(2 * NROUTE);  // both views in a row
+    auto dispensers = c.take<uint32_t>(2 * NROUTE);
+    auto route_list = c.take<int32_t>(NROUTE * items);
+    auto bounds = c.take<uint32_t>(DIRECT_MAX_CTAS * DIRECT_BOUNDS);
+    // rows whose output range is at most 2^18 columns (they are among the first 2^18 rows)
+    const int64_t base_rows = std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC);
+    const uint32_t blocks_per_row = (uint32_t)((std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC) + BASE_BLOCK - 1) / BASE_BLOCK);
+    auto parts_list = c.take<int2>(base_rows * DIRECT_MAX_PARTS);
+    auto block_base = c.take<uint32_t>(base_rows * blocks_per_row);
     auto work_prefix = c.take<int64_t>(items + 1);
     auto itemoff = c.take<int64_t>(items + 1);
     auto heavy_id = c.take<uint8_t>(std::max<int64_t>(n, 1));
-    auto heavy_mask = c.take<uint64_t>(std::max<int64_t>(m, 1));
+    const int64_t mask_stride = (items + 3) / 4 * 4;
+    auto heavy_mask = c.take<uint32_t>(HEAVY_PLANES * mask_stride);
     auto items8 = c.take<uint32_t>(items);
     auto adeg = c.take<int32_t>(std::max<int64_t>(m, 1));
     auto part_bounds = c.take<int64_t>(MAX_PARTS + 1);
@@ -237,7 +249,9 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     // full-output mode: the upper view's own per-row arrays and the second descriptor array
     uint2* desc_hi = nullptr;
     int64_t *u_work = nullptr, *u_itemoff = nullptr, *u_class_start_dev = nullptr, *hi_begin = nullptr, *work_sum = nullptr;
-    int32_t *u_perm = nullptr, *u_cnt = nullptr, *cnt_tot = nullptr;
+    int32_t *u_perm = nullptr, *u_cnt = nullptr, *cnt_tot = nullptr, *u_route_list = nullptr;
+    int2* u_parts_list = nullptr;
+    uint32_t* u_block_base = nullptr;
     uint4* u_hdr = nullptr;
     uint8_t* u_cls = nullptr;
     if (full) {
@@ -250,12 +264,17 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         u_itemoff = c.take<int64_t>(items + 1);
         u_class_start_dev = c.take<int64_t>(NCLASS + 1);
         cnt_tot = c.take<int32_t>(m);
+        u_route_list = c.take<int32_t>(NROUTE * items);
+        u_parts_list = c.take<int2>(base_rows * DIRECT_MAX_PARTS);
+        u_block_base = c.take<uint32_t>(base_rows * blocks_per_row);
         hi_begin = c.take<int64_t>(items + 1);
         work_sum = c.take<int64_t>(m);
     }
     if (pl) {
         pl->desc_hi = desc_hi; pl->cnt_tot = cnt_tot; pl->hi_begin = hi_begin; pl->work_sum = work_sum;
-        pl->row_counter = row_counter; pl->gacc = gacc; pl->gslots = gslots;
+        pl->route_count = route_count; pl->dispensers = dispensers; pl->route_list = route_list; pl->bounds = bounds; pl->parts_list = parts_list;
+        pl->block_base = block_base; pl->blocks_per_row = blocks_per_row;
+        pl->dev.mask_stride = mask_stride;
         pl->work_prefix = work_prefix; pl->part_bounds = part_bounds; pl->itemoff = itemoff;
         pl->ub = ub; pl->ub_off = ub_off;
         pl->dev.heavy_id = heavy_id; pl->dev.heavy_mask = heavy_mask; pl->facts = facts;
@@ -270,7 +289,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         pl->class_start_dev = class_start_dev; pl->work_total_dev = work_total_dev;
         pl->state_bin = state_bin; pl->state_items = state_items; pl->state_col = state_col; pl->items8 = items8;
         pl->zero_all = zero; pl->zero_all_bytes = zero_words * sizeof(int64_t);
-        pl->zero_bin = zero; pl->zero_bin_bytes = bin_words * sizeof(int64_t);
+        pl->rows_cap = items; pl->zero_bin = zero; pl->zero_bin_bytes = bin_words * sizeof(int64_t);
         pl->dev.nheavy = facts + 1;
         if (up) {
             // the upper view shares everything that describes A and the scratch space; its rows are its own
@@ -280,6 +299,8 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
             up->perm = u_perm; up->hdr = u_hdr; up->cnt = u_cnt; up->cls = u_cls; up->itemoff = u_itemoff;
             up->class_start_dev = u_class_start_dev; up->work_total_dev = u_work_total_dev;
             up->state_bin = u_state_bin; up->state_items = u_state_items;
+            up->route_count = route_count + NROUTE; up->dispensers = dispensers + NROUTE; up->route_list = u_route_list;
+            up->parts_list = u_parts_list; up->block_base = u_block_base;
         }
     }
     return (c.off + ALIGN - 1) / ALIGN * ALIGN;
@@ -641,45 +662,127 @@ spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, cudaStream_t st) {
     const size_t smem = CtaRowSmem<int32_t, THREADS, false>::bytes(cb, 0);
     auto kern = rows_cta_kernel<int32_t, THREADS, false>;
     SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<(unsigned)count, THREADS, smem, st>>>(pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr,
-                                                  nullptr, 0u, nullptr, nullptr, 0u);
+    kern<<<(unsigned)count, THREADS, smem, st>>>(pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr, nullptr, 0, 0,
+                                                 pl->block_base, pl->blocks_per_row);
     note_launches(1);
     return SPSYRK_OK;
 }
 
-template <typename V, int THREADS>
-spsyrk_status_t launch_numeric_cta(spsyrk_plan_s* pl, int c, uint32_t acc_slots_or_zero, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
+// Shared-memory shapes of the heavy-row kernels and the rule that goes with them.  The small rank kernel is launched
+// for three widths of its bitmap, so that rows in the lower part of the range leave room for more CTAs per SM.
+constexpr int RANK_SMALL_THREADS = 256, RANK_MID_THREADS = 512, RANK_BIG_THREADS = 1024, DENSE8_THREADS = 512;
+constexpr size_t SMEM_PER_CTA = 226 * 1024;
+
+struct HeavyShapes {
+    RouteRule rule;
+    uint32_t columns;  // of the widest bitmap
+    uint32_t dense8_columns;
+};
+
+template <typename V>
+HeavyShapes heavy_shapes(const spsyrk_plan_s* pl) {
     using Acc = typename AccOf<V>::type;
-    const int64_t count = numeric_count(pl, c);
+    HeavyShapes h;
+    h.columns = row_chunk_bits(pl, ROW_CHUNK_BITS_MAX_NUMERIC);
+    const uint32_t cb = h.columns;
+    RouteRule& r = h.rule;
+    r.wide = ROW_CHUNK_BITS_MAX_NUMERIC;
+    r.bits0 = std::min(cb, 65536u);
+    r.bits1 = std::min(cb, 131072u);
+    r.slots_small = std::min(cb, (uint32_t)(16384 / sizeof(Acc)));
+    r.slots_mid = std::min(cb, (uint32_t)(65536 / sizeof(Acc)));
+    r.slots_big = std::min(cb, (uint32_t)((SMEM_PER_CTA - RankSmem<V, RANK_BIG_THREADS>::bytes(cb, 0)) / sizeof(Acc)) / 1024 * 1024);
+    // whole blocks of the table, two CTAs per SM; 2^18 columns are at most DIRECT_MAX_CHUNKS chunks
+    r.chunk = std::min(cb, (uint32_t)((SMEM_PER_CTA / 2 - 1024 - DirectSmem<V, DIRECT_THREADS>::bytes(0)) / (sizeof(Acc) * 32 + 32 + 4)) * 32 / BASE_BLOCK * BASE_BLOCK);
+    static_assert(ROW_CHUNK_BITS_MAX_NUMERIC / BASE_BLOCK <= DIRECT_MAX_CHUNKS, "a row's chunk bounds fit a CTA's scratch");
+    const uint64_t umax = pl->dev.mode == SPSYRK_TRIL ? (uint64_t)pl->dev.r1 : (uint64_t)pl->dev.m;
+    h.dense8_columns = (uint32_t)std::min<uint64_t>(umax, (SMEM_PER_CTA - Dense8Smem<DENSE8_THREADS>::bytes(0)) / 16 * 16);
+    r.dense8 = h.dense8_columns;
+    r.binary = pl->dev.binary;
+    return h;
+}
+
+// which kernel computes which heavy row; the counts of the symbolic pass are known
+spsyrk_status_t route_heavy(spsyrk_plan_s* pl, cudaStream_t st) {
+    const int64_t count = pl->class_start[NCLASS] - pl->class_start[6];
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->route_count, 0, NROUTE * sizeof(uint32_t), st));
     if (count <= 0) return SPSYRK_OK;
-    const int32_t* rows_of_class = pl->perm + numeric_first(pl, c);
-    const uint32_t cb = row_chunk_bits(pl, ROW_CHUNK_BITS_MAX_NUMERIC);
-    uint32_t slots = acc_slots_or_zero;
-    if (slots == 0) {
-        const size_t fixed = CtaRowSmem<V, THREADS, true>::bytes(cb, 0);
-        slots = (uint32_t)((LARGE_SMEM_BUDGET - fixed) / sizeof(Acc));
-        slots = std::min(slots, cb);  // a chunk never has more slots than bits
-    }
-    const size_t smem = CtaRowSmem<V, THREADS, true>::bytes(cb, slots);
-    auto kern = rows_cta_kernel<V, THREADS, true>;
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // rows that overflow the shared-memory tile go to the persistent variant with global accumulators
-    const bool use_global = acc_slots_or_zero == 0 && pl->gslots >= cb;
-    const uint32_t gslots = use_global ? pl->gslots : 0u;
-    kern<<<(unsigned)count, THREADS, smem, st>>>(pl->dev, rows_of_class, cb, slots, nullptr, pl->out_begin, pl->out_end,
-                                                  c_colidx, static_cast<V*>(c_vals), 0u, nullptr, nullptr, gslots);
+    const HeavyShapes h = pl->dtype == SPSYRK_I32 ? heavy_shapes<int32_t>(pl) : heavy_shapes<double>(pl);
+    route_rows_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->route_list,
+                                                                       pl->rows_cap, pl->parts_list, pl->route_count);
     note_launches(1);
-    if (use_global) {
-        auto gkern = rows_cta_kernel<V, THREADS, true, true>;
-        const size_t gsmem = CtaRowSmem<V, THREADS, true>::bytes(cb, 0);
-        SPSYRK_CUDA_TRY(cudaFuncSetAttribute(gkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem));
-        SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->row_counter, 0, sizeof(uint32_t), st));
-        const unsigned grid = (unsigned)std::min<int64_t>(std::min<int64_t>(pl->sm_count, GLOBAL_ACC_CTAS), count);
-        gkern<<<grid, THREADS, gsmem, st>>>(pl->dev, rows_of_class, cb, slots, nullptr, pl->out_begin, pl->out_end,
-                                            c_colidx, static_cast<V*>(c_vals), (uint32_t)count, pl->row_counter,
-                                            reinterpret_cast<Acc*>(pl->gacc), gslots);
+    SPSYRK_CUDA_TRY(cudaGetLastError());
+    return SPSYRK_OK;
+}
+
+// as many CTAs as are resident at once, at most one per row
+template <typename Kernel>
+cudaError_t persistent_grid(const spsyrk_plan_s* pl, Kernel kern, int threads, size_t smem, int64_t count, unsigned* grid) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int per_sm = 1;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    *grid = (unsigned)std::min<int64_t>(count, (int64_t)pl->sm_count * std::max(per_sm, 1));
+    return e;
+}
+
+template <typename V>
+spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
+    using Acc = typename AccOf<V>::type;
+    static_assert(sizeof(Acc) == sizeof(typename AccOf<std::conditional_t<std::is_same<V, int32_t>::value, int32_t, double>>::type), "the rule's shapes");
+    uint32_t any = 0;
+    for (int k = 0; k < NROUTE; ++k) any |= pl->route_n[k];
+    if (!any) return SPSYRK_OK;
+    const HeavyShapes h = heavy_shapes<V>(pl);
+    V* cv = static_cast<V*>(c_vals);
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->dispensers, 0, NROUTE * sizeof(uint32_t), st));
+    const int64_t row_lo = pl->sub_active ? pl->sub_row_lo : 0, row_hi = pl->sub_active ? pl->sub_row_hi : INT64_MAX;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(c_colidx) | reinterpret_cast<uintptr_t>(c_vals) | reinterpret_cast<uintptr_t>(pl->dev.jaccard)) & 15u) == 0;
+    auto args = [&](int k) {
+        return HeavyArgs{pl->route_list + k * (pl->rows_cap), pl->route_n[k], pl->dispensers + k, row_lo, row_hi, pl->out_begin, pl->out_end, c_colidx, aligned,
+                         pl->parts_list, k == ROUTE_DIRECT ? pl->route_n[ROUTE_PARTS] : 0u, pl->bounds, pl->block_base, pl->blocks_per_row};
+    };
+    unsigned grid = 0;
+    auto rank = [&](auto kern, int threads, int k, uint32_t columns, uint32_t slots, size_t smem) -> cudaError_t {
+        if (!pl->route_n[k]) return cudaSuccess;
+        const cudaError_t e = persistent_grid(pl, kern, threads, smem, pl->route_n[k], &grid);
+        if (e != cudaSuccess) return e;
+        kern<<<grid, threads, smem, st>>>(pl->dev, args(k), columns, slots, cv);
+        note_launches(1);
+        return cudaGetLastError();
+    };
+    if (const int64_t units = (int64_t)pl->route_n[ROUTE_DIRECT] + pl->route_n[ROUTE_PARTS]) {
+        auto kern = rows_direct_kernel<V, DIRECT_THREADS>;
+        const size_t smem = DirectSmem<V, DIRECT_THREADS>::bytes(h.rule.chunk);
+        SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DIRECT_THREADS, smem, std::min<int64_t>(units, DIRECT_MAX_CTAS), &grid));
+        kern<<<grid, DIRECT_THREADS, smem, st>>>(pl->dev, args(ROUTE_DIRECT), h.rule.chunk, cv);
         note_launches(1);
     }
+    using Small = RankSmem<V, RANK_SMALL_THREADS>;
+    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_BIG_THREADS, 1>, RANK_BIG_THREADS, ROUTE_RANK_BIG, h.columns, h.rule.slots_big, RankSmem<V, RANK_BIG_THREADS>::bytes(h.columns, h.rule.slots_big)));
+    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_MID_THREADS, 2>, RANK_MID_THREADS, ROUTE_RANK_MID, h.columns, h.rule.slots_mid, RankSmem<V, RANK_MID_THREADS>::bytes(h.columns, h.rule.slots_mid)));
+    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_SMALL_THREADS, 4>, RANK_SMALL_THREADS, ROUTE_RANK2, h.columns, h.rule.slots_small, Small::bytes(h.columns, h.rule.slots_small)));
+    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_SMALL_THREADS, 4>, RANK_SMALL_THREADS, ROUTE_RANK1, h.rule.bits1, h.rule.slots_small, Small::bytes(h.rule.bits1, h.rule.slots_small)));
+    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_SMALL_THREADS, 4>, RANK_SMALL_THREADS, ROUTE_RANK0, h.rule.bits0, h.rule.slots_small, Small::bytes(h.rule.bits0, h.rule.slots_small)));
+    if (pl->route_n[ROUTE_DENSE8]) {
+        auto kern = rows_dense8_kernel<V, DENSE8_THREADS, 3>;
+        const size_t smem = Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns);
+        SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DENSE8_THREADS, smem, pl->route_n[ROUTE_DENSE8], &grid));
+        kern<<<grid, DENSE8_THREADS, smem, st>>>(pl->dev, args(ROUTE_DENSE8), h.dense8_columns, cv);
+        note_launches(1);
+    }
+    if (pl->route_n[ROUTE_WIDE]) {
+        constexpr int THREADS = 1024;
+        const size_t fixed = CtaRowSmem<V, THREADS, true>::bytes(h.columns, 0);
+        const uint32_t slots = std::min((uint32_t)((LARGE_SMEM_BUDGET - fixed) / sizeof(Acc)), h.columns);
+        const size_t smem = CtaRowSmem<V, THREADS, true>::bytes(h.columns, slots);
+        auto kern = rows_cta_kernel<V, THREADS, true>;
+        SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const HeavyArgs a = args(ROUTE_WIDE);
+        kern<<<pl->route_n[ROUTE_WIDE], THREADS, smem, st>>>(pl->dev, a.list, h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv, row_lo, row_hi,
+                                                             nullptr, 0u);
+        note_launches(1);
+    }
+    SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
 }
 
@@ -688,10 +791,8 @@ spsyrk_status_t numeric_typed(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals
     if (pl->map_filled) launch_numeric_map_all<V>(pl, c_colidx, c_vals, st);
     else if (pl->key64) launch_numeric_warp_all<V, uint64_t>(pl, c_colidx, c_vals, st);
     else launch_numeric_warp_all<V, uint32_t>(pl, c_colidx, c_vals, st);
-    spsyrk_status_t s = launch_numeric_cta<V, 512>(pl, 6, BLOCK_ACC_SLOTS, c_colidx, c_vals, st);
-    if (s != SPSYRK_OK) return s;
-    mark(pl, pl->ev_num, 7, st);
-    s = launch_numeric_cta<V, 1024>(pl, 7, 0u, c_colidx, c_vals, st);
+    mark(pl, pl->ev_num, 7, st);  // the heavy rows of both classes are timed as one
+    const spsyrk_status_t s = launch_heavy<V>(pl, c_colidx, c_vals, st);
     if (s != SPSYRK_OK) return s;
     mark(pl, pl->ev_num, 8, st);
     SPSYRK_CUDA_TRY(cudaGetLastError());
@@ -713,17 +814,48 @@ __global__ void upper_begin_kernel(const int64_t* __restrict__ c_rowptr, const i
     if (r < rows) hi_begin[r] = c_rowptr[r] + cnt_lo[r];
 }
 
-// prefix sums of per-row counts into out[rows + 1]; the total and the error word are on their way to the host
+// prefix sums, and for the host the total, the error word and the lengths of the heavy rows' lists (both views)
+struct CountsOut {
+    int64_t* out;
+    int64_t n;
+    const uint32_t *err, *routes;
+    int64_t* host;
+    __device__ __forceinline__ void operator()(int64_t i, int64_t ex) const { out[i] = ex; }
+    __device__ __forceinline__ void total(int64_t t) const {
+        uint32_t w[1 + 2 * NROUTE];
+        w[0] = *err;
+#pragma unroll
+        for (int k = 0; k < 2 * NROUTE; ++k) w[1 + k] = routes[k];
+        out[n] = t;
+        host[0] = t;
+#pragma unroll
+        for (int k = 0; k < 1 + 2 * NROUTE; ++k) host[1 + k] = (int64_t)w[k];
+    }
+};
+static_assert(2 + 2 * NROUTE <= 32, "the totals take the first half of the host block");
+
+// prefix sums of per-row counts into out[rows + 1]; what the host needs is on its way
 cudaError_t scan_counts(spsyrk_plan_s* pl, const int32_t* counts, int64_t rows, int64_t* out, cudaStream_t st) {
     if (rows == 0) return cudaMemsetAsync(out, 0, sizeof(int64_t), st);
-    return scan_launch(ScanArray<int32_t>{counts}, rows, ScanIntoHost{out, rows, pl->dev.err, pl->host.dev}, pl->partials, pl->dev.err, st);
+    return scan_launch(ScanArray<int32_t>{counts}, rows, CountsOut{out, rows, pl->dev.err, pl->route_count, pl->host.dev}, pl->partials, pl->dev.err, st);
 }
-// waits for them
-spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, int64_t* total, cudaStream_t st) {
+// waits for it
+spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, bool routes, int64_t* total, cudaStream_t st) {
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    if (rows == 0) { *total = 0; return SPSYRK_OK; }
-    const spsyrk_status_t s = status_of((uint32_t)pl->host.host[1]);
-    if (s == SPSYRK_OK) *total = pl->host.host[0];
+    spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
+    if (rows == 0) {
+        *total = 0;
+        if (routes) std::memset(pl->route_n, 0, sizeof(pl->route_n));
+        if (routes && up) std::memset(up->route_n, 0, sizeof(up->route_n));
+        return SPSYRK_OK;
+    }
+    const int64_t* h = pl->host.host;
+    const spsyrk_status_t s = status_of((uint32_t)h[1]);
+    if (s == SPSYRK_OK) *total = h[0];
+    for (int k = 0; routes && k < NROUTE; ++k) {
+        pl->route_n[k] = (uint32_t)h[2 + k];
+        if (up) up->route_n[k] = (uint32_t)h[2 + NROUTE + k];
+    }
     return s;
 }
 
@@ -747,8 +879,7 @@ spsyrk_status_t symbolic_view(spsyrk_plan_s* pl, bool with_map, cudaStream_t st)
     s = launch_symbolic_cta<1024>(pl, 7, st);
     if (s != SPSYRK_OK) return s;
     mark(pl, pl->ev_sym, 8, st);
-    SPSYRK_CUDA_TRY(cudaGetLastError());
-    return SPSYRK_OK;
+    return route_heavy(pl, st);
 }
 
 }  // namespace
@@ -837,7 +968,6 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
     P.rowptr = d_rowptr; P.colidx = d_colidx; P.vals = d_vals;
     pl->dtype = dtype;
     pl->user_mode = mode;
-    pl->rows_cap = m;
     pl->key64 = m > (int64_t(1) << 22);
     pl->s0 = 0;
     pl->s1 = (int32_t)m;
@@ -880,10 +1010,10 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
         heavy_assign_kernel<<<hb, 256, 0, st>>>(pl->colcnt, n, pl->facts, pl->heavy_id);
         const unsigned mb = (unsigned)std::min<int64_t>((m * 32 + 255) / 256, (int64_t)pl->sm_count * 8);
         switch (g) {
-            case 4: heavy_mask_kernel<4><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
-            case 8: heavy_mask_kernel<8><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
-            case 16: heavy_mask_kernel<16><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
-            default: heavy_mask_kernel<32><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask); break;
+            case 4: heavy_mask_kernel<4><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
+            case 8: heavy_mask_kernel<8><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
+            case 16: heavy_mask_kernel<16><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
+            default: heavy_mask_kernel<32><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
         }
         note_launches(3);
         PLAN_TRY(cudaGetLastError());
@@ -953,7 +1083,7 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t
         upper_begin_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(d_c_rowptr, pl->cnt, rows, pl->hi_begin);
         note_launches(1);
     }
-    s = collect_total(pl, rows, nnz_out, st);
+    s = collect_total(pl, rows, true, nnz_out, st);
     if (s != SPSYRK_OK) return s;
     pl->have_symbolic = true;
     pl->map_filled = with_map;
@@ -1029,6 +1159,8 @@ spsyrk_status_t spsyrk_numeric_rows(spsyrk_plan_t plan, int64_t row_begin, int64
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
         views[v]->sub_active = true;
+        views[v]->sub_row_lo = row_begin - pl->dev.r0;
+        views[v]->sub_row_hi = row_end - pl->dev.r0;
         for (int c = 0; c < NCLASS; ++c) { views[v]->sub_lo[c] = pos[v][2 * c]; views[v]->sub_hi[c] = pos[v][2 * c + 1]; }
     }
     const spsyrk_status_t s = spsyrk_numeric(plan, d_c_rowptr, d_c_colidx, d_c_vals, cuda_stream);
@@ -1048,13 +1180,14 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
     spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, st);
     if (s != SPSYRK_OK) return s;
     s = launch_symbolic_cta<1024>(pl, 7, st);
+    if (s == SPSYRK_OK) s = route_heavy(pl, st);
     if (s != SPSYRK_OK) return s;
     if (rows > 0) {
         onepass_slots_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev, pl->cls, pl->cnt, pl->diag, rows, pl->ub);
         note_launches(1);
     }
     SPSYRK_CUDA_TRY(scan_counts(pl, pl->ub, rows, pl->ub_off, st));
-    s = collect_total(pl, rows, slot_entries, st);
+    s = collect_total(pl, rows, true, slot_entries, st);
     if (s != SPSYRK_OK) return s;
     pl->have_onepass = true;
     return SPSYRK_OK;
@@ -1085,7 +1218,7 @@ spsyrk_status_t spsyrk_onepass_numeric(spsyrk_plan_t plan, int32_t* d_slot_colid
     pl->map_filled = map_was;
     if (s != SPSYRK_OK) return s;
     SPSYRK_CUDA_TRY(scan_counts(pl, pl->cnt, rows, d_c_rowptr, st));
-    return collect_total(pl, rows, nnz_out, st);
+    return collect_total(pl, rows, false, nnz_out, st);
 }
 
 spsyrk_status_t spsyrk_onepass_row_begin(spsyrk_plan_t plan, int64_t* d_row_begin, void* cuda_stream) {

@@ -1,4 +1,5 @@
-// Steps a4 / a6 for heavy rows: one CTA per output row.
+// Step a4 for heavy rows, and step a6 for those whose output range has more than 2^18 columns (the others:
+// rows_heavy.cuh): one CTA per output row.
 //
 // The output columns j of row i lie in [0, U), U = i + 1 (TRIL) or m (FULL).  The range is cut
 // into chunks of `chunk_bits` columns.  For each chunk a shared-memory bitmap records which j
@@ -37,21 +38,14 @@ struct CtaRowSmem {
     }
 };
 
-// GLOBAL_ACC: the variant for rows whose output does not fit the shared-memory accumulator tile.
-// Instead of walking the lists once per tile, it accumulates the whole row in one pass into a
-// global-memory slice owned by the CTA (global atomics, served by L2).  It runs as a persistent grid:
-// CTAs fetch rows from a counter, so that the slice indexed by blockIdx.x is never shared.  The
-// two variants are launched over the same row list and each skips the rows of the other.
-template <typename V, int THREADS, bool NUMERIC, bool GLOBAL_ACC = false>
+template <typename V, int THREADS, bool NUMERIC>
 __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) rows_cta_kernel(PlanDev P, const int32_t* __restrict__ rows,
                                                            uint32_t chunk_bits, uint32_t acc_slots,
                                                            int32_t* __restrict__ cnt,
                                                            const int64_t* __restrict__ c_rowptr, const int64_t* __restrict__ c_rowend,
                                                            int32_t* __restrict__ c_colidx, V* __restrict__ c_vals,
-                                                           uint32_t nrows = 0, uint32_t* row_counter = nullptr,
-                                                           typename AccOf<V>::type* gscratch = nullptr, uint32_t gslots = 0) {
+                                                           int64_t row_lo, int64_t row_hi, uint32_t* __restrict__ block_base, uint32_t blocks_per_row) {
     using Acc = typename AccOf<V>::type;
-    __shared__ uint32_t s_row;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t scratch[33];
     __shared__ uint32_t s_sel[2];
@@ -67,20 +61,14 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     size_t words = (size_t)cw * (NUMERIC ? 2 : 1) + 5 * THREADS + 1;
     words = (words + 3) & ~size_t(3);
     Acc* la = reinterpret_cast<Acc*>(smem_raw + words * 4);
-    Acc* acc = GLOBAL_ACC ? gscratch + (size_t)blockIdx.x * gslots : la + THREADS;
-    const uint32_t tile_slots = GLOBAL_ACC ? gslots : acc_slots;  // slots accumulated per pass over the lists
+    Acc* acc = la + THREADS;
 
     const int tid = threadIdx.x;
-    auto do_row = [&](const int32_t rloc) {
+    // later rows carry longer column prefixes: hand them out first so that the tail of the launch is light
+    const int32_t rloc = rows[gridDim.x - 1 - blockIdx.x];
+    if (NUMERIC && (rloc < row_lo || rloc >= row_hi)) return;
     const int64_t i = (int64_t)P.r0 + rloc;
     const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
-    if (NUMERIC) {
-        // rows that overflow the shared-memory tile (and are not full) belong to the global variant
-        const int64_t row_cnt = c_rowend[rloc] - c_rowptr[rloc];
-        const bool wants_global = gslots > 0 && row_cnt > (int64_t)acc_slots && U <= chunk_bits && row_cnt < (int64_t)U &&
-                                  row_cnt <= (int64_t)gslots;
-        if (wants_global != GLOBAL_ACC) return;
-    }
     const int64_t p0 = P.rowptr[i];
     const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
     const int64_t out_base = NUMERIC ? c_rowptr[rloc] : 0;
@@ -89,40 +77,27 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     uint32_t total_cnt = 0;
 
     // A row whose range fits one chunk and that holds a column present in every candidate row
-    // (a list as long as the range) is dense: every j occurs, slot = j, no bitmap is needed.
-    bool dense = false;
-    if (U <= chunk_bits) {
+    // (a list as long as the range) is dense: every j occurs, no bitmap is needed to count them.
+    if (!NUMERIC && U <= chunk_bits) {
         int hit = 0;
         for (uint32_t b0 = tid; b0 < deg; b0 += THREADS) hit |= (P.desc[p0 + b0].y == U);
-        dense = __syncthreads_or(hit) != 0;
+        if (__syncthreads_or(hit)) {
+            if (tid == 0) cnt[rloc] = (int32_t)U;
+            return;
+        }
     }
-    if (dense && !NUMERIC) {
-        if (tid == 0) cnt[rloc] = (int32_t)U;
-        return;
-    }
-    // Binary input: a partial product is 1.  In a dense row the heavy columns' share of every count comes
-    // from the per-row bit masks (one population count per entry), and their lists are not walked.
     const bool binary = P.binary != 0;
-    const bool use_masks = NUMERIC && dense && binary && *P.nheavy > 0;
-    const unsigned long long mask_i = use_masks ? P.heavy_mask[i] : 0ull;
-    // Binary input, dense row of at most 255 nonzeros: every count is at most the row's own length, so four
-    // 8-bit counters share a 32-bit word of the accumulator tile and a tile holds four times the columns
-    // (a row of 1e5 columns is one tile: its lists are cut into column ranges once, not once per tile).
-    const bool packed = NUMERIC && !GLOBAL_ACC && std::is_same<V, int32_t>::value && dense && binary && deg <= 255u;
-    const uint32_t row_tile_slots = packed ? tile_slots * 4u : tile_slots;
 
     // One partial product: set its bit, or add it into its slot.
-    auto apply = [&](auto what, auto dense_tag, uint32_t rel, Acc a, Acc v, uint32_t s0) {
+    auto apply = [&](auto what, uint32_t rel, Acc a, Acc v, uint32_t s0) {
         constexpr int WHAT = decltype(what)::value;
-        constexpr bool DENSE = decltype(dense_tag)::value;
         if (WHAT == CTA_SETBITS) {
             if (SPSYRK_IN_RANGE((rel >> 5) < cw, P.err)) atomicOr(&bits[rel >> 5], 1u << (rel & 31));
         } else {
-            if (!SPSYRK_IN_RANGE(DENSE || (rel >> 5) < cw, P.err)) return;
-            const uint32_t slot = (DENSE ? rel : rank[rel >> 5] + __popc(bits[rel >> 5] & ((1u << (rel & 31)) - 1u))) - s0;
-            if (!SPSYRK_IN_RANGE(slot < row_tile_slots, P.err)) return;
-            if (DENSE && packed) atomicAdd(reinterpret_cast<uint32_t*>(acc) + (slot >> 2), 1u << ((slot & 3u) * 8u));  // a product of a binary matrix is 1
-            else atomicAdd(&acc[slot], acc_mul(a, v));
+            if (!SPSYRK_IN_RANGE((rel >> 5) < cw, P.err)) return;
+            const uint32_t slot = rank[rel >> 5] + __popc(bits[rel >> 5] & ((1u << (rel & 31)) - 1u)) - s0;
+            if (!SPSYRK_IN_RANGE(slot < acc_slots, P.err)) return;
+            atomicAdd(&acc[slot], acc_mul(a, v));
         }
     };
 
@@ -135,7 +110,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     // `resume`: the range starts where the previous call's range ended (consecutive slot tiles of a row
     // with at most THREADS lists), so each list's lower end is remembered instead of searched again.
     // ones_tag: the partial products are ones (binary input, or the bit-setting pass): only row ids are read
-    auto for_each_product = [&](auto what, auto dense_tag, auto ones_tag, uint32_t lo, uint32_t hi, bool whole, uint32_t c0, uint32_t s0,
+    auto for_each_product = [&](auto what, auto ones_tag, uint32_t lo, uint32_t hi, bool whole, uint32_t c0, uint32_t s0,
                                 bool resume) {
         constexpr int WHAT = decltype(what)::value;
         constexpr bool ONES = decltype(ones_tag)::value || WHAT != CTA_ACCUM;
@@ -144,8 +119,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
             Acc a = Acc(0);
             if (tid == 0) s_nlong = 0;
             if (b0 + tid < deg) {
-                uint2 d = P.desc[p0 + b0 + tid];
-                if (WHAT == CTA_ACCUM && use_masks && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
+                const uint2 d = P.desc[p0 + b0 + tid];
                 if (whole) {
                     substart = d.x;
                     sublen = d.y;
@@ -225,7 +199,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
                         }
 #pragma unroll
                         for (int u = 0; u < UNR; ++u)
-                            if (q[u] != 0xffffffffu) apply(what, dense_tag, rel[u], av[u], val[u], s0);
+                            if (q[u] != 0xffffffffu) apply(what, rel[u], av[u], val[u], s0);
                     }
                 }
             }
@@ -253,14 +227,14 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
                         }
                     }
 #pragma unroll
-                    for (int u = 0; u < UNR; ++u) apply(what, dense_tag, rel[u], fa, val[u], s0);
+                    for (int u = 0; u < UNR; ++u) apply(what, rel[u], fa, val[u], s0);
                 }
                 for (; e < len; e += THREADS) {
                     if constexpr (!ONES) {
                         const ColRec<V> rec = recp[e];
-                        apply(what, dense_tag, (uint32_t)rec.j - c0, fa, (Acc)rec.v, s0);
+                        apply(what, (uint32_t)rec.j - c0, fa, (Acc)rec.v, s0);
                     } else {
-                        apply(what, dense_tag, (uint32_t)rowp[e] - c0, fa, Acc(1), s0);
+                        apply(what, (uint32_t)rowp[e] - c0, fa, Acc(1), s0);
                     }
                 }
             }
@@ -269,8 +243,8 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     };
     const std::integral_constant<int, CTA_SETBITS> SET{};
     const std::integral_constant<int, CTA_ACCUM> ACC{};
-    const std::true_type IS_DENSE{};
-    const std::false_type NOT_DENSE{};
+    const std::true_type ONES{};
+    const std::false_type VALUES{};
 
     for (uint32_t c0 = 0; c0 < U; c0 += chunk_bits) {
         const uint32_t c1 = min(c0 + chunk_bits, U);
@@ -278,14 +252,45 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
         const uint32_t cwa = (c1 - c0 + 31) >> 5;  // words of the bitmap this chunk uses
         const uint32_t per = (cwa + THREADS - 1) / THREADS;
         const uint32_t w0 = tid * per;
-        uint32_t tot = c1 - c0;
-        if (!dense) {
+        uint32_t tot;
+        {
             for (uint32_t w = tid; w < cwa; w += THREADS) bits[w] = 0;
             __syncthreads();
-            for_each_product(SET, NOT_DENSE, IS_DENSE, c0, c1, single_chunk, c0, 0u, false);
-            uint32_t s = 0;
-            for (uint32_t w = w0; w < w0 + per && w < cwa; ++w) s += __popc(bits[w]);
-            uint32_t ex = block_exclusive_scan<uint32_t, THREADS>(s, scratch, &tot);
+            for_each_product(SET, ONES, c0, c1, single_chunk, c0, 0u, false);
+            uint32_t ex = 0;
+            if constexpr (!NUMERIC) {
+                // a warp counts a block of BASE_BLOCK columns at a time; rows of at most blocks_per_row blocks keep the
+                // counts before each block, which lets the numeric pass compute parts of a row apart
+                constexpr uint32_t BW = BASE_BLOCK / 32;
+                const uint32_t nblk = (cwa + BW - 1) / BW;
+                for (uint32_t blk = tid >> 5; blk < nblk; blk += THREADS / 32) {
+                    uint32_t s = 0;
+#pragma unroll
+                    for (uint32_t q = 0; q < BW / 32; ++q) {
+                        const uint32_t w = blk * BW + q * 32 + (tid & 31);
+                        if (w < cwa) s += __popc(bits[w]);
+                    }
+                    s = warp_reduce_sum<uint32_t>(s);
+                    if ((tid & 31) == 0) loff[blk] = s;  // (at most 256 blocks in a chunk: the list offsets' space)
+                }
+                __syncthreads();
+                if (tid < 32) {
+                    uint32_t run = 0;
+                    for (uint32_t b0 = 0; b0 < nblk; b0 += 32) {
+                        const uint32_t v = b0 + tid < nblk ? loff[b0 + tid] : 0u;
+                        const uint32_t incl = warp_inclusive_scan<uint32_t>(v);
+                        if (b0 + tid < nblk && single_chunk && nblk <= blocks_per_row) block_base[(uint64_t)i * blocks_per_row + b0 + tid] = run + incl - v;
+                        run += __shfl_sync(FULL_MASK, incl, 31);
+                    }
+                    if (tid == 0) s_sel[0] = run;
+                }
+                __syncthreads();
+                tot = s_sel[0];
+            } else {
+                uint32_t s = 0;
+                for (uint32_t w = w0; w < w0 + per && w < cwa; ++w) s += __popc(bits[w]);
+                ex = block_exclusive_scan<uint32_t, THREADS>(s, scratch, &tot);
+            }
             if (NUMERIC) {
                 for (uint32_t w = w0; w < w0 + per && w < cwa; ++w) { rank[w] = ex; ex += __popc(bits[w]); }
                 __syncthreads();
@@ -293,7 +298,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
         }
         if (NUMERIC) {
             const int64_t ob = out_base + total_cnt;
-            if (!dense) {  // (a dense row writes its column ids, c0 + slot, with its values below)
+            {
                 // column ids straight from the bitmap
                 for (uint32_t w = tid; w < cwa; w += THREADS) {
                     uint32_t b = bits[w], r = rank[w];
@@ -305,14 +310,11 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
                     }
                 }
             }
-            for (uint32_t s0 = 0; s0 < tot; s0 += row_tile_slots) {
-                const uint32_t s1 = min(s0 + row_tile_slots, tot);
+            for (uint32_t s0 = 0; s0 < tot; s0 += acc_slots) {
+                const uint32_t s1 = min(s0 + acc_slots, tot);
                 const bool single_tile = (s0 == 0 && s1 == tot);
                 uint32_t jlo = c0, jhi = c1;
-                if (!single_tile && dense) {
-                    jlo = c0 + s0;
-                    jhi = c0 + s1;
-                } else if (!single_tile) {
+                if (!single_tile) {
                     if (tid < 2) {
                         const uint32_t sl = tid == 0 ? s0 : s1;
                         uint32_t res;
@@ -335,46 +337,20 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
                     jlo = s_sel[0];
                     jhi = s_sel[1];
                 }
-                if (packed) {
-                    // slot t of a dense row is column c0 + s0 + t; word w holds slots 4 w .. 4 w + 3
-                    const uint64_t* mk = P.heavy_mask + c0 + s0;
-                    uint32_t* acc32 = reinterpret_cast<uint32_t*>(acc);
-                    for (uint32_t w = tid; w < (s1 - s0 + 3u) / 4u; w += THREADS) {
-                        uint32_t word = 0;
-                        if (use_masks) {
-#pragma unroll
-                            for (uint32_t q = 0; q < 4; ++q)
-                                if (4u * w + q < s1 - s0) word |= (uint32_t)__popcll((unsigned long long)mk[4u * w + q] & mask_i) << (8u * q);
-                        }
-                        acc32[w] = word;
-                    }
-                } else if (use_masks) {
-                    // slot t of a dense row is column c0 + s0 + t
-                    const uint64_t* mk = P.heavy_mask + c0 + s0;
-                    for (uint32_t t = tid; t < s1 - s0; t += THREADS) acc[t] = Acc(__popcll((unsigned long long)mk[t] & mask_i));
-                } else {
-                    for (uint32_t t = tid; t < s1 - s0; t += THREADS) acc[t] = Acc(0);
-                }
+                for (uint32_t t = tid; t < s1 - s0; t += THREADS) acc[t] = Acc(0);
                 __syncthreads();
                 const bool resume = s0 > 0 && deg <= THREADS;
                 const bool whole_row = single_chunk && single_tile;
-                if (binary) {  // (the tags are std::true_type / std::false_type: here "the products are ones")
-                    if (dense) for_each_product(ACC, IS_DENSE, IS_DENSE, jlo, jhi, whole_row, c0, s0, resume);
-                    else for_each_product(ACC, NOT_DENSE, IS_DENSE, jlo, jhi, whole_row, c0, s0, resume);
-                } else {
-                    if (dense) for_each_product(ACC, IS_DENSE, NOT_DENSE, jlo, jhi, whole_row, c0, s0, resume);
-                    else for_each_product(ACC, NOT_DENSE, NOT_DENSE, jlo, jhi, whole_row, c0, s0, resume);
-                }
+                if (binary) for_each_product(ACC, ONES, jlo, jhi, whole_row, c0, s0, resume);
+                else for_each_product(ACC, VALUES, jlo, jhi, whole_row, c0, s0, resume);
                 for (uint32_t t = tid; t < s1 - s0; t += THREADS) {
                     if (!SPSYRK_IN_RANGE(ob + s0 + t < out_end, P.err)) continue;
-                    const V cv = packed ? (V)((reinterpret_cast<const uint32_t*>(acc)[t >> 2] >> ((t & 3u) * 8u)) & 0xffu)
-                                        : (V)(GLOBAL_ACC ? __ldcg(acc + t) : acc[t]);
+                    const V cv = (V)acc[t];
                     c_vals[ob + s0 + t] = cv;
-                    if (dense) c_colidx[ob + s0 + t] = (int32_t)(c0 + s0 + t);
                     if constexpr (std::is_same<V, int32_t>::value) {
                         if (P.jaccard) {
-                            // J = c / (|a_i| + |a_j| - c); the column id was written above (dense rows: it is the slot's column)
-                            const int64_t j = dense ? (int64_t)(c0 + s0 + t) : (int64_t)c_colidx[ob + s0 + t];
+                            // J = c / (|a_i| + |a_j| - c); the column id was written above
+                            const int64_t j = c_colidx[ob + s0 + t];
                             const int64_t na_j = P.adeg[j];
                             P.jaccard[ob + s0 + t] = __fdiv_rn((float)cv, (float)((int64_t)deg + na_j - (int64_t)cv));
                         }
@@ -387,22 +363,6 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
         __syncthreads();
     }
     if (!NUMERIC && tid == 0) cnt[rloc] = (int32_t)total_cnt;
-    };  // do_row
-
-    if (GLOBAL_ACC) {
-        for (;;) {
-            if (tid == 0) s_row = atomicAdd(row_counter, 1u);
-            __syncthreads();
-            const uint32_t r = s_row;
-            __syncthreads();
-            if (r >= nrows) break;
-            do_row(rows[nrows - 1 - r]);
-            __syncthreads();
-        }
-    } else {
-        // later rows carry longer column prefixes: hand them out first so that the tail of the launch is light
-        do_row(rows[gridDim.x - 1 - blockIdx.x]);
-    }
 }
 
 }  // namespace spsyrk

@@ -1,0 +1,585 @@
+// Step a6 for heavy rows whose output range [0, U) has at most 2^18 columns: the symbolic pass leaves the number of
+// entries of every row, and a row goes to the kernel that suits it (route_rows_kernel):
+//   rank   : a bitmap of the columns that occur, prefix population counts turn it into column -> slot, partial products
+//            are added into slots.  Two walks over the lists, shared memory by the row's entries.  Sparse rows.
+//   direct : accumulators indexed by column, for a chunk of columns at a time.  One walk, no ranks, but every column
+//            of the range is swept.  Rows that fill their range, or have more entries than slots fit an SM.  A long
+//            row is cut into parts of whole chunks: the symbolic pass has left the number of entries before every block of columns.
+//   dense8 : rows of a binary matrix in which every column occurs: four 8-bit counters per word, the heaviest
+//            columns counted through bit masks.
+// All are persistent: a CTA takes its next row from a counter, so that no launch waits for its longest row's wave and
+// a CTA's buffers stay where they are.
+//
+// Before, every heavy row went through a bitmap, 32-bit ranks and one size of slots (512 threads up to 32768 products, 1024
+// above), rows with more entries than slots into global slices with L2 atomics, dense rows of binary matrices
+// through a 200 KB tile with one CTA per SM.  Large power-law workload (96 000 heavy rows, 1.46e9 products, single precision):
+// 7.3 + 7.4 + 0.6 ms before, rank 5.9 ms (0.6e9 products) and direct 8.8 ms now; binary Zipf workload of 50000 rows
+// (1.25e9 counts and similarities): 10.8 ms before, dense8 4.4 ms = 3.4 TB/s of output.
+#pragma once
+#include "transpose.cuh"
+
+namespace spsyrk {
+
+enum : int { ROUTE_RANK0 = 0, ROUTE_RANK1, ROUTE_RANK2, ROUTE_RANK_MID, ROUTE_RANK_BIG, ROUTE_DIRECT, ROUTE_PARTS, ROUTE_DENSE8, ROUTE_WIDE, NROUTE };
+
+constexpr int DIRECT_MAX_PARTS = 8;
+constexpr int64_t DIRECT_PART_WORK = 131072;  // products of a part of a row, at least
+
+// What the choice needs to know; bytes are shared memory of the kernels as launched
+struct RouteRule {
+    uint32_t slots_small, slots_mid, slots_big;  // slots of the rank kernels
+    uint32_t bits0, bits1;                       // columns of the two narrower bitmaps of the small rank kernel
+    uint32_t wide;                               // ranges above this go to the chunked kernel
+    uint32_t chunk;                              // columns per chunk of the direct kernel
+    uint32_t dense8;                             // columns the packed counters of one row may have
+    int binary;
+};
+
+// One thread per heavy row (classes 6 and 7, the last rows first: they carry the longest lists).
+static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, RouteRule R, const int32_t* __restrict__ rows, int64_t count,
+                                                                const int32_t* __restrict__ cnt, int32_t* __restrict__ lists, int64_t cap,
+                                                                int2* __restrict__ parts_list, uint32_t* __restrict__ counters) {
+    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int route = -1, parts = 1;
+    int32_t rloc = 0;
+    if (n < count) {
+        rloc = rows[count - 1 - n];
+        const int64_t i = (int64_t)P.r0 + rloc;
+        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const uint32_t entries = (uint32_t)cnt[rloc];
+        const int64_t w = P.work[rloc], deg = P.rowptr[i + 1] - P.rowptr[i];
+        const uint32_t chunks = (U + R.chunk - 1) / R.chunk;
+        // Direct against rank: a product costs about 25 cycles of an SM per 32 in one walk against 38 in two, a column of the
+        // range 1/8 against 1/40 of a cycle, a chunk after the first about 3000 for its searches and barriers.
+        if (U > R.wide) route = ROUTE_WIDE;
+        else if (R.binary && entries == U && deg <= 255 && U <= R.dense8) route = ROUTE_DENSE8;
+        else if (entries > R.slots_big || w >= (int64_t)(U / 4) + (int64_t)(chunks - 1) * 7000) {
+            // one CTA on the longest row (1e6 products) took as long as all the others together
+            parts = (int)min(min(w / DIRECT_PART_WORK, (int64_t)DIRECT_MAX_PARTS), (int64_t)chunks);
+            route = parts > 1 ? ROUTE_PARTS : ROUTE_DIRECT;
+        }
+        else if (entries <= R.slots_small) route = U <= R.bits0 ? ROUTE_RANK0 : U <= R.bits1 ? ROUTE_RANK1 : ROUTE_RANK2;
+        else route = entries <= R.slots_mid ? ROUTE_RANK_MID : ROUTE_RANK_BIG;
+    }
+#pragma unroll
+    for (int k = 0; k < NROUTE; ++k) {  // one atomic per warp and route
+        if (k == ROUTE_PARTS) continue;
+        const unsigned votes = __ballot_sync(FULL_MASK, route == k);
+        if (route == k) {
+            const int leader = __ffs(votes) - 1;
+            uint32_t base = 0;
+            if (lane_id() == leader) base = atomicAdd(&counters[k], (uint32_t)__popc(votes));
+            base = __shfl_sync(votes, base, leader);
+            lists[(int64_t)k * cap + base + __popc(votes & ((1u << lane_id()) - 1u))] = rloc;
+        }
+    }
+    if (route == ROUTE_PARTS) {
+        const uint32_t base = atomicAdd(&counters[ROUTE_PARTS], (uint32_t)parts);
+        for (int k = 0; k < parts; ++k) parts_list[base + k] = make_int2(rloc, k | parts << 8);
+    }
+}
+
+// The lists of a row, up to THREADS of them at a time, flattened through a prefix sum of their lengths
+template <typename Acc, int THREADS>
+struct ListBatch {
+    uint32_t off[THREADS + 1];
+    uint32_t start[THREADS];
+    Acc a[THREADS];
+    uint32_t warp_sum[THREADS / 32];
+};
+
+// Every thread brings one list (len may be 0).  Contains barriers, the last statement is one.
+template <typename Acc, int THREADS>
+__device__ __forceinline__ void batch_fill(ListBatch<Acc, THREADS>& B, uint32_t start, uint32_t len, Acc a) {
+    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const uint32_t incl = warp_inclusive_scan<uint32_t>(len);
+    if (lane == 31) B.warp_sum[warp] = incl;
+    __syncthreads();
+    const uint32_t ws = lane < THREADS / 32 ? B.warp_sum[lane] : 0u;
+    const uint32_t before = warp_reduce_sum<uint32_t>(lane < warp ? ws : 0u);
+    B.off[tid] = before + incl - len;
+    B.start[tid] = start;
+    B.a[tid] = a;
+    if (tid == THREADS - 1) B.off[THREADS] = before + incl;
+    __syncthreads();
+}
+
+// Every warp takes a contiguous run of the flattened items and its lanes interleave inside it: loads are coalesced and UNR
+// of them in flight; a lane steps from list to list as its items advance.  fn(position in the column lists, a).
+template <typename Acc, int THREADS, int UNR, typename Load, typename Apply>
+__device__ __forceinline__ void batch_walk(const ListBatch<Acc, THREADS>& B, Load load, Apply apply) {
+    constexpr uint32_t NW = THREADS / 32;
+    const uint32_t T = B.off[THREADS];
+    const uint32_t per_warp = ((T + NW - 1) / NW + 31u) & ~31u;
+    const uint32_t wfirst = min((uint32_t)(threadIdx.x >> 5) * per_warp, T), last = min(wfirst + per_warp, T);
+    const uint32_t first = wfirst + lane_id();
+    if (first >= last) return;
+    uint32_t lo = 0, hi = THREADS;  // last list whose offset is <= first
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (B.off[mid] <= first) lo = mid; else hi = mid;
+    }
+    uint32_t cur = lo, next = B.off[cur + 1], shift = B.start[cur] - B.off[cur];
+    Acc a = B.a[cur];
+    using L = decltype(load(0u));
+    for (uint32_t item0 = first; item0 < last; item0 += UNR * 32) {
+        L v[UNR];
+        Acc av[UNR];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            const uint32_t item = item0 + u * 32;
+            if (item < last) {
+                if (item >= next) {
+                    do { ++cur; } while (item >= B.off[cur + 1]);
+                    next = B.off[cur + 1];
+                    shift = B.start[cur] - B.off[cur];
+                    a = B.a[cur];
+                }
+                v[u] = load(shift + item);
+                av[u] = a;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < UNR; ++u)
+            if (item0 + u * 32 < last) apply(v[u], av[u]);
+    }
+}
+
+struct HeavyArgs {
+    const int32_t* list;
+    uint32_t count;
+    uint32_t* dispenser;
+    int64_t row_lo, row_hi;    // rows of the plan's range to compute
+    const int64_t* out_begin;  // where each row's part of the output starts / ends
+    const int64_t* out_end;
+    int32_t* c_colidx;
+    bool aligned;              // the output arrays start on 16-byte boundaries
+    // direct kernel
+    const int2* parts;         // parts of long rows: (row, part | parts << 8), computed before the list
+    uint32_t nparts;
+    uint32_t* bounds;          // scratch of DIRECT_BOUNDS words per CTA
+    const uint32_t* block_base;  // [absolute row * blocks_per_row + block]: entries of the row before the block of columns
+    uint32_t blocks_per_row;
+};
+
+// The rows of a persistent CTA, one after the other.  Thread 0 draws the number after next while the row is computed.
+struct RowQueue {
+    uint32_t n;
+    __device__ __forceinline__ explicit RowQueue(const HeavyArgs& H) { n = threadIdx.x == 0 ? atomicAdd(H.dispenser, 1u) : 0u; }
+    // the next row (or part of one), or -1; contains barriers, after which the row before is finished by all threads
+    __device__ __forceinline__ int2 next(const HeavyArgs& H, int2* s_row) {
+        if (threadIdx.x == 0) {
+            int2 r = make_int2(-1, 0);
+            while (n < H.nparts + H.count) {
+                const int2 c = n < H.nparts ? H.parts[n] : make_int2(H.list[n - H.nparts], 1 << 8);
+                n = atomicAdd(H.dispenser, 1u);
+                if (c.x >= H.row_lo && c.x < H.row_hi) { r = c; break; }  // (a row range: spsyrk_numeric_rows)
+            }
+            *s_row = r;
+        }
+        __syncthreads();
+        const int2 r = *s_row;
+        __syncthreads();
+        return r;
+    }
+};
+
+template <typename V>
+__device__ __forceinline__ void store_jaccard(const PlanDev& P, int64_t at, int32_t j, int32_t c, int32_t deg) {
+    // |a_i| + |a_j| - c < 2^31: the sum of two row lengths minus what they share
+    P.jaccard[at] = __fdiv_rn((float)c, (float)(uint32_t)(deg + P.adeg[j] - c));
+}
+
+// ---------------------------------------------------------------------------------------------
+// rank
+// ---------------------------------------------------------------------------------------------
+template <typename V, int THREADS>
+struct RankSmem {
+    using Acc = typename AccOf<V>::type;
+    static size_t bytes(uint32_t columns, uint32_t slots) {
+        return (size_t)columns / 8 + (size_t)columns / 32 + (size_t)slots * sizeof(Acc) + sizeof(ListBatch<Acc, THREADS>) + 16;
+    }
+};
+
+// Bound by latency and by the shared-memory pipe (adds of doubles are compare-and-swap loops, 21 cycles per 32): what
+// counts is how many rows an SM has under way, so the bitmap has 16-bit ranks per 64 columns (a rank per 32-bit
+// word: twice the shared memory) and the slots come in three sizes.
+template <typename V, int THREADS, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, HeavyArgs H, uint32_t columns, uint32_t slots, V* __restrict__ c_vals) {
+    using Acc = typename AccOf<V>::type;
+    constexpr int NW = THREADS / 32;
+    extern __shared__ __align__(16) unsigned char rk_smem[];
+    __shared__ int2 s_row;
+    __shared__ uint32_t s_warp[NW];
+    unsigned long long* bits = reinterpret_cast<unsigned long long*>(rk_smem);                 // [columns / 64]
+    Acc* acc = reinterpret_cast<Acc*>(bits + columns / 64);                                   // [slots]
+    ListBatch<Acc, THREADS>& B = *reinterpret_cast<ListBatch<Acc, THREADS>*>(acc + slots);
+    uint16_t* rank = reinterpret_cast<uint16_t*>(reinterpret_cast<unsigned char*>(acc + slots) + (sizeof(ListBatch<Acc, THREADS>) + 15) / 16 * 16);  // [columns / 64]
+    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const bool ones = P.binary != 0;
+    const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
+    uint32_t* bits32 = reinterpret_cast<uint32_t*>(bits);
+    for (uint32_t w = tid; w < columns / 64; w += THREADS) bits[w] = 0;
+
+    RowQueue queue(H);
+    for (;;) {
+        const int32_t rloc = queue.next(H, &s_row).x;
+        if (rloc < 0) break;
+        const int64_t i = (int64_t)P.r0 + rloc;
+        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const int64_t p0 = P.rowptr[i];
+        const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
+        const int64_t ob = H.out_begin[rloc];
+        const uint32_t entries = (uint32_t)(H.out_end[rloc] - ob);
+        auto fill = [&](uint32_t b0) {
+            const bool on = b0 + tid < deg;
+            const uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
+            const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
+            batch_fill<Acc, THREADS>(B, d.x, d.y, a);
+        };
+        // the columns that occur
+        for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+            if (b0) __syncthreads();
+            fill(b0);
+            batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) {
+                if (SPSYRK_IN_RANGE((uint32_t)j < columns, P.err)) atomicOr(&bits32[(uint32_t)j >> 5], 1u << ((uint32_t)j & 31u));
+            });
+        }
+        for (uint32_t t = tid; t < entries; t += THREADS) acc[t] = Acc(0);
+        __syncthreads();
+        // ranks: a warp owns consecutive words, 32 per step
+        const uint32_t words = (U + 63u) / 64u;
+        const uint32_t per_warp = ((words + NW - 1) / NW + 31u) & ~31u;
+        const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
+        uint32_t sum = 0;
+        for (uint32_t w = w0 + lane; w < w1; w += 32) sum += __popcll(bits[w]);
+        sum = warp_reduce_sum<uint32_t>(sum);
+        if (lane == 0) s_warp[warp] = sum;
+        __syncthreads();
+        uint32_t run = warp_reduce_sum<uint32_t>(lane < warp ? s_warp[lane < NW ? lane : 0] : 0u);
+        for (uint32_t w = w0; w < w1; w += 32) {
+            const uint32_t c = w + lane < w1 ? __popcll(bits[w + lane]) : 0u;
+            const uint32_t incl = warp_inclusive_scan<uint32_t>(c);
+            if (w + lane < w1) rank[w + lane] = (uint16_t)(run + incl - c);
+            run += __shfl_sync(FULL_MASK, incl, 31);
+        }
+        __syncthreads();
+        // the products
+        auto add = [&](uint32_t j, Acc p) {
+            if (!SPSYRK_IN_RANGE(j < columns, P.err)) return;
+            const uint32_t slot = rank[j >> 6] + __popcll(bits[j >> 6] & ((1ull << (j & 63u)) - 1ull));
+            if (SPSYRK_IN_RANGE(slot < entries && slot < slots, P.err)) atomicAdd(&acc[slot], p);
+        };
+        for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+            if (deg > THREADS) {  // (one batch: the lists are still there)
+                if (b0) __syncthreads();
+                fill(b0);
+            }
+            if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
+            else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc a) { add((uint32_t)r.j, acc_mul(a, (Acc)r.v)); });
+        }
+        __syncthreads();
+        // out: sums by slot, column ids from the bitmap, which is cleared for the next row
+        for (uint32_t t = tid; t < entries; t += THREADS) c_vals[ob + t] = (V)acc[t];
+        for (uint32_t w = tid; w < words; w += THREADS) {
+            unsigned long long b = bits[w];
+            if (b == 0) continue;
+            bits[w] = 0;
+            uint32_t r = rank[w];
+            while (b) {
+                const int32_t j = (int32_t)(w * 64u) + __ffsll((long long)b) - 1;
+                b &= b - 1;
+                if (SPSYRK_IN_RANGE(r < entries, P.err)) {
+                    H.c_colidx[ob + r] = j;
+                    if constexpr (std::is_same<V, int32_t>::value)
+                        if (P.jaccard) store_jaccard<V>(P, ob + r, j, acc[r], (int32_t)deg);
+                }
+                ++r;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// direct
+// ---------------------------------------------------------------------------------------------
+template <typename V, int THREADS>
+struct DirectSmem {
+    using Acc = typename AccOf<V>::type;
+    static size_t bytes(uint32_t chunk) {
+        return (size_t)chunk * (sizeof(Acc) + 1) + (size_t)chunk / 32 * 4 + sizeof(ListBatch<Acc, THREADS>) + 16;
+    }
+};
+
+constexpr int DIRECT_THREADS = 512;
+constexpr int DIRECT_MAX_CHUNKS = 32;  // 2^18 columns in chunks of BASE_BLOCK columns at least
+constexpr int DIRECT_MAX_CTAS = 320;
+constexpr size_t DIRECT_BOUNDS = (size_t)DIRECT_MAX_CHUNKS * DIRECT_THREADS;
+
+// Where the lists of a row pass from one chunk to the next: bounds[c * THREADS + l] = entries of list l in columns below
+// (c + 1) * chunk, for every list and the boundaries k0 <= c < k1 at once: all searches together take little longer than
+// those of one boundary.  At most THREADS lists.
+template <int THREADS>
+__device__ __forceinline__ void list_bounds(const PlanDev& P, int64_t p0, uint32_t deg, uint32_t chunk, uint32_t k0, uint32_t k1, uint32_t* __restrict__ bounds) {
+    constexpr int ILP = 4;
+    const uint32_t total = k1 > k0 ? deg * (k1 - k0) : 0u;
+    for (uint32_t s0 = threadIdx.x; s0 < total; s0 += ILP * THREADS) {
+        const int32_t* lst[ILP];
+        uint32_t lo[ILP], len[ILP], most = 0;
+        int32_t key[ILP];
+#pragma unroll
+        for (int u = 0; u < ILP; ++u) {
+            const uint32_t s = s0 + u * THREADS, c = s / deg;
+            const uint2 d = s < total ? P.desc[p0 + (s - c * deg)] : make_uint2(0u, 0u);
+            lst[u] = P.at_row + d.x;
+            lo[u] = 0;
+            len[u] = d.y;
+            key[u] = (int32_t)((k0 + c + 1) * chunk);
+            most = max(most, d.y);
+        }
+        for (; most > 0; most >>= 1) {
+            int32_t v[ILP];
+#pragma unroll
+            for (int u = 0; u < ILP; ++u) v[u] = len[u] ? lst[u][lo[u] + (len[u] >> 1)] : 0;
+#pragma unroll
+            for (int u = 0; u < ILP; ++u) {
+                if (len[u]) {
+                    const uint32_t half = len[u] >> 1;
+                    if (v[u] < key[u]) { lo[u] += half + 1; len[u] -= half + 1; } else len[u] = half;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < ILP; ++u) {
+            const uint32_t s = s0 + u * THREADS, c = s / deg;
+            if (s < total && SPSYRK_IN_RANGE(k0 + c < (uint32_t)DIRECT_MAX_CHUNKS, P.err)) bounds[(k0 + c) * THREADS + (s - c * deg)] = lo[u];
+        }
+    }
+}
+
+// a row's bits of the heavy columns (planes in use: 32 columns each)
+struct HeavyMask {
+    uint32_t w[HEAVY_PLANES];
+};
+__device__ __forceinline__ HeavyMask load_heavy_mask(const PlanDev& P, int64_t i, int planes) {
+    HeavyMask k;
+#pragma unroll
+    for (int p = 0; p < HEAVY_PLANES; ++p) k.w[p] = p < planes ? P.heavy_mask[p * P.mask_stride + i] : 0u;
+    return k;
+}
+__device__ __forceinline__ int heavy_planes(const PlanDev& P) { return (int)((min(*P.nheavy, (uint32_t)HEAVY_MAX) + 31u) / 32u); }
+
+// Bound by the adds in shared memory.  Two CTAs of 512 threads per SM: one searches and sweeps while the other adds.
+// A column that occurs is marked by a plain byte store (a bitmap needs an atomic or a look first; accumulators that
+// start as a special NaN need a compare-and-swap loop of their own, which took five times the built-in add).
+template <typename V, int THREADS>
+__global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, HeavyArgs H, uint32_t chunk, V* __restrict__ c_vals) {
+    using Acc = typename AccOf<V>::type;
+    constexpr int NW = THREADS / 32;
+    extern __shared__ __align__(16) unsigned char dr_smem[];
+    __shared__ int2 s_row;
+    __shared__ uint32_t s_warp[NW];
+    Acc* acc = reinterpret_cast<Acc*>(dr_smem);                                          // [chunk]
+    uint8_t* occurs = reinterpret_cast<uint8_t*>(acc + chunk);                           // [chunk]
+    uint32_t* votes = reinterpret_cast<uint32_t*>(occurs + chunk);                       // [chunk / 32]
+    ListBatch<Acc, THREADS>& B = *reinterpret_cast<ListBatch<Acc, THREADS>*>(votes + chunk / 32);
+    uint32_t* const bounds = H.bounds + blockIdx.x * DIRECT_BOUNDS;
+    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const bool ones = P.binary != 0;
+    const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
+    for (uint32_t t = tid; t < chunk; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
+
+    RowQueue queue(H);
+    for (;;) {
+        const int2 unit = queue.next(H, &s_row);
+        const int32_t rloc = unit.x;
+        if (rloc < 0) break;
+        const int64_t i = (int64_t)P.r0 + rloc;
+        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const int64_t p0 = P.rowptr[i];
+        const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
+        const int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
+        const bool dense = oe - ob == (int64_t)U;  // every column occurs
+        const int planes = ones && dense ? heavy_planes(P) : 0;
+        const bool use_masks = planes > 0;
+        const HeavyMask mine = load_heavy_mask(P, i, planes);
+        const uint32_t nchunks = (U + chunk - 1) / chunk, part = unit.y & 0xff, parts = (uint32_t)unit.y >> 8;
+        const uint32_t ca = nchunks * part / parts, cb = nchunks * (part + 1) / parts;  // chunks of this part
+        const bool one_batch = deg <= THREADS;
+        if (one_batch && nchunks > 1) {
+            list_bounds<THREADS>(P, p0, deg, chunk, ca > 0 ? ca - 1 : 0u, min(cb, nchunks - 1), bounds);
+            __syncthreads();
+        }
+        uint32_t done = dense ? ca * chunk : ca > 0 ? H.block_base[(uint64_t)i * H.blocks_per_row + ca * chunk / BASE_BLOCK] : 0u;  // entries before the chunk
+        uint32_t passed = one_batch && ca > 0 && (uint32_t)tid < deg ? bounds[(ca - 1) * THREADS + tid] : 0u;  // this thread's list up to the chunk
+        for (uint32_t c = ca; c < cb; ++c) {
+            const uint32_t c0 = c * chunk, c1 = min(c0 + chunk, U), cn = c1 - c0;
+            if (use_masks) {
+                for (uint32_t t = tid; t < cn; t += THREADS) {
+                    uint32_t n = 0;
+#pragma unroll
+                    for (int p = 0; p < HEAVY_PLANES; ++p)
+                        if (p < planes) n += __popc(P.heavy_mask[p * P.mask_stride + c0 + t] & mine.w[p]);
+                    acc[t] = (Acc)(int32_t)n;
+                }
+            }
+            auto add = [&](uint32_t j, Acc p) {
+                const uint32_t rel = j - c0;
+                if (!SPSYRK_IN_RANGE(rel < cn, P.err)) return;
+                if (!dense) occurs[rel] = 1;
+                atomicAdd(&acc[rel], p);
+            };
+            for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+                const bool on = b0 + tid < deg;
+                uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
+                if (use_masks && on && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
+                uint32_t lo = 0, hi = d.y;  // the list's entries in [c0, c1)
+                if (d.y > 0 && nchunks > 1) {
+                    const int32_t* lst = P.at_row + d.x;
+                    lo = one_batch ? passed : c0 == 0 ? 0u : lower_bound_i32(lst, d.y, (int32_t)c0);
+                    if (c1 < U) hi = one_batch ? bounds[c * THREADS + tid] : lo + lower_bound_i32(lst + lo, d.y - lo, (int32_t)c1);
+                    passed = hi;
+                }
+                const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
+                if (b0) __syncthreads();
+                batch_fill<Acc, THREADS>(B, d.x + lo, hi - lo, a);
+                if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
+                else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc av) { add((uint32_t)r.j, acc_mul(av, (Acc)r.v)); });
+            }
+            __syncthreads();
+            // entries of every group of 32 columns, their prefix sums; a warp owns consecutive groups
+            const uint32_t words = (cn + 31u) / 32u;
+            const uint32_t per_warp = (words + NW - 1) / NW;
+            const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
+            uint32_t tot = cn, run = 0;
+            if (!dense) {
+                uint32_t sum = 0;
+                for (uint32_t w = w0; w < w1; ++w) {
+                    const uint32_t t = w * 32u + lane;
+                    const unsigned b = __ballot_sync(FULL_MASK, t < cn && occurs[t] != 0);
+                    if (lane == 0) votes[w] = b;
+                    sum += __popc(b);
+                }
+                if (lane == 0) s_warp[warp] = sum;
+                __syncthreads();
+                const uint32_t ws = lane < NW ? s_warp[lane] : 0u;
+                run = warp_reduce_sum<uint32_t>(lane < warp ? ws : 0u);
+                tot = warp_reduce_sum<uint32_t>(ws);
+            }
+            for (uint32_t w = w0; w < w1; ++w) {
+                const uint32_t b = dense ? 0xffffffffu : votes[w];
+                const uint32_t t = w * 32u + lane;
+                if (((b >> lane) & 1u) && t < cn) {
+                    const int64_t at = ob + done + (dense ? t : run + __popc(b & ((1u << lane) - 1u)));
+                    const Acc v = acc[t];
+                    acc[t] = Acc(0);
+                    occurs[t] = 0;
+                    if (SPSYRK_IN_RANGE(at < oe, P.err)) {
+                        c_vals[at] = (V)v;
+                        H.c_colidx[at] = (int32_t)(c0 + t);
+                        if constexpr (std::is_same<V, int32_t>::value)
+                            if (P.jaccard) store_jaccard<V>(P, at, (int32_t)(c0 + t), v, (int32_t)deg);
+                    }
+                }
+                run += __popc(b);
+            }
+            done += tot;
+            __syncthreads();
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// dense8
+// ---------------------------------------------------------------------------------------------
+template <int THREADS>
+struct Dense8Smem {
+    static size_t bytes(uint32_t columns) { return ((size_t)columns + 15) / 16 * 16 + 16 + sizeof(ListBatch<int32_t, THREADS>); }
+};
+
+// A dense row of a binary matrix with at most 255 nonzeros: every count is at most the row's own length, so a word holds
+// four counters and a row is one tile.  The counters start at the overlap of the rows' heavy-column masks (read as
+// planes of 32 columns, four rows j at a time), the remaining lists, short ones, are walked, and the row leaves four
+// entries per thread: groups of four are aligned in the output, where the row starts at any offset.
+template <typename V, int THREADS, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, HeavyArgs H, uint32_t columns, V* __restrict__ c_vals) {
+    extern __shared__ __align__(16) unsigned char d8_smem[];
+    __shared__ int2 s_row;
+    uint32_t* acc = reinterpret_cast<uint32_t*>(d8_smem);  // four columns per word
+    ListBatch<int32_t, THREADS>& B = *reinterpret_cast<ListBatch<int32_t, THREADS>*>(d8_smem + ((size_t)columns + 15) / 16 * 16 + 16);
+    const int tid = threadIdx.x;
+    const int planes = heavy_planes(P);
+    RowQueue queue(H);
+    for (;;) {
+        const int32_t rloc = queue.next(H, &s_row).x;
+        if (rloc < 0) break;
+        const int64_t i = (int64_t)P.r0 + rloc;
+        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const int64_t p0 = P.rowptr[i];
+        const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);  // at most 255: one batch
+        const int64_t ob = H.out_begin[rloc];
+        const uint32_t words = (U + 3u) / 4u;
+        uint2 d = (uint32_t)tid < deg ? P.desc[p0 + tid] : make_uint2(0u, 0u);
+        if (planes > 0) {
+            if (d.y > 0 && P.heavy_id[P.colidx[p0 + tid]] != 0xff) d.y = 0;  // counted through the masks
+            const HeavyMask mine = load_heavy_mask(P, i, planes);
+            for (uint32_t w = tid; w < words; w += THREADS) {
+                uint32_t n0 = 0, n1 = 0, n2 = 0, n3 = 0;
+#pragma unroll
+                for (int p = 0; p < HEAVY_PLANES; ++p) {  // (planes are padded to whole groups of four rows)
+                    if (p >= planes) break;
+                    const uint4 k = *reinterpret_cast<const uint4*>(P.heavy_mask + p * P.mask_stride + 4 * (int64_t)w);
+                    n0 += __popc(k.x & mine.w[p]); n1 += __popc(k.y & mine.w[p]);
+                    n2 += __popc(k.z & mine.w[p]); n3 += __popc(k.w & mine.w[p]);
+                }
+                acc[w] = n0 | (n1 << 8) | (n2 << 16) | (n3 << 24);
+            }
+        } else {
+            for (uint32_t w = tid; w < words; w += THREADS) acc[w] = 0;
+        }
+        batch_fill<int32_t, THREADS>(B, d.x, d.y, 0);
+        batch_walk<int32_t, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, int32_t) {
+            if (SPSYRK_IN_RANGE((uint32_t)j < U, P.err)) atomicAdd(&acc[(uint32_t)j >> 2], 1u << (((uint32_t)j & 3u) * 8u));
+        });
+        __syncthreads();
+        auto one = [&](uint32_t j) {
+            const int32_t c = (int32_t)((acc[j >> 2] >> ((j & 3u) * 8u)) & 0xffu);
+            c_vals[ob + j] = (V)c;
+            H.c_colidx[ob + j] = (int32_t)j;
+            if constexpr (std::is_same<V, int32_t>::value)
+                if (P.jaccard) store_jaccard<V>(P, ob + j, (int32_t)j, c, (int32_t)deg);
+        };
+        if (!H.aligned) {
+            for (uint32_t j = tid; j < U; j += THREADS) one(j);
+            continue;
+        }
+        // columns [head, tail) leave in whole groups: (ob + j) % 4 == 0
+        const uint32_t head = min((uint32_t)((4 - (ob & 3)) & 3), U), groups = (U - head) / 4u, tail = head + 4u * groups;
+        if ((uint32_t)tid < head) one((uint32_t)tid);
+        if ((uint32_t)tid < U - tail) one(tail + tid);
+        for (uint32_t g = tid; g < groups; g += THREADS) {
+            const uint32_t j = head + 4u * g;
+            // counters j .. j + 3 straddle two words unless head is 0 (the word after the last group's is inside the buffer)
+            const uint32_t q = __funnelshift_r(acc[j >> 2], acc[(j >> 2) + 1], (j & 3u) * 8u);
+            const int32_t c[4] = {(int32_t)(q & 0xffu), (int32_t)((q >> 8) & 0xffu), (int32_t)((q >> 16) & 0xffu), (int32_t)(q >> 24)};
+            *reinterpret_cast<int4*>(H.c_colidx + ob + j) = make_int4((int)j, (int)j + 1, (int)j + 2, (int)j + 3);
+            if constexpr (sizeof(V) == 8) {
+                double2* o = reinterpret_cast<double2*>(c_vals + ob + j);
+                o[0] = make_double2(c[0], c[1]);
+                o[1] = make_double2(c[2], c[3]);
+            } else if constexpr (std::is_same<V, float>::value) {
+                *reinterpret_cast<float4*>(c_vals + ob + j) = make_float4((float)c[0], (float)c[1], (float)c[2], (float)c[3]);
+            } else {
+                *reinterpret_cast<int4*>(c_vals + ob + j) = make_int4(c[0], c[1], c[2], c[3]);
+                if (P.jaccard) {
+                    float s[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) s[k] = __fdiv_rn((float)c[k], (float)(uint32_t)((int32_t)deg + P.adeg[j + k] - c[k]));
+                    *reinterpret_cast<float4*>(P.jaccard + ob + j) = make_float4(s[0], s[1], s[2], s[3]);
+                }
+            }
+        }
+    }
+}
+
+}  // namespace spsyrk

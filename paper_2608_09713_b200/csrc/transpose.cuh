@@ -20,6 +20,12 @@
 
 namespace spsyrk {
 
+// granularity of the per-row entry counts that the symbolic pass keeps for the heavy rows (columns)
+constexpr uint32_t BASE_BLOCK = 8192;
+
+constexpr int HEAVY_PLANES = 4;
+constexpr int HEAVY_MAX = 32 * HEAVY_PLANES;
+
 struct PlanDev {
     int32_t m, n;
     int64_t nnz;
@@ -36,13 +42,16 @@ struct PlanDev {
     int64_t* work;  // per row of the range
     uint32_t* err;
     // Binary input (every stored value is exactly one): a partial product is 1 and an entry of the
-    // product is an intersection count.  Then the heaviest columns (at most 64, chosen by their number
-    // of entries) are also kept as one bit per row, heavy_mask[i] bit b = row i stores heavy column b, so
-    // that their share of a count is popcount(heavy_mask[i] & heavy_mask[j]) instead of one list walk each.
+    // product is an intersection count.  Then the heaviest columns (at most HEAVY_MAX, chosen by their number
+    // of entries) are also kept as one bit per row, in planes of 32 columns: bit b of heavy_mask[p * mask_stride + i] =
+    // row i stores heavy column 32 p + b, so that their share of a count is the population count of two rows' common
+    // bits instead of one list walk each.  (On the Zipf workloads 128 columns leave 0.7 of 16 products per entry
+    // to the walks, 64 columns 1.5.)
     int32_t binary;               // 0 / 1, valid after the plan's analysis
     const uint32_t* nheavy;       // heavy columns in use (0: none), device memory, written when the matrix is binary
     const uint8_t* heavy_id;      // [n] bit number of a heavy column, 0xff otherwise
-    const uint64_t* heavy_mask;   // [m]
+    const uint32_t* heavy_mask;   // [HEAVY_PLANES][mask_stride]
+    int64_t mask_stride;          // m rounded up to four
     float* jaccard;               // optional: the numeric pass also writes c / (|a_i| + |a_j| - c) here (int32 values)
     const int32_t* adeg;          // [m] stored entries per row of A (|a_i| of the Jaccard formula)
 };
@@ -52,33 +61,44 @@ struct PlanDev {
 // per-row bit masks.  Launched for binary matrices only.
 // facts[0] = 1 if some stored value differs from one; facts[1] = heavy columns; facts[32..] histogram.
 // ---------------------------------------------------------------------------------------------
-// histogram of floor(log2(column length)) over the columns
-static __global__ void __launch_bounds__(256) heavy_hist_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ hist32) {
-    __shared__ uint32_t h[32];
-    if (threadIdx.x < 32) h[threadIdx.x] = 0;
+// histogram of the column lengths, four bins per octave
+constexpr int HEAVY_BINS = 128;
+__device__ __forceinline__ int heavy_bin(uint32_t d) {
+    const int e = 31 - __clz(d);
+    return 4 * e + (int)((d >> (e - 2)) & 3u);
+}
+static __global__ void __launch_bounds__(256) heavy_hist_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ hist) {
+    __shared__ uint32_t h[HEAVY_BINS];
+    if (threadIdx.x < HEAVY_BINS) h[threadIdx.x] = 0;
     __syncthreads();
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; k < n; k += stride) {
         const uint32_t d = colcnt[k];
-        if (d >= 256u) atomicAdd(&h[31 - __clz(d)], 1u);  // lighter columns are never candidates
+        if (d >= 256u) atomicAdd(&h[heavy_bin(d)], 1u);  // lighter columns are never candidates
     }
     __syncthreads();
-    if (threadIdx.x < 32 && h[threadIdx.x]) atomicAdd(&hist32[threadIdx.x], h[threadIdx.x]);
+    if (threadIdx.x < HEAVY_BINS && h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
 }
 
-// Columns of at least the threshold get a bit number; the threshold is the smallest power of two such that at most 64
-// columns have that many entries or more.
+// Columns of at least the threshold get a bit number; the threshold is the smallest bin such that at most HEAVY_MAX
+// columns lie in it and above.
 static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ facts,
                                                                  uint8_t* __restrict__ heavy_id) {
     __shared__ uint32_t s_thr;
     if (threadIdx.x < 32) {
-        const int b = 31 - (int)threadIdx.x;  // lane l looks at lengths of 2^(31 - l) and more
-        const uint32_t c = facts[32 + b];
-        const uint32_t upto = warp_inclusive_scan<uint32_t>(c);
-        const unsigned fits = __ballot_sync(FULL_MASK, b >= 8 && upto <= 64u);
-        const unsigned used = __ballot_sync(FULL_MASK, c > 0) & (fits == FULL_MASK ? FULL_MASK : ((1u << __popc(fits)) - 1u));
-        if (threadIdx.x == 0) s_thr = used ? 1u << (31 - (31 - __clz(used))) : 0xffffffffu;
+        const int e = 31 - (int)threadIdx.x;  // lane l looks at the octave from 2^(31 - l)
+        uint32_t c[4], sum = 0;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) { c[f] = facts[32 + 4 * e + f]; sum += c[f]; }
+        uint32_t above = warp_inclusive_scan<uint32_t>(sum) - sum, cand = 0xffffffffu;
+#pragma unroll
+        for (int f = 3; f >= 0; --f) {
+            above += c[f];
+            if (e >= 8 && above <= (uint32_t)HEAVY_MAX && c[f]) cand = (uint32_t)(4 + f) << (e - 2);
+        }
+        cand = __reduce_min_sync(FULL_MASK, cand);
+        if (threadIdx.x == 0) s_thr = cand;
     }
     __syncthreads();
     const uint32_t thr = s_thr;
@@ -87,7 +107,7 @@ static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t
         uint8_t id = 0xff;
         if (colcnt[k] >= thr) {
             const uint32_t b = atomicAdd(&facts[1], 1u);
-            if (b < 64u) id = (uint8_t)b;
+            if (b < (uint32_t)HEAVY_MAX) id = (uint8_t)b;
         }
         heavy_id[k] = id;
     }
@@ -96,23 +116,28 @@ static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t
 template <int G>
 static __global__ void __launch_bounds__(256) heavy_mask_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, int32_t m,
                                                                const uint32_t* __restrict__ facts, const uint8_t* __restrict__ heavy_id,
-                                                               uint64_t* __restrict__ heavy_mask) {
-    if (facts[1] == 0) return;  // no heavy column: nothing reads the masks (a fixed grid walks the rows, so the launch costs nothing then)
+                                                               uint32_t* __restrict__ heavy_mask, int64_t mask_stride) {
+    if (facts[1] == 0) return;  // no heavy column: nothing reads the masks
     const int gl = threadIdx.x & (G - 1);
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x) / G; base < m; base += groups) {  // uniform per CTA
         const int64_t gid = base + threadIdx.x / G;
-        unsigned long long mk = 0;
+        uint32_t mk[HEAVY_PLANES] = {};
         if (gid < m) {
             const int64_t p0 = rowptr[gid], p1 = rowptr[gid + 1];
             for (int64_t p = p0 + gl; p < p1; p += G) {
                 const uint8_t id = heavy_id[colidx[p]];
-                if (id != 0xff) mk |= 1ull << id;
+#pragma unroll
+                for (int q = 0; q < HEAVY_PLANES; ++q)
+                    if ((id >> 5) == q) mk[q] |= 1u << (id & 31);  // (0xff belongs to no plane)
             }
         }
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) mk |= __shfl_xor_sync(FULL_MASK, mk, o);
-        if (gid < m && gl == 0) heavy_mask[gid] = mk;
+        for (int q = 0; q < HEAVY_PLANES; ++q) {
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) mk[q] |= __shfl_xor_sync(FULL_MASK, mk[q], o);
+            if (gid < m && gl == 0) heavy_mask[q * mask_stride + gid] = mk[q];
+        }
     }
 }
 
