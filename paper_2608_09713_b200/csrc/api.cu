@@ -57,7 +57,6 @@ constexpr size_t ALIGN = 256;
 constexpr int64_t BLOCK_CLASS_MAX_WORK = 32768;  // class 6 (block class) up to here, class 7 above
 constexpr uint32_t ROW_CHUNK_BITS_MAX_NUMERIC = 1u << 18;
 constexpr uint32_t ROW_CHUNK_BITS_MAX_SYMBOLIC = 1u << 20;
-constexpr int TRANSPOSE_RADIX_BITS = 8;
 constexpr size_t LARGE_SMEM_BUDGET = 200 * 1024;
 constexpr int64_t MAX_PARTS = 65536;
 
@@ -124,8 +123,7 @@ struct spsyrk_plan_s {
     // radix sort buffers of the transpose (nnz entries each) and its histograms
     uint32_t *rx_key_a, *rx_row_a, *rx_pos_a, *rx_key_b, *rx_row_b, *rx_pos_b;
     void *rx_val_a, *rx_val_b;
-    uint32_t* rx_hist;
-    int64_t* rx_offsets;
+    RadixState rx;
     int32_t* blockhist;
     int64_t* offsets;
     int64_t* partials;
@@ -183,10 +181,13 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto hdr = c.take<uint4>(m);
     auto cnt = c.take<int32_t>(m);
     auto cls = c.take<uint8_t>(items);
+    const int npass = radix_passes((uint64_t)std::max<int64_t>(n - 1, 1));
+    const size_t rx_words = radix_state_words(radix_tiles(nnz), radix_wide(nnz), npass);
     // counters in one piece, so that one memset clears them: the binning's, then the plan's, then the column counts
     const int views = full ? 2 : 1;
     const size_t bin_words = views * (1 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(items));
-    auto zero = c.take<int64_t>(bin_words + 32 + (32 + HEAVY_BINS) / 2 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2);
+    auto zero = c.take<int64_t>(bin_words + 32 + (32 + HEAVY_BINS) / 2 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2 +
+                                RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES + rx_words);
     Carver cz(zero);
     auto take_words = [&](size_t words) { int64_t* q = zero ? zero + cz.off : nullptr; cz.off += words; return q; };
     auto work_total_dev = reinterpret_cast<unsigned long long*>(take_words(1));
@@ -198,8 +199,11 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto facts = reinterpret_cast<uint32_t*>(take_words((32 + HEAVY_BINS) / 2));  // [0..1] binary analysis, [32..] its histogram
     auto state_col = take_words(scan_partials_count(std::max<int64_t>(n, 1)));
     auto colcnt = reinterpret_cast<uint32_t*>(take_words((size_t)(n + 1) / 2));
+    RadixState rx;
+    rx.bins = reinterpret_cast<unsigned long long*>(take_words(RX_MAX_PASSES * RX_BINS));
+    rx.tickets = reinterpret_cast<uint32_t*>(take_words(RX_MAX_PASSES));
+    rx.words = take_words(rx_words);
     const size_t zero_words = cz.off;
-    const int64_t rx_hist_n = (int64_t)(1 << TRANSPOSE_RADIX_BITS) * std::max<int64_t>(radix_tiles(nnz), 1);
     // The two buffer sets of the radix sort (key, row, position, value per nonzero) are reused: the set that
     // the last pass does not read receives the column lists that pass writes (row ids and records), and the
     // set it does read holds, once the sort is over, the block descriptors and the heavy-row accumulator slices.
@@ -215,17 +219,14 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto rx_row_b = cb.take<uint32_t>(nnz);
     auto rx_pos_b = cb.take<uint32_t>(nnz);
     auto rx_val_b = cb.take<char>(nnz * sv);
-    const int npass = (bits_for((uint64_t)std::max<int64_t>(n - 1, 1)) + TRANSPOSE_RADIX_BITS - 1) / TRANSPOSE_RADIX_BITS;
     const bool last_reads_a = npass >= 2 && (npass % 2) == 0;  // pass p writes set A when p is even; one pass reads the input itself (and row ids kept in set B)
     Carver c_free(last_reads_a ? set_b : set_a), c_src(last_reads_a ? set_a : set_b);
     auto at_row = c_free.take<int32_t>(nnz + 4);  // the symbolic gathers read aligned 16-byte pieces: up to 3 entries past the end
     auto at_rec = c_free.take<char>(nnz * (sv == 8 ? 16 : 8));
     auto desc_blk = c_src.take<uint2>(nnz);
-    auto rx_hist = c.take<uint32_t>(rx_hist_n);
-    auto rx_offsets = c.take<int64_t>(rx_hist_n + 1);
     auto blockhist = c.take<int32_t>(NCLASS * nb);
     auto offsets = c.take<int64_t>(NCLASS * nb + 1);
-    auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(std::max<int64_t>(items + 1, NCLASS * nb), rx_hist_n)));
+    auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(items + 1, NCLASS * nb)));
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
     auto route_count = c.take<uint32_t>(2 * NROUTE);  // both views in a row
     auto dispensers = c.take<uint32_t>(2 * NROUTE);
@@ -284,7 +285,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         pl->desc_full = desc; pl->desc_blk = desc_blk;
         pl->perm = perm; pl->hdr = hdr; pl->cnt = cnt; pl->cls = cls; pl->colcnt = colcnt;
         pl->rx_key_a = rx_key_a; pl->rx_row_a = rx_row_a; pl->rx_pos_a = rx_pos_a; pl->rx_key_b = rx_key_b; pl->rx_row_b = rx_row_b;
-        pl->rx_pos_b = rx_pos_b; pl->rx_val_a = rx_val_a; pl->rx_val_b = rx_val_b; pl->rx_hist = rx_hist; pl->rx_offsets = rx_offsets;
+        pl->rx_pos_b = rx_pos_b; pl->rx_val_a = rx_val_a; pl->rx_val_b = rx_val_b; pl->rx = rx;
         pl->blockhist = blockhist; pl->offsets = offsets; pl->partials = partials;
         pl->class_start_dev = class_start_dev; pl->work_total_dev = work_total_dev;
         pl->state_bin = state_bin; pl->state_items = state_items; pl->state_col = state_col; pl->items8 = items8;
@@ -359,10 +360,10 @@ int group_width(int64_t nnz, int64_t m) {
 // VB: unsigned integer of the value's width (values are only moved)
 template <typename VB>
 spsyrk_status_t sort_by_column(spsyrk_plan_s* pl, cudaStream_t st) {
-    constexpr int BITS = TRANSPOSE_RADIX_BITS;
     const PlanDev& P = pl->dev;
     if (P.nnz == 0) return SPSYRK_OK;
-    const int npass = (bits_for((uint64_t)std::max<int64_t>(P.n - 1, 1)) + BITS - 1) / BITS;
+    const int npass = radix_passes((uint64_t)std::max<int64_t>(P.n - 1, 1));
+    SPSYRK_CUDA_TRY(radix_bins<true>(pl->colcnt, P.n, npass, pl->rx.bins, st));  // from the column counts: n numbers, not nnz keys
     const uint32_t* src_key = reinterpret_cast<const uint32_t*>(P.colidx);
     const uint32_t* src_row = pl->rx_row_b;
     const VB* src_val = static_cast<const VB*>(P.vals);
@@ -375,12 +376,10 @@ spsyrk_status_t sort_by_column(spsyrk_plan_s* pl, cudaStream_t st) {
         VB* dst_val = static_cast<VB*>(to_a ? pl->rx_val_a : pl->rx_val_b);
         if (p == npass - 1) {
             EmitTransposeFinal<VB> emit{P, pl->desc_hi};
-            SPSYRK_CUDA_TRY((radix_pass3<BITS, VB>(src_key, src_row, src_val, src_pos, P.nnz, p * BITS, pl->rx_hist, pl->rx_offsets,
-                                                   pl->partials, emit, P.err, st)));
+            SPSYRK_CUDA_TRY((radix_pass<VB, true>(src_key, src_row, src_val, src_pos, P.nnz, p, pl->rx, emit, P.err, st)));
         } else {
             EmitArrays3<VB> emit{dst_key, dst_row, dst_val, dst_pos};
-            SPSYRK_CUDA_TRY((radix_pass3<BITS, VB>(src_key, src_row, src_val, src_pos, P.nnz, p * BITS, pl->rx_hist, pl->rx_offsets,
-                                                   pl->partials, emit, P.err, st)));
+            SPSYRK_CUDA_TRY((radix_pass<VB, true>(src_key, src_row, src_val, src_pos, P.nnz, p, pl->rx, emit, P.err, st)));
         }
         src_key = dst_key;
         src_row = dst_row;

@@ -16,7 +16,6 @@ using namespace spsyrk;
 namespace {
 
 constexpr size_t ALIGN = 256;
-constexpr int PERMUTE_RADIX_BITS = 8;
 
 struct PermuteWs {
     uint32_t* len;   // m: lengths of B's rows
@@ -25,8 +24,9 @@ struct PermuteWs {
     uint32_t* err;
     uint32_t *key_a, *pay_a, *key_b, *pay_b;  // nnz each
     void *val_a, *val_b;
-    uint32_t* hist;
-    int64_t* offsets;
+    RadixState rs[2];  // sort by column, sort by row
+    void* zero;
+    size_t zero_bytes;
 };
 
 size_t carve(PermuteWs* w, void* ws, int64_t m, int64_t n, int64_t nnz, size_t sv) {
@@ -40,11 +40,10 @@ size_t carve(PermuteWs* w, void* ws, int64_t m, int64_t n, int64_t nnz, size_t s
     };
     const int64_t items = std::max<int64_t>(std::max(m, n), 1);
     const int64_t ne = std::max<int64_t>(nnz, 1);
-    const int64_t hist_n = (int64_t)(1 << PERMUTE_RADIX_BITS) * std::max<int64_t>(radix_tiles(nnz), 1);
     PermuteWs t;
     t.len = (uint32_t*)take(items * 4);
     t.seen = (uint32_t*)take(items * 4);
-    t.partials = (int64_t*)take(scan_partials_count(std::max<int64_t>(items + 1, hist_n)) * 8);
+    t.partials = (int64_t*)take(scan_partials_count(items + 1) * 8);
     t.err = (uint32_t*)take(4);
     t.key_a = (uint32_t*)take(ne * 4);
     t.pay_a = (uint32_t*)take(ne * 4);
@@ -52,8 +51,17 @@ size_t carve(PermuteWs* w, void* ws, int64_t m, int64_t n, int64_t nnz, size_t s
     t.pay_b = (uint32_t*)take(ne * 4);
     t.val_a = take(ne * sv);
     t.val_b = take(ne * sv);
-    t.hist = (uint32_t*)take(hist_n * 4);
-    t.offsets = (int64_t*)take((hist_n + 1) * 8);
+    const size_t words[2] = {radix_state_words(radix_tiles(nnz), radix_wide(nnz), radix_passes((uint64_t)std::max<int64_t>(n - 1, 1))),
+                             radix_state_words(radix_tiles(nnz), radix_wide(nnz), radix_passes((uint64_t)std::max<int64_t>(m - 1, 1)))};
+    t.zero_bytes = (2 * (RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES) + words[0] + words[1]) * 8;
+    t.zero = take(t.zero_bytes);
+    unsigned long long* z = (unsigned long long*)t.zero;
+    for (int k = 0; k < 2; ++k) {
+        t.rs[k].bins = z;
+        t.rs[k].tickets = (uint32_t*)(z + RX_MAX_PASSES * RX_BINS);
+        t.rs[k].words = z + RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES;
+        z += RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES + words[k];
+    }
     if (w) *w = t;
     return (off + ALIGN - 1) / ALIGN * ALIGN;
 }
@@ -122,7 +130,7 @@ int group_width(int64_t nnz, int64_t m) {
 template <typename V>
 spsyrk_status_t permute_sort(const PermuteWs& w, int64_t m, int64_t n, int64_t nnz, const void* vals, bool sort_columns,
                              int32_t* b_colidx, void* b_vals, cudaStream_t st) {
-    constexpr int BITS = PERMUTE_RADIX_BITS;
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(w.zero, 0, w.zero_bytes, st));
     // after the expand: key_a = new column, pay_a = new row
     const uint32_t* key = w.key_a;
     const uint32_t* pay = w.pay_a;
@@ -132,27 +140,29 @@ spsyrk_status_t permute_sort(const PermuteWs& w, int64_t m, int64_t n, int64_t n
     auto other_pay = [&]() { return in_a ? w.pay_b : w.pay_a; };
     auto other_val = [&]() { return static_cast<V*>(in_a ? w.val_b : w.val_a); };
     if (sort_columns) {
-        const int npass = (bits_for((uint64_t)std::max<int64_t>(n - 1, 1)) + BITS - 1) / BITS;
+        const int npass = radix_passes((uint64_t)std::max<int64_t>(n - 1, 1));
+        SPSYRK_CUDA_TRY(radix_bins<false>(key, nnz, npass, w.rs[0].bins, st));
         for (int p = 0; p < npass; ++p) {
             EmitArrays<V> emit{other_key(), other_pay(), other_val()};
-            SPSYRK_CUDA_TRY((radix_pass<BITS, V>(key, pay, val, nnz, p * BITS, w.hist, w.offsets, w.partials, emit, w.err, st)));
+            SPSYRK_CUDA_TRY((radix_pass<V, false>(key, pay, val, nullptr, nnz, p, w.rs[0], emit, w.err, st)));
             key = emit.keys; pay = emit.pa; val = emit.pb;
             in_a = !in_a;
         }
     }
     // now sort by the new row: the row array becomes the key, the column array the payload
     std::swap(key, pay);
-    const int npass = (bits_for((uint64_t)std::max<int64_t>(m - 1, 1)) + BITS - 1) / BITS;
+    const int npass = radix_passes((uint64_t)std::max<int64_t>(m - 1, 1));
+    SPSYRK_CUDA_TRY(radix_bins<false>(key, nnz, npass, w.rs[1].bins, st));
     for (int p = 0; p < npass; ++p) {
         if (p == npass - 1) {
             EmitPermuted<V> emit{b_colidx, static_cast<V*>(b_vals)};
-            SPSYRK_CUDA_TRY((radix_pass<BITS, V>(key, pay, val, nnz, p * BITS, w.hist, w.offsets, w.partials, emit, w.err, st)));
+            SPSYRK_CUDA_TRY((radix_pass<V, false>(key, pay, val, nullptr, nnz, p, w.rs[1], emit, w.err, st)));
         } else {
             // the roles of the two uint32 buffers of a pair are swapped with the arrays
             uint32_t* dk = in_a ? w.pay_b : w.pay_a;
             uint32_t* dp = in_a ? w.key_b : w.key_a;
             EmitArrays<V> emit{dk, dp, other_val()};
-            SPSYRK_CUDA_TRY((radix_pass<BITS, V>(key, pay, val, nnz, p * BITS, w.hist, w.offsets, w.partials, emit, w.err, st)));
+            SPSYRK_CUDA_TRY((radix_pass<V, false>(key, pay, val, nullptr, nnz, p, w.rs[1], emit, w.err, st)));
             key = dk; pay = dp; val = emit.pb;
             in_a = !in_a;
         }

@@ -3,14 +3,17 @@
 // in ascending row order leave every column's segment in ascending row order, with no atomics and
 // no per-segment sort, and every pass reads and writes memory in long runs.
 //
-// One pass = three launches: per-tile digit histogram, device-wide scan of the digit-major
-// histogram, scatter.  In the scatter a warp owns a contiguous slice of the tile, keeps its elements
-// in registers and ranks them 32 at a time (elements with equal digits find each other through one
-// warp vote per digit bit, the lowest lane bumps the warp's counter), an exclusive prefix over the
-// warps makes the ranks tile-wide and stable, every element is dropped into its slot of the
-// digit-major tile in shared memory and the tile is written out in runs.  There is no waiting
-// between CTAs.
+// A pass is one launch (single-pass partition with decoupled look-back: Adinets & Merrill, "Onesweep", 2022): the
+// sizes of all digits of all passes are known beforehand, a CTA takes its tile's number from a counter,
+// ranks its elements, publishes the tile's count of every digit, drops the elements into their slots of the
+// digit-major tile in shared memory, adds up what the tiles before it have published, one thread per digit, and
+// writes the tile out in runs.  In the ranking a warp owns a contiguous slice of the tile, keeps its
+// elements in registers and ranks them 32 at a time (elements with equal digits find each other through one
+// warp vote per digit bit, the lowest lane bumps the warp's counter); an exclusive prefix over the
+// warps makes the ranks tile-wide and stable.  A tile only waits for tiles that running CTAs hold.
+// (Per-tile histograms and their device-wide scan before: three more launches per pass and the keys read twice.)
 #pragma once
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -25,42 +28,95 @@ constexpr int RX_CHUNK = RX_TILE / RX_WARPS;    // contiguous elements per warp
 
 inline int64_t radix_tiles(int64_t n) { return n > 0 ? (n + RX_TILE - 1) / RX_TILE : 0; }
 
-template <int BITS>
-__global__ void __launch_bounds__(RX_THREADS) radix_hist_kernel(const uint32_t* __restrict__ keys, int64_t n, int shift,
-                                                                uint32_t* __restrict__ hist, int64_t ntiles) {
-    constexpr int NB = 1 << BITS;
-    __shared__ uint32_t h[RX_WARPS][NB];  // one histogram per warp keeps the atomics apart
-    for (int d = threadIdx.x; d < RX_WARPS * NB; d += RX_THREADS) (&h[0][0])[d] = 0;
-    __syncthreads();
-    const int warp = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * RX_TILE;
-    uint32_t k[RX_ITEMS];
+constexpr int RX_BITS = 8;
+constexpr int RX_BINS = 1 << RX_BITS;
+constexpr int RX_MAX_PASSES = 4;
+inline int radix_passes(uint64_t max_key);
+
+// State of a sort, all zero at its start: sizes of the digits of every pass, a tile counter per pass, and per pass, tile
+// and digit a word value << 2 | kind (see scan_look_back; 32-bit words while counts stay below 2^30).
+struct RadixState {
+    unsigned long long* bins;  // [passes][RX_BINS]
+    uint32_t* tickets;         // [RX_MAX_PASSES]
+    void* words;               // [passes][tiles][RX_BINS]
+};
+inline bool radix_wide(int64_t n) { return n >= (int64_t(1) << 30); }
+inline size_t radix_state_words(int64_t tiles, bool wide, int passes) { return (size_t)passes * tiles * RX_BINS / (wide ? 1 : 2); }  // 64-bit words
+
+__device__ __forceinline__ uint32_t ld_status(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_status(uint32_t* p, uint32_t v) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+
+// One thread per digit: the tile's count is published with radix_publish as soon as it is known; radix_look_back returns how
+// many elements of the digit the tiles before hold and publishes the sum.
+template <typename S>
+__device__ __forceinline__ void radix_publish(S* words, int64_t tile, int digit, uint32_t count) {
+    st_status(words + tile * RX_BINS + digit, (S)(((S)count << 2) | (tile == 0 ? (S)SCAN_PREFIX : (S)SCAN_PARTIAL)));
+}
+template <typename S>
+__device__ __forceinline__ int64_t radix_look_back(S* words, int64_t tile, int digit, uint32_t count, uint32_t* err) {
+    if (tile == 0) return 0;
+    constexpr int W = 8;  // tiles per round trip
+    S before = 0;
+    bool done = false;
+    for (int64_t last = tile - 1; !done; last -= W) {
+        S v[W];
 #pragma unroll
-    for (int it = 0; it < RX_ITEMS; ++it) {
-        const int64_t e = base + it * RX_THREADS + threadIdx.x;
-        k[it] = e < n ? keys[e] : 0u;
-    }
+        for (int k = 0; k < W; ++k) v[k] = last - k >= 0 ? ld_status(words + (last - k) * RX_BINS + digit) : (S)SCAN_PREFIX;
 #pragma unroll
-    for (int it = 0; it < RX_ITEMS; ++it) {
-        const int64_t e = base + it * RX_THREADS + threadIdx.x;
-        if (e < n) atomicAdd(&h[warp][(k[it] >> shift) & (NB - 1)], 1u);
+        for (int k = 0; k < W; ++k) {
+            if (done) continue;
+            for (int polls = 0; (v[k] & 3) == 0; ++polls) {
+                if (polls == SPIN_LIMIT) {  // the host sees ERRW_INTERNAL; the sum is too small, nothing is indexed out of range
+                    if (err) atomicOr(err, ERRW_INTERNAL);
+                    v[k] = (S)SCAN_PREFIX;
+                    break;
+                }
+                v[k] = ld_status(words + (last - k) * RX_BINS + digit);
+            }
+            before += v[k] >> 2;
+            done = (v[k] & 3) == (S)SCAN_PREFIX;
+        }
     }
-    __syncthreads();
-    for (int d = threadIdx.x; d < NB; d += RX_THREADS) {
-        uint32_t t = 0;
-#pragma unroll
-        for (int w = 0; w < RX_WARPS; ++w) t += h[w][d];
-        hist[(int64_t)d * ntiles + blockIdx.x] = t;
-    }
+    st_status(words + tile * RX_BINS + digit, (S)(((S)(before + count) << 2) | (S)SCAN_PREFIX));
+    return (int64_t)before;
 }
 
-// A functor that declares `static constexpr bool NEIGHBOURS = true` is also handed the keys next to the
-// element in the tile's sorted order.
-constexpr uint32_t NO_KEY = 0xffffffffu;
-template <typename E, typename = void>
-struct emit_wants_neighbours : std::false_type {};
-template <typename E>
-struct emit_wants_neighbours<E, std::void_t<decltype(E::NEIGHBOURS)>> : std::bool_constant<E::NEIGHBOURS> {};
+// Sizes of all digits of 32-bit keys: weights[k] elements of key k (keys = nullptr), or the keys themselves
+template <bool COUNTED>
+static __global__ void __launch_bounds__(RX_THREADS) radix_bins_kernel(const uint32_t* __restrict__ in, int64_t n, int passes, unsigned long long* __restrict__ bins) {
+    __shared__ uint32_t h[RX_MAX_PASSES][RX_BINS];
+    for (int d = threadIdx.x; d < RX_MAX_PASSES * RX_BINS; d += RX_THREADS) (&h[0][0])[d] = 0;
+    __syncthreads();
+    // a CTA counts fewer than 2^32 elements: the sum of all weights of a matrix is below 2^31, and keys are one each
+    const int64_t stride = (int64_t)gridDim.x * RX_THREADS;
+    constexpr int UNR = 4;
+    for (int64_t e = (int64_t)blockIdx.x * RX_THREADS + threadIdx.x; e < n; e += UNR * stride) {
+        uint32_t v[UNR];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) v[u] = e + u * stride < n ? in[e + u * stride] : 0u;
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            if (e + u * stride >= n || (COUNTED && v[u] == 0)) continue;
+            const uint32_t key = COUNTED ? (uint32_t)(e + u * stride) : v[u];
+            for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (p * RX_BITS)) & (RX_BINS - 1)], COUNTED ? v[u] : 1u);
+        }
+    }
+    __syncthreads();
+    for (int d = threadIdx.x; d < passes * RX_BINS; d += RX_THREADS)
+        if ((&h[0][0])[d]) atomicAdd(&bins[d], (unsigned long long)(&h[0][0])[d]);
+}
+template <bool COUNTED>
+inline cudaError_t radix_bins(const uint32_t* in, int64_t n, int passes, unsigned long long* bins, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    const int64_t ctas = std::min<int64_t>((n + RX_THREADS * 4 - 1) / (RX_THREADS * 4), 148 * 4);
+    radix_bins_kernel<COUNTED><<<(unsigned)ctas, RX_THREADS, 0, st>>>(in, n, passes, bins);
+    note_launches(1);
+    return cudaGetLastError();
+}
 
 template <int BITS, typename PB, bool HAS_PC = false>
 struct RadixSmem {
@@ -82,15 +138,19 @@ struct RadixSmem {
 // read back slot by slot and written out in runs.
 // HAS_PC: a third payload pc (32 bits; nullptr = the element's own index) travels along and the functor is
 // called as emit(dest, key, pa, pb, pc).
-template <int BITS, typename PB, typename Emit, bool HAS_PC = false>
+// An element whose position is not in [0, n) is dropped: it takes keys that were not counted (a matrix that failed its
+// checks, which the caller learns of later).
+template <int BITS, typename PB, typename Emit, bool HAS_PC, typename S>
 __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pa,
                                                                       const PB* __restrict__ pb, const uint32_t* __restrict__ pc,
-                                                                      int64_t n, int shift, const int64_t* __restrict__ goff_all,
-                                                                      int64_t ntiles, Emit emit, uint32_t* err) {
+                                                                      int64_t n, int shift, const unsigned long long* __restrict__ bins,
+                                                                      S* __restrict__ words, uint32_t* __restrict__ ticket, Emit emit, uint32_t* err) {
     constexpr int NB = 1 << BITS;
     static_assert(BITS <= 12, "digit width");
     extern __shared__ __align__(16) unsigned char rx_smem[];
     __shared__ uint32_t scratch[33];
+    __shared__ int64_t scratch64[33];
+    __shared__ uint32_t s_tile;
     int64_t* goff = reinterpret_cast<int64_t*>(rx_smem);               // [NB]
     PB* s_pb = reinterpret_cast<PB*>(goff + NB);                       // [TILE] sorted order
     uint32_t* s_key = reinterpret_cast<uint32_t*>(s_pb + RX_TILE);     // [TILE] sorted order
@@ -100,7 +160,10 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
     uint32_t* bin_start = wcount + RX_WARPS * NB;                      // [NB]
 
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    const int64_t tile_base = (int64_t)blockIdx.x * RX_TILE;
+    static_assert(NB == RX_BINS && NB <= RX_THREADS, "one thread per digit");
+    if (tid == 0) s_tile = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const int64_t tile = s_tile, tile_base = tile * RX_TILE;
     const int tile_n = (int)min((int64_t)RX_TILE, n - tile_base);
     uint32_t k[RX_ITEMS], a[RX_ITEMS];
     PB b[RX_ITEMS];
@@ -145,42 +208,23 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
         __syncwarp();
     }
     __syncthreads();
-    // exclusive prefix over the warps per digit; digit totals; this tile's global offsets
-    for (int d = tid; d < NB; d += RX_THREADS) {
-        uint32_t run = 0;
+    // exclusive prefix over the warps per digit; the digit totals are published at once
+    uint32_t total_d = 0;
+    if (tid < NB) {
 #pragma unroll
         for (int w = 0; w < RX_WARPS; ++w) {
-            const uint32_t c = wcount[w * NB + d];
-            wcount[w * NB + d] = run;
-            run += c;
+            const uint32_t c = wcount[w * NB + tid];
+            wcount[w * NB + tid] = total_d;
+            total_d += c;
         }
-        bin_start[d] = run;
-        goff[d] = goff_all[(int64_t)d * ntiles + blockIdx.x];
+        radix_publish<S>(words, tile, tid, total_d);
     }
+    uint32_t tot;
+    const uint32_t first_d = block_exclusive_scan<uint32_t, RX_THREADS>(total_d, scratch, &tot);
+    if (tid < NB) bin_start[tid] = first_d;
     __syncthreads();
-    {
-        // exclusive scan of the digit totals: thread t owns digits [t * PER, t * PER + PER)
-        constexpr int PER = (NB + RX_THREADS - 1) / RX_THREADS;
-        uint32_t s = 0;
-#pragma unroll
-        for (int q = 0; q < PER; ++q)
-            if (tid * PER + q < NB) s += bin_start[tid * PER + q];
-        uint32_t tot;
-        uint32_t ex = block_exclusive_scan<uint32_t, RX_THREADS>(s, scratch, &tot);
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            if (tid * PER + q < NB) {
-                const uint32_t t = bin_start[tid * PER + q];
-                bin_start[tid * PER + q] = ex;
-                ex += t;
-            }
-        }
-    }
-    __syncthreads();
-    // a warp's first slot of digit d = start of the digit + the elements of the warps before it; slot q of
-    // digit d goes to goff[d] + (q - bin_start[d]): fold the tables
+    // a warp's first slot of digit d = start of the digit + the elements of the warps before it
     for (int e = tid; e < RX_WARPS * NB; e += RX_THREADS) wcount[e] += bin_start[e & (NB - 1)];
-    for (int d = tid; d < NB; d += RX_THREADS) goff[d] -= (int64_t)bin_start[d];
     __syncthreads();
     // elements into their slots
 #pragma unroll
@@ -196,17 +240,17 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
             if constexpr (HAS_PC) s_pc[q] = pc ? pc[tile_base + t] : (uint32_t)(tile_base + t);
         }
     }
+    // slot q of digit d goes to (elements of smaller digits) + (of this digit in the tiles before) + q - first slot of d
+    int64_t tot64;
+    const int64_t base_d = block_exclusive_scan<int64_t, RX_THREADS>(tid < NB ? (int64_t)bins[tid] : 0, scratch64, &tot64);
+    if (tid < NB) goff[tid] = base_d + radix_look_back<S>(words, tile, tid, total_d, err) - (int64_t)first_d;
     __syncthreads();
     for (int q = tid; q < tile_n; q += RX_THREADS) {
         const uint32_t key = s_key[q];
         const int64_t dest = goff[(key >> shift) & (NB - 1)] + q;
-        if (!SPSYRK_IN_RANGE(dest >= 0 && dest < n, err)) continue;
+        if (dest < 0 || dest >= n) continue;
         if constexpr (HAS_PC) {
             emit(dest, key, s_pa[q], s_pb[q], s_pc[q]);
-        } else if constexpr (emit_wants_neighbours<Emit>::value) {
-            // the keys of the slots before and after (NO_KEY at the ends of the tile): in the last pass of a
-            // sort equal keys are adjacent, so a functor can tell where a run of one key starts and ends
-            emit(dest, key, s_pa[q], s_pb[q], q > 0 ? s_key[q - 1] : NO_KEY, q + 1 < tile_n ? s_key[q + 1] : NO_KEY);
         } else {
             emit(dest, key, s_pa[q], s_pb[q]);
         }
@@ -239,36 +283,26 @@ struct EmitArrays3 {
     }
 };
 
-// hist: NB * ntiles uint32; offsets: NB * ntiles + 1 int64; partials: scan_partials_count(NB * ntiles) int64
-template <int BITS, typename PB, bool HAS_PC, typename Emit>
-inline cudaError_t radix_pass_impl(const uint32_t* keys, const uint32_t* pa, const PB* pb, const uint32_t* pc, int64_t n, int shift,
-                                   uint32_t* hist, int64_t* offsets, int64_t* partials, Emit emit, uint32_t* err, cudaStream_t st) {
-    constexpr int NB = 1 << BITS;
+// pass `pass` of a sort whose state has been set up (zeroed, bins counted)
+template <typename PB, bool HAS_PC, typename Emit, typename S>
+inline cudaError_t radix_pass_launch(const uint32_t* keys, const uint32_t* pa, const PB* pb, const uint32_t* pc, int64_t n, int pass, const RadixState& rs,
+                                     Emit emit, uint32_t* err, cudaStream_t st) {
     const int64_t nt = radix_tiles(n);
-    if (nt == 0) return cudaSuccess;
-    radix_hist_kernel<BITS><<<(unsigned)nt, RX_THREADS, 0, st>>>(keys, n, shift, hist, nt);
-    cudaError_t e = exclusive_scan_i64<uint32_t>(hist, (int64_t)NB * nt, offsets, partials, err, st);
+    auto kern = radix_scatter_kernel<RX_BITS, PB, Emit, HAS_PC, S>;
+    const size_t smem = RadixSmem<RX_BITS, PB, HAS_PC>::bytes();
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    auto kern = radix_scatter_kernel<BITS, PB, Emit, HAS_PC>;
-    const size_t smem = RadixSmem<BITS, PB, HAS_PC>::bytes();
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nt, RX_THREADS, smem, st>>>(keys, pa, pb, pc, n, shift, offsets, nt, emit, err);
-    note_launches(2);
+    kern<<<(unsigned)nt, RX_THREADS, smem, st>>>(keys, pa, pb, pc, n, pass * RX_BITS, rs.bins + pass * RX_BINS, static_cast<S*>(rs.words) + (size_t)pass * nt * RX_BINS,
+                                                 rs.tickets + pass, emit, err);
+    note_launches(1);
     return cudaGetLastError();
 }
-
-template <int BITS, typename PB, typename Emit>
-inline cudaError_t radix_pass(const uint32_t* keys, const uint32_t* pa, const PB* pb, int64_t n, int shift, uint32_t* hist,
-                              int64_t* offsets, int64_t* partials, Emit emit, uint32_t* err, cudaStream_t st) {
-    return radix_pass_impl<BITS, PB, false>(keys, pa, pb, nullptr, n, shift, hist, offsets, partials, emit, err, st);
-}
-
-// the same with a third 32-bit payload (pc == nullptr: the element's own index)
-template <int BITS, typename PB, typename Emit>
-inline cudaError_t radix_pass3(const uint32_t* keys, const uint32_t* pa, const PB* pb, const uint32_t* pc, int64_t n, int shift,
-                               uint32_t* hist, int64_t* offsets, int64_t* partials, Emit emit, uint32_t* err, cudaStream_t st) {
-    return radix_pass_impl<BITS, PB, true>(keys, pa, pb, pc, n, shift, hist, offsets, partials, emit, err, st);
+template <typename PB, bool HAS_PC, typename Emit>
+inline cudaError_t radix_pass(const uint32_t* keys, const uint32_t* pa, const PB* pb, const uint32_t* pc, int64_t n, int pass, const RadixState& rs, Emit emit,
+                              uint32_t* err, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    return radix_wide(n) ? radix_pass_launch<PB, HAS_PC, Emit, unsigned long long>(keys, pa, pb, pc, n, pass, rs, emit, err, st)
+                         : radix_pass_launch<PB, HAS_PC, Emit, uint32_t>(keys, pa, pb, pc, n, pass, rs, emit, err, st);
 }
 
 inline int bits_for(uint64_t max_value) {
@@ -276,5 +310,7 @@ inline int bits_for(uint64_t max_value) {
     while (b < 64 && (max_value >> b)) ++b;
     return b;
 }
+
+inline int radix_passes(uint64_t max_key) { return (bits_for(max_key) + RX_BITS - 1) / RX_BITS; }
 
 }  // namespace spsyrk
