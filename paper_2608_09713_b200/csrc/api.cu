@@ -138,8 +138,7 @@ struct spsyrk_plan_s {
     int32_t* route_list;    // NROUTE lists of rows_cap each
     uint32_t* route_count;  // NROUTE list lengths (device) ...
     uint32_t route_n[NROUTE];  // ... and as the host knows them after the symbolic pass
-    uint32_t* bounds;       // scratch of the direct kernel
-    int2* parts_list;       // parts of the longest rows
+    int2* rank_parts;       // parts of the longest rows
     uint32_t* block_base;   // entries of a heavy row before every block of columns, [row][blocks_per_row]
     uint32_t blocks_per_row;
     uint32_t* dispensers;   // NROUTE counters the persistent kernels take their rows from
@@ -162,6 +161,7 @@ struct spsyrk_plan_s {
     bool key64;
     bool diag;  // the light-row kernels handle the diagonal apart (lower-triangle mode, whole column range)
     int sm_count;
+    int device;
     // optional per-class timing of the symbolic and numeric launches
     bool timing;
     cudaEvent_t ev_sym[NCLASS + 1];
@@ -231,11 +231,10 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto route_count = c.take<uint32_t>(2 * NROUTE);  // both views in a row
     auto dispensers = c.take<uint32_t>(2 * NROUTE);
     auto route_list = c.take<int32_t>(NROUTE * items);
-    auto bounds = c.take<uint32_t>(DIRECT_MAX_CTAS * DIRECT_BOUNDS);
     // rows whose output range is at most 2^18 columns (they are among the first 2^18 rows)
     const int64_t base_rows = std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC);
     const uint32_t blocks_per_row = (uint32_t)((std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC) + BASE_BLOCK - 1) / BASE_BLOCK);
-    auto parts_list = c.take<int2>(base_rows * DIRECT_MAX_PARTS);
+    auto rank_parts = c.take<int2>(base_rows * MAX_ROW_PARTS);
     auto block_base = c.take<uint32_t>(base_rows * blocks_per_row);
     auto work_prefix = c.take<int64_t>(items + 1);
     auto itemoff = c.take<int64_t>(items + 1);
@@ -251,7 +250,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     uint2* desc_hi = nullptr;
     int64_t *u_work = nullptr, *u_itemoff = nullptr, *u_class_start_dev = nullptr, *hi_begin = nullptr, *work_sum = nullptr;
     int32_t *u_perm = nullptr, *u_cnt = nullptr, *cnt_tot = nullptr, *u_route_list = nullptr;
-    int2* u_parts_list = nullptr;
+    int2* u_rank_parts = nullptr;
     uint32_t* u_block_base = nullptr;
     uint4* u_hdr = nullptr;
     uint8_t* u_cls = nullptr;
@@ -266,14 +265,14 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         u_class_start_dev = c.take<int64_t>(NCLASS + 1);
         cnt_tot = c.take<int32_t>(m);
         u_route_list = c.take<int32_t>(NROUTE * items);
-        u_parts_list = c.take<int2>(base_rows * DIRECT_MAX_PARTS);
+        u_rank_parts = c.take<int2>(base_rows * MAX_ROW_PARTS);
         u_block_base = c.take<uint32_t>(base_rows * blocks_per_row);
         hi_begin = c.take<int64_t>(items + 1);
         work_sum = c.take<int64_t>(m);
     }
     if (pl) {
         pl->desc_hi = desc_hi; pl->cnt_tot = cnt_tot; pl->hi_begin = hi_begin; pl->work_sum = work_sum;
-        pl->route_count = route_count; pl->dispensers = dispensers; pl->route_list = route_list; pl->bounds = bounds; pl->parts_list = parts_list;
+        pl->route_count = route_count; pl->dispensers = dispensers; pl->route_list = route_list; pl->rank_parts = rank_parts;
         pl->block_base = block_base; pl->blocks_per_row = blocks_per_row;
         pl->dev.mask_stride = mask_stride;
         pl->work_prefix = work_prefix; pl->part_bounds = part_bounds; pl->itemoff = itemoff;
@@ -301,11 +300,61 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
             up->class_start_dev = u_class_start_dev; up->work_total_dev = u_work_total_dev;
             up->state_bin = u_state_bin; up->state_items = u_state_items;
             up->route_count = route_count + NROUTE; up->dispensers = dispensers + NROUTE; up->route_list = u_route_list;
-            up->parts_list = u_parts_list; up->block_base = u_block_base;
+            up->rank_parts = u_rank_parts; up->block_base = u_block_base;
         }
     }
     return (c.off + ALIGN - 1) / ALIGN * ALIGN;
 }
+
+// A chain of kernels that do not depend on one another (see chain_begin).  With `overlap` off every launch is an ordinary one,
+// and so is that of a kernel that fills the GPU for long (`brief` false): its CTAs would start one by one as those of the
+// kernel before end, and a persistent grid that shares its rows out beforehand ends with the last of them.  (All launches
+// overlapped: large Erdos-Renyi product and mirror 36.0 ms against 35.1, large power-law 35.7 against 34.6; the
+// 8192-row power-law product takes 378 us with and 446 without overlap.)
+struct Chain {
+    cudaStream_t st;
+    bool overlap;
+    bool first = true;
+    template <typename... Params, typename... Args>
+    cudaError_t launch(bool brief, void (*kern)(Params...), unsigned grid, int threads, size_t smem, Args... args) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = overlap && brief && !first ? 1 : 0;
+        first = false;
+        note_launches(1);
+        return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    }
+};
+
+inline bool brief_rows(int64_t rows, int64_t resident) { return rows <= 16 * resident; }  // a few rows per CTA
+
+// CTAs of a kernel that an SM holds at once, asked for once per device (and the shared memory it needs is allowed once).  One
+// object per kernel.
+struct Residency {
+    static constexpr int DEVICES = 64;
+    std::atomic<int> per_sm[DEVICES] = {};
+    template <typename Kernel>
+    cudaError_t get(Kernel kern, int threads, size_t smem, int device, int* out) {
+        const bool known = device >= 0 && device < DEVICES;
+        int n = known ? per_sm[device].load(std::memory_order_relaxed) : 0;
+        if (n == 0) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem);
+            if (e != cudaSuccess) return e;
+            n = std::max(n, 1);
+            if (known) per_sm[device].store(n, std::memory_order_relaxed);
+        }
+        *out = n;
+        return cudaSuccess;
+    }
+};
 
 spsyrk_status_t status_of(uint32_t e) {
     if (e & (ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED)) return SPSYRK_ERR_BAD_CSR;
@@ -489,7 +538,7 @@ int64_t map_items_total(const spsyrk_plan_s* pl) { return pl->map_items + (pl->u
 bool use_map(const spsyrk_plan_s* pl) { return pl->map && pl->map_bytes >= (size_t)map_items_total(pl) * sizeof(uint16_t); }
 
 template <int N, bool DIAG>
-spsyrk_status_t launch_symbolic_warp_d(spsyrk_plan_s* pl, int c, cudaStream_t st) {
+spsyrk_status_t launch_symbolic_warp_d(spsyrk_plan_s* pl, int c, Chain& ch) {
     const int64_t count = pl->class_start[c + 1] - pl->class_start[c];
     if (count <= 0) return SPSYRK_OK;
     constexpr int G = warp_class_group(N);
@@ -497,19 +546,18 @@ spsyrk_status_t launch_symbolic_warp_d(spsyrk_plan_s* pl, int c, cudaStream_t st
     constexpr int ROWS = SW * (32 / G);  // rows a CTA works on at a time
     constexpr size_t smem = (size_t)ROWS * SymbolicWarpSmem<N>::GROUP;
     auto kern = symbolic_warp_kernel<N, G, DIAG>;
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static Residency residency;
     int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SW * 32, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    SPSYRK_CUDA_TRY(residency.get(kern, SW * 32, smem, pl->device, &per_sm));
     const int64_t want = (count + ROWS - 1) / ROWS;
     const int64_t cap = (int64_t)pl->sm_count * per_sm;
-    kern<<<(unsigned)std::min(want, cap), SW * 32, smem, st>>>(pl->dev, pl->hdr + pl->class_start[c], count, pl->cnt);
-    note_launches(1);
+    SPSYRK_CUDA_TRY(ch.launch(want <= cap, kern, (unsigned)std::min(want, cap), SW * 32, smem, pl->dev, pl->hdr + pl->class_start[c], count, pl->cnt));
     return SPSYRK_OK;
 }
 
 template <int N>
-spsyrk_status_t launch_symbolic_warp(spsyrk_plan_s* pl, int c, cudaStream_t st) {
-    return pl->diag ? launch_symbolic_warp_d<N, true>(pl, c, st) : launch_symbolic_warp_d<N, false>(pl, c, st);
+spsyrk_status_t launch_symbolic_warp(spsyrk_plan_s* pl, int c, Chain& ch) {
+    return pl->diag ? launch_symbolic_warp_d<N, true>(pl, c, ch) : launch_symbolic_warp_d<N, false>(pl, c, ch);
 }
 
 // the part of class c's row list (rows in ascending order) a numeric launch covers
@@ -519,7 +567,7 @@ inline int64_t numeric_count(const spsyrk_plan_s* pl, int c) {
 }
 
 template <typename V, int N, typename Key, bool DIAG>
-spsyrk_status_t launch_numeric_warp_d(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
+spsyrk_status_t launch_numeric_warp_d(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, Chain& ch) {
     const int64_t count = numeric_count(pl, c);
     if (count <= 0) return SPSYRK_OK;
     constexpr int G = warp_class_group(N);
@@ -529,25 +577,24 @@ spsyrk_status_t launch_numeric_warp_d(spsyrk_plan_s* pl, int c, int32_t* c_colid
     // persistent groups: exactly as many CTAs as are resident at once, each group walks its rows with
     // a stride of the whole grid
     auto kern = numeric_warp_kernel<V, N, G, Key, DIAG>;
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static Residency residency;
     int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    SPSYRK_CUDA_TRY(residency.get(kern, NW * 32, smem, pl->device, &per_sm));
     const int64_t want = (count + ROWS - 1) / ROWS;
     const int64_t cap = (int64_t)pl->sm_count * per_sm;
-    kern<<<(unsigned)std::min(want, cap), NW * 32, smem, st>>>(pl->dev, pl->hdr + numeric_first(pl, c), count, pl->out_begin, pl->out_end,
-                                                               c_colidx, static_cast<V*>(c_vals), pl->cnt_out);
-    note_launches(1);
+    SPSYRK_CUDA_TRY(ch.launch(want <= cap, kern, (unsigned)std::min(want, cap), NW * 32, smem, pl->dev, pl->hdr + numeric_first(pl, c), count, pl->out_begin, pl->out_end,
+                                                               c_colidx, static_cast<V*>(c_vals), pl->cnt_out));
     return SPSYRK_OK;
 }
 
 template <typename V, int N, typename Key>
-spsyrk_status_t launch_numeric_warp(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
-    return pl->diag ? launch_numeric_warp_d<V, N, Key, true>(pl, c, c_colidx, c_vals, st)
-                    : launch_numeric_warp_d<V, N, Key, false>(pl, c, c_colidx, c_vals, st);
+spsyrk_status_t launch_numeric_warp(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, Chain& ch) {
+    return pl->diag ? launch_numeric_warp_d<V, N, Key, true>(pl, c, c_colidx, c_vals, ch)
+                    : launch_numeric_warp_d<V, N, Key, false>(pl, c, c_colidx, c_vals, ch);
 }
 
 template <int N, typename Key, bool DIAG>
-spsyrk_status_t launch_symbolic_sort_d(spsyrk_plan_s* pl, int c, cudaStream_t st) {
+spsyrk_status_t launch_symbolic_sort_d(spsyrk_plan_s* pl, int c, Chain& ch) {
     const int64_t count = pl->class_start[c + 1] - pl->class_start[c];
     if (count <= 0) return SPSYRK_OK;
     constexpr int G = warp_class_group(N);
@@ -555,26 +602,25 @@ spsyrk_status_t launch_symbolic_sort_d(spsyrk_plan_s* pl, int c, cudaStream_t st
     constexpr int ROWS = SW * (32 / G);
     constexpr size_t smem = (size_t)ROWS * SymbolicSortSmem<N>::GROUP;
     auto kern = symbolic_sort_warp_kernel<N, G, Key, DIAG>;
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static Residency residency;
     int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SW * 32, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    SPSYRK_CUDA_TRY(residency.get(kern, SW * 32, smem, pl->device, &per_sm));
     const int64_t want = (count + ROWS - 1) / ROWS;
     const int64_t cap = (int64_t)pl->sm_count * per_sm;
-    kern<<<(unsigned)std::min(want, cap), SW * 32, smem, st>>>(pl->dev, pl->hdr + pl->class_start[c], pl->itemoff + pl->class_start[c],
-                                                               count, pl->cnt, pl->map);
-    note_launches(1);
+    SPSYRK_CUDA_TRY(ch.launch(want <= cap, kern, (unsigned)std::min(want, cap), SW * 32, smem, pl->dev, pl->hdr + pl->class_start[c], pl->itemoff + pl->class_start[c],
+                                                               count, pl->cnt, pl->map));
     return SPSYRK_OK;
 }
 
 template <int N>
-spsyrk_status_t launch_symbolic_sort(spsyrk_plan_s* pl, int c, cudaStream_t st) {
+spsyrk_status_t launch_symbolic_sort(spsyrk_plan_s* pl, int c, Chain& ch) {
     if (pl->key64)
-        return pl->diag ? launch_symbolic_sort_d<N, uint64_t, true>(pl, c, st) : launch_symbolic_sort_d<N, uint64_t, false>(pl, c, st);
-    return pl->diag ? launch_symbolic_sort_d<N, uint32_t, true>(pl, c, st) : launch_symbolic_sort_d<N, uint32_t, false>(pl, c, st);
+        return pl->diag ? launch_symbolic_sort_d<N, uint64_t, true>(pl, c, ch) : launch_symbolic_sort_d<N, uint64_t, false>(pl, c, ch);
+    return pl->diag ? launch_symbolic_sort_d<N, uint32_t, true>(pl, c, ch) : launch_symbolic_sort_d<N, uint32_t, false>(pl, c, ch);
 }
 
 template <typename V, int N, bool DIAG>
-spsyrk_status_t launch_numeric_map_d(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
+spsyrk_status_t launch_numeric_map_d(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, Chain& ch) {
     const int64_t count = numeric_count(pl, c);
     if (count <= 0) return SPSYRK_OK;
     constexpr int G = warp_class_group(N);
@@ -582,55 +628,54 @@ spsyrk_status_t launch_numeric_map_d(spsyrk_plan_s* pl, int c, int32_t* c_colidx
     constexpr int ROWS = NW * (32 / G);
     constexpr size_t smem = (size_t)ROWS * NumericMapSmem<V, N>::GROUP;
     auto kern = numeric_map_warp_kernel<V, N, G, DIAG>;
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static Residency residency;
     int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    SPSYRK_CUDA_TRY(residency.get(kern, NW * 32, smem, pl->device, &per_sm));
     const int64_t want = (count + ROWS - 1) / ROWS;
     const int64_t cap = (int64_t)pl->sm_count * per_sm;
-    kern<<<(unsigned)std::min(want, cap), NW * 32, smem, st>>>(pl->dev, pl->hdr + numeric_first(pl, c), pl->itemoff + numeric_first(pl, c),
-                                                               count, pl->map, pl->out_begin, pl->out_end, c_colidx, static_cast<V*>(c_vals));
-    note_launches(1);
+    SPSYRK_CUDA_TRY(ch.launch(want <= cap, kern, (unsigned)std::min(want, cap), NW * 32, smem, pl->dev, pl->hdr + numeric_first(pl, c), pl->itemoff + numeric_first(pl, c),
+                                                               count, pl->map, pl->out_begin, pl->out_end, c_colidx, static_cast<V*>(c_vals)));
     return SPSYRK_OK;
 }
 
 template <typename V, int N>
-spsyrk_status_t launch_numeric_map(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
-    return pl->diag ? launch_numeric_map_d<V, N, true>(pl, c, c_colidx, c_vals, st)
-                    : launch_numeric_map_d<V, N, false>(pl, c, c_colidx, c_vals, st);
+spsyrk_status_t launch_numeric_map(spsyrk_plan_s* pl, int c, int32_t* c_colidx, void* c_vals, Chain& ch) {
+    return pl->diag ? launch_numeric_map_d<V, N, true>(pl, c, c_colidx, c_vals, ch)
+                    : launch_numeric_map_d<V, N, false>(pl, c, c_colidx, c_vals, ch);
 }
 
-inline void mark(spsyrk_plan_s* pl, cudaEvent_t* ev, int i, cudaStream_t st) {
-    if (pl->timing) cudaEventRecord(ev[i], st);
+inline void mark(spsyrk_plan_s* pl, cudaEvent_t* ev, int i, const Chain& ch) {
+    if (pl->timing) cudaEventRecord(ev[i], ch.st);
 }
 
 template <typename V>
-void launch_numeric_map_all(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
-    mark(pl, pl->ev_num, 1, st);
-    launch_numeric_map<V, 32>(pl, 1, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 2, st);
-    launch_numeric_map<V, 64>(pl, 2, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 3, st);
-    launch_numeric_map<V, 128>(pl, 3, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 4, st);
-    launch_numeric_map<V, 256>(pl, 4, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 5, st);
-    launch_numeric_map<V, 512>(pl, 5, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 6, st);
+void launch_numeric_map_all(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, Chain& ch) {
+    mark(pl, pl->ev_num, 1, ch);
+    launch_numeric_map<V, 32>(pl, 1, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 2, ch);
+    launch_numeric_map<V, 64>(pl, 2, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 3, ch);
+    launch_numeric_map<V, 128>(pl, 3, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 4, ch);
+    launch_numeric_map<V, 256>(pl, 4, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 5, ch);
+    launch_numeric_map<V, 512>(pl, 5, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 6, ch);
 }
 
 template <typename V, typename Key>
-void launch_numeric_warp_all(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
-    mark(pl, pl->ev_num, 1, st);
-    launch_numeric_warp<V, 32, Key>(pl, 1, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 2, st);
-    launch_numeric_warp<V, 64, Key>(pl, 2, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 3, st);
-    launch_numeric_warp<V, 128, Key>(pl, 3, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 4, st);
-    launch_numeric_warp<V, 256, Key>(pl, 4, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 5, st);
-    launch_numeric_warp<V, 512, Key>(pl, 5, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 6, st);
+void launch_numeric_warp_all(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, Chain& ch) {
+    mark(pl, pl->ev_num, 1, ch);
+    launch_numeric_warp<V, 32, Key>(pl, 1, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 2, ch);
+    launch_numeric_warp<V, 64, Key>(pl, 2, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 3, ch);
+    launch_numeric_warp<V, 128, Key>(pl, 3, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 4, ch);
+    launch_numeric_warp<V, 256, Key>(pl, 4, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 5, ch);
+    launch_numeric_warp<V, 512, Key>(pl, 5, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 6, ch);
 }
 
 // bounds[p] = r0 + the smallest r in [0, rows] with prefix[r] * parts >= p * prefix[rows]
@@ -654,16 +699,15 @@ uint32_t row_chunk_bits(const spsyrk_plan_s* pl, uint32_t cap) {
 }
 
 template <int THREADS>
-spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, cudaStream_t st) {
+spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
     const int64_t count = pl->class_start[c + 1] - pl->class_start[c];
     if (count <= 0) return SPSYRK_OK;
     const uint32_t cb = row_chunk_bits(pl, ROW_CHUNK_BITS_MAX_SYMBOLIC);
     const size_t smem = CtaRowSmem<int32_t, THREADS, false>::bytes(cb, 0);
     auto kern = rows_cta_kernel<int32_t, THREADS, false>;
     SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<(unsigned)count, THREADS, smem, st>>>(pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr, nullptr, 0, 0,
-                                                 pl->block_base, pl->blocks_per_row);
-    note_launches(1);
+    SPSYRK_CUDA_TRY(ch.launch(brief_rows(count, (int64_t)pl->sm_count * (2048 / THREADS)), kern, (unsigned)count, THREADS, smem, pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr,
+                              nullptr, 0, 0, pl->block_base, pl->blocks_per_row));
     return SPSYRK_OK;
 }
 
@@ -691,9 +735,8 @@ HeavyShapes heavy_shapes(const spsyrk_plan_s* pl) {
     r.slots_small = std::min(cb, (uint32_t)(16384 / sizeof(Acc)));
     r.slots_mid = std::min(cb, (uint32_t)(65536 / sizeof(Acc)));
     r.slots_big = std::min(cb, (uint32_t)((SMEM_PER_CTA - RankSmem<V, RANK_BIG_THREADS>::bytes(cb, 0)) / sizeof(Acc)) / 1024 * 1024);
-    // whole blocks of the table, two CTAs per SM; 2^18 columns are at most DIRECT_MAX_CHUNKS chunks
-    r.chunk = std::min(cb, (uint32_t)((SMEM_PER_CTA / 2 - 1024 - DirectSmem<V, DIRECT_THREADS>::bytes(0)) / (sizeof(Acc) * 32 + 32 + 4)) * 32 / BASE_BLOCK * BASE_BLOCK);
-    static_assert(ROW_CHUNK_BITS_MAX_NUMERIC / BASE_BLOCK <= DIRECT_MAX_CHUNKS, "a row's chunk bounds fit a CTA's scratch");
+    // two CTAs per SM
+    r.chunk = std::min(cb, (uint32_t)((SMEM_PER_CTA / 2 - 1024 - DirectSmem<V, DIRECT_THREADS>::bytes(0)) / (sizeof(Acc) * 32 + 32 + 4)) * 32);
     const uint64_t umax = pl->dev.mode == SPSYRK_TRIL ? (uint64_t)pl->dev.r1 : (uint64_t)pl->dev.m;
     h.dense8_columns = (uint32_t)std::min<uint64_t>(umax, (SMEM_PER_CTA - Dense8Smem<DENSE8_THREADS>::bytes(0)) / 16 * 16);
     r.dense8 = h.dense8_columns;
@@ -704,14 +747,23 @@ HeavyShapes heavy_shapes(const spsyrk_plan_s* pl) {
 // which kernel computes which heavy row; the counts of the symbolic pass are known
 spsyrk_status_t route_heavy(spsyrk_plan_s* pl, cudaStream_t st) {
     const int64_t count = pl->class_start[NCLASS] - pl->class_start[6];
-    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->route_count, 0, NROUTE * sizeof(uint32_t), st));
     if (count <= 0) return SPSYRK_OK;
     const HeavyShapes h = pl->dtype == SPSYRK_I32 ? heavy_shapes<int32_t>(pl) : heavy_shapes<double>(pl);
-    route_rows_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->route_list,
-                                                                       pl->rows_cap, pl->parts_list, pl->route_count);
+    route_rows_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->block_base,
+                                                                       pl->blocks_per_row, pl->route_list, pl->rows_cap, pl->rank_parts, pl->route_count);
     note_launches(1);
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
+}
+
+// the lists of both views; without heavy rows nothing is launched and nobody looks at the list lengths
+bool heavy_rows(const spsyrk_plan_s* pl) { return pl->class_start[NCLASS] > pl->class_start[6]; }
+spsyrk_status_t route_views(spsyrk_plan_s* pl, cudaStream_t st) {
+    spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
+    if (!heavy_rows(pl) && !(up && heavy_rows(up))) return SPSYRK_OK;
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->route_count, 0, 2 * NROUTE * sizeof(uint32_t), st));
+    const spsyrk_status_t s = route_heavy(pl, st);
+    return s == SPSYRK_OK && up ? route_heavy(up, st) : s;
 }
 
 // as many CTAs as are resident at once, at most one per row
@@ -724,37 +776,38 @@ cudaError_t persistent_grid(const spsyrk_plan_s* pl, Kernel kern, int threads, s
     return e;
 }
 
-template <typename V>
-spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
-    using Acc = typename AccOf<V>::type;
-    static_assert(sizeof(Acc) == sizeof(typename AccOf<std::conditional_t<std::is_same<V, int32_t>::value, int32_t, double>>::type), "the rule's shapes");
+bool any_heavy(const spsyrk_plan_s* pl) {
     uint32_t any = 0;
     for (int k = 0; k < NROUTE; ++k) any |= pl->route_n[k];
-    if (!any) return SPSYRK_OK;
+    return any != 0;
+}
+
+template <typename V>
+spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, Chain& ch) {
+    using Acc = typename AccOf<V>::type;
+    static_assert(sizeof(Acc) == sizeof(typename AccOf<std::conditional_t<std::is_same<V, int32_t>::value, int32_t, double>>::type), "the rule's shapes");
+    if (!any_heavy(pl)) return SPSYRK_OK;
     const HeavyShapes h = heavy_shapes<V>(pl);
     V* cv = static_cast<V*>(c_vals);
-    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->dispensers, 0, NROUTE * sizeof(uint32_t), st));
     const int64_t row_lo = pl->sub_active ? pl->sub_row_lo : 0, row_hi = pl->sub_active ? pl->sub_row_hi : INT64_MAX;
     const bool aligned = ((reinterpret_cast<uintptr_t>(c_colidx) | reinterpret_cast<uintptr_t>(c_vals) | reinterpret_cast<uintptr_t>(pl->dev.jaccard)) & 15u) == 0;
     auto args = [&](int k) {
         return HeavyArgs{pl->route_list + k * (pl->rows_cap), pl->route_n[k], pl->dispensers + k, row_lo, row_hi, pl->out_begin, pl->out_end, c_colidx, aligned,
-                         pl->parts_list, k == ROUTE_DIRECT ? pl->route_n[ROUTE_PARTS] : 0u, pl->bounds, pl->block_base, pl->blocks_per_row};
+                         pl->rank_parts, k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u, pl->block_base, pl->blocks_per_row};
     };
     unsigned grid = 0;
     auto rank = [&](auto kern, int threads, int k, uint32_t columns, uint32_t slots, size_t smem) -> cudaError_t {
-        if (!pl->route_n[k]) return cudaSuccess;
-        const cudaError_t e = persistent_grid(pl, kern, threads, smem, pl->route_n[k], &grid);
+        const int64_t units = (int64_t)pl->route_n[k] + (k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u);
+        if (!units) return cudaSuccess;
+        const cudaError_t e = persistent_grid(pl, kern, threads, smem, units, &grid);
         if (e != cudaSuccess) return e;
-        kern<<<grid, threads, smem, st>>>(pl->dev, args(k), columns, slots, cv);
-        note_launches(1);
-        return cudaGetLastError();
+        return ch.launch(brief_rows(units, grid), kern, grid, threads, smem, pl->dev, args(k), columns, slots, cv);
     };
-    if (const int64_t units = (int64_t)pl->route_n[ROUTE_DIRECT] + pl->route_n[ROUTE_PARTS]) {
+    if (const int64_t units = pl->route_n[ROUTE_DIRECT]) {
         auto kern = rows_direct_kernel<V, DIRECT_THREADS>;
         const size_t smem = DirectSmem<V, DIRECT_THREADS>::bytes(h.rule.chunk);
-        SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DIRECT_THREADS, smem, std::min<int64_t>(units, DIRECT_MAX_CTAS), &grid));
-        kern<<<grid, DIRECT_THREADS, smem, st>>>(pl->dev, args(ROUTE_DIRECT), h.rule.chunk, cv);
-        note_launches(1);
+        SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DIRECT_THREADS, smem, units, &grid));
+        SPSYRK_CUDA_TRY(ch.launch(brief_rows(units, grid), kern, grid, DIRECT_THREADS, smem, pl->dev, args(ROUTE_DIRECT), h.rule.chunk, cv));
     }
     using Small = RankSmem<V, RANK_SMALL_THREADS>;
     SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_BIG_THREADS, 1>, RANK_BIG_THREADS, ROUTE_RANK_BIG, h.columns, h.rule.slots_big, RankSmem<V, RANK_BIG_THREADS>::bytes(h.columns, h.rule.slots_big)));
@@ -766,8 +819,7 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
         auto kern = rows_dense8_kernel<V, DENSE8_THREADS, 3>;
         const size_t smem = Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns);
         SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DENSE8_THREADS, smem, pl->route_n[ROUTE_DENSE8], &grid));
-        kern<<<grid, DENSE8_THREADS, smem, st>>>(pl->dev, args(ROUTE_DENSE8), h.dense8_columns, cv);
-        note_launches(1);
+        SPSYRK_CUDA_TRY(ch.launch(brief_rows(pl->route_n[ROUTE_DENSE8], grid), kern, grid, DENSE8_THREADS, smem, pl->dev, args(ROUTE_DENSE8), h.dense8_columns, cv));
     }
     if (pl->route_n[ROUTE_WIDE]) {
         constexpr int THREADS = 1024;
@@ -777,26 +829,25 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
         auto kern = rows_cta_kernel<V, THREADS, true>;
         SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         const HeavyArgs a = args(ROUTE_WIDE);
-        kern<<<pl->route_n[ROUTE_WIDE], THREADS, smem, st>>>(pl->dev, a.list, h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv, row_lo, row_hi,
-                                                             nullptr, 0u);
-        note_launches(1);
+        SPSYRK_CUDA_TRY(ch.launch(brief_rows(pl->route_n[ROUTE_WIDE], pl->sm_count), kern, pl->route_n[ROUTE_WIDE], THREADS, smem, pl->dev, a.list, h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv,
+                                  row_lo, row_hi, nullptr, 0u));
     }
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
 }
 
 template <typename V>
-spsyrk_status_t numeric_typed(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, cudaStream_t st) {
-    if (pl->map_filled) launch_numeric_map_all<V>(pl, c_colidx, c_vals, st);
-    else if (pl->key64) launch_numeric_warp_all<V, uint64_t>(pl, c_colidx, c_vals, st);
-    else launch_numeric_warp_all<V, uint32_t>(pl, c_colidx, c_vals, st);
-    mark(pl, pl->ev_num, 7, st);  // the heavy rows of both classes are timed as one
-    const spsyrk_status_t s = launch_heavy<V>(pl, c_colidx, c_vals, st);
+spsyrk_status_t numeric_typed(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, Chain& ch) {
+    if (pl->map_filled) launch_numeric_map_all<V>(pl, c_colidx, c_vals, ch);
+    else if (pl->key64) launch_numeric_warp_all<V, uint64_t>(pl, c_colidx, c_vals, ch);
+    else launch_numeric_warp_all<V, uint32_t>(pl, c_colidx, c_vals, ch);
+    mark(pl, pl->ev_num, 7, ch);  // the heavy rows of both classes are timed as one
+    const spsyrk_status_t s = launch_heavy<V>(pl, c_colidx, c_vals, ch);
     if (s != SPSYRK_OK) return s;
-    mark(pl, pl->ev_num, 8, st);
+    mark(pl, pl->ev_num, 8, ch);
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
-    return read_err(pl, st);  // the bounds-checked build reports a skipped access at once (synchronises)
+    return read_err(pl, ch.st);  // the bounds-checked build reports a skipped access at once (synchronises)
 #else
     return SPSYRK_OK;
 #endif
@@ -852,33 +903,33 @@ spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, bool routes, int6
     const spsyrk_status_t s = status_of((uint32_t)h[1]);
     if (s == SPSYRK_OK) *total = h[0];
     for (int k = 0; routes && k < NROUTE; ++k) {
-        pl->route_n[k] = (uint32_t)h[2 + k];
-        if (up) up->route_n[k] = (uint32_t)h[2 + NROUTE + k];
+        pl->route_n[k] = heavy_rows(pl) ? (uint32_t)h[2 + k] : 0u;
+        if (up) up->route_n[k] = heavy_rows(up) ? (uint32_t)h[2 + NROUTE + k] : 0u;
     }
     return s;
 }
 
 // the per-class count kernels of one view (entries per row into its cnt array)
-spsyrk_status_t symbolic_view(spsyrk_plan_s* pl, bool with_map, cudaStream_t st) {
+spsyrk_status_t symbolic_view(spsyrk_plan_s* pl, bool with_map, Chain& ch) {
     pl->map_filled = false;
-    mark(pl, pl->ev_sym, 1, st);
-    if (with_map) launch_symbolic_sort<32>(pl, 1, st); else launch_symbolic_warp<32>(pl, 1, st);
-    mark(pl, pl->ev_sym, 2, st);
-    if (with_map) launch_symbolic_sort<64>(pl, 2, st); else launch_symbolic_warp<64>(pl, 2, st);
-    mark(pl, pl->ev_sym, 3, st);
-    if (with_map) launch_symbolic_sort<128>(pl, 3, st); else launch_symbolic_warp<128>(pl, 3, st);
-    mark(pl, pl->ev_sym, 4, st);
-    if (with_map) launch_symbolic_sort<256>(pl, 4, st); else launch_symbolic_warp<256>(pl, 4, st);
-    mark(pl, pl->ev_sym, 5, st);
-    if (with_map) launch_symbolic_sort<512>(pl, 5, st); else launch_symbolic_warp<512>(pl, 5, st);
-    mark(pl, pl->ev_sym, 6, st);
-    spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, st);
+    mark(pl, pl->ev_sym, 1, ch);
+    if (with_map) launch_symbolic_sort<32>(pl, 1, ch); else launch_symbolic_warp<32>(pl, 1, ch);
+    mark(pl, pl->ev_sym, 2, ch);
+    if (with_map) launch_symbolic_sort<64>(pl, 2, ch); else launch_symbolic_warp<64>(pl, 2, ch);
+    mark(pl, pl->ev_sym, 3, ch);
+    if (with_map) launch_symbolic_sort<128>(pl, 3, ch); else launch_symbolic_warp<128>(pl, 3, ch);
+    mark(pl, pl->ev_sym, 4, ch);
+    if (with_map) launch_symbolic_sort<256>(pl, 4, ch); else launch_symbolic_warp<256>(pl, 4, ch);
+    mark(pl, pl->ev_sym, 5, ch);
+    if (with_map) launch_symbolic_sort<512>(pl, 5, ch); else launch_symbolic_warp<512>(pl, 5, ch);
+    mark(pl, pl->ev_sym, 6, ch);
+    spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, ch);
     if (s != SPSYRK_OK) return s;
-    mark(pl, pl->ev_sym, 7, st);
-    s = launch_symbolic_cta<1024>(pl, 7, st);
+    mark(pl, pl->ev_sym, 7, ch);
+    s = launch_symbolic_cta<1024>(pl, 7, ch);
     if (s != SPSYRK_OK) return s;
-    mark(pl, pl->ev_sym, 8, st);
-    return route_heavy(pl, st);
+    mark(pl, pl->ev_sym, 8, ch);
+    return SPSYRK_OK;
 }
 
 }  // namespace
@@ -974,6 +1025,7 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
         int dev_id = 0;
         pl->sm_count = 148;
         if (cudaGetDevice(&dev_id) == cudaSuccess) cudaDeviceGetAttribute(&pl->sm_count, cudaDevAttrMultiProcessorCount, dev_id);
+        pl->device = dev_id;
     }
     spsyrk_plan_s* up = nullptr;
     if (full) {
@@ -1061,15 +1113,20 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     const bool with_map = use_map(pl);
-    spsyrk_status_t s = symbolic_view(pl, with_map, st);
+    Chain ch{st, !pl->timing};
+    spsyrk_status_t s = symbolic_view(pl, with_map, ch);
     if (s != SPSYRK_OK) return s;
     const int32_t* counts = pl->cnt;
-    if (pl->upper_active) {
-        spsyrk_plan_s* up = pl->upper;
+    spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
+    if (up) {
         up->map = with_map ? pl->map + pl->map_items : nullptr;  // the upper parts' words follow the lower parts'
         up->map_bytes = with_map ? (size_t)up->map_items * sizeof(uint16_t) : 0;
-        s = symbolic_view(up, with_map, st);
+        s = symbolic_view(up, with_map, ch);
         if (s != SPSYRK_OK) return s;
+    }
+    s = route_views(pl, st);
+    if (s != SPSYRK_OK) return s;
+    if (up) {
         if (rows > 0) {
             add_counts_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->cnt, up->cnt, rows, pl->cnt_tot);
             note_launches(1);
@@ -1098,11 +1155,13 @@ spsyrk_status_t spsyrk_numeric(spsyrk_plan_t plan, const int64_t* d_c_rowptr, in
     const int64_t work_all = pl->work_total + (pl->upper_active ? pl->upper->work_total : 0);
     if (work_all > 0 && (!d_c_colidx || !d_c_vals)) return SPSYRK_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (any_heavy(pl) || (pl->upper_active && any_heavy(pl->upper))) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->dispensers, 0, 2 * NROUTE * sizeof(uint32_t), st));
+    Chain ch{st, !pl->timing};
     auto run = [&](spsyrk_plan_s* v) {
         switch (v->dtype) {
-            case SPSYRK_F64: return numeric_typed<double>(v, d_c_colidx, d_c_vals, st);
-            case SPSYRK_F32: return numeric_typed<float>(v, d_c_colidx, d_c_vals, st);
-            default: return numeric_typed<int32_t>(v, d_c_colidx, d_c_vals, st);
+            case SPSYRK_F64: return numeric_typed<double>(v, d_c_colidx, d_c_vals, ch);
+            case SPSYRK_F32: return numeric_typed<float>(v, d_c_colidx, d_c_vals, ch);
+            default: return numeric_typed<int32_t>(v, d_c_colidx, d_c_vals, ch);
         }
     };
     pl->out_begin = d_c_rowptr;
@@ -1176,10 +1235,11 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     pl->have_onepass = false;
     // heavy rows: their counts come from their own kernels (bitmaps), as in the symbolic pass
-    spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, st);
+    Chain ch{st, !pl->timing};
+    spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, ch);
     if (s != SPSYRK_OK) return s;
-    s = launch_symbolic_cta<1024>(pl, 7, st);
-    if (s == SPSYRK_OK) s = route_heavy(pl, st);
+    s = launch_symbolic_cta<1024>(pl, 7, ch);
+    if (s == SPSYRK_OK) s = route_views(pl, st);
     if (s != SPSYRK_OK) return s;
     if (rows > 0) {
         onepass_slots_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev, pl->cls, pl->cnt, pl->diag, rows, pl->ub);
@@ -1207,11 +1267,13 @@ spsyrk_status_t spsyrk_onepass_numeric(spsyrk_plan_t plan, int32_t* d_slot_colid
     pl->cnt_out = pl->cnt;
     pl->out_begin = pl->ub_off;
     pl->out_end = pl->ub_off + 1;
+    if (any_heavy(pl)) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->dispensers, 0, 2 * NROUTE * sizeof(uint32_t), st));
+    Chain ch{st, !pl->timing};
     spsyrk_status_t s;
     switch (pl->dtype) {
-        case SPSYRK_F64: s = numeric_typed<double>(pl, d_slot_colidx, d_slot_vals, st); break;
-        case SPSYRK_F32: s = numeric_typed<float>(pl, d_slot_colidx, d_slot_vals, st); break;
-        default: s = numeric_typed<int32_t>(pl, d_slot_colidx, d_slot_vals, st); break;
+        case SPSYRK_F64: s = numeric_typed<double>(pl, d_slot_colidx, d_slot_vals, ch); break;
+        case SPSYRK_F32: s = numeric_typed<float>(pl, d_slot_colidx, d_slot_vals, ch); break;
+        default: s = numeric_typed<int32_t>(pl, d_slot_colidx, d_slot_vals, ch); break;
     }
     pl->cnt_out = nullptr;
     pl->map_filled = map_was;

@@ -55,6 +55,16 @@ struct ScopedHostBlock : HostBlock {
         if (_e != cudaSuccess) return SPSYRK_ERR_CUDA;         \
     } while (0)
 
+// Kernels that do not depend on one another (the row classes of a pass, the two views of the full-output mode) are launched as a
+// chain (programmatic dependent launch): a kernel of the chain may start when every CTA of the one before has started,
+// so that small launches run side by side and the tail of one is filled by the next.  A kernel calls chain_begin first;
+// one thread of it waits at the end for the kernel before, so that the last kernel's end is the end of all of
+// them, which is what the next ordinary launch waits for.  (Launched the ordinary way both calls do nothing.)
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_end() {
+    if (blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __host__ __device__ constexpr int ilog2_ce(int v) { return v <= 1 ? 0 : 1 + ilog2_ce(v >> 1); }
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     __shared__ uint32_t scratch[33];
     __shared__ uint32_t s_sel[2];
     __shared__ uint32_t s_nlong;
+    chain_begin();
     const uint32_t cw = chunk_bits >> 5;
     uint32_t* bits = reinterpret_cast<uint32_t*>(smem_raw);
     uint32_t* rank = bits + cw;  // numeric only
@@ -66,7 +67,10 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     const int tid = threadIdx.x;
     // later rows carry longer column prefixes: hand them out first so that the tail of the launch is light
     const int32_t rloc = rows[gridDim.x - 1 - blockIdx.x];
-    if (NUMERIC && (rloc < row_lo || rloc >= row_hi)) return;
+    if (NUMERIC && (rloc < row_lo || rloc >= row_hi)) {
+        chain_end();
+        return;
+    }
     const int64_t i = (int64_t)P.r0 + rloc;
     const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
     const int64_t p0 = P.rowptr[i];
@@ -82,7 +86,11 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
         int hit = 0;
         for (uint32_t b0 = tid; b0 < deg; b0 += THREADS) hit |= (P.desc[p0 + b0].y == U);
         if (__syncthreads_or(hit)) {
+            const uint32_t nblk = (U + BASE_BLOCK - 1) / BASE_BLOCK;
+            if (nblk <= blocks_per_row)
+                for (uint32_t blk = tid; blk < nblk; blk += THREADS) block_base[(uint64_t)i * blocks_per_row + blk] = blk * BASE_BLOCK;
             if (tid == 0) cnt[rloc] = (int32_t)U;
+            chain_end();
             return;
         }
     }
@@ -363,6 +371,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
         __syncthreads();
     }
     if (!NUMERIC && tid == 0) cnt[rloc] = (int32_t)total_cnt;
+    chain_end();
 }
 
 }  // namespace spsyrk

@@ -2,9 +2,10 @@
 // entries of every row, and a row goes to the kernel that suits it (route_rows_kernel):
 //   rank   : a bitmap of the columns that occur, prefix population counts turn it into column -> slot, partial products
 //            are added into slots.  Two walks over the lists, shared memory by the row's entries.  Sparse rows.
-//   direct : accumulators indexed by column, for a chunk of columns at a time.  One walk, no ranks, but every column
-//            of the range is swept.  Rows that fill their range, or have more entries than slots fit an SM.  A long
-//            row is cut into parts of whole chunks: the symbolic pass has left the number of entries before every block of columns.
+//   direct : accumulators indexed by column, one walk, no ranks, but every column of the range is swept: short ranges that
+//            the row fills, and dense rows of binary matrices that dense8 does not take (chunk by chunk).
+// A row with more entries than slots fit an SM is cut into parts of whole blocks of columns: the symbolic pass has left
+// the number of entries before every block.
 //   dense8 : rows of a binary matrix in which every column occurs: four 8-bit counters per word, the heaviest
 //            columns counted through bit masks.
 // All are persistent: a CTA takes its next row from a counter, so that no launch waits for its longest row's wave and
@@ -13,17 +14,21 @@
 // Before, every heavy row went through a bitmap, 32-bit ranks and one size of slots (512 threads up to 32768 products, 1024
 // above), rows with more entries than slots into global slices with L2 atomics, dense rows of binary matrices
 // through a 200 KB tile with one CTA per SM.  Large power-law workload (96 000 heavy rows, 1.46e9 products, single precision):
-// 7.3 + 7.4 + 0.6 ms before, rank 5.9 ms (0.6e9 products) and direct 8.8 ms now; binary Zipf workload of 50000 rows
-// (1.25e9 counts and similarities): 10.8 ms before, dense8 4.4 ms = 3.4 TB/s of output.
+// 15.3 ms before, 12.2 now; binary Zipf workload of 50000 rows (1.25e9 counts and similarities): 10.8 ms before, dense8
+// 4.4 ms = 3.4 TB/s of output.
 #pragma once
 #include "transpose.cuh"
 
 namespace spsyrk {
 
-enum : int { ROUTE_RANK0 = 0, ROUTE_RANK1, ROUTE_RANK2, ROUTE_RANK_MID, ROUTE_RANK_BIG, ROUTE_DIRECT, ROUTE_PARTS, ROUTE_DENSE8, ROUTE_WIDE, NROUTE };
+enum : int { ROUTE_RANK0 = 0, ROUTE_RANK1, ROUTE_RANK2, ROUTE_RANK_MID, ROUTE_RANK_BIG, ROUTE_RANK_PARTS, ROUTE_DIRECT, ROUTE_DENSE8, ROUTE_WIDE, NROUTE };
 
-constexpr int DIRECT_MAX_PARTS = 8;
-constexpr int64_t DIRECT_PART_WORK = 131072;  // products of a part of a row, at least
+// A row of the rank kernel is cut into parts of at most slots_big entries; every part but the last has more than
+// slots_big - BASE_BLOCK, so 2^18 columns make at most 22 parts of 20480 doubles.
+constexpr int MAX_ROW_PARTS = 24;
+
+// a row or part of one: blocks [first, end) of BASE_BLOCK columns
+__host__ __device__ __forceinline__ int pack_blocks(uint32_t first, uint32_t end) { return (int)(first | end << 8); }
 
 // What the choice needs to know; bytes are shared memory of the kernels as launched
 struct RouteRule {
@@ -37,10 +42,11 @@ struct RouteRule {
 
 // One thread per heavy row (classes 6 and 7, the last rows first: they carry the longest lists).
 static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, RouteRule R, const int32_t* __restrict__ rows, int64_t count,
-                                                                const int32_t* __restrict__ cnt, int32_t* __restrict__ lists, int64_t cap,
-                                                                int2* __restrict__ parts_list, uint32_t* __restrict__ counters) {
+                                                                const int32_t* __restrict__ cnt, const uint32_t* __restrict__ block_base, uint32_t blocks_per_row,
+                                                                int32_t* __restrict__ lists, int64_t cap, int2* __restrict__ rank_parts,
+                                                                uint32_t* __restrict__ counters) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int route = -1, parts = 1;
+    int route = -1;
     int32_t rloc = 0;
     if (n < count) {
         rloc = rows[count - 1 - n];
@@ -48,22 +54,42 @@ static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, Route
         const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
         const uint32_t entries = (uint32_t)cnt[rloc];
         const int64_t w = P.work[rloc], deg = P.rowptr[i + 1] - P.rowptr[i];
-        const uint32_t chunks = (U + R.chunk - 1) / R.chunk;
-        // Direct against rank: a product costs about 25 cycles of an SM per 32 in one walk against 38 in two, a column of the
-        // range 1/8 against 1/40 of a cycle, a chunk after the first about 3000 for its searches and barriers.
-        if (U > R.wide) route = ROUTE_WIDE;
-        else if (R.binary && entries == U && deg <= 255 && U <= R.dense8) route = ROUTE_DENSE8;
-        else if (entries > R.slots_big || w >= (int64_t)(U / 4) + (int64_t)(chunks - 1) * 7000) {
-            // one CTA on the longest row (1e6 products) took as long as all the others together
-            parts = (int)min(min(w / DIRECT_PART_WORK, (int64_t)DIRECT_MAX_PARTS), (int64_t)chunks);
-            route = parts > 1 ? ROUTE_PARTS : ROUTE_DIRECT;
+        const uint32_t blocks = (U + BASE_BLOCK - 1) / BASE_BLOCK;
+        const bool dense = entries == U;
+        if (U > R.wide) {
+            route = ROUTE_WIDE;
+        } else if (R.binary && dense && deg <= 255 && U <= R.dense8) {
+            route = ROUTE_DENSE8;
+        } else if ((R.binary && dense) || (U <= R.chunk && w >= (int64_t)(U / 4))) {
+            // one chunk: a product takes about 25 cycles of an SM per 32 in one walk against 75 in two, a column 1/8 against
+            // 1/40.  (Longer ranges in chunks of 8192 columns: 14 ms per 1e9 products for the searches, barriers and
+            // sweeps of every chunk, against 6.7 in parts of the rank kernel.)
+            route = ROUTE_DIRECT;
+        } else if (entries <= R.slots_small) {
+            route = U <= R.bits0 ? ROUTE_RANK0 : U <= R.bits1 ? ROUTE_RANK1 : ROUTE_RANK2;
+        } else if (entries <= R.slots_big) {
+            route = entries <= R.slots_mid ? ROUTE_RANK_MID : ROUTE_RANK_BIG;
+        } else {
+            // as many blocks as the slots hold (a block has fewer entries than that)
+            uint32_t end[MAX_ROW_PARTS];
+            int parts = 0;
+            const uint32_t* base = block_base + (uint64_t)i * blocks_per_row;
+            uint32_t from = 0;
+            for (uint32_t b = 1; b <= blocks; ++b) {
+                const uint32_t upto = b < blocks ? base[b] : entries;
+                if (upto - from > R.slots_big && parts < MAX_ROW_PARTS - 1) {
+                    end[parts++] = b - 1;
+                    from = base[b - 1];
+                }
+            }
+            end[parts++] = blocks;
+            const uint32_t at = atomicAdd(&counters[ROUTE_RANK_PARTS], (uint32_t)parts);
+            for (int k = 0; k < parts; ++k) rank_parts[at + k] = make_int2(rloc, pack_blocks(k ? end[k - 1] : 0u, end[k]));
         }
-        else if (entries <= R.slots_small) route = U <= R.bits0 ? ROUTE_RANK0 : U <= R.bits1 ? ROUTE_RANK1 : ROUTE_RANK2;
-        else route = entries <= R.slots_mid ? ROUTE_RANK_MID : ROUTE_RANK_BIG;
     }
 #pragma unroll
     for (int k = 0; k < NROUTE; ++k) {  // one atomic per warp and route
-        if (k == ROUTE_PARTS) continue;
+        if (k == ROUTE_RANK_PARTS) continue;
         const unsigned votes = __ballot_sync(FULL_MASK, route == k);
         if (route == k) {
             const int leader = __ffs(votes) - 1;
@@ -72,10 +98,6 @@ static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, Route
             base = __shfl_sync(votes, base, leader);
             lists[(int64_t)k * cap + base + __popc(votes & ((1u << lane_id()) - 1u))] = rloc;
         }
-    }
-    if (route == ROUTE_PARTS) {
-        const uint32_t base = atomicAdd(&counters[ROUTE_PARTS], (uint32_t)parts);
-        for (int k = 0; k < parts; ++k) parts_list[base + k] = make_int2(rloc, k | parts << 8);
     }
 }
 
@@ -154,10 +176,8 @@ struct HeavyArgs {
     const int64_t* out_end;
     int32_t* c_colidx;
     bool aligned;              // the output arrays start on 16-byte boundaries
-    // direct kernel
-    const int2* parts;         // parts of long rows: (row, part | parts << 8), computed before the list
+    const int2* parts;         // parts of rows (row, pack_blocks), computed before the list
     uint32_t nparts;
-    uint32_t* bounds;          // scratch of DIRECT_BOUNDS words per CTA
     const uint32_t* block_base;  // [absolute row * blocks_per_row + block]: entries of the row before the block of columns
     uint32_t blocks_per_row;
 };
@@ -171,7 +191,7 @@ struct RowQueue {
         if (threadIdx.x == 0) {
             int2 r = make_int2(-1, 0);
             while (n < H.nparts + H.count) {
-                const int2 c = n < H.nparts ? H.parts[n] : make_int2(H.list[n - H.nparts], 1 << 8);
+                const int2 c = n < H.nparts ? H.parts[n] : make_int2(H.list[n - H.nparts], pack_blocks(0u, 255u));  // 255: to the end
                 n = atomicAdd(H.dispenser, 1u);
                 if (c.x >= H.row_lo && c.x < H.row_hi) { r = c; break; }  // (a row range: spsyrk_numeric_rows)
             }
@@ -221,20 +241,33 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
     uint32_t* bits32 = reinterpret_cast<uint32_t*>(bits);
     for (uint32_t w = tid; w < columns / 64; w += THREADS) bits[w] = 0;
 
+    chain_begin();
     RowQueue queue(H);
     for (;;) {
-        const int32_t rloc = queue.next(H, &s_row).x;
+        const int2 unit = queue.next(H, &s_row);
+        const int32_t rloc = unit.x;
         if (rloc < 0) break;
         const int64_t i = (int64_t)P.r0 + rloc;
-        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const uint32_t whole = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const uint32_t b_first = unit.y & 0xff, b_end = (uint32_t)unit.y >> 8;
+        const uint32_t c0 = b_first * BASE_BLOCK, c1 = min(b_end * BASE_BLOCK, whole), U = c1 - c0;  // columns [c0, c1)
         const int64_t p0 = P.rowptr[i];
         const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
-        const int64_t ob = H.out_begin[rloc];
-        const uint32_t entries = (uint32_t)(H.out_end[rloc] - ob);
+        int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
+        if (c1 < whole) oe = ob + H.block_base[(uint64_t)i * H.blocks_per_row + b_end];
+        if (c0 > 0) ob += H.block_base[(uint64_t)i * H.blocks_per_row + b_first];
+        uint32_t entries = (uint32_t)(oe - ob);
+        if (!SPSYRK_IN_RANGE(ob >= H.out_begin[rloc] && oe <= H.out_end[rloc] && entries <= slots && U <= columns, P.err)) entries = 0;
         auto fill = [&](uint32_t b0) {
             const bool on = b0 + tid < deg;
-            const uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
+            uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
             const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
+            if (d.y > 0 && U < whole) {
+                const int32_t* lst = P.at_row + d.x;
+                const uint32_t hi = c1 < whole ? lower_bound_i32(lst, d.y, (int32_t)c1) : d.y;
+                const uint32_t lo = c0 > 0 ? lower_bound_i32(lst, hi, (int32_t)c0) : 0u;
+                d = make_uint2(d.x + lo, hi - lo);
+            }
             batch_fill<Acc, THREADS>(B, d.x, d.y, a);
         };
         // the columns that occur
@@ -242,7 +275,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
             if (b0) __syncthreads();
             fill(b0);
             batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) {
-                if (SPSYRK_IN_RANGE((uint32_t)j < columns, P.err)) atomicOr(&bits32[(uint32_t)j >> 5], 1u << ((uint32_t)j & 31u));
+                const uint32_t rel = (uint32_t)j - c0;
+                if (SPSYRK_IN_RANGE(rel < columns, P.err)) atomicOr(&bits32[rel >> 5], 1u << (rel & 31u));
             });
         }
         for (uint32_t t = tid; t < entries; t += THREADS) acc[t] = Acc(0);
@@ -266,6 +300,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
         __syncthreads();
         // the products
         auto add = [&](uint32_t j, Acc p) {
+            j -= c0;
             if (!SPSYRK_IN_RANGE(j < columns, P.err)) return;
             const uint32_t slot = rank[j >> 6] + __popcll(bits[j >> 6] & ((1ull << (j & 63u)) - 1ull));
             if (SPSYRK_IN_RANGE(slot < entries && slot < slots, P.err)) atomicAdd(&acc[slot], p);
@@ -287,7 +322,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
             bits[w] = 0;
             uint32_t r = rank[w];
             while (b) {
-                const int32_t j = (int32_t)(w * 64u) + __ffsll((long long)b) - 1;
+                const int32_t j = (int32_t)(c0 + w * 64u) + __ffsll((long long)b) - 1;
                 b &= b - 1;
                 if (SPSYRK_IN_RANGE(r < entries, P.err)) {
                     H.c_colidx[ob + r] = j;
@@ -298,6 +333,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
             }
         }
     }
+    chain_end();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -312,50 +348,6 @@ struct DirectSmem {
 };
 
 constexpr int DIRECT_THREADS = 512;
-constexpr int DIRECT_MAX_CHUNKS = 32;  // 2^18 columns in chunks of BASE_BLOCK columns at least
-constexpr int DIRECT_MAX_CTAS = 320;
-constexpr size_t DIRECT_BOUNDS = (size_t)DIRECT_MAX_CHUNKS * DIRECT_THREADS;
-
-// Where the lists of a row pass from one chunk to the next: bounds[c * THREADS + l] = entries of list l in columns below
-// (c + 1) * chunk, for every list and the boundaries k0 <= c < k1 at once: all searches together take little longer than
-// those of one boundary.  At most THREADS lists.
-template <int THREADS>
-__device__ __forceinline__ void list_bounds(const PlanDev& P, int64_t p0, uint32_t deg, uint32_t chunk, uint32_t k0, uint32_t k1, uint32_t* __restrict__ bounds) {
-    constexpr int ILP = 4;
-    const uint32_t total = k1 > k0 ? deg * (k1 - k0) : 0u;
-    for (uint32_t s0 = threadIdx.x; s0 < total; s0 += ILP * THREADS) {
-        const int32_t* lst[ILP];
-        uint32_t lo[ILP], len[ILP], most = 0;
-        int32_t key[ILP];
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            const uint32_t s = s0 + u * THREADS, c = s / deg;
-            const uint2 d = s < total ? P.desc[p0 + (s - c * deg)] : make_uint2(0u, 0u);
-            lst[u] = P.at_row + d.x;
-            lo[u] = 0;
-            len[u] = d.y;
-            key[u] = (int32_t)((k0 + c + 1) * chunk);
-            most = max(most, d.y);
-        }
-        for (; most > 0; most >>= 1) {
-            int32_t v[ILP];
-#pragma unroll
-            for (int u = 0; u < ILP; ++u) v[u] = len[u] ? lst[u][lo[u] + (len[u] >> 1)] : 0;
-#pragma unroll
-            for (int u = 0; u < ILP; ++u) {
-                if (len[u]) {
-                    const uint32_t half = len[u] >> 1;
-                    if (v[u] < key[u]) { lo[u] += half + 1; len[u] -= half + 1; } else len[u] = half;
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            const uint32_t s = s0 + u * THREADS, c = s / deg;
-            if (s < total && SPSYRK_IN_RANGE(k0 + c < (uint32_t)DIRECT_MAX_CHUNKS, P.err)) bounds[(k0 + c) * THREADS + (s - c * deg)] = lo[u];
-        }
-    }
-}
 
 // a row's bits of the heavy columns (planes in use: 32 columns each)
 struct HeavyMask {
@@ -383,16 +375,15 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
     uint8_t* occurs = reinterpret_cast<uint8_t*>(acc + chunk);                           // [chunk]
     uint32_t* votes = reinterpret_cast<uint32_t*>(occurs + chunk);                       // [chunk / 32]
     ListBatch<Acc, THREADS>& B = *reinterpret_cast<ListBatch<Acc, THREADS>*>(votes + chunk / 32);
-    uint32_t* const bounds = H.bounds + blockIdx.x * DIRECT_BOUNDS;
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool ones = P.binary != 0;
     const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
     for (uint32_t t = tid; t < chunk; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
 
+    chain_begin();
     RowQueue queue(H);
     for (;;) {
-        const int2 unit = queue.next(H, &s_row);
-        const int32_t rloc = unit.x;
+        const int32_t rloc = queue.next(H, &s_row).x;
         if (rloc < 0) break;
         const int64_t i = (int64_t)P.r0 + rloc;
         const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
@@ -403,17 +394,9 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
         const int planes = ones && dense ? heavy_planes(P) : 0;
         const bool use_masks = planes > 0;
         const HeavyMask mine = load_heavy_mask(P, i, planes);
-        const uint32_t nchunks = (U + chunk - 1) / chunk, part = unit.y & 0xff, parts = (uint32_t)unit.y >> 8;
-        const uint32_t ca = nchunks * part / parts, cb = nchunks * (part + 1) / parts;  // chunks of this part
-        const bool one_batch = deg <= THREADS;
-        if (one_batch && nchunks > 1) {
-            list_bounds<THREADS>(P, p0, deg, chunk, ca > 0 ? ca - 1 : 0u, min(cb, nchunks - 1), bounds);
-            __syncthreads();
-        }
-        uint32_t done = dense ? ca * chunk : ca > 0 ? H.block_base[(uint64_t)i * H.blocks_per_row + ca * chunk / BASE_BLOCK] : 0u;  // entries before the chunk
-        uint32_t passed = one_batch && ca > 0 && (uint32_t)tid < deg ? bounds[(ca - 1) * THREADS + tid] : 0u;  // this thread's list up to the chunk
-        for (uint32_t c = ca; c < cb; ++c) {
-            const uint32_t c0 = c * chunk, c1 = min(c0 + chunk, U), cn = c1 - c0;
+        uint32_t done = 0;  // entries of the chunks before
+        for (uint32_t c0 = 0; c0 < U; c0 += chunk) {
+            const uint32_t c1 = min(c0 + chunk, U), cn = c1 - c0;
             if (use_masks) {
                 for (uint32_t t = tid; t < cn; t += THREADS) {
                     uint32_t n = 0;
@@ -434,11 +417,9 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
                 uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
                 if (use_masks && on && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
                 uint32_t lo = 0, hi = d.y;  // the list's entries in [c0, c1)
-                if (d.y > 0 && nchunks > 1) {
-                    const int32_t* lst = P.at_row + d.x;
-                    lo = one_batch ? passed : c0 == 0 ? 0u : lower_bound_i32(lst, d.y, (int32_t)c0);
-                    if (c1 < U) hi = one_batch ? bounds[c * THREADS + tid] : lo + lower_bound_i32(lst + lo, d.y - lo, (int32_t)c1);
-                    passed = hi;
+                if (d.y > 0 && U > chunk) {
+                    if (c1 < U) hi = lower_bound_i32(P.at_row + d.x, d.y, (int32_t)c1);
+                    if (c0 > 0) lo = lower_bound_i32(P.at_row + d.x, hi, (int32_t)c0);
                 }
                 const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
                 if (b0) __syncthreads();
@@ -487,6 +468,7 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
             __syncthreads();
         }
     }
+    chain_end();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -509,6 +491,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, H
     ListBatch<int32_t, THREADS>& B = *reinterpret_cast<ListBatch<int32_t, THREADS>*>(d8_smem + ((size_t)columns + 15) / 16 * 16 + 16);
     const int tid = threadIdx.x;
     const int planes = heavy_planes(P);
+    chain_begin();
     RowQueue queue(H);
     for (;;) {
         const int32_t rloc = queue.next(H, &s_row).x;
@@ -580,6 +563,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, H
             }
         }
     }
+    chain_end();
 }
 
 }  // namespace spsyrk

@@ -107,6 +107,7 @@ numeric_warp_kernel(PlanDev P, const uint4* __restrict__ hdr, int64_t nrows, con
     static_assert(R >= 1 && (R & (R - 1)) == 0, "keys per lane");
     extern __shared__ __align__(16) unsigned char nw_smem[];
 
+    chain_begin();
     const int lane = lane_id(), gl = lane & (G - 1);
     const int gq = threadIdx.x / G;  // group inside the CTA
     unsigned char* gs = nw_smem + (size_t)gq * SM::GROUP;
@@ -343,6 +344,7 @@ numeric_warp_kernel(PlanDev P, const uint4* __restrict__ hdr, int64_t nrows, con
         hB = hA; lB = lNew; hA = hNew;
     }
     cp_async_wait<0>();
+    chain_end();
     (void)c_rowend;
 }
 
@@ -373,6 +375,7 @@ __global__ void __launch_bounds__(symbolic_warps(N) * 32) symbolic_warp_kernel(P
     constexpr int SHIFT = 32 - ilog2_ce(T);
     extern __shared__ __align__(16) unsigned char sw_smem[];
 
+    chain_begin();
     const int lane = lane_id(), gl = lane & (G - 1);
     const int gq = threadIdx.x / G;
     unsigned char* gs = sw_smem + (size_t)gq * SM::GROUP;
@@ -492,6 +495,7 @@ __global__ void __launch_bounds__(symbolic_warps(N) * 32) symbolic_warp_kernel(P
         hB = hA; lB = lNew; hA = hNew;
     }
     cp_async_wait<0>();
+    chain_end();
 }
 
 // =============================================================================================
@@ -533,6 +537,7 @@ symbolic_sort_warp_kernel(PlanDev P, const uint4* __restrict__ hdr, const int64_
     constexpr Key PAD = ~Key(0);
     extern __shared__ __align__(16) unsigned char ss_smem[];
 
+    chain_begin();
     const int lane = lane_id(), gl = lane & (G - 1);
     const int gq = threadIdx.x / G;
     unsigned char* gs = ss_smem + (size_t)gq * SM::GROUP;
@@ -694,6 +699,7 @@ symbolic_sort_warp_kernel(PlanDev P, const uint4* __restrict__ hdr, const int64_
         hB = hA; lB = lNew; hA = hNew;
     }
     cp_async_wait<0>();
+    chain_end();
 }
 
 template <typename V, int N>
@@ -722,6 +728,7 @@ numeric_map_warp_kernel(PlanDev P, const uint4* __restrict__ hdr, const int64_t*
     constexpr int R = N / G;
     extern __shared__ __align__(16) unsigned char nm_smem[];
 
+    chain_begin();
     const int lane = lane_id(), gl = lane & (G - 1);
     const int gq = threadIdx.x / G;
     unsigned char* gs = nm_smem + (size_t)gq * SM::GROUP;
@@ -898,6 +905,7 @@ numeric_map_warp_kernel(PlanDev P, const uint4* __restrict__ hdr, const int64_t*
         hB = hA; lB = lNew; hA = hNew; ioB = ioNew;
     }
     cp_async_wait<0>();
+    chain_end();
 }
 
 }  // namespace spsyrk
