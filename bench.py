@@ -416,7 +416,7 @@ def roofline_and_variants(a, args, line, ctx, headline):
     diag_apart = True  # lower-triangle mode over the whole column range: light rows are classed without their diagonal products
     cls = class_of_rows(work - (deg if diag_apart else 0), deg, work)
     dom = int(np.argmax(num_ms))
-    sel = cls == dom
+    sel = cls == dom if dom <= 5 else cls >= 6  # the heavy rows of both classes are timed as one
     # Column lists that fit in L2 are read from DRAM once, not once per multiply-add: the launch's
     # algorithmic bytes are then its rows of A, the column lists once, and its output.
     at_bytes = a.nnz * (4 + sv)
@@ -429,7 +429,7 @@ def roofline_and_variants(a, args, line, ctx, headline):
     if dom <= 5:
         kernel = ("numeric_map_warp_kernel<N=%d>" if line["config"]["item_map"] else "numeric_warp_kernel<N=%d>") % (16 << dom)
     else:
-        kernel = "rows_cta_kernel<%d threads, numeric>" % (256 if dom == 6 else 1024)
+        kernel = "rows_rank_kernel / rows_direct_kernel / rows_dense8_kernel (all heavy rows)"
     traffic = None
     if NCU_TRAFFIC_BYTES_PER_MAC is not None and dom == 4 and a.vals.dtype == np.float64 and not lists_in_l2 and line["config"]["item_map"]:
         traffic = NCU_TRAFFIC_BYTES_PER_MAC * float(work[sel].sum())
