@@ -139,7 +139,8 @@ struct RadixSmem {
 // HAS_PC: a third payload pc (32 bits; nullptr = the element's own index) travels along and the functor is
 // called as emit(dest, key, pa, pb, pc).
 // An element whose position is not in [0, n) is dropped: it takes keys that were not counted (a matrix that failed its
-// checks, which the caller learns of later).
+// checks, which the caller learns of later).  Then places of the output also stay unwritten, and what the next pass reads
+// there is whatever the memory held: an emit that indexes by a payload tests it.
 template <int BITS, typename PB, typename Emit, bool HAS_PC, typename S>
 __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pa,
                                                                       const PB* __restrict__ pb, const uint32_t* __restrict__ pc,

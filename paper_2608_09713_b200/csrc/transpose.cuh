@@ -151,8 +151,8 @@ template <> struct alignas(8) ColRec<int32_t> { int32_t j; int32_t v; };
 // G lanes per row, one sweep over the nonzeros of A: the checks of the row pointers (a row indexes nothing unless its own
 // two are sane) and of the column ids (in range, strictly ascending inside the row), the column histogram (its scan gives
 // colptr), the explicit row id of every nonzero (the radix sort's first payload), the row lengths, and whether
-// every stored value is one.  Nothing waits for the checks: the kernels up to the plan's one synchronisation index
-// nothing by what they would have found wrong.
+// every stored value is one.  Nothing waits for the checks: the kernels up to the plan's one synchronisation test what
+// they index by, or look at the error word first.
 template <int G, typename V>
 static __global__ void __launch_bounds__(256) row_expand_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
                                                                 const V* __restrict__ vals, int32_t m, int32_t n, int64_t nnz,
@@ -191,7 +191,9 @@ struct EmitTransposeFinal {
     PlanDev P;
     uint2* desc_hi;  // null in lower-triangle mode
     __device__ __forceinline__ void operator()(int64_t s, uint32_t k, uint32_t row, VB val, uint32_t p) const {
-        if (k >= (uint32_t)P.n) return;  // not a canonical matrix: reported when the plan synchronises
+        // A matrix that failed its checks (reported when the plan synchronises): keys that were not counted leave places of a
+        // pass's output unwritten, so the next pass may bring any key and any position.
+        if (k >= (uint32_t)P.n || (int64_t)p >= P.nnz) return;
         const int64_t cs = P.colptr[k];
         P.at_row[s] = (int32_t)row;
         if constexpr (sizeof(VB) == 8) static_cast<uint4*>(P.at_rec)[s] = make_uint4(row, 0u, (uint32_t)val, (uint32_t)(val >> 32));

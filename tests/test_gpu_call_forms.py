@@ -1,0 +1,60 @@
+"""Calls outside the common sequence: matrices that fail their checks in a workspace with old contents, one plan on
+several streams and threads, row ranges, similarities of values other than one; against the CPU oracle or against the
+same product computed the common way."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_09713_b200 import workloads as W
+from test_gpu_parity import B, dev, run_and_compare  # noqa: F401  (B is the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def random_csr(m, n, per_row, dtype, seed, ones=False):
+    """CSR with 1 to 2 * per_row - 1 entries per row, uniform columns."""
+    rng = np.random.default_rng(seed)
+    rows = [np.unique(rng.integers(0, n, rng.integers(1, 2 * per_row))) for _ in range(m)]
+    rowptr = np.zeros(m + 1, dtype=np.int64)
+    np.cumsum([r.size for r in rows], out=rowptr[1:])
+    vals = np.ones(rowptr[-1]) if ones else rng.integers(1, 9, rowptr[-1]) if dtype == np.int32 else rng.uniform(-1, 1, rowptr[-1])
+    return W.CSR(m, n, rowptr, np.concatenate(rows).astype(np.int32), vals.astype(dtype))
+
+
+# ------------------------------------------------------------------ matrices that fail their checks
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("fault", ["column ids", "one column id", "row pointers", "duplicate"])
+def test_bad_csr_writes_nothing_outside_the_workspace(B, fault, mode):
+    """Three radix passes (n = 2^17 + 3).  The workspace holds words of an earlier use: valid column ids and, as
+    often, positions that would lead behind the workspace, where words that must not change lie."""
+    a = random_csr(3000, (1 << 17) + 3, 8, np.float64, 1)
+    nnz = a.colidx.size
+    rng = np.random.default_rng(2)
+    rowptr, colidx, vals = dev(a)
+    if fault == "column ids":
+        colidx[torch.from_numpy(rng.integers(0, nnz, nnz // 4)).cuda()] = a.n + 5
+    elif fault == "one column id":
+        colidx[7] = a.n + 5
+    elif fault == "row pointers":
+        rowptr[100], rowptr[200] = int(rowptr[150]), 3
+    else:
+        p = int(rowptr[40])
+        colidx[p + 1] = colidx[p]
+    size = B.spsyrk_plan_workspace_bytes(a.m, a.n, nnz, torch.float64, mode)
+    total = 4 * size
+    buf = torch.empty(total, dtype=torch.uint8, device="cuda")
+    words = buf.view(torch.int32)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    near = torch.randint(0, a.n, words.shape, generator=g, device="cuda", dtype=torch.int32)
+    far = torch.randint(size // 8 + 1, (total - size) // 8 - 1, words.shape, generator=g, device="cuda", dtype=torch.int32)
+    words.copy_(torch.where(torch.rand(words.shape, generator=g, device="cuda") < 0.5, near, far))
+    behind = buf[size:].clone()
+    with pytest.raises(B.SpsyrkError) as e:
+        B.spsyrk_plan(a.m, a.n, rowptr, colidx, vals, mode=mode, workspace=buf[:size])
+    assert e.value.status == 2
+    assert torch.equal(buf[size:], behind)
+    plan = B.spsyrk_plan(a.m, a.n, *dev(a), mode=mode, workspace=buf[:size])  # the next plan in the same workspace
+    run_and_compare(B, a, mode, plan=plan)
+    assert torch.equal(buf[size:], behind)
