@@ -204,10 +204,11 @@ struct RowQueue {
     }
 };
 
+// The same formula in the same arithmetic as spsyrk_jaccard: the values need not be ones, so the denominator can be
+// anything a sum of 64 bits holds.
 template <typename V>
 __device__ __forceinline__ void store_jaccard(const PlanDev& P, int64_t at, int32_t j, int32_t c, int32_t deg) {
-    // |a_i| + |a_j| - c < 2^31: the sum of two row lengths minus what they share
-    P.jaccard[at] = __fdiv_rn((float)c, (float)(uint32_t)(deg + P.adeg[j] - c));
+    P.jaccard[at] = __fdiv_rn((float)c, (float)((int64_t)deg + P.adeg[j] - c));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, H
                 if (P.jaccard) {
                     float s[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) s[k] = __fdiv_rn((float)c[k], (float)(uint32_t)((int32_t)deg + P.adeg[j + k] - c[k]));
+                    for (int k = 0; k < 4; ++k) s[k] = __fdiv_rn((float)c[k], (float)(uint32_t)((int32_t)deg + P.adeg[j + k] - c[k]));  // (ones: the sum is a union's size)
                     *reinterpret_cast<float4*>(P.jaccard + ob + j) = make_float4(s[0], s[1], s[2], s[3]);
                 }
             }

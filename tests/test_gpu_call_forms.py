@@ -58,3 +58,21 @@ def test_bad_csr_writes_nothing_outside_the_workspace(B, fault, mode):
     plan = B.spsyrk_plan(a.m, a.n, *dev(a), mode=mode, workspace=buf[:size])  # the next plan in the same workspace
     run_and_compare(B, a, mode, plan=plan)
     assert torch.equal(buf[size:], behind)
+
+
+# ------------------------------------------------------------------ similarities
+@pytest.mark.parametrize("m,n,per_row", [(900, 3000, 120), (20000, 700, 20), (12000, 400, 3)])
+def test_similarities_of_values_other_than_one(B, m, n, per_row):
+    """The fused similarity is spsyrk_jaccard's to the bit for any int32 values: the denominators are negative or zero for
+    many entries (direct, rank and light rows)."""
+    a = random_csr(m, n, per_row, np.int32, m)
+    d = dev(a)
+    rp, ci, cv, plan = B.tril_syrk(a.m, a.n, *d)
+    jac = torch.full((cv.numel(),), -7.0, dtype=torch.float32, device="cuda")
+    B.spsyrk_plan_set_jaccard(plan, jac)
+    B.spsyrk_numeric(plan, rp, ci, cv)
+    want = B.spsyrk_jaccard(a.m, 0, a.m, d[0], rp, ci, cv)
+    assert torch.equal(jac.view(torch.int32), want.view(torch.int32))
+    denominator = (d[0][1:] - d[0][:-1])
+    rows = torch.repeat_interleave(torch.arange(m, device="cuda"), rp[1:] - rp[:-1])
+    assert int((denominator[rows] + denominator[ci.long()] - cv < 0).sum()) > 1000
