@@ -357,7 +357,7 @@ struct Residency {
 };
 
 spsyrk_status_t status_of(uint32_t e) {
-    if (e & (ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED)) return SPSYRK_ERR_BAD_CSR;
+    if (e & ERRW_BAD_CSR) return SPSYRK_ERR_BAD_CSR;
     if (e) return SPSYRK_ERR_INTERNAL;
     return SPSYRK_OK;
 }
@@ -392,11 +392,18 @@ void launch_block_desc(spsyrk_plan_s* pl, cudaStream_t st) {
     note_launches(1);
 }
 
+// analyse: the binary analysis is due (a new plan's first view); at least two CTAs, at most what the GPU holds beside others
 template <int G>
-void launch_row_work(spsyrk_plan_s* pl, cudaStream_t st) {
-    const int64_t rows = pl->dev.r1 - pl->dev.r0, nb = bin_blocks(rows);
-    row_work_kernel<G><<<(unsigned)nb, BIN_THREADS, 0, st>>>(pl->dev, pl->cls, BLOCK_CLASS_MAX_WORK, pl->diag, bin_tile(rows), pl->blockhist, nb,
-                                                             pl->work_total_dev);
+void launch_row_work(spsyrk_plan_s* pl, bool analyse, cudaStream_t st) {
+    const PlanDev& P = pl->dev;
+    const int64_t rows = P.r1 - P.r0, nb = bin_blocks(rows);
+    HeavyArrays heavy{pl->colcnt, pl->facts, pl->heavy_id, pl->heavy_mask, 0u};
+    if (analyse) heavy.ctas = (unsigned)std::min<int64_t>(2 + std::max<int64_t>(P.n, (int64_t)P.m * G) / BIN_THREADS, (int64_t)pl->sm_count * 8);
+    if (nb > 0)
+        row_work_kernel<G><<<(unsigned)nb + heavy.ctas, BIN_THREADS, 0, st>>>(P, pl->cls, BLOCK_CLASS_MAX_WORK, pl->diag, bin_tile(rows), pl->blockhist, nb,
+                                                                             pl->work_total_dev, heavy);
+    else if (analyse) heavy_analysis_kernel<G><<<heavy.ctas, BIN_THREADS, 0, st>>>(P, heavy);
+    else return;
     note_launches(1);
 }
 
@@ -412,7 +419,7 @@ spsyrk_status_t sort_by_column(spsyrk_plan_s* pl, cudaStream_t st) {
     const PlanDev& P = pl->dev;
     if (P.nnz == 0) return SPSYRK_OK;
     const int npass = radix_passes((uint64_t)std::max<int64_t>(P.n - 1, 1));
-    SPSYRK_CUDA_TRY(radix_bins<true>(pl->colcnt, P.n, npass, pl->rx.bins, st));  // from the column counts: n numbers, not nnz keys
+    SPSYRK_CUDA_TRY(radix_bins<true>(pl->colcnt, P.n, npass, pl->rx.bins, st, HeavyHistogram{pl->facts}));  // from the column counts: n numbers, not nnz keys
     const uint32_t* src_key = reinterpret_cast<const uint32_t*>(P.colidx);
     const uint32_t* src_row = pl->rx_row_b;
     const VB* src_val = static_cast<const VB*>(P.vals);
@@ -447,25 +454,26 @@ __global__ void plan_facts_kernel(PlanFacts f) { f.publish(0); }
 
 // Work estimate + binning of one view's current row range (dev.desc, dev.mode and diag are set).  The facts the host
 // needs are on their way to `host` when this returns.
-spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, cudaStream_t st) {
+spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, bool analyse, cudaStream_t st) {
     const int64_t rows = pl->dev.r1 - pl->dev.r0, nb = bin_blocks(rows);
     pl->have_symbolic = false;
     pl->have_onepass = false;
     pl->map_filled = false;
     const PlanDev& P = pl->dev;
     const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->facts, P.err, host};
+    if (P.nnz == 0) analyse = false;
+    switch (group_width(P.nnz, P.m)) {
+        case 4: launch_row_work<4>(pl, analyse, st); break;
+        case 8: launch_row_work<8>(pl, analyse, st); break;
+        case 16: launch_row_work<16>(pl, analyse, st); break;
+        default: launch_row_work<32>(pl, analyse, st); break;
+    }
     if (rows == 0) {
         SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->class_start_dev, 0, (NCLASS + 1) * sizeof(int64_t), st));
         plan_facts_kernel<<<1, 1, 0, st>>>(facts);
         note_launches(1);
         SPSYRK_CUDA_TRY(cudaGetLastError());
         return SPSYRK_OK;
-    }
-    switch (group_width(P.nnz, P.m)) {
-        case 4: launch_row_work<4>(pl, st); break;
-        case 8: launch_row_work<8>(pl, st); break;
-        case 16: launch_row_work<16>(pl, st); break;
-        default: launch_row_work<32>(pl, st); break;
     }
     SPSYRK_CUDA_TRY(scan_launch(ScanArray<int32_t>{pl->blockhist}, NCLASS * nb, BinStarts{pl->offsets, (uint32_t)nb, pl->class_start_dev}, pl->state_bin, P.err, st, true));
     row_scatter_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(P, pl->cls, bin_tile(rows), pl->offsets, nb, pl->diag, pl->perm, pl->hdr, pl->items8, pl->cnt);
@@ -484,7 +492,7 @@ spsyrk_status_t bin_collect(spsyrk_plan_s* pl, const int64_t* host) {
 }
 
 // Descriptors, work estimate and binning of the plan's current block of output rows and columns; synchronises once.
-// fresh: the counters of the binning are zero already.
+// fresh: a new plan's first call (the counters of the binning are zero already, the binary analysis is due).
 spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st) {
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     const bool whole = pl->s0 <= 0 && pl->s1 >= pl->dev.m;
@@ -510,7 +518,7 @@ spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st)
             }
         }
     }
-    spsyrk_status_t s = bin_launch(pl, pl->host.dev, st);
+    spsyrk_status_t s = bin_launch(pl, pl->host.dev, fresh, st);
     if (s != SPSYRK_OK) return s;
     spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
     if (up) {
@@ -519,7 +527,7 @@ spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st)
         up->dev.desc = pl->desc_hi;
         up->dev.jaccard = pl->dev.jaccard;
         up->diag = false;
-        s = bin_launch(up, pl->host.dev + 16, st);
+        s = bin_launch(up, pl->host.dev + 16, false, st);
         if (s != SPSYRK_OK) return s;
         if (rows > 0) {
             add_work_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev.work, up->dev.work, rows, pl->work_sum);
@@ -1041,7 +1049,8 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
     PLAN_TRY(pl->host.acquire());
     PLAN_TRY(cudaMemsetAsync(pl->zero_all, 0, pl->zero_all_bytes, st));
     // 1. one sweep over A (checks, column histogram, row ids, row lengths, values all one?); 2. transpose: the histogram's
-    // scan gives colptr; stable radix sort by column; 3. work estimate and row binning.  One synchronisation at the end.
+    // scan gives colptr; stable radix sort by column; 3. work estimate, row binning and binary analysis.  One synchronisation at
+    // the end: nothing of the plan is under way when the call returns.
     const int g = group_width(nnz, m);
     switch (g) {
         case 4: launch_row_expand<4>(pl, st); break;
@@ -1054,21 +1063,6 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
     if (s != SPSYRK_OK) return fail(s);
     s = estimate_and_bin(pl, true, st);
     if (s != SPSYRK_OK) return fail(s);
-    // 4. binary input: heavy columns as bit masks per row
-    if (P.binary) {
-        const unsigned hb = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)pl->sm_count * 16);
-        heavy_hist_kernel<<<hb, 256, 0, st>>>(pl->colcnt, n, pl->facts + 32);
-        heavy_assign_kernel<<<hb, 256, 0, st>>>(pl->colcnt, n, pl->facts, pl->heavy_id);
-        const unsigned mb = (unsigned)std::min<int64_t>((m * 32 + 255) / 256, (int64_t)pl->sm_count * 8);
-        switch (g) {
-            case 4: heavy_mask_kernel<4><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
-            case 8: heavy_mask_kernel<8><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
-            case 16: heavy_mask_kernel<16><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
-            default: heavy_mask_kernel<32><<<mb, 256, 0, st>>>(d_rowptr, d_colidx, P.m, pl->facts, pl->heavy_id, pl->heavy_mask, P.mask_stride); break;
-        }
-        note_launches(3);
-        PLAN_TRY(cudaGetLastError());
-    }
 #undef PLAN_TRY
     *plan = pl;
     return SPSYRK_OK;

@@ -18,6 +18,7 @@ enum : uint32_t {
     ERRW_UNSORTED = 4u,
     ERRW_INTERNAL = 8u,
     ERRW_UPPER = 16u,
+    ERRW_BAD_CSR = ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED,
 };
 
 // Bounds-checked build (-DSPSYRK_CHECKED, a second library next to the regular one): every index into a

@@ -85,9 +85,14 @@ __device__ __forceinline__ int64_t radix_look_back(S* words, int64_t tile, int d
     return (int64_t)before;
 }
 
-// Sizes of all digits of 32-bit keys: weights[k] elements of key k (keys = nullptr), or the keys themselves
-template <bool COUNTED>
-static __global__ void __launch_bounds__(RX_THREADS) radix_bins_kernel(const uint32_t* __restrict__ in, int64_t n, int passes, unsigned long long* __restrict__ bins) {
+// Sizes of all digits of 32-bit keys: in[k] elements of key k (COUNTED), or the keys themselves.  also(x) is called with
+// every non-zero count (every key).
+struct RadixBinsOnly {
+    __device__ __forceinline__ void operator()(uint32_t) const {}
+};
+template <bool COUNTED, typename Also>
+static __global__ void __launch_bounds__(RX_THREADS) radix_bins_kernel(const uint32_t* __restrict__ in, int64_t n, int passes, unsigned long long* __restrict__ bins,
+                                                                       Also also) {
     __shared__ uint32_t h[RX_MAX_PASSES][RX_BINS];
     for (int d = threadIdx.x; d < RX_MAX_PASSES * RX_BINS; d += RX_THREADS) (&h[0][0])[d] = 0;
     __syncthreads();
@@ -102,6 +107,7 @@ static __global__ void __launch_bounds__(RX_THREADS) radix_bins_kernel(const uin
         for (int u = 0; u < UNR; ++u) {
             if (e + u * stride >= n || (COUNTED && v[u] == 0)) continue;
             const uint32_t key = COUNTED ? (uint32_t)(e + u * stride) : v[u];
+            also(v[u]);
             for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (p * RX_BITS)) & (RX_BINS - 1)], COUNTED ? v[u] : 1u);
         }
     }
@@ -109,11 +115,11 @@ static __global__ void __launch_bounds__(RX_THREADS) radix_bins_kernel(const uin
     for (int d = threadIdx.x; d < passes * RX_BINS; d += RX_THREADS)
         if ((&h[0][0])[d]) atomicAdd(&bins[d], (unsigned long long)(&h[0][0])[d]);
 }
-template <bool COUNTED>
-inline cudaError_t radix_bins(const uint32_t* in, int64_t n, int passes, unsigned long long* bins, cudaStream_t st) {
+template <bool COUNTED, typename Also = RadixBinsOnly>
+inline cudaError_t radix_bins(const uint32_t* in, int64_t n, int passes, unsigned long long* bins, cudaStream_t st, Also also = {}) {
     if (n <= 0) return cudaSuccess;
     const int64_t ctas = std::min<int64_t>((n + RX_THREADS * 4 - 1) / (RX_THREADS * 4), 148 * 4);
-    radix_bins_kernel<COUNTED><<<(unsigned)ctas, RX_THREADS, 0, st>>>(in, n, passes, bins);
+    radix_bins_kernel<COUNTED, Also><<<(unsigned)ctas, RX_THREADS, 0, st>>>(in, n, passes, bins, also);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -58,7 +58,7 @@ struct PlanDev {
 
 // ---------------------------------------------------------------------------------------------
 // Analysis of a binary matrix (every stored value is one, see row_expand_kernel): choice of the heavy columns, the
-// per-row bit masks.  Launched for binary matrices only.
+// per-row bit masks.  The host does not know yet whether the matrix is binary: the CTAs return at once if it is not.
 // facts[0] = 1 if some stored value differs from one; facts[1] = heavy columns; facts[32..] histogram.
 // ---------------------------------------------------------------------------------------------
 // histogram of the column lengths, four bins per octave
@@ -67,24 +67,17 @@ __device__ __forceinline__ int heavy_bin(uint32_t d) {
     const int e = 31 - __clz(d);
     return 4 * e + (int)((d >> (e - 2)) & 3u);
 }
-static __global__ void __launch_bounds__(256) heavy_hist_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[HEAVY_BINS];
-    if (threadIdx.x < HEAVY_BINS) h[threadIdx.x] = 0;
-    __syncthreads();
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; k < n; k += stride) {
-        const uint32_t d = colcnt[k];
-        if (d >= 256u) atomicAdd(&h[heavy_bin(d)], 1u);  // lighter columns are never candidates
+// (few columns are that long: a look at the flag and an atomic each, beside the digit counts of the sort)
+struct HeavyHistogram {
+    uint32_t* facts;
+    __device__ __forceinline__ void operator()(uint32_t d) const {
+        if (d >= 256u && facts[0] == 0) atomicAdd(&facts[32 + heavy_bin(d)], 1u);  // lighter columns are never candidates
     }
-    __syncthreads();
-    if (threadIdx.x < HEAVY_BINS && h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
-}
+};
 
 // Columns of at least the threshold get a bit number; the threshold is the smallest bin such that at most HEAVY_MAX
-// columns lie in it and above.
-static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* __restrict__ facts,
-                                                                 uint8_t* __restrict__ heavy_id) {
+// columns lie in it and above.  Part `part` of `parts`, BIN_THREADS threads.
+static __device__ void heavy_assign(const uint32_t* __restrict__ colcnt, int64_t n, uint32_t* facts, uint8_t* heavy_id, int64_t part, int64_t parts) {
     __shared__ uint32_t s_thr;
     if (threadIdx.x < 32) {
         const int e = 31 - (int)threadIdx.x;  // lane l looks at the octave from 2^(31 - l)
@@ -102,8 +95,8 @@ static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t
     }
     __syncthreads();
     const uint32_t thr = s_thr;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
+    if (thr == 0xffffffffu) return;  // no heavy column: nothing reads the bit numbers
+    for (int64_t k = part * BIN_THREADS + threadIdx.x; k < n; k += parts * BIN_THREADS) {
         uint8_t id = 0xff;
         if (colcnt[k] >= thr) {
             const uint32_t b = atomicAdd(&facts[1], 1u);
@@ -113,20 +106,19 @@ static __global__ void __launch_bounds__(256) heavy_assign_kernel(const uint32_t
     }
 }
 
+// The rows' masks, G lanes per row; the bit numbers were written by other CTAs of the same launch.
 template <int G>
-static __global__ void __launch_bounds__(256) heavy_mask_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, int32_t m,
-                                                               const uint32_t* __restrict__ facts, const uint8_t* __restrict__ heavy_id,
-                                                               uint32_t* __restrict__ heavy_mask, int64_t mask_stride) {
-    if (facts[1] == 0) return;  // no heavy column: nothing reads the masks
+static __device__ void heavy_masks(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, int32_t m, const uint8_t* heavy_id,
+                                   uint32_t* __restrict__ heavy_mask, int64_t mask_stride, int64_t part, int64_t parts) {
     const int gl = threadIdx.x & (G - 1);
-    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
-    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x) / G; base < m; base += groups) {  // uniform per CTA
+    constexpr int GROUPS = BIN_THREADS / G;
+    for (int64_t base = part * GROUPS; base < m; base += parts * GROUPS) {  // uniform per CTA
         const int64_t gid = base + threadIdx.x / G;
         uint32_t mk[HEAVY_PLANES] = {};
         if (gid < m) {
             const int64_t p0 = rowptr[gid], p1 = rowptr[gid + 1];
             for (int64_t p = p0 + gl; p < p1; p += G) {
-                const uint8_t id = heavy_id[colidx[p]];
+                const uint8_t id = __ldcg(heavy_id + colidx[p]);
 #pragma unroll
                 for (int q = 0; q < HEAVY_PLANES; ++q)
                     if ((id >> 5) == q) mk[q] |= 1u << (id & 31);  // (0xff belongs to no plane)
@@ -140,6 +132,45 @@ static __global__ void __launch_bounds__(256) heavy_mask_kernel(const int64_t* _
         }
     }
 }
+
+// The analysis as one of `ctas` CTAs beside the work estimate (which it does not depend on): as launches of their own
+// the two steps cost every plan 6 us, binary or not.  The CTAs that start first hand out the bit numbers and
+// return; the others wait for them, and then build the masks.
+struct HeavyArrays {
+    const uint32_t* colcnt;
+    uint32_t* facts;  // [2] CTAs that have started, [3] CTAs whose share of the bit numbers is written
+    uint8_t* heavy_id;
+    uint32_t* heavy_mask;
+    uint32_t ctas;
+};
+template <int G>
+static __device__ void heavy_analysis(const PlanDev& P, const HeavyArrays& H) {
+    __shared__ uint32_t s_ticket;
+    // the matrix is not binary, or it failed its checks and has column ids that index nothing
+    if (H.facts[0] != 0 || (*P.err & ERRW_BAD_CSR) != 0) return;
+    if (threadIdx.x == 0) s_ticket = atomicAdd(&H.facts[2], 1u);
+    __syncthreads();
+    const uint32_t ticket = s_ticket, assigning = (H.ctas + 3) / 4;
+    if (ticket < assigning) {
+        heavy_assign(H.colcnt, P.n, H.facts, H.heavy_id, ticket, assigning);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) atomicAdd(&H.facts[3], 1u);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        int polls = 0;
+        while (ld_status(&H.facts[3]) < assigning && polls < SPIN_LIMIT) ++polls;
+        if (polls == SPIN_LIMIT) atomicOr(P.err, ERRW_INTERNAL);
+        __threadfence();
+    }
+    __syncthreads();
+    if (ld_status(&H.facts[1]) == 0) return;  // no heavy column: nothing reads the masks
+    heavy_masks<G>(P.rowptr, P.colidx, P.m, H.heavy_id, H.heavy_mask, P.mask_stride, ticket - assigning, H.ctas - assigning);
+}
+// without rows to estimate the work of
+template <int G>
+static __global__ void __launch_bounds__(BIN_THREADS) heavy_analysis_kernel(PlanDev P, HeavyArrays H) { heavy_analysis<G>(P, H); }
 
 // One entry of a column list as a record: what the light-row numeric kernel gathers (one aligned
 // asynchronous copy per entry, whatever the list's offset).
@@ -235,11 +266,15 @@ static __global__ void __launch_bounds__(256) block_desc_kernel(PlanDev P, const
 //   diag: the light-row kernels leave the diagonal products out of their item lists (lower-triangle mode
 //   over the whole column range), so a light row is classed by w minus its number of nonzeros
 // A group takes UNR rows at a time, so that the loads of one row do not wait for those of the row before (one at a time:
-// 438 us for 4.2e6 rows of 16 nonzeros).
+// 438 us for 4.2e6 rows of 16 nonzeros).  The CTAs behind `nblocks` do the binary analysis.
 template <int G>
 static __global__ void __launch_bounds__(BIN_THREADS) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, bool diag, int64_t tile,
                                                                       int32_t* __restrict__ blockhist, int64_t nblocks,
-                                                                      unsigned long long* __restrict__ work_total) {
+                                                                      unsigned long long* __restrict__ work_total, HeavyArrays heavy) {
+    if (blockIdx.x >= nblocks) {
+        heavy_analysis<G>(P, heavy);
+        return;
+    }
     constexpr int GROUPS = BIN_THREADS / G;
     constexpr int UNR = 4;
     __shared__ int32_t hist[NCLASS];
@@ -250,7 +285,7 @@ static __global__ void __launch_bounds__(BIN_THREADS) row_work_kernel(PlanDev P,
     const int gl = threadIdx.x & (G - 1), group = threadIdx.x / G;
     const int64_t rows = P.r1 - P.r0;
     const int64_t t0 = (int64_t)blockIdx.x * tile, t1 = min(t0 + tile, rows);
-    const bool sane = (*P.err & (ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED)) == 0;  // a matrix that failed its checks has no descriptors
+    const bool sane = (*P.err & ERRW_BAD_CSR) == 0;  // a matrix that failed its checks has no descriptors
     unsigned long long mine = 0;    // work of the rows this thread owned
     for (int64_t base = t0; base < t1; base += GROUPS * UNR) {
         int64_t p0[UNR], w[UNR];

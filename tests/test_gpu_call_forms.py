@@ -76,3 +76,26 @@ def test_similarities_of_values_other_than_one(B, m, n, per_row):
     denominator = (d[0][1:] - d[0][:-1])
     rows = torch.repeat_interleave(torch.arange(m, device="cuda"), rp[1:] - rp[:-1])
     assert int((denominator[rows] + denominator[ci.long()] - cv < 0).sum()) > 1000
+
+
+# ------------------------------------------------------------------ streams and threads
+def test_nothing_of_a_plan_is_under_way_when_it_returns(B):
+    """Binary matrix with many columns (its heavy columns are looked for among 2^26): the stream is idle when the plan returns,
+    so the product may be taken on another stream."""
+    m, n = 4000, 1 << 26
+    rng = np.random.default_rng(4)
+    a = random_csr(m, 300, 40, np.float32, 4, ones=True)
+    spread = np.sort(rng.choice(n, 300, replace=False)).astype(np.int32)
+    a = W.CSR(m, n, a.rowptr, spread[a.colidx], a.vals)
+    d = dev(a)
+    ref = oracle.syrk(m, n, a.rowptr, a.colidx, a.vals, oracle.TRIL)
+    torch.cuda.synchronize()
+    other = torch.cuda.Stream()
+    for _ in range(3):
+        plan = B.spsyrk_plan(m, n, *d)
+        assert torch.cuda.current_stream().query()
+        with torch.cuda.stream(other):
+            rp, ci, cv, _ = B.tril_syrk(m, n, *d, plan=plan)
+        torch.cuda.synchronize()
+        assert np.array_equal(rp.cpu().numpy(), ref.rowptr) and np.array_equal(ci.cpu().numpy(), ref.colidx)
+        assert np.array_equal(cv.cpu().numpy().astype(np.float64), ref.vals)
