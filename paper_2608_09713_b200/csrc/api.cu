@@ -713,7 +713,7 @@ spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
     const uint32_t cb = row_chunk_bits(pl, ROW_CHUNK_BITS_MAX_SYMBOLIC);
     const size_t smem = CtaRowSmem<int32_t, THREADS, false>::bytes(cb, 0);
     auto kern = rows_cta_kernel<int32_t, THREADS, false>;
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<int32_t, THREADS, false>>()));
     SPSYRK_CUDA_TRY(ch.launch(brief_rows(count, (int64_t)pl->sm_count * (2048 / THREADS)), kern, (unsigned)count, THREADS, smem, pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr,
                               nullptr, 0, 0, pl->block_base, pl->blocks_per_row));
     return SPSYRK_OK;
@@ -722,6 +722,7 @@ spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
 // Shared-memory shapes of the heavy-row kernels and the rule that goes with them.  The small rank kernel is launched
 // for three widths of its bitmap, so that rows in the lower part of the range leave room for more CTAs per SM.
 constexpr int RANK_SMALL_THREADS = 256, RANK_MID_THREADS = 512, RANK_BIG_THREADS = 1024, DENSE8_THREADS = 512;
+template <int T, int C> struct RankShape { static constexpr int THREADS = T, CTAS = C; };
 constexpr size_t SMEM_PER_CTA = 226 * 1024;
 
 struct HeavyShapes {
@@ -775,11 +776,11 @@ spsyrk_status_t route_views(spsyrk_plan_s* pl, cudaStream_t st) {
 }
 
 // as many CTAs as are resident at once, at most one per row
-template <typename Kernel>
-cudaError_t persistent_grid(const spsyrk_plan_s* pl, Kernel kern, int threads, size_t smem, int64_t count, unsigned* grid) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <auto Kernel>
+cudaError_t persistent_grid(const spsyrk_plan_s* pl, int threads, size_t smem, int64_t count, unsigned* grid) {
+    cudaError_t e = allow_shared_memory<Kernel>();
     int per_sm = 1;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem);
     *grid = (unsigned)std::min<int64_t>(count, (int64_t)pl->sm_count * std::max(per_sm, 1));
     return e;
 }
@@ -804,29 +805,31 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
                          pl->rank_parts, k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u, pl->block_base, pl->blocks_per_row};
     };
     unsigned grid = 0;
-    auto rank = [&](auto kern, int threads, int k, uint32_t columns, uint32_t slots, size_t smem) -> cudaError_t {
-        const int64_t units = (int64_t)pl->route_n[k] + (k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u);
-        if (!units) return cudaSuccess;
-        const cudaError_t e = persistent_grid(pl, kern, threads, smem, units, &grid);
-        if (e != cudaSuccess) return e;
-        return ch.launch(brief_rows(units, grid), kern, grid, threads, smem, pl->dev, args(k), columns, slots, cv);
-    };
     if (const int64_t units = pl->route_n[ROUTE_DIRECT]) {
-        auto kern = rows_direct_kernel<V, DIRECT_THREADS>;
+        constexpr auto kern = rows_direct_kernel<V, DIRECT_THREADS>;
         const size_t smem = DirectSmem<V, DIRECT_THREADS>::bytes(h.rule.chunk);
-        SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DIRECT_THREADS, smem, units, &grid));
+        SPSYRK_CUDA_TRY(persistent_grid<kern>(pl, DIRECT_THREADS, smem, units, &grid));
         SPSYRK_CUDA_TRY(ch.launch(brief_rows(units, grid), kern, grid, DIRECT_THREADS, smem, pl->dev, args(ROUTE_DIRECT), h.rule.chunk, cv));
     }
-    using Small = RankSmem<V, RANK_SMALL_THREADS>;
-    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_BIG_THREADS, 1>, RANK_BIG_THREADS, ROUTE_RANK_BIG, h.columns, h.rule.slots_big, RankSmem<V, RANK_BIG_THREADS>::bytes(h.columns, h.rule.slots_big)));
-    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_MID_THREADS, 2>, RANK_MID_THREADS, ROUTE_RANK_MID, h.columns, h.rule.slots_mid, RankSmem<V, RANK_MID_THREADS>::bytes(h.columns, h.rule.slots_mid)));
-    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_SMALL_THREADS, 4>, RANK_SMALL_THREADS, ROUTE_RANK2, h.columns, h.rule.slots_small, Small::bytes(h.columns, h.rule.slots_small)));
-    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_SMALL_THREADS, 4>, RANK_SMALL_THREADS, ROUTE_RANK1, h.rule.bits1, h.rule.slots_small, Small::bytes(h.rule.bits1, h.rule.slots_small)));
-    SPSYRK_CUDA_TRY(rank(rows_rank_kernel<V, RANK_SMALL_THREADS, 4>, RANK_SMALL_THREADS, ROUTE_RANK0, h.rule.bits0, h.rule.slots_small, Small::bytes(h.rule.bits0, h.rule.slots_small)));
+    auto rank = [&](auto shape, int k, uint32_t columns, uint32_t slots) -> cudaError_t {
+        using Shape = decltype(shape);
+        constexpr auto kern = rows_rank_kernel<V, Shape::THREADS, Shape::CTAS>;
+        const int64_t units = (int64_t)pl->route_n[k] + (k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u);
+        if (!units) return cudaSuccess;
+        const size_t smem = RankSmem<V, Shape::THREADS>::bytes(columns, slots);
+        const cudaError_t e = persistent_grid<kern>(pl, Shape::THREADS, smem, units, &grid);
+        if (e != cudaSuccess) return e;
+        return ch.launch(brief_rows(units, grid), kern, grid, Shape::THREADS, smem, pl->dev, args(k), columns, slots, cv);
+    };
+    SPSYRK_CUDA_TRY(rank(RankShape<RANK_BIG_THREADS, 1>{}, ROUTE_RANK_BIG, h.columns, h.rule.slots_big));
+    SPSYRK_CUDA_TRY(rank(RankShape<RANK_MID_THREADS, 2>{}, ROUTE_RANK_MID, h.columns, h.rule.slots_mid));
+    SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK2, h.columns, h.rule.slots_small));
+    SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK1, h.rule.bits1, h.rule.slots_small));
+    SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK0, h.rule.bits0, h.rule.slots_small));
     if (pl->route_n[ROUTE_DENSE8]) {
-        auto kern = rows_dense8_kernel<V, DENSE8_THREADS, 3>;
+        constexpr auto kern = rows_dense8_kernel<V, DENSE8_THREADS, 3>;
         const size_t smem = Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns);
-        SPSYRK_CUDA_TRY(persistent_grid(pl, kern, DENSE8_THREADS, smem, pl->route_n[ROUTE_DENSE8], &grid));
+        SPSYRK_CUDA_TRY(persistent_grid<kern>(pl, DENSE8_THREADS, smem, pl->route_n[ROUTE_DENSE8], &grid));
         SPSYRK_CUDA_TRY(ch.launch(brief_rows(pl->route_n[ROUTE_DENSE8], grid), kern, grid, DENSE8_THREADS, smem, pl->dev, args(ROUTE_DENSE8), h.dense8_columns, cv));
     }
     if (pl->route_n[ROUTE_WIDE]) {
@@ -835,7 +838,7 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
         const uint32_t slots = std::min((uint32_t)((LARGE_SMEM_BUDGET - fixed) / sizeof(Acc)), h.columns);
         const size_t smem = CtaRowSmem<V, THREADS, true>::bytes(h.columns, slots);
         auto kern = rows_cta_kernel<V, THREADS, true>;
-        SPSYRK_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<V, THREADS, true>>()));
         const HeavyArgs a = args(ROUTE_WIDE);
         SPSYRK_CUDA_TRY(ch.launch(brief_rows(pl->route_n[ROUTE_WIDE], pl->sm_count), kern, pl->route_n[ROUTE_WIDE], THREADS, smem, pl->dev, a.list, h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv,
                                   row_lo, row_hi, nullptr, 0u));

@@ -2,6 +2,7 @@
 // stable class binning.  Header-only; included by every translation unit of libspsyrk.
 #pragma once
 #include <cuda_runtime.h>
+#include <atomic>
 #include <stdint.h>
 #include <type_traits>
 
@@ -55,6 +56,24 @@ struct ScopedHostBlock : HostBlock {
         cudaError_t _e = (expr);                               \
         if (_e != cudaSuccess) return SPSYRK_ERR_CUDA;         \
     } while (0)
+
+// Lets a kernel take all the shared memory of an SM that its static arrays leave, once per device.  A kernel that is
+// launched with several sizes must not have its limit set to each of them in turn: another thread's limit can come between.
+template <auto Kernel>
+inline cudaError_t allow_shared_memory() {
+    static std::atomic<uint64_t> done{0};  // a bit per device
+    int device = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = device < 64 ? uint64_t(1) << device : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    cudaFuncAttributes a{};
+    e = cudaFuncGetAttributes(&a, Kernel);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 // Kernels that do not depend on one another (the row classes of a pass, the two views of the full-output mode) are launched as a
 // chain (programmatic dependent launch): a kernel of the chain may start when every CTA of the one before has started,

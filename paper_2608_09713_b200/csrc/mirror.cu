@@ -306,8 +306,8 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     a.place_stride = three ? sp.pieces : sp.nchunks;
     a.cnt = w.cnt; a.fstart = w.fstart; a.f_colidx = f_colidx; a.f_vals = f_vals; a.err = w.err;
     const size_t split_smem = MirrorSplitSmem<VB>::bytes(1 << sp.lbits), place_smem = MirrorPlaceSmem<VB>::bytes(1 << sp.hbits);
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(mirror_split_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem));
-    SPSYRK_CUDA_TRY(cudaFuncSetAttribute(mirror_place_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)place_smem));
+    SPSYRK_CUDA_TRY(allow_shared_memory<mirror_split_kernel<VB>>());
+    SPSYRK_CUDA_TRY(allow_shared_memory<mirror_place_kernel<VB>>());
     mirror_mark(0, st);
 #define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf)
     if (g <= 16) ROWS(4); else ROWS(16);
@@ -329,7 +329,7 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         mirror_mid_count_kernel<<<units, MS_THREADS, 0, st>>>(a, w.hist);
         SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.partials, w.err, st));
         const size_t mid_smem = MirrorMidSmem<VB>::bytes(1 << sp.mbits);
-        SPSYRK_CUDA_TRY(cudaFuncSetAttribute(mirror_mid_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
+        SPSYRK_CUDA_TRY(allow_shared_memory<mirror_mid_kernel<VB>>());
         mirror_mid_kernel<VB><<<units, MS_THREADS, mid_smem, st>>>(a);
         note_launches(2);
         mirror_mark(pass++, st);

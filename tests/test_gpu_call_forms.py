@@ -1,6 +1,8 @@
 """Calls outside the common sequence: matrices that fail their checks in a workspace with old contents, one plan on
 several streams and threads, row ranges, similarities of values other than one; against the CPU oracle or against the
 same product computed the common way."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -99,3 +101,55 @@ def test_nothing_of_a_plan_is_under_way_when_it_returns(B):
         torch.cuda.synchronize()
         assert np.array_equal(rp.cpu().numpy(), ref.rowptr) and np.array_equal(ci.cpu().numpy(), ref.colidx)
         assert np.array_equal(cv.cpu().numpy().astype(np.float64), ref.vals)
+
+
+def heavy_matrix(m, dtype, seed):
+    """Rows with more than 32 nonzeros over columns of about 40 entries, in every part of the range, among rows with one
+    nonzero; a few rows that outgrow the smaller slot counts."""
+    rng = np.random.default_rng(seed)
+    n = max(m // 40, 64)
+    rows = {i: np.array([rng.integers(n)]) for i in range(m)}
+    for i in rng.choice(m, 300, replace=False):
+        rows[i] = np.sort(rng.choice(n, 34, replace=False))
+    for i in rng.choice(np.arange(m // 2, m), 20, replace=False):
+        rows[i] = np.sort(rng.choice(n, min(400, n), replace=False))
+    rowptr = np.zeros(m + 1, dtype=np.int64)
+    np.cumsum([rows[i].size for i in range(m)], out=rowptr[1:])
+    vals = rng.integers(1, 9, rowptr[-1]) if dtype == np.int32 else rng.uniform(-1, 1, rowptr[-1])
+    return W.CSR(m, n, rowptr, np.concatenate([rows[i] for i in range(m)]).astype(np.int32), vals.astype(dtype))
+
+
+def test_plans_of_several_threads(B):
+    """Every thread has its own matrix, plan and stream; the kernels of the heavy rows are launched with many sizes of shared
+    memory side by side, the mirror's with several."""
+    sizes = (150000, 140000, 70000, 20000)
+    mats = [heavy_matrix(m, np.int32, m) for m in sizes]
+    want = []
+    for a in mats:
+        rp, ci, cv, _ = B.tril_syrk(a.m, a.n, *dev(a))
+        want.append((rp, ci, cv) + tuple(B.spsyrk_mirror(a.m, rp, ci, cv)))
+    torch.cuda.synchronize()
+    failures = []
+
+    def work(k):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                a = mats[k]
+                d = dev(a)
+                rp, ci, cv, plan = B.tril_syrk(a.m, a.n, *d)
+                ci.fill_(-1)
+                for _ in range(1500):
+                    B.spsyrk_numeric(plan, rp, ci, cv)
+                f = B.spsyrk_mirror(a.m, rp, ci, cv)
+                torch.cuda.current_stream().synchronize()
+                if not all(torch.equal(x, y) for x, y in zip((rp, ci, cv) + tuple(f), want[k])):
+                    failures.append((k, "another result"))
+        except Exception as e:  # noqa: BLE001 (reported by the assertion)
+            failures.append((k, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(sizes))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures
