@@ -141,7 +141,6 @@ struct spsyrk_plan_s {
     int2* rank_parts;       // parts of the longest rows
     uint32_t* block_base;   // entries of a heavy row before every block of columns, [row][blocks_per_row]
     uint32_t blocks_per_row;
-    uint32_t* dispensers;   // NROUTE counters the persistent kernels take their rows from
     int64_t sub_row_lo, sub_row_hi;  // with sub_active: the rows (of the plan's range) to compute
     uint32_t* facts;       // binary analysis (device): differs-from-one flag, heavy columns, threshold, histogram
     uint8_t* heavy_id;
@@ -229,7 +228,6 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(items + 1, NCLASS * nb)));
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
     auto route_count = c.take<uint32_t>(2 * NROUTE);  // both views in a row
-    auto dispensers = c.take<uint32_t>(2 * NROUTE);
     auto route_list = c.take<int32_t>(NROUTE * items);
     // rows whose output range is at most 2^18 columns (they are among the first 2^18 rows)
     const int64_t base_rows = std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC);
@@ -272,7 +270,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     }
     if (pl) {
         pl->desc_hi = desc_hi; pl->cnt_tot = cnt_tot; pl->hi_begin = hi_begin; pl->work_sum = work_sum;
-        pl->route_count = route_count; pl->dispensers = dispensers; pl->route_list = route_list; pl->rank_parts = rank_parts;
+        pl->route_count = route_count; pl->route_list = route_list; pl->rank_parts = rank_parts;
         pl->block_base = block_base; pl->blocks_per_row = blocks_per_row;
         pl->dev.mask_stride = mask_stride;
         pl->work_prefix = work_prefix; pl->part_bounds = part_bounds; pl->itemoff = itemoff;
@@ -299,7 +297,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
             up->perm = u_perm; up->hdr = u_hdr; up->cnt = u_cnt; up->cls = u_cls; up->itemoff = u_itemoff;
             up->class_start_dev = u_class_start_dev; up->work_total_dev = u_work_total_dev;
             up->state_bin = u_state_bin; up->state_items = u_state_items;
-            up->route_count = route_count + NROUTE; up->dispensers = dispensers + NROUTE; up->route_list = u_route_list;
+            up->route_count = route_count + NROUTE; up->route_list = u_route_list;
             up->rank_parts = u_rank_parts; up->block_base = u_block_base;
         }
     }
@@ -775,14 +773,14 @@ spsyrk_status_t route_views(spsyrk_plan_s* pl, cudaStream_t st) {
     return s == SPSYRK_OK && up ? route_heavy(up, st) : s;
 }
 
-// as many CTAs as are resident at once, at most one per row
-template <auto Kernel>
-cudaError_t persistent_grid(const spsyrk_plan_s* pl, int threads, size_t smem, int64_t count, unsigned* grid) {
+// A launch of one CTA per row or part of one (the CTAs that start take the others over): a brief one if there are few per CTA
+template <auto Kernel, typename... Args>
+cudaError_t launch_rows(const spsyrk_plan_s* pl, Chain& ch, int64_t units, int threads, size_t smem, Args... args) {
     cudaError_t e = allow_shared_memory<Kernel>();
     int per_sm = 1;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem);
-    *grid = (unsigned)std::min<int64_t>(count, (int64_t)pl->sm_count * std::max(per_sm, 1));
-    return e;
+    if (e != cudaSuccess) return e;
+    return ch.launch(brief_rows(units, (int64_t)pl->sm_count * std::max(per_sm, 1)), Kernel, (unsigned)units, threads, smem, args...);
 }
 
 bool any_heavy(const spsyrk_plan_s* pl) {
@@ -801,37 +799,28 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
     const int64_t row_lo = pl->sub_active ? pl->sub_row_lo : 0, row_hi = pl->sub_active ? pl->sub_row_hi : INT64_MAX;
     const bool aligned = ((reinterpret_cast<uintptr_t>(c_colidx) | reinterpret_cast<uintptr_t>(c_vals) | reinterpret_cast<uintptr_t>(pl->dev.jaccard)) & 15u) == 0;
     auto args = [&](int k) {
-        return HeavyArgs{pl->route_list + k * (pl->rows_cap), pl->route_n[k], pl->dispensers + k, row_lo, row_hi, pl->out_begin, pl->out_end, c_colidx, aligned,
+        return HeavyArgs{pl->route_list + k * (pl->rows_cap), pl->route_n[k], row_lo, row_hi, pl->out_begin, pl->out_end, c_colidx, aligned,
                          pl->rank_parts, k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u, pl->block_base, pl->blocks_per_row};
     };
-    unsigned grid = 0;
     if (const int64_t units = pl->route_n[ROUTE_DIRECT]) {
-        constexpr auto kern = rows_direct_kernel<V, DIRECT_THREADS>;
-        const size_t smem = DirectSmem<V, DIRECT_THREADS>::bytes(h.rule.chunk);
-        SPSYRK_CUDA_TRY(persistent_grid<kern>(pl, DIRECT_THREADS, smem, units, &grid));
-        SPSYRK_CUDA_TRY(ch.launch(brief_rows(units, grid), kern, grid, DIRECT_THREADS, smem, pl->dev, args(ROUTE_DIRECT), h.rule.chunk, cv));
+        SPSYRK_CUDA_TRY((launch_rows<rows_direct_kernel<V, DIRECT_THREADS>>(pl, ch, units, DIRECT_THREADS, DirectSmem<V, DIRECT_THREADS>::bytes(h.rule.chunk), pl->dev,
+                                                                            args(ROUTE_DIRECT), h.rule.chunk, cv)));
     }
     auto rank = [&](auto shape, int k, uint32_t columns, uint32_t slots) -> cudaError_t {
         using Shape = decltype(shape);
-        constexpr auto kern = rows_rank_kernel<V, Shape::THREADS, Shape::CTAS>;
         const int64_t units = (int64_t)pl->route_n[k] + (k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u);
         if (!units) return cudaSuccess;
-        const size_t smem = RankSmem<V, Shape::THREADS>::bytes(columns, slots);
-        const cudaError_t e = persistent_grid<kern>(pl, Shape::THREADS, smem, units, &grid);
-        if (e != cudaSuccess) return e;
-        return ch.launch(brief_rows(units, grid), kern, grid, Shape::THREADS, smem, pl->dev, args(k), columns, slots, cv);
+        return launch_rows<rows_rank_kernel<V, Shape::THREADS, Shape::CTAS>>(pl, ch, units, Shape::THREADS, RankSmem<V, Shape::THREADS>::bytes(columns, slots), pl->dev,
+                                                                             args(k), columns, slots, cv);
     };
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_BIG_THREADS, 1>{}, ROUTE_RANK_BIG, h.columns, h.rule.slots_big));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_MID_THREADS, 2>{}, ROUTE_RANK_MID, h.columns, h.rule.slots_mid));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK2, h.columns, h.rule.slots_small));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK1, h.rule.bits1, h.rule.slots_small));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK0, h.rule.bits0, h.rule.slots_small));
-    if (pl->route_n[ROUTE_DENSE8]) {
-        constexpr auto kern = rows_dense8_kernel<V, DENSE8_THREADS, 3>;
-        const size_t smem = Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns);
-        SPSYRK_CUDA_TRY(persistent_grid<kern>(pl, DENSE8_THREADS, smem, pl->route_n[ROUTE_DENSE8], &grid));
-        SPSYRK_CUDA_TRY(ch.launch(brief_rows(pl->route_n[ROUTE_DENSE8], grid), kern, grid, DENSE8_THREADS, smem, pl->dev, args(ROUTE_DENSE8), h.dense8_columns, cv));
-    }
+    if (const int64_t units = pl->route_n[ROUTE_DENSE8])
+        SPSYRK_CUDA_TRY((launch_rows<rows_dense8_kernel<V, DENSE8_THREADS, 3>>(pl, ch, units, DENSE8_THREADS, Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns), pl->dev,
+                                                                               args(ROUTE_DENSE8), h.dense8_columns, cv)));
     if (pl->route_n[ROUTE_WIDE]) {
         constexpr int THREADS = 1024;
         const size_t fixed = CtaRowSmem<V, THREADS, true>::bytes(h.columns, 0);
@@ -1152,7 +1141,6 @@ spsyrk_status_t spsyrk_numeric(spsyrk_plan_t plan, const int64_t* d_c_rowptr, in
     const int64_t work_all = pl->work_total + (pl->upper_active ? pl->upper->work_total : 0);
     if (work_all > 0 && (!d_c_colidx || !d_c_vals)) return SPSYRK_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (any_heavy(pl) || (pl->upper_active && any_heavy(pl->upper))) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->dispensers, 0, 2 * NROUTE * sizeof(uint32_t), st));
     Chain ch{st, !pl->timing};
     auto run = [&](spsyrk_plan_s* v) {
         switch (v->dtype) {
@@ -1264,7 +1252,6 @@ spsyrk_status_t spsyrk_onepass_numeric(spsyrk_plan_t plan, int32_t* d_slot_colid
     pl->cnt_out = pl->cnt;
     pl->out_begin = pl->ub_off;
     pl->out_end = pl->ub_off + 1;
-    if (any_heavy(pl)) SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->dispensers, 0, 2 * NROUTE * sizeof(uint32_t), st));
     Chain ch{st, !pl->timing};
     spsyrk_status_t s;
     switch (pl->dtype) {

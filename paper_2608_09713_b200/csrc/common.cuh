@@ -81,9 +81,10 @@ inline cudaError_t allow_shared_memory() {
 // one thread of it waits at the end for the kernel before, so that the last kernel's end is the end of all of
 // them, which is what the next ordinary launch waits for.  (Launched the ordinary way both calls do nothing.)
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void chain_end() {
-    if (blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+__device__ __forceinline__ void chain_end(bool this_cta) {  // true in one CTA
+    if (this_cta && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+__device__ __forceinline__ void chain_end() { chain_end(blockIdx.x == 0); }
 
 __host__ __device__ constexpr int ilog2_ce(int v) { return v <= 1 ? 0 : 1 + ilog2_ce(v >> 1); }
 

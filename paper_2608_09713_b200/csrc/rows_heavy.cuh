@@ -8,8 +8,10 @@
 // the number of entries before every block.
 //   dense8 : rows of a binary matrix in which every column occurs: four 8-bit counters per word, the heaviest
 //            columns counted through bit masks.
-// All are persistent: a CTA takes its next row from a counter, so that no launch waits for its longest row's wave and
-// a CTA's buffers stay where they are.
+// All are launched with a CTA per row or part of one, the longest lists first, so that the GPU hands the rows out as CTAs end.
+// (Persistent CTAs that drew their rows from a counter in the plan lost rows when two passes of one plan overlapped; the
+// same rows dealt out beforehand took 1.14 times as long on the large power-law workload.)  In dense8, whose rows are short and
+// alike, a CTA that has finished takes over one that has not started (cluster launch control).
 //
 // Before, every heavy row went through a bitmap, 32-bit ranks and one size of slots (512 threads up to 32768 products, 1024
 // above), rows with more entries than slots into global slices with L2 atomics, dense rows of binary matrices
@@ -170,7 +172,6 @@ __device__ __forceinline__ void batch_walk(const ListBatch<Acc, THREADS>& B, Loa
 struct HeavyArgs {
     const int32_t* list;
     uint32_t count;
-    uint32_t* dispenser;
     int64_t row_lo, row_hi;    // rows of the plan's range to compute
     const int64_t* out_begin;  // where each row's part of the output starts / ends
     const int64_t* out_end;
@@ -182,23 +183,85 @@ struct HeavyArgs {
     uint32_t blocks_per_row;
 };
 
-// The rows of a persistent CTA, one after the other.  Thread 0 draws the number after next while the row is computed.
+// A row, or a part of one, by its number in the launch
+__device__ __forceinline__ int2 heavy_unit(const HeavyArgs& H, uint32_t n) {
+    const int2 u = n < H.nparts ? H.parts[n] : make_int2(H.list[n - H.nparts], pack_blocks(0u, 255u));  // 255: to the end
+    return u.x >= H.row_lo && u.x < H.row_hi ? u : make_int2(-1, 0);  // (a row range: spsyrk_numeric_rows)
+}
+
+// The rows of a CTA, one after the other: its own, then those of CTAs that have not started.  Thread 0 asks for the next CTA
+// while the row is computed (clusterlaunchcontrol.try_cancel; the answer arrives in shared memory and completes a phase
+// of the barrier).  After a refusal nothing is asked for any more, and a CTA does not end with a request under way.
+// (50000 dense rows of up to 50000 columns, counts and similarities: 4.38 ms, with a CTA per row 4.52; the rank kernels
+// gain nothing: 12.6 against 12.5 ms on the large power-law workload.)
+struct RowQueueShared {
+    uint4 answer;
+    unsigned long long barrier;
+    int2 unit;
+};
 struct RowQueue {
-    uint32_t n;
-    __device__ __forceinline__ explicit RowQueue(const HeavyArgs& H) { n = threadIdx.x == 0 ? atomicAdd(H.dispenser, 1u) : 0u; }
+    static constexpr uint32_t NONE = 0xffffffffu;
+    RowQueueShared* s;
+    uint32_t answer_at, barrier_at;  // shared-memory addresses
+    uint32_t n, phase = 0;
+    bool asked = false;
+    bool has_first;  // this CTA has handled the launch's first row: it ends the chain
+
+    __device__ __forceinline__ explicit RowQueue(RowQueueShared* shared) : s(shared), n(blockIdx.x), has_first(blockIdx.x == 0) {
+        answer_at = (uint32_t)__cvta_generic_to_shared(&s->answer);
+        barrier_at = (uint32_t)__cvta_generic_to_shared(&s->barrier);
+        if (threadIdx.x == 0) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barrier_at) : "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+    }
+    __device__ __forceinline__ void ask() {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the answer before has been read
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 16;" ::"r"(barrier_at) : "memory");
+        asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer_at), "r"(barrier_at)
+                     : "memory");
+        asked = true;
+    }
+    __device__ __forceinline__ uint32_t take(uint32_t* err) {
+        if (!asked) return NONE;
+        asked = false;
+        uint32_t done = 0;
+        for (int polls = 0; !done; ++polls) {
+            if (polls == SPIN_LIMIT) {
+                atomicOr(err, ERRW_INTERNAL);
+                return NONE;
+            }
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(done)
+                         : "r"(barrier_at), "r"(phase)
+                         : "memory");
+        }
+        phase ^= 1u;
+        uint32_t cta;
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b128 h;\n\tld.shared.b128 h, [%1];\n\tmov.u32 %0, 0xffffffff;\n\t"
+                     "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+                     "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+                     : "=r"(cta)
+                     : "r"(answer_at)
+                     : "memory");
+        if (cta == 0) has_first = true;
+        return cta;
+    }
     // the next row (or part of one), or -1; contains barriers, after which the row before is finished by all threads
-    __device__ __forceinline__ int2 next(const HeavyArgs& H, int2* s_row) {
+    __device__ __forceinline__ int2 next(const HeavyArgs& H, uint32_t* err) {
         if (threadIdx.x == 0) {
             int2 r = make_int2(-1, 0);
-            while (n < H.nparts + H.count) {
-                const int2 c = n < H.nparts ? H.parts[n] : make_int2(H.list[n - H.nparts], pack_blocks(0u, 255u));  // 255: to the end
-                n = atomicAdd(H.dispenser, 1u);
-                if (c.x >= H.row_lo && c.x < H.row_hi) { r = c; break; }  // (a row range: spsyrk_numeric_rows)
+            if (asked) n = take(err);
+            while (n != NONE) {
+                r = heavy_unit(H, n);
+                ask();
+                if (r.x >= 0) break;
+                n = take(err);
             }
-            *s_row = r;
+            s->unit = r;
         }
         __syncthreads();
-        const int2 r = *s_row;
+        const int2 r = s->unit;
         __syncthreads();
         return r;
     }
@@ -230,7 +293,6 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
     using Acc = typename AccOf<V>::type;
     constexpr int NW = THREADS / 32;
     extern __shared__ __align__(16) unsigned char rk_smem[];
-    __shared__ int2 s_row;
     __shared__ uint32_t s_warp[NW];
     unsigned long long* bits = reinterpret_cast<unsigned long long*>(rk_smem);                 // [columns / 64]
     Acc* acc = reinterpret_cast<Acc*>(bits + columns / 64);                                   // [slots]
@@ -240,14 +302,10 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
     const bool ones = P.binary != 0;
     const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
     uint32_t* bits32 = reinterpret_cast<uint32_t*>(bits);
-    for (uint32_t w = tid; w < columns / 64; w += THREADS) bits[w] = 0;
-
     chain_begin();
-    RowQueue queue(H);
-    for (;;) {
-        const int2 unit = queue.next(H, &s_row);
-        const int32_t rloc = unit.x;
-        if (rloc < 0) break;
+    const int2 unit = heavy_unit(H, blockIdx.x);
+    const int32_t rloc = unit.x;
+    if (rloc >= 0) {
         const int64_t i = (int64_t)P.r0 + rloc;
         const uint32_t whole = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
         const uint32_t b_first = unit.y & 0xff, b_end = (uint32_t)unit.y >> 8;
@@ -258,7 +316,9 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
         if (c1 < whole) oe = ob + H.block_base[(uint64_t)i * H.blocks_per_row + b_end];
         if (c0 > 0) ob += H.block_base[(uint64_t)i * H.blocks_per_row + b_first];
         uint32_t entries = (uint32_t)(oe - ob);
+        const uint32_t words = (U + 63u) / 64u;
         if (!SPSYRK_IN_RANGE(ob >= H.out_begin[rloc] && oe <= H.out_end[rloc] && entries <= slots && U <= columns, P.err)) entries = 0;
+        for (uint32_t w = tid; w < words; w += THREADS) bits[w] = 0;  // (seen by all behind the first batch's barriers)
         auto fill = [&](uint32_t b0) {
             const bool on = b0 + tid < deg;
             uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
@@ -283,7 +343,6 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
         for (uint32_t t = tid; t < entries; t += THREADS) acc[t] = Acc(0);
         __syncthreads();
         // ranks: a warp owns consecutive words, 32 per step
-        const uint32_t words = (U + 63u) / 64u;
         const uint32_t per_warp = ((words + NW - 1) / NW + 31u) & ~31u;
         const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
         uint32_t sum = 0;
@@ -315,12 +374,11 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
             else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc a) { add((uint32_t)r.j, acc_mul(a, (Acc)r.v)); });
         }
         __syncthreads();
-        // out: sums by slot, column ids from the bitmap, which is cleared for the next row
+        // out: sums by slot, column ids from the bitmap
         for (uint32_t t = tid; t < entries; t += THREADS) c_vals[ob + t] = (V)acc[t];
         for (uint32_t w = tid; w < words; w += THREADS) {
             unsigned long long b = bits[w];
             if (b == 0) continue;
-            bits[w] = 0;
             uint32_t r = rank[w];
             while (b) {
                 const int32_t j = (int32_t)(c0 + w * 64u) + __ffsll((long long)b) - 1;
@@ -370,7 +428,6 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
     using Acc = typename AccOf<V>::type;
     constexpr int NW = THREADS / 32;
     extern __shared__ __align__(16) unsigned char dr_smem[];
-    __shared__ int2 s_row;
     __shared__ uint32_t s_warp[NW];
     Acc* acc = reinterpret_cast<Acc*>(dr_smem);                                          // [chunk]
     uint8_t* occurs = reinterpret_cast<uint8_t*>(acc + chunk);                           // [chunk]
@@ -379,13 +436,9 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool ones = P.binary != 0;
     const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
-    for (uint32_t t = tid; t < chunk; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
-
     chain_begin();
-    RowQueue queue(H);
-    for (;;) {
-        const int32_t rloc = queue.next(H, &s_row).x;
-        if (rloc < 0) break;
+    const int32_t rloc = heavy_unit(H, blockIdx.x).x;
+    if (rloc >= 0) {
         const int64_t i = (int64_t)P.r0 + rloc;
         const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
         const int64_t p0 = P.rowptr[i];
@@ -398,7 +451,9 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
         uint32_t done = 0;  // entries of the chunks before
         for (uint32_t c0 = 0; c0 < U; c0 += chunk) {
             const uint32_t c1 = min(c0 + chunk, U), cn = c1 - c0;
-            if (use_masks) {
+            if (!use_masks) {
+                for (uint32_t t = tid; t < cn; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
+            } else {
                 for (uint32_t t = tid; t < cn; t += THREADS) {
                     uint32_t n = 0;
 #pragma unroll
@@ -454,8 +509,6 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
                 if (((b >> lane) & 1u) && t < cn) {
                     const int64_t at = ob + done + (dense ? t : run + __popc(b & ((1u << lane) - 1u)));
                     const Acc v = acc[t];
-                    acc[t] = Acc(0);
-                    occurs[t] = 0;
                     if (SPSYRK_IN_RANGE(at < oe, P.err)) {
                         c_vals[at] = (V)v;
                         H.c_colidx[at] = (int32_t)(c0 + t);
@@ -487,15 +540,15 @@ struct Dense8Smem {
 template <typename V, int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, HeavyArgs H, uint32_t columns, V* __restrict__ c_vals) {
     extern __shared__ __align__(16) unsigned char d8_smem[];
-    __shared__ int2 s_row;
+    __shared__ RowQueueShared s_queue;
     uint32_t* acc = reinterpret_cast<uint32_t*>(d8_smem);  // four columns per word
     ListBatch<int32_t, THREADS>& B = *reinterpret_cast<ListBatch<int32_t, THREADS>*>(d8_smem + ((size_t)columns + 15) / 16 * 16 + 16);
     const int tid = threadIdx.x;
     const int planes = heavy_planes(P);
     chain_begin();
-    RowQueue queue(H);
+    RowQueue queue(&s_queue);
     for (;;) {
-        const int32_t rloc = queue.next(H, &s_row).x;
+        const int32_t rloc = queue.next(H, P.err).x;
         if (rloc < 0) break;
         const int64_t i = (int64_t)P.r0 + rloc;
         const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
@@ -564,7 +617,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, H
             }
         }
     }
-    chain_end();
+    chain_end(queue.has_first);
 }
 
 }  // namespace spsyrk

@@ -153,3 +153,25 @@ def test_plans_of_several_threads(B):
     for t in threads:
         t.join()
     assert not failures
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_one_plan_on_two_streams(B, mode):
+    """Two numeric passes of one plan, and passes over row ranges of it, under way at the same time: every entry is written in
+    all of them."""
+    a = W.rmat(14, 16, 7)
+    rp, ci, cv, plan = B.tril_syrk(a.m, a.n, *dev(a), mode=mode)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = [(torch.full_like(ci, -1), torch.zeros_like(cv)) for _ in range(4)]
+    torch.cuda.synchronize()
+    for st, out in zip(streams, outs):
+        B.spsyrk_numeric(plan, rp, *out, stream=st)
+    for k in range(4):
+        for st, out in zip(streams, outs[2:]):
+            B.spsyrk_numeric_rows(plan, a.m * k // 4, a.m * (k + 1) // 4, rp, *out, stream=st)
+    torch.cuda.synchronize()
+    scale = cv.abs().clamp(min=1e-30)
+    for c, v in outs:
+        assert torch.equal(c, ci)
+        assert float(((v - cv).abs() / scale).max()) <= 1e-5  # (sums of positive products: any order of additions)
