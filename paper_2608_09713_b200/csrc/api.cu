@@ -19,7 +19,7 @@ static std::atomic<long long> g_launches{0};
 void note_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 // Allocating pinned memory takes a millisecond or more, so blocks given back are kept for the next user, up to
-// HOST_POOL_MAX of 512 bytes each.  Blocks are portable: any device's kernels may write them.
+// HOST_POOL_MAX of 1280 bytes each.  Blocks are portable: any device's kernels may write them.
 static std::mutex g_host_mutex;
 static std::vector<int64_t*> g_host_pool;
 constexpr size_t HOST_POOL_MAX = 64;
@@ -109,7 +109,7 @@ struct spsyrk_plan_s {
     int64_t* ub_off;
     int32_t* cnt_out;
     bool have_onepass;
-    HostBlock host;  // words 0..31: facts of the two views; 32..63: the position search of spsyrk_numeric_rows (upper view: unused)
+    HostBlock host;  // words 0..31: facts of the two views; the rest: the position search of spsyrk_numeric_rows (upper view: unused)
     int64_t rows_cap;
     // workspace views
     int32_t* perm;
@@ -141,7 +141,8 @@ struct spsyrk_plan_s {
     int2* rank_parts;       // parts of the longest rows
     uint32_t* block_base;   // entries of a heavy row before every block of columns, [row][blocks_per_row]
     uint32_t blocks_per_row;
-    int64_t sub_row_lo, sub_row_hi;  // with sub_active: the rows (of the plan's range) to compute
+    RoutePieces sub_route[NROUTE];  // with sub_active: the pieces of the heavy rows' lists to compute
+    unsigned long long* route_state;  // both views: [ticket, words of the look-back] each, as many as their heavy rows need
     uint32_t* facts;       // binary analysis (device): differs-from-one flag, heavy columns, threshold, histogram
     uint8_t* heavy_id;
     uint32_t* heavy_mask;
@@ -229,6 +230,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
     auto route_count = c.take<uint32_t>(2 * NROUTE);  // both views in a row
     auto route_list = c.take<int32_t>(NROUTE * items);
+    auto route_state = c.take<unsigned long long>(views * (1 + (size_t)route_tiles(m) * NROUTE));
     // rows whose output range is at most 2^18 columns (they are among the first 2^18 rows)
     const int64_t base_rows = std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC);
     const uint32_t blocks_per_row = (uint32_t)((std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC) + BASE_BLOCK - 1) / BASE_BLOCK);
@@ -270,7 +272,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     }
     if (pl) {
         pl->desc_hi = desc_hi; pl->cnt_tot = cnt_tot; pl->hi_begin = hi_begin; pl->work_sum = work_sum;
-        pl->route_count = route_count; pl->route_list = route_list; pl->rank_parts = rank_parts;
+        pl->route_count = route_count; pl->route_list = route_list; pl->route_state = route_state; pl->rank_parts = rank_parts;
         pl->block_base = block_base; pl->blocks_per_row = blocks_per_row;
         pl->dev.mask_stride = mask_stride;
         pl->work_prefix = work_prefix; pl->part_bounds = part_bounds; pl->itemoff = itemoff;
@@ -713,7 +715,7 @@ spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
     auto kern = rows_cta_kernel<int32_t, THREADS, false>;
     SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<int32_t, THREADS, false>>()));
     SPSYRK_CUDA_TRY(ch.launch(brief_rows(count, (int64_t)pl->sm_count * (2048 / THREADS)), kern, (unsigned)count, THREADS, smem, pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr,
-                              nullptr, 0, 0, pl->block_base, pl->blocks_per_row));
+                              nullptr, pl->block_base, pl->blocks_per_row));
     return SPSYRK_OK;
 }
 
@@ -751,26 +753,29 @@ HeavyShapes heavy_shapes(const spsyrk_plan_s* pl) {
     return h;
 }
 
+int64_t heavy_rows(const spsyrk_plan_s* pl) { return pl->class_start[NCLASS] - pl->class_start[6]; }
+
 // which kernel computes which heavy row; the counts of the symbolic pass are known
-spsyrk_status_t route_heavy(spsyrk_plan_s* pl, cudaStream_t st) {
-    const int64_t count = pl->class_start[NCLASS] - pl->class_start[6];
+spsyrk_status_t route_heavy(spsyrk_plan_s* pl, unsigned long long* state, cudaStream_t st) {
+    const int64_t count = heavy_rows(pl);
     if (count <= 0) return SPSYRK_OK;
     const HeavyShapes h = pl->dtype == SPSYRK_I32 ? heavy_shapes<int32_t>(pl) : heavy_shapes<double>(pl);
-    route_rows_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->block_base,
-                                                                       pl->blocks_per_row, pl->route_list, pl->rows_cap, pl->rank_parts, pl->route_count);
+    route_rows_kernel<<<(unsigned)route_tiles(count), ROUTE_THREADS, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->block_base,
+                                                                              pl->blocks_per_row, pl->route_list, pl->rows_cap, pl->rank_parts, pl->route_count,
+                                                                              state + 1, state);
     note_launches(1);
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
 }
 
 // the lists of both views; without heavy rows nothing is launched and nobody looks at the list lengths
-bool heavy_rows(const spsyrk_plan_s* pl) { return pl->class_start[NCLASS] > pl->class_start[6]; }
 spsyrk_status_t route_views(spsyrk_plan_s* pl, cudaStream_t st) {
     spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
+    const size_t words = 1 + (size_t)route_tiles(heavy_rows(pl)) * NROUTE, up_words = up ? 1 + (size_t)route_tiles(heavy_rows(up)) * NROUTE : 0;
     if (!heavy_rows(pl) && !(up && heavy_rows(up))) return SPSYRK_OK;
-    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->route_count, 0, 2 * NROUTE * sizeof(uint32_t), st));
-    const spsyrk_status_t s = route_heavy(pl, st);
-    return s == SPSYRK_OK && up ? route_heavy(up, st) : s;
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->route_state, 0, (words + up_words) * sizeof(unsigned long long), st));
+    const spsyrk_status_t s = route_heavy(pl, pl->route_state, st);
+    return s == SPSYRK_OK && up ? route_heavy(up, pl->route_state + words, st) : s;
 }
 
 // A launch of one CTA per row or part of one (the CTAs that start take the others over): a brief one if there are few per CTA
@@ -783,32 +788,26 @@ cudaError_t launch_rows(const spsyrk_plan_s* pl, Chain& ch, int64_t units, int t
     return ch.launch(brief_rows(units, (int64_t)pl->sm_count * std::max(per_sm, 1)), Kernel, (unsigned)units, threads, smem, args...);
 }
 
-bool any_heavy(const spsyrk_plan_s* pl) {
-    uint32_t any = 0;
-    for (int k = 0; k < NROUTE; ++k) any |= pl->route_n[k];
-    return any != 0;
-}
-
 template <typename V>
 spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals, Chain& ch) {
     using Acc = typename AccOf<V>::type;
     static_assert(sizeof(Acc) == sizeof(typename AccOf<std::conditional_t<std::is_same<V, int32_t>::value, int32_t, double>>::type), "the rule's shapes");
-    if (!any_heavy(pl)) return SPSYRK_OK;
+    if (!heavy_rows(pl)) return SPSYRK_OK;
     const HeavyShapes h = heavy_shapes<V>(pl);
     V* cv = static_cast<V*>(c_vals);
-    const int64_t row_lo = pl->sub_active ? pl->sub_row_lo : 0, row_hi = pl->sub_active ? pl->sub_row_hi : INT64_MAX;
+    auto pieces = [&](int k) { return pl->sub_active ? pl->sub_route[k] : RoutePieces{{0u, 0u}, {pl->route_n[k], 0u}}; };
     const bool aligned = ((reinterpret_cast<uintptr_t>(c_colidx) | reinterpret_cast<uintptr_t>(c_vals) | reinterpret_cast<uintptr_t>(pl->dev.jaccard)) & 15u) == 0;
     auto args = [&](int k) {
-        return HeavyArgs{pl->route_list + k * (pl->rows_cap), pl->route_n[k], row_lo, row_hi, pl->out_begin, pl->out_end, c_colidx, aligned,
-                         pl->rank_parts, k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u, pl->block_base, pl->blocks_per_row};
+        return HeavyArgs{pl->route_list + k * (pl->rows_cap), pieces(k), pl->out_begin, pl->out_end, c_colidx, aligned,
+                         pl->rank_parts, k == ROUTE_RANK_BIG ? pieces(ROUTE_RANK_PARTS) : RoutePieces{}, pl->block_base, pl->blocks_per_row};
     };
-    if (const int64_t units = pl->route_n[ROUTE_DIRECT]) {
+    if (const int64_t units = pieces(ROUTE_DIRECT).total()) {
         SPSYRK_CUDA_TRY((launch_rows<rows_direct_kernel<V, DIRECT_THREADS>>(pl, ch, units, DIRECT_THREADS, DirectSmem<V, DIRECT_THREADS>::bytes(h.rule.chunk), pl->dev,
                                                                             args(ROUTE_DIRECT), h.rule.chunk, cv)));
     }
     auto rank = [&](auto shape, int k, uint32_t columns, uint32_t slots) -> cudaError_t {
         using Shape = decltype(shape);
-        const int64_t units = (int64_t)pl->route_n[k] + (k == ROUTE_RANK_BIG ? pl->route_n[ROUTE_RANK_PARTS] : 0u);
+        const int64_t units = (int64_t)pieces(k).total() + (k == ROUTE_RANK_BIG ? pieces(ROUTE_RANK_PARTS).total() : 0u);
         if (!units) return cudaSuccess;
         return launch_rows<rows_rank_kernel<V, Shape::THREADS, Shape::CTAS>>(pl, ch, units, Shape::THREADS, RankSmem<V, Shape::THREADS>::bytes(columns, slots), pl->dev,
                                                                              args(k), columns, slots, cv);
@@ -818,19 +817,21 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK2, h.columns, h.rule.slots_small));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK1, h.rule.bits1, h.rule.slots_small));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK0, h.rule.bits0, h.rule.slots_small));
-    if (const int64_t units = pl->route_n[ROUTE_DENSE8])
+    if (const int64_t units = pieces(ROUTE_DENSE8).total())
         SPSYRK_CUDA_TRY((launch_rows<rows_dense8_kernel<V, DENSE8_THREADS, 3>>(pl, ch, units, DENSE8_THREADS, Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns), pl->dev,
                                                                                args(ROUTE_DENSE8), h.dense8_columns, cv)));
-    if (pl->route_n[ROUTE_WIDE]) {
+    const RoutePieces wide = pieces(ROUTE_WIDE);
+    for (int k = 0; k < 2; ++k) {
+        if (!wide.count[k]) continue;
         constexpr int THREADS = 1024;
         const size_t fixed = CtaRowSmem<V, THREADS, true>::bytes(h.columns, 0);
         const uint32_t slots = std::min((uint32_t)((LARGE_SMEM_BUDGET - fixed) / sizeof(Acc)), h.columns);
         const size_t smem = CtaRowSmem<V, THREADS, true>::bytes(h.columns, slots);
         auto kern = rows_cta_kernel<V, THREADS, true>;
         SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<V, THREADS, true>>()));
-        const HeavyArgs a = args(ROUTE_WIDE);
-        SPSYRK_CUDA_TRY(ch.launch(brief_rows(pl->route_n[ROUTE_WIDE], pl->sm_count), kern, pl->route_n[ROUTE_WIDE], THREADS, smem, pl->dev, a.list, h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv,
-                                  row_lo, row_hi, nullptr, 0u));
+        SPSYRK_CUDA_TRY(ch.launch(brief_rows(wide.count[k], pl->sm_count), kern, wide.count[k], THREADS, smem, pl->dev,
+                                  pl->route_list + ROUTE_WIDE * pl->rows_cap + wide.first[k], h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv,
+                                  nullptr, 0u));
     }
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
@@ -1161,11 +1162,18 @@ spsyrk_status_t spsyrk_numeric(spsyrk_plan_t plan, const int64_t* d_c_rowptr, in
 }
 
 namespace {
-// out[(2 * c) + e] = first position of class c's row list (ascending local row ids) whose row is >= bound[e]
+// out[(2 * c) + e] = first position of class c's row list (ascending local row ids) whose row is >= bound[e]; behind them the
+// pieces of the heavy rows' lists (route_positions), where there are any
+constexpr int POSITION_WORDS = 2 * NCLASS + 4 * NROUTE;
+static_assert(32 + 2 * POSITION_WORDS <= HOST_WORDS, "the positions of both views in the rest of the host block");
 __global__ void class_positions_kernel(const int32_t* __restrict__ perm, const int64_t* __restrict__ class_start_dev, int64_t lo_row,
-                                       int64_t hi_row, int64_t* __restrict__ out) {
+                                       int64_t hi_row, bool heavy, const int32_t* __restrict__ lists, int64_t cap, const int2* __restrict__ rank_parts,
+                                       const uint32_t* __restrict__ lengths, const uint8_t* __restrict__ cls, int64_t* __restrict__ out) {
     const int t = threadIdx.x;
-    if (t >= 2 * NCLASS) return;
+    if (t >= 2 * NCLASS) {
+        if (heavy && t < POSITION_WORDS) route_positions(t - 2 * NCLASS, lists, cap, rank_parts, lengths, cls, lo_row, hi_row, out + 2 * NCLASS);
+        return;
+    }
     const int c = t >> 1;
     const int64_t bound = (t & 1) ? hi_row : lo_row;
     int64_t lo = class_start_dev[c], hi = class_start_dev[c + 1];
@@ -1192,19 +1200,27 @@ spsyrk_status_t spsyrk_numeric_rows(spsyrk_plan_t plan, int64_t row_begin, int64
     spsyrk_plan_s* views[2] = {pl, pl->upper_active ? pl->upper : nullptr};
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
-        class_positions_kernel<<<1, 32, 0, st>>>(views[v]->perm, views[v]->class_start_dev, row_begin - pl->dev.r0, row_end - pl->dev.r0,
-                                                 dev_pos + v * 2 * NCLASS);
+        class_positions_kernel<<<1, 64, 0, st>>>(views[v]->perm, views[v]->class_start_dev, row_begin - pl->dev.r0, row_end - pl->dev.r0, heavy_rows(views[v]) > 0,
+                                                 views[v]->route_list, pl->rows_cap, views[v]->rank_parts, views[v]->route_count, views[v]->cls,
+                                                 dev_pos + v * POSITION_WORDS);
         note_launches(1);
     }
+    static_assert(POSITION_WORDS <= 64, "one thread per position");
     SPSYRK_CUDA_TRY(cudaGetLastError());
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    const int64_t(*pos)[2 * NCLASS] = reinterpret_cast<const int64_t(*)[2 * NCLASS]>(pl->host.host + 32);
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
+        const int64_t* pos = pl->host.host + 32 + v * POSITION_WORDS;
         views[v]->sub_active = true;
-        views[v]->sub_row_lo = row_begin - pl->dev.r0;
-        views[v]->sub_row_hi = row_end - pl->dev.r0;
-        for (int c = 0; c < NCLASS; ++c) { views[v]->sub_lo[c] = pos[v][2 * c]; views[v]->sub_hi[c] = pos[v][2 * c + 1]; }
+        for (int c = 0; c < NCLASS; ++c) { views[v]->sub_lo[c] = pos[2 * c]; views[v]->sub_hi[c] = pos[2 * c + 1]; }
+        pos += 2 * NCLASS;
+        for (int k = 0; k < NROUTE; ++k) {
+            RoutePieces& r = views[v]->sub_route[k];
+            for (int e = 0; e < 2; ++e) {
+                r.first[e] = heavy_rows(views[v]) ? (uint32_t)pos[4 * k + 2 * e] : 0u;
+                r.count[e] = heavy_rows(views[v]) ? (uint32_t)(pos[4 * k + 2 * e + 1] - pos[4 * k + 2 * e]) : 0u;
+            }
+        }
     }
     const spsyrk_status_t s = spsyrk_numeric(plan, d_c_rowptr, d_c_colidx, d_c_vals, cuda_stream);
     for (int v = 0; v < 2; ++v)

@@ -40,7 +40,7 @@ void note_launches(int n);
 // Pinned host memory that kernels write the facts the host waits for into (class sizes, entry counts, the error word):
 // one synchronisation and no copy, where a copy into ordinary memory took 3 us of device time and as much again
 // on the host, up to five in a row.  Blocks of HOST_WORDS words come from a pool (defined in api.cu).
-constexpr int HOST_WORDS = 64;
+constexpr int HOST_WORDS = 160;
 struct HostBlock {
     int64_t* host = nullptr;
     int64_t* dev = nullptr;  // the same memory as kernels see it

@@ -52,11 +52,11 @@ __device__ __forceinline__ void st_status(uint32_t* p, uint32_t v) { asm volatil
 
 // One thread per digit: the tile's count is published with radix_publish as soon as it is known; radix_look_back returns how
 // many elements of the digit the tiles before hold and publishes the sum.
-template <typename S>
+template <typename S, int BINS = RX_BINS>
 __device__ __forceinline__ void radix_publish(S* words, int64_t tile, int digit, uint32_t count) {
-    st_status(words + tile * RX_BINS + digit, (S)(((S)count << 2) | (tile == 0 ? (S)SCAN_PREFIX : (S)SCAN_PARTIAL)));
+    st_status(words + tile * BINS + digit, (S)(((S)count << 2) | (tile == 0 ? (S)SCAN_PREFIX : (S)SCAN_PARTIAL)));
 }
-template <typename S>
+template <typename S, int BINS = RX_BINS>
 __device__ __forceinline__ int64_t radix_look_back(S* words, int64_t tile, int digit, uint32_t count, uint32_t* err) {
     if (tile == 0) return 0;
     constexpr int W = 8;  // tiles per round trip
@@ -65,7 +65,7 @@ __device__ __forceinline__ int64_t radix_look_back(S* words, int64_t tile, int d
     for (int64_t last = tile - 1; !done; last -= W) {
         S v[W];
 #pragma unroll
-        for (int k = 0; k < W; ++k) v[k] = last - k >= 0 ? ld_status(words + (last - k) * RX_BINS + digit) : (S)SCAN_PREFIX;
+        for (int k = 0; k < W; ++k) v[k] = last - k >= 0 ? ld_status(words + (last - k) * BINS + digit) : (S)SCAN_PREFIX;
 #pragma unroll
         for (int k = 0; k < W; ++k) {
             if (done) continue;
@@ -75,13 +75,13 @@ __device__ __forceinline__ int64_t radix_look_back(S* words, int64_t tile, int d
                     v[k] = (S)SCAN_PREFIX;
                     break;
                 }
-                v[k] = ld_status(words + (last - k) * RX_BINS + digit);
+                v[k] = ld_status(words + (last - k) * BINS + digit);
             }
             before += v[k] >> 2;
             done = (v[k] & 3) == (S)SCAN_PREFIX;
         }
     }
-    st_status(words + tile * RX_BINS + digit, (S)(((S)(before + count) << 2) | (S)SCAN_PREFIX));
+    st_status(words + tile * BINS + digit, (S)(((S)(before + count) << 2) | (S)SCAN_PREFIX));
     return (int64_t)before;
 }
 

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
                                                            int32_t* __restrict__ cnt,
                                                            const int64_t* __restrict__ c_rowptr, const int64_t* __restrict__ c_rowend,
                                                            int32_t* __restrict__ c_colidx, V* __restrict__ c_vals,
-                                                           int64_t row_lo, int64_t row_hi, uint32_t* __restrict__ block_base, uint32_t blocks_per_row) {
+                                                           uint32_t* __restrict__ block_base, uint32_t blocks_per_row) {
     using Acc = typename AccOf<V>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t scratch[33];
@@ -67,10 +67,6 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     const int tid = threadIdx.x;
     // later rows carry longer column prefixes: hand them out first so that the tail of the launch is light
     const int32_t rloc = rows[gridDim.x - 1 - blockIdx.x];
-    if (NUMERIC && (rloc < row_lo || rloc >= row_hi)) {
-        chain_end();
-        return;
-    }
     const int64_t i = (int64_t)P.r0 + rloc;
     const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
     const int64_t p0 = P.rowptr[i];

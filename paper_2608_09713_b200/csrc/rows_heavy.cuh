@@ -42,14 +42,27 @@ struct RouteRule {
     int binary;
 };
 
-// One thread per heavy row (classes 6 and 7, the last rows first: they carry the longest lists).
-static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, RouteRule R, const int32_t* __restrict__ rows, int64_t count,
-                                                                const int32_t* __restrict__ cnt, const uint32_t* __restrict__ block_base, uint32_t blocks_per_row,
-                                                                int32_t* __restrict__ lists, int64_t cap, int2* __restrict__ rank_parts,
-                                                                uint32_t* __restrict__ counters) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// One thread per heavy row: class 7, then class 6, each with the last rows first (they carry the longest lists).  The lists
+// keep that order, so that the rows of a range are two pieces of each: a tile's place in a list comes from the tiles before it by
+// look-back, as in the radix passes.  `words` ([tiles][NROUTE]) and `ticket` are zero at the start.
+constexpr int ROUTE_THREADS = 256;
+inline int64_t route_tiles(int64_t rows) { return (rows + ROUTE_THREADS - 1) / ROUTE_THREADS; }
+static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDev P, RouteRule R, const int32_t* __restrict__ rows, int64_t count,
+                                                                          const int32_t* __restrict__ cnt, const uint32_t* __restrict__ block_base, uint32_t blocks_per_row,
+                                                                          int32_t* __restrict__ lists, int64_t cap, int2* __restrict__ rank_parts,
+                                                                          uint32_t* __restrict__ lengths, unsigned long long* words, unsigned long long* ticket) {
+    constexpr int NW = ROUTE_THREADS / 32;
+    __shared__ uint32_t s_before[NW][NROUTE];  // rows (parts) of the tile's warps before
+    __shared__ int64_t s_base[NROUTE];
+    __shared__ uint32_t s_tile;
+    if (threadIdx.x == 0) s_tile = (uint32_t)atomicAdd(ticket, 1ull);
+    __syncthreads();
+    const int64_t tile = s_tile, n = tile * ROUTE_THREADS + threadIdx.x;
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
     int route = -1;
     int32_t rloc = 0;
+    uint32_t end[MAX_ROW_PARTS];
+    uint32_t parts = 0;
     if (n < count) {
         rloc = rows[count - 1 - n];
         const int64_t i = (int64_t)P.r0 + rloc;
@@ -73,8 +86,7 @@ static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, Route
             route = entries <= R.slots_mid ? ROUTE_RANK_MID : ROUTE_RANK_BIG;
         } else {
             // as many blocks as the slots hold (a block has fewer entries than that)
-            uint32_t end[MAX_ROW_PARTS];
-            int parts = 0;
+            route = ROUTE_RANK_PARTS;
             const uint32_t* base = block_base + (uint64_t)i * blocks_per_row;
             uint32_t from = 0;
             for (uint32_t b = 1; b <= blocks; ++b) {
@@ -85,22 +97,71 @@ static __global__ void __launch_bounds__(256) route_rows_kernel(PlanDev P, Route
                 }
             }
             end[parts++] = blocks;
-            const uint32_t at = atomicAdd(&counters[ROUTE_RANK_PARTS], (uint32_t)parts);
-            for (int k = 0; k < parts; ++k) rank_parts[at + k] = make_int2(rloc, pack_blocks(k ? end[k - 1] : 0u, end[k]));
         }
     }
+    uint32_t mine = 0;  // rows (parts) of this route in the lanes before
 #pragma unroll
-    for (int k = 0; k < NROUTE; ++k) {  // one atomic per warp and route
-        if (k == ROUTE_RANK_PARTS) continue;
-        const unsigned votes = __ballot_sync(FULL_MASK, route == k);
-        if (route == k) {
-            const int leader = __ffs(votes) - 1;
-            uint32_t base = 0;
-            if (lane_id() == leader) base = atomicAdd(&counters[k], (uint32_t)__popc(votes));
-            base = __shfl_sync(votes, base, leader);
-            lists[(int64_t)k * cap + base + __popc(votes & ((1u << lane_id()) - 1u))] = rloc;
+    for (int k = 0; k < NROUTE; ++k) {
+        uint32_t all;
+        if (k == ROUTE_RANK_PARTS) {
+            const uint32_t incl = warp_inclusive_scan<uint32_t>(parts);
+            all = __shfl_sync(FULL_MASK, incl, 31);
+            if (route == k) mine = incl - parts;
+        } else {
+            const unsigned votes = __ballot_sync(FULL_MASK, route == k);
+            all = __popc(votes);
+            if (route == k) mine = __popc(votes & ((1u << lane) - 1u));
         }
+        if (lane == 0) s_before[warp][k] = all;
     }
+    __syncthreads();
+    if (threadIdx.x < NROUTE) {
+        uint32_t total = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const uint32_t c = s_before[w][threadIdx.x];
+            s_before[w][threadIdx.x] = total;
+            total += c;
+        }
+        radix_publish<unsigned long long, NROUTE>(words, tile, threadIdx.x, total);
+        const int64_t base = radix_look_back<unsigned long long, NROUTE>(words, tile, threadIdx.x, total, P.err);
+        s_base[threadIdx.x] = base;
+        if (tile == gridDim.x - 1) lengths[threadIdx.x] = (uint32_t)(base + total);
+    }
+    __syncthreads();
+    if (route < 0) return;
+    const int64_t at = s_base[route] + s_before[warp][route] + mine;
+    if (route == ROUTE_RANK_PARTS) {
+        for (uint32_t k = 0; k < parts; ++k) rank_parts[at + k] = make_int2(rloc, pack_blocks(k ? end[k - 1] : 0u, end[k]));
+    } else {
+        lists[(int64_t)route * cap + at] = rloc;
+    }
+}
+
+// What of a route's list a launch takes: two pieces (the rows of a range among those of class 7 and among those of class 6)
+struct RoutePieces {
+    uint32_t first[2], count[2];
+    __host__ __device__ __forceinline__ uint32_t total() const { return count[0] + count[1]; }
+    __host__ __device__ __forceinline__ uint32_t at(uint32_t n) const { return n < count[0] ? first[0] + n : first[1] + (n - count[0]); }
+};
+
+// For every route, both pieces of the rows [lo_row, hi_row): out[(route * 2 + piece) * 2] = first, [.. + 1] = one past the
+// last.  A list is descending inside a class; one thread per bound.
+static __device__ void route_positions(int t, const int32_t* lists, int64_t cap, const int2* rank_parts, const uint32_t* lengths, const uint8_t* cls, int64_t lo_row,
+                                       int64_t hi_row, int64_t* out) {
+    const int k = t >> 2, piece = (t >> 1) & 1;
+    const int64_t bound = (t & 1) ? lo_row : hi_row;
+    auto row = [&](uint32_t n) { return k == ROUTE_RANK_PARTS ? rank_parts[n].x : lists[(int64_t)k * cap + n]; };
+    auto first_not = [](uint32_t lo, uint32_t hi, auto before) {  // first position in [lo, hi) that does not lie before
+        while (lo < hi) {
+            const uint32_t mid = lo + (hi - lo) / 2;
+            if (before(mid)) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    const uint32_t len = lengths[k];
+    const uint32_t split = first_not(0u, len, [&](uint32_t n) { return cls[row(n)] == 7; });
+    out[t] = first_not(piece ? split : 0u, piece ? len : split, [&](uint32_t n) { return (int64_t)row(n) >= bound; });
 }
 
 // The lists of a row, up to THREADS of them at a time, flattened through a prefix sum of their lengths
@@ -171,22 +232,31 @@ __device__ __forceinline__ void batch_walk(const ListBatch<Acc, THREADS>& B, Loa
 
 struct HeavyArgs {
     const int32_t* list;
-    uint32_t count;
-    int64_t row_lo, row_hi;    // rows of the plan's range to compute
+    RoutePieces rows;
     const int64_t* out_begin;  // where each row's part of the output starts / ends
     const int64_t* out_end;
     int32_t* c_colidx;
     bool aligned;              // the output arrays start on 16-byte boundaries
     const int2* parts;         // parts of rows (row, pack_blocks), computed before the list
-    uint32_t nparts;
+    RoutePieces part_rows;
     const uint32_t* block_base;  // [absolute row * blocks_per_row + block]: entries of the row before the block of columns
     uint32_t blocks_per_row;
 };
 
 // A row, or a part of one, by its number in the launch
 __device__ __forceinline__ int2 heavy_unit(const HeavyArgs& H, uint32_t n) {
-    const int2 u = n < H.nparts ? H.parts[n] : make_int2(H.list[n - H.nparts], pack_blocks(0u, 255u));  // 255: to the end
-    return u.x >= H.row_lo && u.x < H.row_hi ? u : make_int2(-1, 0);  // (a row range: spsyrk_numeric_rows)
+    const uint32_t np = H.part_rows.total();
+    return n < np ? H.parts[H.part_rows.at(n)] : make_int2(H.list[H.rows.at(n - np)], pack_blocks(0u, 255u));  // 255: to the end
+}
+
+// The order in which dense8 takes `count` rows of a list: the first of each of 64 segments, the second of each, ...  Rows next
+// to each other are equally long, and CTAs that all count while all others count, and write while all write, leave the
+// memory idle half the time: 50000 dense rows 5.58 ms in the list's order, 4.36 so; 20000 rows 0.92 against 0.84; 5000 rows
+// 0.110 against 0.109; 3000 rows 57.6 against 59.1 us (the longest rows first matter more).
+__device__ __forceinline__ uint32_t spread_rows(uint32_t n, uint32_t count) {
+    constexpr uint32_t SEGMENTS = 64, MIN_LENGTH = 64;
+    const uint32_t length = count / SEGMENTS;
+    return length >= MIN_LENGTH && n < length * SEGMENTS ? n % SEGMENTS * length + n / SEGMENTS : n;
 }
 
 // The rows of a CTA, one after the other: its own, then those of CTAs that have not started.  Thread 0 asks for the next CTA
@@ -252,11 +322,9 @@ struct RowQueue {
         if (threadIdx.x == 0) {
             int2 r = make_int2(-1, 0);
             if (asked) n = take(err);
-            while (n != NONE) {
-                r = heavy_unit(H, n);
+            if (n != NONE) {
+                r = heavy_unit(H, spread_rows(n, H.rows.total()));  // (dense8 has no parts)
                 ask();
-                if (r.x >= 0) break;
-                n = take(err);
             }
             s->unit = r;
         }
@@ -305,91 +373,89 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, Hea
     chain_begin();
     const int2 unit = heavy_unit(H, blockIdx.x);
     const int32_t rloc = unit.x;
-    if (rloc >= 0) {
-        const int64_t i = (int64_t)P.r0 + rloc;
-        const uint32_t whole = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
-        const uint32_t b_first = unit.y & 0xff, b_end = (uint32_t)unit.y >> 8;
-        const uint32_t c0 = b_first * BASE_BLOCK, c1 = min(b_end * BASE_BLOCK, whole), U = c1 - c0;  // columns [c0, c1)
-        const int64_t p0 = P.rowptr[i];
-        const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
-        int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
-        if (c1 < whole) oe = ob + H.block_base[(uint64_t)i * H.blocks_per_row + b_end];
-        if (c0 > 0) ob += H.block_base[(uint64_t)i * H.blocks_per_row + b_first];
-        uint32_t entries = (uint32_t)(oe - ob);
-        const uint32_t words = (U + 63u) / 64u;
-        if (!SPSYRK_IN_RANGE(ob >= H.out_begin[rloc] && oe <= H.out_end[rloc] && entries <= slots && U <= columns, P.err)) entries = 0;
-        for (uint32_t w = tid; w < words; w += THREADS) bits[w] = 0;  // (seen by all behind the first batch's barriers)
-        auto fill = [&](uint32_t b0) {
-            const bool on = b0 + tid < deg;
-            uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
-            const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
-            if (d.y > 0 && U < whole) {
-                const int32_t* lst = P.at_row + d.x;
-                const uint32_t hi = c1 < whole ? lower_bound_i32(lst, d.y, (int32_t)c1) : d.y;
-                const uint32_t lo = c0 > 0 ? lower_bound_i32(lst, hi, (int32_t)c0) : 0u;
-                d = make_uint2(d.x + lo, hi - lo);
-            }
-            batch_fill<Acc, THREADS>(B, d.x, d.y, a);
-        };
-        // the columns that occur
-        for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+    const int64_t i = (int64_t)P.r0 + rloc;
+    const uint32_t whole = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+    const uint32_t b_first = unit.y & 0xff, b_end = (uint32_t)unit.y >> 8;
+    const uint32_t c0 = b_first * BASE_BLOCK, c1 = min(b_end * BASE_BLOCK, whole), U = c1 - c0;  // columns [c0, c1)
+    const int64_t p0 = P.rowptr[i];
+    const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
+    int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
+    if (c1 < whole) oe = ob + H.block_base[(uint64_t)i * H.blocks_per_row + b_end];
+    if (c0 > 0) ob += H.block_base[(uint64_t)i * H.blocks_per_row + b_first];
+    uint32_t entries = (uint32_t)(oe - ob);
+    const uint32_t words = (U + 63u) / 64u;
+    if (!SPSYRK_IN_RANGE(ob >= H.out_begin[rloc] && oe <= H.out_end[rloc] && entries <= slots && U <= columns, P.err)) entries = 0;
+    for (uint32_t w = tid; w < words; w += THREADS) bits[w] = 0;  // (seen by all behind the first batch's barriers)
+    auto fill = [&](uint32_t b0) {
+        const bool on = b0 + tid < deg;
+        uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
+        const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
+        if (d.y > 0 && U < whole) {
+            const int32_t* lst = P.at_row + d.x;
+            const uint32_t hi = c1 < whole ? lower_bound_i32(lst, d.y, (int32_t)c1) : d.y;
+            const uint32_t lo = c0 > 0 ? lower_bound_i32(lst, hi, (int32_t)c0) : 0u;
+            d = make_uint2(d.x + lo, hi - lo);
+        }
+        batch_fill<Acc, THREADS>(B, d.x, d.y, a);
+    };
+    // the columns that occur
+    for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+        if (b0) __syncthreads();
+        fill(b0);
+        batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) {
+            const uint32_t rel = (uint32_t)j - c0;
+            if (SPSYRK_IN_RANGE(rel < columns, P.err)) atomicOr(&bits32[rel >> 5], 1u << (rel & 31u));
+        });
+    }
+    for (uint32_t t = tid; t < entries; t += THREADS) acc[t] = Acc(0);
+    __syncthreads();
+    // ranks: a warp owns consecutive words, 32 per step
+    const uint32_t per_warp = ((words + NW - 1) / NW + 31u) & ~31u;
+    const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
+    uint32_t sum = 0;
+    for (uint32_t w = w0 + lane; w < w1; w += 32) sum += __popcll(bits[w]);
+    sum = warp_reduce_sum<uint32_t>(sum);
+    if (lane == 0) s_warp[warp] = sum;
+    __syncthreads();
+    uint32_t run = warp_reduce_sum<uint32_t>(lane < warp ? s_warp[lane < NW ? lane : 0] : 0u);
+    for (uint32_t w = w0; w < w1; w += 32) {
+        const uint32_t c = w + lane < w1 ? __popcll(bits[w + lane]) : 0u;
+        const uint32_t incl = warp_inclusive_scan<uint32_t>(c);
+        if (w + lane < w1) rank[w + lane] = (uint16_t)(run + incl - c);
+        run += __shfl_sync(FULL_MASK, incl, 31);
+    }
+    __syncthreads();
+    // the products
+    auto add = [&](uint32_t j, Acc p) {
+        j -= c0;
+        if (!SPSYRK_IN_RANGE(j < columns, P.err)) return;
+        const uint32_t slot = rank[j >> 6] + __popcll(bits[j >> 6] & ((1ull << (j & 63u)) - 1ull));
+        if (SPSYRK_IN_RANGE(slot < entries && slot < slots, P.err)) atomicAdd(&acc[slot], p);
+    };
+    for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+        if (deg > THREADS) {  // (one batch: the lists are still there)
             if (b0) __syncthreads();
             fill(b0);
-            batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) {
-                const uint32_t rel = (uint32_t)j - c0;
-                if (SPSYRK_IN_RANGE(rel < columns, P.err)) atomicOr(&bits32[rel >> 5], 1u << (rel & 31u));
-            });
         }
-        for (uint32_t t = tid; t < entries; t += THREADS) acc[t] = Acc(0);
-        __syncthreads();
-        // ranks: a warp owns consecutive words, 32 per step
-        const uint32_t per_warp = ((words + NW - 1) / NW + 31u) & ~31u;
-        const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
-        uint32_t sum = 0;
-        for (uint32_t w = w0 + lane; w < w1; w += 32) sum += __popcll(bits[w]);
-        sum = warp_reduce_sum<uint32_t>(sum);
-        if (lane == 0) s_warp[warp] = sum;
-        __syncthreads();
-        uint32_t run = warp_reduce_sum<uint32_t>(lane < warp ? s_warp[lane < NW ? lane : 0] : 0u);
-        for (uint32_t w = w0; w < w1; w += 32) {
-            const uint32_t c = w + lane < w1 ? __popcll(bits[w + lane]) : 0u;
-            const uint32_t incl = warp_inclusive_scan<uint32_t>(c);
-            if (w + lane < w1) rank[w + lane] = (uint16_t)(run + incl - c);
-            run += __shfl_sync(FULL_MASK, incl, 31);
-        }
-        __syncthreads();
-        // the products
-        auto add = [&](uint32_t j, Acc p) {
-            j -= c0;
-            if (!SPSYRK_IN_RANGE(j < columns, P.err)) return;
-            const uint32_t slot = rank[j >> 6] + __popcll(bits[j >> 6] & ((1ull << (j & 63u)) - 1ull));
-            if (SPSYRK_IN_RANGE(slot < entries && slot < slots, P.err)) atomicAdd(&acc[slot], p);
-        };
-        for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
-            if (deg > THREADS) {  // (one batch: the lists are still there)
-                if (b0) __syncthreads();
-                fill(b0);
+        if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
+        else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc a) { add((uint32_t)r.j, acc_mul(a, (Acc)r.v)); });
+    }
+    __syncthreads();
+    // out: sums by slot, column ids from the bitmap
+    for (uint32_t t = tid; t < entries; t += THREADS) c_vals[ob + t] = (V)acc[t];
+    for (uint32_t w = tid; w < words; w += THREADS) {
+        unsigned long long b = bits[w];
+        if (b == 0) continue;
+        uint32_t r = rank[w];
+        while (b) {
+            const int32_t j = (int32_t)(c0 + w * 64u) + __ffsll((long long)b) - 1;
+            b &= b - 1;
+            if (SPSYRK_IN_RANGE(r < entries, P.err)) {
+                H.c_colidx[ob + r] = j;
+                if constexpr (std::is_same<V, int32_t>::value)
+                    if (P.jaccard) store_jaccard<V>(P, ob + r, j, acc[r], (int32_t)deg);
             }
-            if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
-            else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc a) { add((uint32_t)r.j, acc_mul(a, (Acc)r.v)); });
-        }
-        __syncthreads();
-        // out: sums by slot, column ids from the bitmap
-        for (uint32_t t = tid; t < entries; t += THREADS) c_vals[ob + t] = (V)acc[t];
-        for (uint32_t w = tid; w < words; w += THREADS) {
-            unsigned long long b = bits[w];
-            if (b == 0) continue;
-            uint32_t r = rank[w];
-            while (b) {
-                const int32_t j = (int32_t)(c0 + w * 64u) + __ffsll((long long)b) - 1;
-                b &= b - 1;
-                if (SPSYRK_IN_RANGE(r < entries, P.err)) {
-                    H.c_colidx[ob + r] = j;
-                    if constexpr (std::is_same<V, int32_t>::value)
-                        if (P.jaccard) store_jaccard<V>(P, ob + r, j, acc[r], (int32_t)deg);
-                }
-                ++r;
-            }
+            ++r;
         }
     }
     chain_end();
@@ -438,89 +504,87 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
     const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
     chain_begin();
     const int32_t rloc = heavy_unit(H, blockIdx.x).x;
-    if (rloc >= 0) {
-        const int64_t i = (int64_t)P.r0 + rloc;
-        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
-        const int64_t p0 = P.rowptr[i];
-        const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
-        const int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
-        const bool dense = oe - ob == (int64_t)U;  // every column occurs
-        const int planes = ones && dense ? heavy_planes(P) : 0;
-        const bool use_masks = planes > 0;
-        const HeavyMask mine = load_heavy_mask(P, i, planes);
-        uint32_t done = 0;  // entries of the chunks before
-        for (uint32_t c0 = 0; c0 < U; c0 += chunk) {
-            const uint32_t c1 = min(c0 + chunk, U), cn = c1 - c0;
-            if (!use_masks) {
-                for (uint32_t t = tid; t < cn; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
-            } else {
-                for (uint32_t t = tid; t < cn; t += THREADS) {
-                    uint32_t n = 0;
+    const int64_t i = (int64_t)P.r0 + rloc;
+    const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+    const int64_t p0 = P.rowptr[i];
+    const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
+    const int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
+    const bool dense = oe - ob == (int64_t)U;  // every column occurs
+    const int planes = ones && dense ? heavy_planes(P) : 0;
+    const bool use_masks = planes > 0;
+    const HeavyMask mine = load_heavy_mask(P, i, planes);
+    uint32_t done = 0;  // entries of the chunks before
+    for (uint32_t c0 = 0; c0 < U; c0 += chunk) {
+        const uint32_t c1 = min(c0 + chunk, U), cn = c1 - c0;
+        if (!use_masks) {
+            for (uint32_t t = tid; t < cn; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
+        } else {
+            for (uint32_t t = tid; t < cn; t += THREADS) {
+                uint32_t n = 0;
 #pragma unroll
-                    for (int p = 0; p < HEAVY_PLANES; ++p)
-                        if (p < planes) n += __popc(P.heavy_mask[p * P.mask_stride + c0 + t] & mine.w[p]);
-                    acc[t] = (Acc)(int32_t)n;
-                }
+                for (int p = 0; p < HEAVY_PLANES; ++p)
+                    if (p < planes) n += __popc(P.heavy_mask[p * P.mask_stride + c0 + t] & mine.w[p]);
+                acc[t] = (Acc)(int32_t)n;
             }
-            auto add = [&](uint32_t j, Acc p) {
-                const uint32_t rel = j - c0;
-                if (!SPSYRK_IN_RANGE(rel < cn, P.err)) return;
-                if (!dense) occurs[rel] = 1;
-                atomicAdd(&acc[rel], p);
-            };
-            for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
-                const bool on = b0 + tid < deg;
-                uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
-                if (use_masks && on && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
-                uint32_t lo = 0, hi = d.y;  // the list's entries in [c0, c1)
-                if (d.y > 0 && U > chunk) {
-                    if (c1 < U) hi = lower_bound_i32(P.at_row + d.x, d.y, (int32_t)c1);
-                    if (c0 > 0) lo = lower_bound_i32(P.at_row + d.x, hi, (int32_t)c0);
-                }
-                const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
-                if (b0) __syncthreads();
-                batch_fill<Acc, THREADS>(B, d.x + lo, hi - lo, a);
-                if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
-                else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc av) { add((uint32_t)r.j, acc_mul(av, (Acc)r.v)); });
-            }
-            __syncthreads();
-            // entries of every group of 32 columns, their prefix sums; a warp owns consecutive groups
-            const uint32_t words = (cn + 31u) / 32u;
-            const uint32_t per_warp = (words + NW - 1) / NW;
-            const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
-            uint32_t tot = cn, run = 0;
-            if (!dense) {
-                uint32_t sum = 0;
-                for (uint32_t w = w0; w < w1; ++w) {
-                    const uint32_t t = w * 32u + lane;
-                    const unsigned b = __ballot_sync(FULL_MASK, t < cn && occurs[t] != 0);
-                    if (lane == 0) votes[w] = b;
-                    sum += __popc(b);
-                }
-                if (lane == 0) s_warp[warp] = sum;
-                __syncthreads();
-                const uint32_t ws = lane < NW ? s_warp[lane] : 0u;
-                run = warp_reduce_sum<uint32_t>(lane < warp ? ws : 0u);
-                tot = warp_reduce_sum<uint32_t>(ws);
-            }
-            for (uint32_t w = w0; w < w1; ++w) {
-                const uint32_t b = dense ? 0xffffffffu : votes[w];
-                const uint32_t t = w * 32u + lane;
-                if (((b >> lane) & 1u) && t < cn) {
-                    const int64_t at = ob + done + (dense ? t : run + __popc(b & ((1u << lane) - 1u)));
-                    const Acc v = acc[t];
-                    if (SPSYRK_IN_RANGE(at < oe, P.err)) {
-                        c_vals[at] = (V)v;
-                        H.c_colidx[at] = (int32_t)(c0 + t);
-                        if constexpr (std::is_same<V, int32_t>::value)
-                            if (P.jaccard) store_jaccard<V>(P, at, (int32_t)(c0 + t), v, (int32_t)deg);
-                    }
-                }
-                run += __popc(b);
-            }
-            done += tot;
-            __syncthreads();
         }
+        auto add = [&](uint32_t j, Acc p) {
+            const uint32_t rel = j - c0;
+            if (!SPSYRK_IN_RANGE(rel < cn, P.err)) return;
+            if (!dense) occurs[rel] = 1;
+            atomicAdd(&acc[rel], p);
+        };
+        for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+            const bool on = b0 + tid < deg;
+            uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
+            if (use_masks && on && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
+            uint32_t lo = 0, hi = d.y;  // the list's entries in [c0, c1)
+            if (d.y > 0 && U > chunk) {
+                if (c1 < U) hi = lower_bound_i32(P.at_row + d.x, d.y, (int32_t)c1);
+                if (c0 > 0) lo = lower_bound_i32(P.at_row + d.x, hi, (int32_t)c0);
+            }
+            const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
+            if (b0) __syncthreads();
+            batch_fill<Acc, THREADS>(B, d.x + lo, hi - lo, a);
+            if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
+            else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc av) { add((uint32_t)r.j, acc_mul(av, (Acc)r.v)); });
+        }
+        __syncthreads();
+        // entries of every group of 32 columns, their prefix sums; a warp owns consecutive groups
+        const uint32_t words = (cn + 31u) / 32u;
+        const uint32_t per_warp = (words + NW - 1) / NW;
+        const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
+        uint32_t tot = cn, run = 0;
+        if (!dense) {
+            uint32_t sum = 0;
+            for (uint32_t w = w0; w < w1; ++w) {
+                const uint32_t t = w * 32u + lane;
+                const unsigned b = __ballot_sync(FULL_MASK, t < cn && occurs[t] != 0);
+                if (lane == 0) votes[w] = b;
+                sum += __popc(b);
+            }
+            if (lane == 0) s_warp[warp] = sum;
+            __syncthreads();
+            const uint32_t ws = lane < NW ? s_warp[lane] : 0u;
+            run = warp_reduce_sum<uint32_t>(lane < warp ? ws : 0u);
+            tot = warp_reduce_sum<uint32_t>(ws);
+        }
+        for (uint32_t w = w0; w < w1; ++w) {
+            const uint32_t b = dense ? 0xffffffffu : votes[w];
+            const uint32_t t = w * 32u + lane;
+            if (((b >> lane) & 1u) && t < cn) {
+                const int64_t at = ob + done + (dense ? t : run + __popc(b & ((1u << lane) - 1u)));
+                const Acc v = acc[t];
+                if (SPSYRK_IN_RANGE(at < oe, P.err)) {
+                    c_vals[at] = (V)v;
+                    H.c_colidx[at] = (int32_t)(c0 + t);
+                    if constexpr (std::is_same<V, int32_t>::value)
+                        if (P.jaccard) store_jaccard<V>(P, at, (int32_t)(c0 + t), v, (int32_t)deg);
+                }
+            }
+            run += __popc(b);
+        }
+        done += tot;
+        __syncthreads();
     }
     chain_end();
 }
