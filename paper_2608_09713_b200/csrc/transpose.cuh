@@ -266,9 +266,11 @@ static __global__ void __launch_bounds__(256) block_desc_kernel(PlanDev P, const
 //   diag: the light-row kernels leave the diagonal products out of their item lists (lower-triangle mode
 //   over the whole column range), so a light row is classed by w minus its number of nonzeros
 // A group takes UNR rows at a time, so that the loads of one row do not wait for those of the row before (one at a time:
-// 438 us for 4.2e6 rows of 16 nonzeros).  The CTAs behind `nblocks` do the binary analysis.
+// 438 us for 4.2e6 rows of 16 nonzeros).  The CTAs behind `nblocks` do the binary analysis.  Six CTAs per SM are asked for: left
+// to itself the compiler serialises the loads of long rows beside the analysis (524288 rows of a power-law matrix, whole
+// plan: 859 us without the bound, 749 with it).
 template <int G>
-static __global__ void __launch_bounds__(BIN_THREADS) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, bool diag, int64_t tile,
+static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, bool diag, int64_t tile,
                                                                       int32_t* __restrict__ blockhist, int64_t nblocks,
                                                                       unsigned long long* __restrict__ work_total, HeavyArrays heavy) {
     if (blockIdx.x >= nblocks) {
