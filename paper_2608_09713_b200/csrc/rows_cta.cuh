@@ -65,8 +65,10 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
     Acc* acc = la + THREADS;
 
     const int tid = threadIdx.x;
-    // later rows carry longer column prefixes: hand them out first so that the tail of the launch is light
-    const int32_t rloc = rows[gridDim.x - 1 - blockIdx.x];
+    // later rows carry longer column prefixes: hand them out first so that the tail of the launch is light (the class lists
+    // of the counting pass are ascending, the lists of the numeric pass start with the last rows already; in the wrong
+    // order the numeric pass of 524288 power-law rows with 4 edges each takes 11.9 ms instead of 10.4)
+    const int32_t rloc = rows[NUMERIC ? blockIdx.x : gridDim.x - 1 - blockIdx.x];
     const int64_t i = (int64_t)P.r0 + rloc;
     const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
     const int64_t p0 = P.rowptr[i];
