@@ -10,8 +10,8 @@
 //            columns counted through bit masks.
 // All are launched with a CTA per row or part of one, the longest lists first, so that the GPU hands the rows out as CTAs end.
 // (Persistent CTAs that drew their rows from a counter in the plan lost rows when two passes of one plan overlapped; the
-// same rows dealt out beforehand took 1.14 times as long on the large power-law workload.)  In dense8, whose rows are short and
-// alike, a CTA that has finished takes over one that has not started (cluster launch control).
+// same rows dealt out beforehand took 1.14 times as long on the large power-law workload.)  In direct and dense8 a CTA
+// that has finished takes over one that has not started (cluster launch control) and keeps its accumulators.
 //
 // Before, every heavy row went through a bitmap, 32-bit ranks and one size of slots (512 threads up to 32768 products, 1024
 // above), rows with more entries than slots into global slices with L2 atomics, dense rows of binary matrices
@@ -262,8 +262,8 @@ __device__ __forceinline__ uint32_t spread_rows(uint32_t n, uint32_t count) {
 // The rows of a CTA, one after the other: its own, then those of CTAs that have not started.  Thread 0 asks for the next CTA
 // while the row is computed (clusterlaunchcontrol.try_cancel; the answer arrives in shared memory and completes a phase
 // of the barrier).  After a refusal nothing is asked for any more, and a CTA does not end with a request under way.
-// (50000 dense rows of up to 50000 columns, counts and similarities: 4.38 ms, with a CTA per row 4.52; the rank kernels
-// gain nothing: 12.6 against 12.5 ms on the large power-law workload.)
+// (With a CTA per row: dense8 on 50000 rows 4.52 ms instead of 4.38, direct on 8192 equal rows 273 us instead of 257.  The
+// rank kernels, whose rows take longest, gain nothing: 12.6 against 12.5 ms on the large power-law workload.)
 struct RowQueueShared {
     uint4 answer;
     unsigned long long barrier;
@@ -318,12 +318,13 @@ struct RowQueue {
         return cta;
     }
     // the next row (or part of one), or -1; contains barriers, after which the row before is finished by all threads
+    template <bool SPREAD>
     __device__ __forceinline__ int2 next(const HeavyArgs& H, uint32_t* err) {
         if (threadIdx.x == 0) {
             int2 r = make_int2(-1, 0);
             if (asked) n = take(err);
             if (n != NONE) {
-                r = heavy_unit(H, spread_rows(n, H.rows.total()));  // (dense8 has no parts)
+                r = heavy_unit(H, SPREAD ? spread_rows(n, H.rows.total()) : n);  // (no parts where rows are spread)
                 ask();
             }
             s->unit = r;
@@ -494,6 +495,7 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
     using Acc = typename AccOf<V>::type;
     constexpr int NW = THREADS / 32;
     extern __shared__ __align__(16) unsigned char dr_smem[];
+    __shared__ RowQueueShared s_queue;
     __shared__ uint32_t s_warp[NW];
     Acc* acc = reinterpret_cast<Acc*>(dr_smem);                                          // [chunk]
     uint8_t* occurs = reinterpret_cast<uint8_t*>(acc + chunk);                           // [chunk]
@@ -502,91 +504,96 @@ __global__ void __launch_bounds__(THREADS, 2) rows_direct_kernel(PlanDev P, Heav
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool ones = P.binary != 0;
     const ColRec<V>* __restrict__ recs = static_cast<const ColRec<V>*>(P.at_rec);
+    for (uint32_t t = tid; t < chunk; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }  // (later the sweep leaves them so)
     chain_begin();
-    const int32_t rloc = heavy_unit(H, blockIdx.x).x;
-    const int64_t i = (int64_t)P.r0 + rloc;
-    const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
-    const int64_t p0 = P.rowptr[i];
-    const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
-    const int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
-    const bool dense = oe - ob == (int64_t)U;  // every column occurs
-    const int planes = ones && dense ? heavy_planes(P) : 0;
-    const bool use_masks = planes > 0;
-    const HeavyMask mine = load_heavy_mask(P, i, planes);
-    uint32_t done = 0;  // entries of the chunks before
-    for (uint32_t c0 = 0; c0 < U; c0 += chunk) {
-        const uint32_t c1 = min(c0 + chunk, U), cn = c1 - c0;
-        if (!use_masks) {
-            for (uint32_t t = tid; t < cn; t += THREADS) { acc[t] = Acc(0); occurs[t] = 0; }
-        } else {
-            for (uint32_t t = tid; t < cn; t += THREADS) {
-                uint32_t n = 0;
+    RowQueue queue(&s_queue);
+    for (;;) {
+        const int32_t rloc = queue.next<false>(H, P.err).x;
+        if (rloc < 0) break;
+        const int64_t i = (int64_t)P.r0 + rloc;
+        const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
+        const int64_t p0 = P.rowptr[i];
+        const uint32_t deg = (uint32_t)(P.rowptr[i + 1] - p0);
+        const int64_t ob = H.out_begin[rloc], oe = H.out_end[rloc];
+        const bool dense = oe - ob == (int64_t)U;  // every column occurs
+        const int planes = ones && dense ? heavy_planes(P) : 0;
+        const bool use_masks = planes > 0;
+        const HeavyMask mine = load_heavy_mask(P, i, planes);
+        uint32_t done = 0;  // entries of the chunks before
+        for (uint32_t c0 = 0; c0 < U; c0 += chunk) {
+            const uint32_t c1 = min(c0 + chunk, U), cn = c1 - c0;
+            if (use_masks) {
+                for (uint32_t t = tid; t < cn; t += THREADS) {
+                    uint32_t n = 0;
 #pragma unroll
-                for (int p = 0; p < HEAVY_PLANES; ++p)
-                    if (p < planes) n += __popc(P.heavy_mask[p * P.mask_stride + c0 + t] & mine.w[p]);
-                acc[t] = (Acc)(int32_t)n;
-            }
-        }
-        auto add = [&](uint32_t j, Acc p) {
-            const uint32_t rel = j - c0;
-            if (!SPSYRK_IN_RANGE(rel < cn, P.err)) return;
-            if (!dense) occurs[rel] = 1;
-            atomicAdd(&acc[rel], p);
-        };
-        for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
-            const bool on = b0 + tid < deg;
-            uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
-            if (use_masks && on && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
-            uint32_t lo = 0, hi = d.y;  // the list's entries in [c0, c1)
-            if (d.y > 0 && U > chunk) {
-                if (c1 < U) hi = lower_bound_i32(P.at_row + d.x, d.y, (int32_t)c1);
-                if (c0 > 0) lo = lower_bound_i32(P.at_row + d.x, hi, (int32_t)c0);
-            }
-            const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
-            if (b0) __syncthreads();
-            batch_fill<Acc, THREADS>(B, d.x + lo, hi - lo, a);
-            if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
-            else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc av) { add((uint32_t)r.j, acc_mul(av, (Acc)r.v)); });
-        }
-        __syncthreads();
-        // entries of every group of 32 columns, their prefix sums; a warp owns consecutive groups
-        const uint32_t words = (cn + 31u) / 32u;
-        const uint32_t per_warp = (words + NW - 1) / NW;
-        const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
-        uint32_t tot = cn, run = 0;
-        if (!dense) {
-            uint32_t sum = 0;
-            for (uint32_t w = w0; w < w1; ++w) {
-                const uint32_t t = w * 32u + lane;
-                const unsigned b = __ballot_sync(FULL_MASK, t < cn && occurs[t] != 0);
-                if (lane == 0) votes[w] = b;
-                sum += __popc(b);
-            }
-            if (lane == 0) s_warp[warp] = sum;
-            __syncthreads();
-            const uint32_t ws = lane < NW ? s_warp[lane] : 0u;
-            run = warp_reduce_sum<uint32_t>(lane < warp ? ws : 0u);
-            tot = warp_reduce_sum<uint32_t>(ws);
-        }
-        for (uint32_t w = w0; w < w1; ++w) {
-            const uint32_t b = dense ? 0xffffffffu : votes[w];
-            const uint32_t t = w * 32u + lane;
-            if (((b >> lane) & 1u) && t < cn) {
-                const int64_t at = ob + done + (dense ? t : run + __popc(b & ((1u << lane) - 1u)));
-                const Acc v = acc[t];
-                if (SPSYRK_IN_RANGE(at < oe, P.err)) {
-                    c_vals[at] = (V)v;
-                    H.c_colidx[at] = (int32_t)(c0 + t);
-                    if constexpr (std::is_same<V, int32_t>::value)
-                        if (P.jaccard) store_jaccard<V>(P, at, (int32_t)(c0 + t), v, (int32_t)deg);
+                    for (int p = 0; p < HEAVY_PLANES; ++p)
+                        if (p < planes) n += __popc(P.heavy_mask[p * P.mask_stride + c0 + t] & mine.w[p]);
+                    acc[t] = (Acc)(int32_t)n;
                 }
             }
-            run += __popc(b);
+            auto add = [&](uint32_t j, Acc p) {
+                const uint32_t rel = j - c0;
+                if (!SPSYRK_IN_RANGE(rel < cn, P.err)) return;
+                if (!dense) occurs[rel] = 1;
+                atomicAdd(&acc[rel], p);
+            };
+            for (uint32_t b0 = 0; b0 < deg; b0 += THREADS) {
+                const bool on = b0 + tid < deg;
+                uint2 d = on ? P.desc[p0 + b0 + tid] : make_uint2(0u, 0u);
+                if (use_masks && on && P.heavy_id[P.colidx[p0 + b0 + tid]] != 0xff) d.y = 0;  // counted through the masks
+                uint32_t lo = 0, hi = d.y;  // the list's entries in [c0, c1)
+                if (d.y > 0 && U > chunk) {
+                    if (c1 < U) hi = lower_bound_i32(P.at_row + d.x, d.y, (int32_t)c1);
+                    if (c0 > 0) lo = lower_bound_i32(P.at_row + d.x, hi, (int32_t)c0);
+                }
+                const Acc a = on ? (Acc) static_cast<const V*>(P.vals)[p0 + b0 + tid] : Acc(0);
+                if (b0) __syncthreads();
+                batch_fill<Acc, THREADS>(B, d.x + lo, hi - lo, a);
+                if (ones) batch_walk<Acc, THREADS, 8>(B, [&](uint32_t q) { return P.at_row[q]; }, [&](int32_t j, Acc) { add((uint32_t)j, Acc(1)); });
+                else batch_walk<Acc, THREADS, 4>(B, [&](uint32_t q) { return recs[q]; }, [&](const ColRec<V>& r, Acc av) { add((uint32_t)r.j, acc_mul(av, (Acc)r.v)); });
+            }
+            __syncthreads();
+            // entries of every group of 32 columns, their prefix sums; a warp owns consecutive groups
+            const uint32_t words = (cn + 31u) / 32u;
+            const uint32_t per_warp = (words + NW - 1) / NW;
+            const uint32_t w0 = min(warp * per_warp, words), w1 = min(w0 + per_warp, words);
+            uint32_t tot = cn, run = 0;
+            if (!dense) {
+                uint32_t sum = 0;
+                for (uint32_t w = w0; w < w1; ++w) {
+                    const uint32_t t = w * 32u + lane;
+                    const unsigned b = __ballot_sync(FULL_MASK, t < cn && occurs[t] != 0);
+                    if (lane == 0) votes[w] = b;
+                    sum += __popc(b);
+                }
+                if (lane == 0) s_warp[warp] = sum;
+                __syncthreads();
+                const uint32_t ws = lane < NW ? s_warp[lane] : 0u;
+                run = warp_reduce_sum<uint32_t>(lane < warp ? ws : 0u);
+                tot = warp_reduce_sum<uint32_t>(ws);
+            }
+            for (uint32_t w = w0; w < w1; ++w) {
+                const uint32_t b = dense ? 0xffffffffu : votes[w];
+                const uint32_t t = w * 32u + lane;
+                if (((b >> lane) & 1u) && t < cn) {
+                    const int64_t at = ob + done + (dense ? t : run + __popc(b & ((1u << lane) - 1u)));
+                    const Acc v = acc[t];
+                    acc[t] = Acc(0);
+                    occurs[t] = 0;
+                    if (SPSYRK_IN_RANGE(at < oe, P.err)) {
+                        c_vals[at] = (V)v;
+                        H.c_colidx[at] = (int32_t)(c0 + t);
+                        if constexpr (std::is_same<V, int32_t>::value)
+                            if (P.jaccard) store_jaccard<V>(P, at, (int32_t)(c0 + t), v, (int32_t)deg);
+                    }
+                }
+                run += __popc(b);
+            }
+            done += tot;
+            __syncthreads();
         }
-        done += tot;
-        __syncthreads();
     }
-    chain_end();
+    chain_end(queue.has_first);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -612,7 +619,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, H
     chain_begin();
     RowQueue queue(&s_queue);
     for (;;) {
-        const int32_t rloc = queue.next(H, P.err).x;
+        const int32_t rloc = queue.next<true>(H, P.err).x;
         if (rloc < 0) break;
         const int64_t i = (int64_t)P.r0 + rloc;
         const uint32_t U = P.mode == SPSYRK_TRIL ? (uint32_t)i + 1u : (uint32_t)P.m;
