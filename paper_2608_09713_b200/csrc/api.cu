@@ -136,7 +136,7 @@ struct spsyrk_plan_s {
     unsigned long long* work_total_dev;
     // heavy rows by the kernel that computes them (rows_heavy.cuh)
     int32_t* route_list;    // NROUTE lists of rows_cap each
-    uint32_t* route_count;  // NROUTE list lengths (device) ...
+    uint32_t* route_count;  // 2 * NROUTE list lengths (device) ...
     uint32_t route_n[NROUTE];  // ... and as the host knows them after the symbolic pass
     int2* rank_parts;       // parts of the longest rows
     uint32_t* block_base;   // entries of a heavy row before every block of columns, [row][blocks_per_row]
@@ -228,7 +228,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto offsets = c.take<int64_t>(NCLASS * nb + 1);
     auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(items + 1, NCLASS * nb)));
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
-    auto route_count = c.take<uint32_t>(2 * NROUTE);  // both views in a row
+    auto route_count = c.take<uint32_t>(2 * 2 * NROUTE);  // of every view: the lengths, the lengths of class 7's part
     auto route_list = c.take<int32_t>(NROUTE * items);
     auto route_state = c.take<unsigned long long>(views * (1 + (size_t)route_tiles(m) * NROUTE));
     // rows whose output range is at most 2^18 columns (they are among the first 2^18 rows)
@@ -299,7 +299,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
             up->perm = u_perm; up->hdr = u_hdr; up->cnt = u_cnt; up->cls = u_cls; up->itemoff = u_itemoff;
             up->class_start_dev = u_class_start_dev; up->work_total_dev = u_work_total_dev;
             up->state_bin = u_state_bin; up->state_items = u_state_items;
-            up->route_count = route_count + NROUTE; up->route_list = u_route_list;
+            up->route_count = route_count + 2 * NROUTE; up->route_list = u_route_list;
             up->rank_parts = u_rank_parts; up->block_base = u_block_base;
         }
     }
@@ -761,8 +761,8 @@ spsyrk_status_t route_heavy(spsyrk_plan_s* pl, unsigned long long* state, cudaSt
     if (count <= 0) return SPSYRK_OK;
     const HeavyShapes h = pl->dtype == SPSYRK_I32 ? heavy_shapes<int32_t>(pl) : heavy_shapes<double>(pl);
     route_rows_kernel<<<(unsigned)route_tiles(count), ROUTE_THREADS, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->block_base,
-                                                                              pl->blocks_per_row, pl->route_list, pl->rows_cap, pl->rank_parts, pl->route_count,
-                                                                              state + 1, state);
+                                                                              pl->blocks_per_row, pl->route_list, pl->rows_cap, pl->rank_parts,
+                                                                              pl->class_start[NCLASS] - pl->class_start[7], pl->route_count, state + 1, state);
     note_launches(1);
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
@@ -876,7 +876,7 @@ struct CountsOut {
         uint32_t w[1 + 2 * NROUTE];
         w[0] = *err;
 #pragma unroll
-        for (int k = 0; k < 2 * NROUTE; ++k) w[1 + k] = routes[k];
+        for (int k = 0; k < 2 * NROUTE; ++k) w[1 + k] = routes[k < NROUTE ? k : k + NROUTE];
         out[n] = t;
         host[0] = t;
 #pragma unroll
@@ -1168,10 +1168,10 @@ constexpr int POSITION_WORDS = 2 * NCLASS + 4 * NROUTE;
 static_assert(32 + 2 * POSITION_WORDS <= HOST_WORDS, "the positions of both views in the rest of the host block");
 __global__ void class_positions_kernel(const int32_t* __restrict__ perm, const int64_t* __restrict__ class_start_dev, int64_t lo_row,
                                        int64_t hi_row, bool heavy, const int32_t* __restrict__ lists, int64_t cap, const int2* __restrict__ rank_parts,
-                                       const uint32_t* __restrict__ lengths, const uint8_t* __restrict__ cls, int64_t* __restrict__ out) {
+                                       const uint32_t* __restrict__ lengths, int64_t* __restrict__ out) {
     const int t = threadIdx.x;
     if (t >= 2 * NCLASS) {
-        if (heavy && t < POSITION_WORDS) route_positions(t - 2 * NCLASS, lists, cap, rank_parts, lengths, cls, lo_row, hi_row, out + 2 * NCLASS);
+        if (heavy && t < POSITION_WORDS) route_positions(t - 2 * NCLASS, lists, cap, rank_parts, lengths, lo_row, hi_row, out + 2 * NCLASS);
         return;
     }
     const int c = t >> 1;
@@ -1201,7 +1201,7 @@ spsyrk_status_t spsyrk_numeric_rows(spsyrk_plan_t plan, int64_t row_begin, int64
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
         class_positions_kernel<<<1, 64, 0, st>>>(views[v]->perm, views[v]->class_start_dev, row_begin - pl->dev.r0, row_end - pl->dev.r0, heavy_rows(views[v]) > 0,
-                                                 views[v]->route_list, pl->rows_cap, views[v]->rank_parts, views[v]->route_count, views[v]->cls,
+                                                 views[v]->route_list, pl->rows_cap, views[v]->rank_parts, views[v]->route_count,
                                                  dev_pos + v * POSITION_WORDS);
         note_launches(1);
     }

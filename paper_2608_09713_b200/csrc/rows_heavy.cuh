@@ -45,12 +45,14 @@ struct RouteRule {
 // One thread per heavy row: class 7, then class 6, each with the last rows first (they carry the longest lists).  The lists
 // keep that order, so that the rows of a range are two pieces of each: a tile's place in a list comes from the tiles before it by
 // look-back, as in the radix passes.  `words` ([tiles][NROUTE]) and `ticket` are zero at the start.
+// lengths[NROUTE ..] are the lengths of class 7's part (its `long_rows` rows come first).
 constexpr int ROUTE_THREADS = 256;
 inline int64_t route_tiles(int64_t rows) { return (rows + ROUTE_THREADS - 1) / ROUTE_THREADS; }
 static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDev P, RouteRule R, const int32_t* __restrict__ rows, int64_t count,
                                                                           const int32_t* __restrict__ cnt, const uint32_t* __restrict__ block_base, uint32_t blocks_per_row,
                                                                           int32_t* __restrict__ lists, int64_t cap, int2* __restrict__ rank_parts,
-                                                                          uint32_t* __restrict__ lengths, unsigned long long* words, unsigned long long* ticket) {
+                                                                          int64_t long_rows, uint32_t* __restrict__ lengths, unsigned long long* words,
+                                                                          unsigned long long* ticket) {
     constexpr int NW = ROUTE_THREADS / 32;
     __shared__ uint32_t s_before[NW][NROUTE];  // rows (parts) of the tile's warps before
     __shared__ int64_t s_base[NROUTE];
@@ -129,6 +131,17 @@ static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDe
         if (tile == gridDim.x - 1) lengths[threadIdx.x] = (uint32_t)(base + total);
     }
     __syncthreads();
+    // the place in every list at which class 6 begins, from the tile that holds its first row (or the last tile: there is none)
+    if (tile == min(long_rows / ROUTE_THREADS, (int64_t)gridDim.x - 1)) {
+        const int first = (int)(long_rows - tile * ROUTE_THREADS), lane_of_first = first & 31;
+#pragma unroll
+        for (int k = 0; k < NROUTE; ++k) {
+            const uint32_t before = k == ROUTE_RANK_PARTS ? warp_reduce_sum<uint32_t>(lane < lane_of_first ? parts : 0u)
+                                                          : __popc(__ballot_sync(FULL_MASK, route == k) & ((1u << lane_of_first) - 1u));
+            if (first < ROUTE_THREADS && warp == first >> 5 && lane == 0) lengths[NROUTE + k] = (uint32_t)s_base[k] + s_before[warp][k] + before;
+        }
+        if (first >= ROUTE_THREADS && threadIdx.x < NROUTE) lengths[NROUTE + threadIdx.x] = lengths[threadIdx.x];
+    }
     if (route < 0) return;
     const int64_t at = s_base[route] + s_before[warp][route] + mine;
     if (route == ROUTE_RANK_PARTS) {
@@ -147,21 +160,17 @@ struct RoutePieces {
 
 // For every route, both pieces of the rows [lo_row, hi_row): out[(route * 2 + piece) * 2] = first, [.. + 1] = one past the
 // last.  A list is descending inside a class; one thread per bound.
-static __device__ void route_positions(int t, const int32_t* lists, int64_t cap, const int2* rank_parts, const uint32_t* lengths, const uint8_t* cls, int64_t lo_row,
-                                       int64_t hi_row, int64_t* out) {
+static __device__ void route_positions(int t, const int32_t* lists, int64_t cap, const int2* rank_parts, const uint32_t* lengths, int64_t lo_row, int64_t hi_row,
+                                       int64_t* out) {
     const int k = t >> 2, piece = (t >> 1) & 1;
     const int64_t bound = (t & 1) ? lo_row : hi_row;
-    auto row = [&](uint32_t n) { return k == ROUTE_RANK_PARTS ? rank_parts[n].x : lists[(int64_t)k * cap + n]; };
-    auto first_not = [](uint32_t lo, uint32_t hi, auto before) {  // first position in [lo, hi) that does not lie before
-        while (lo < hi) {
-            const uint32_t mid = lo + (hi - lo) / 2;
-            if (before(mid)) lo = mid + 1; else hi = mid;
-        }
-        return lo;
-    };
-    const uint32_t len = lengths[k];
-    const uint32_t split = first_not(0u, len, [&](uint32_t n) { return cls[row(n)] == 7; });
-    out[t] = first_not(piece ? split : 0u, piece ? len : split, [&](uint32_t n) { return (int64_t)row(n) >= bound; });
+    uint32_t lo = piece ? lengths[NROUTE + k] : 0u, hi = piece ? lengths[k] : lengths[NROUTE + k];
+    while (lo < hi) {
+        const uint32_t mid = lo + (hi - lo) / 2;
+        const int64_t row = k == ROUTE_RANK_PARTS ? rank_parts[mid].x : lists[(int64_t)k * cap + mid];
+        if (row >= bound) lo = mid + 1; else hi = mid;
+    }
+    out[t] = lo;
 }
 
 // The lists of a row, up to THREADS of them at a time, flattened through a prefix sum of their lengths
