@@ -60,6 +60,17 @@ constexpr uint32_t ROW_CHUNK_BITS_MAX_SYMBOLIC = 1u << 20;
 constexpr size_t LARGE_SMEM_BUDGET = 200 * 1024;
 constexpr int64_t MAX_PARTS = 65536;
 
+// Shared-memory shapes of the heavy-row kernels (see heavy_shapes)
+constexpr int RANK_SMALL_THREADS = 256, RANK_MID_THREADS = 512, RANK_BIG_THREADS = 1024, DENSE8_THREADS = 512;
+template <int T, int C> struct RankShape { static constexpr int THREADS = T, CTAS = C; };
+constexpr size_t SMEM_PER_CTA = 226 * 1024;
+// slots of the largest rank kernel, one CTA per SM: doubles 21504 beside a bitmap of 2^18 columns, 23552 beside 2^17, 24576 beside 2^16
+template <typename V>
+uint32_t rank_slots_big(uint32_t columns) {
+    using Acc = typename AccOf<V>::type;
+    return std::min(columns, (uint32_t)((SMEM_PER_CTA - RankSmem<V, RANK_BIG_THREADS>::bytes(columns, 0)) / sizeof(Acc)) / 1024 * 1024);
+}
+
 size_t dtype_size(spsyrk_dtype_t t) { return t == SPSYRK_F64 ? 8 : 4; }
 
 struct Carver {
@@ -110,7 +121,7 @@ struct spsyrk_plan_s {
     int32_t* cnt_out;
     bool have_onepass;
     HostBlock host;  // words 0..31: facts of the two views; the rest: the position search of spsyrk_numeric_rows (upper view: unused)
-    int64_t rows_cap;
+    int64_t route_cap;
     // workspace views
     int32_t* perm;
     uint4* hdr;  // per-row headers in class order
@@ -135,7 +146,7 @@ struct spsyrk_plan_s {
     int64_t* class_start_dev;  // NCLASS + 1
     unsigned long long* work_total_dev;
     // heavy rows by the kernel that computes them (rows_heavy.cuh)
-    int32_t* route_list;    // NROUTE lists of rows_cap each
+    int32_t* route_list;    // NROUTE lists, route_cap apart
     uint32_t* route_count;  // 2 * NROUTE list lengths (device) ...
     uint32_t route_n[NROUTE];  // ... and as the host knows them after the symbolic pass
     int2* rank_parts;       // parts of the longest rows
@@ -172,29 +183,29 @@ namespace {
 
 size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t n, int64_t nnz, size_t sv, bool full) {
     Carver c(ws);
-    const int64_t items = std::max<int64_t>(std::max(m, n), 1);
-    const int64_t nb = bin_blocks_max(items);
+    const int64_t rows = std::max<int64_t>(m, 1);  // output rows; only the column pointers, counts and bit numbers go by columns
+    const int64_t nb = bin_blocks_max(rows);
     auto colptr = c.take<int64_t>(n + 1);
     auto desc = c.take<uint2>(nnz);
     auto work = c.take<int64_t>(m);
     auto perm = c.take<int32_t>(m);
     auto hdr = c.take<uint4>(m);
     auto cnt = c.take<int32_t>(m);
-    auto cls = c.take<uint8_t>(items);
+    auto cls = c.take<uint8_t>(rows);
     const int npass = radix_passes((uint64_t)std::max<int64_t>(n - 1, 1));
     const size_t rx_words = radix_state_words(radix_tiles(nnz), radix_wide(nnz), npass);
     // counters in one piece, so that one memset clears them: the binning's, then the plan's, then the column counts
     const int views = full ? 2 : 1;
-    const size_t bin_words = views * (1 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(items));
+    const size_t bin_words = views * (1 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(rows));
     auto zero = c.take<int64_t>(bin_words + 32 + (32 + HEAVY_BINS) / 2 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2 +
                                 RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES + rx_words);
     Carver cz(zero);
     auto take_words = [&](size_t words) { int64_t* q = zero ? zero + cz.off : nullptr; cz.off += words; return q; };
     auto work_total_dev = reinterpret_cast<unsigned long long*>(take_words(1));
-    auto state_bin = take_words(scan_partials_count(NCLASS * nb)), state_items = take_words(scan_partials_count(items));
+    auto state_bin = take_words(scan_partials_count(NCLASS * nb)), state_items = take_words(scan_partials_count(rows));
     unsigned long long* u_work_total_dev = full ? reinterpret_cast<unsigned long long*>(take_words(1)) : nullptr;
     int64_t* u_state_bin = full ? take_words(scan_partials_count(NCLASS * nb)) : nullptr;
-    int64_t* u_state_items = full ? take_words(scan_partials_count(items)) : nullptr;
+    int64_t* u_state_items = full ? take_words(scan_partials_count(rows)) : nullptr;
     auto err = reinterpret_cast<uint32_t*>(take_words(32));
     auto facts = reinterpret_cast<uint32_t*>(take_words((32 + HEAVY_BINS) / 2));  // [0..1] binary analysis, [32..] its histogram
     auto state_col = take_words(scan_partials_count(std::max<int64_t>(n, 1)));
@@ -226,26 +237,34 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     auto desc_blk = c_src.take<uint2>(nnz);
     auto blockhist = c.take<int32_t>(NCLASS * nb);
     auto offsets = c.take<int64_t>(NCLASS * nb + 1);
-    auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(items + 1, NCLASS * nb)));
+    auto partials = c.take<int64_t>(scan_partials_count(std::max<int64_t>(rows + 1, NCLASS * nb)));
     auto class_start_dev = c.take<int64_t>(NCLASS + 1);
     auto route_count = c.take<uint32_t>(2 * 2 * NROUTE);  // of every view: the lengths, the lengths of class 7's part
-    auto route_list = c.take<int32_t>(NROUTE * items);
+    // every route but the last takes rows of ranges of at most 2^18 columns, and there are no more of those than that
+    static_assert(ROUTE_WIDE == NROUTE - 1, "the list that may hold all rows is the last");
+    const int64_t route_cap = std::min<int64_t>(rows, ROW_CHUNK_BITS_MAX_NUMERIC);
+    auto route_list = c.take<int32_t>(ROUTE_WIDE * route_cap + rows);
     auto route_state = c.take<unsigned long long>(views * (1 + (size_t)route_tiles(m) * NROUTE));
-    // rows whose output range is at most 2^18 columns (they are among the first 2^18 rows)
-    const int64_t base_rows = std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC);
-    const uint32_t blocks_per_row = (uint32_t)((std::min<int64_t>(items, ROW_CHUNK_BITS_MAX_NUMERIC) + BASE_BLOCK - 1) / BASE_BLOCK);
-    auto rank_parts = c.take<int2>(base_rows * MAX_ROW_PARTS);
-    auto block_base = c.take<uint32_t>(base_rows * blocks_per_row);
-    auto work_prefix = c.take<int64_t>(items + 1);
-    auto itemoff = c.take<int64_t>(items + 1);
+    // Rows that the rank kernel takes in parts: their range has at most 2^18 columns and more than the slots hold
+    const int64_t ranged = std::min<int64_t>(m, ROW_CHUNK_BITS_MAX_NUMERIC);
+    const int64_t slots = rank_slots_big<double>(pow2_at_least((uint64_t)m, 1024u, ROW_CHUNK_BITS_MAX_NUMERIC)), part = slots - BASE_BLOCK;
+    const bool cut = m > slots;
+    // parts of all such rows: a row of U columns has fewer than U / part + 2 of them; U is the row's number or m
+    const int64_t parts_of_m = cut && m <= ROW_CHUNK_BITS_MAX_NUMERIC ? m * std::min<int64_t>(m / part + 1, MAX_ROW_PARTS) : 0;
+    const int64_t parts_by_row = cut ? (ranged - slots) + ((ranged - slots) * (ranged + slots + 1) / 2) / part : 0;
+    const uint32_t blocks_per_row = cut ? (uint32_t)((ranged + BASE_BLOCK - 1) / BASE_BLOCK) : 0u;
+    auto rank_parts = c.take<int2>(full ? std::max(parts_of_m, parts_by_row) : parts_by_row);
+    auto block_base = c.take<uint32_t>(ranged * blocks_per_row);
+    auto work_prefix = c.take<int64_t>(rows + 1);
+    auto itemoff = c.take<int64_t>(rows + 1);
     auto heavy_id = c.take<uint8_t>(std::max<int64_t>(n, 1));
-    const int64_t mask_stride = (items + 3) / 4 * 4;
+    const int64_t mask_stride = (rows + 3) / 4 * 4;
     auto heavy_mask = c.take<uint32_t>(HEAVY_PLANES * mask_stride);
-    auto items8 = c.take<uint32_t>(items);
+    auto items8 = c.take<uint32_t>(rows);
     auto adeg = c.take<int32_t>(std::max<int64_t>(m, 1));
     auto part_bounds = c.take<int64_t>(MAX_PARTS + 1);
     auto ub = c.take<int32_t>(std::max<int64_t>(m, 1));
-    auto ub_off = c.take<int64_t>(items + 1);
+    auto ub_off = c.take<int64_t>(rows + 1);
     // full-output mode: the upper view's own per-row arrays and the second descriptor array
     uint2* desc_hi = nullptr;
     int64_t *u_work = nullptr, *u_itemoff = nullptr, *u_class_start_dev = nullptr, *hi_begin = nullptr, *work_sum = nullptr;
@@ -260,14 +279,14 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         u_perm = c.take<int32_t>(m);
         u_hdr = c.take<uint4>(m);
         u_cnt = c.take<int32_t>(m);
-        u_cls = c.take<uint8_t>(items);
-        u_itemoff = c.take<int64_t>(items + 1);
+        u_cls = c.take<uint8_t>(rows);
+        u_itemoff = c.take<int64_t>(rows + 1);
         u_class_start_dev = c.take<int64_t>(NCLASS + 1);
         cnt_tot = c.take<int32_t>(m);
-        u_route_list = c.take<int32_t>(NROUTE * items);
-        u_rank_parts = c.take<int2>(base_rows * MAX_ROW_PARTS);
-        u_block_base = c.take<uint32_t>(base_rows * blocks_per_row);
-        hi_begin = c.take<int64_t>(items + 1);
+        u_route_list = c.take<int32_t>(ROUTE_WIDE * route_cap + rows);
+        u_rank_parts = c.take<int2>(parts_of_m);
+        u_block_base = c.take<uint32_t>(parts_of_m ? ranged * blocks_per_row : 0);
+        hi_begin = c.take<int64_t>(rows + 1);
         work_sum = c.take<int64_t>(m);
     }
     if (pl) {
@@ -289,7 +308,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
         pl->class_start_dev = class_start_dev; pl->work_total_dev = work_total_dev;
         pl->state_bin = state_bin; pl->state_items = state_items; pl->state_col = state_col; pl->items8 = items8;
         pl->zero_all = zero; pl->zero_all_bytes = zero_words * sizeof(int64_t);
-        pl->rows_cap = items; pl->zero_bin = zero; pl->zero_bin_bytes = bin_words * sizeof(int64_t);
+        pl->route_cap = route_cap; pl->zero_bin = zero; pl->zero_bin_bytes = bin_words * sizeof(int64_t);
         pl->dev.nheavy = facts + 1;
         if (up) {
             // the upper view shares everything that describes A and the scratch space; its rows are its own
@@ -721,10 +740,6 @@ spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
 
 // Shared-memory shapes of the heavy-row kernels and the rule that goes with them.  The small rank kernel is launched
 // for three widths of its bitmap, so that rows in the lower part of the range leave room for more CTAs per SM.
-constexpr int RANK_SMALL_THREADS = 256, RANK_MID_THREADS = 512, RANK_BIG_THREADS = 1024, DENSE8_THREADS = 512;
-template <int T, int C> struct RankShape { static constexpr int THREADS = T, CTAS = C; };
-constexpr size_t SMEM_PER_CTA = 226 * 1024;
-
 struct HeavyShapes {
     RouteRule rule;
     uint32_t columns;  // of the widest bitmap
@@ -743,7 +758,7 @@ HeavyShapes heavy_shapes(const spsyrk_plan_s* pl) {
     r.bits1 = std::min(cb, 131072u);
     r.slots_small = std::min(cb, (uint32_t)(16384 / sizeof(Acc)));
     r.slots_mid = std::min(cb, (uint32_t)(65536 / sizeof(Acc)));
-    r.slots_big = std::min(cb, (uint32_t)((SMEM_PER_CTA - RankSmem<V, RANK_BIG_THREADS>::bytes(cb, 0)) / sizeof(Acc)) / 1024 * 1024);
+    r.slots_big = rank_slots_big<V>(cb);
     // two CTAs per SM
     r.chunk = std::min(cb, (uint32_t)((SMEM_PER_CTA / 2 - 1024 - DirectSmem<V, DIRECT_THREADS>::bytes(0)) / (sizeof(Acc) * 32 + 32 + 4)) * 32);
     const uint64_t umax = pl->dev.mode == SPSYRK_TRIL ? (uint64_t)pl->dev.r1 : (uint64_t)pl->dev.m;
@@ -761,7 +776,7 @@ spsyrk_status_t route_heavy(spsyrk_plan_s* pl, unsigned long long* state, cudaSt
     if (count <= 0) return SPSYRK_OK;
     const HeavyShapes h = pl->dtype == SPSYRK_I32 ? heavy_shapes<int32_t>(pl) : heavy_shapes<double>(pl);
     route_rows_kernel<<<(unsigned)route_tiles(count), ROUTE_THREADS, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->block_base,
-                                                                              pl->blocks_per_row, pl->route_list, pl->rows_cap, pl->rank_parts,
+                                                                              pl->blocks_per_row, pl->route_list, pl->route_cap, pl->rank_parts,
                                                                               pl->class_start[NCLASS] - pl->class_start[7], pl->route_count, state + 1, state);
     note_launches(1);
     SPSYRK_CUDA_TRY(cudaGetLastError());
@@ -798,7 +813,7 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
     auto pieces = [&](int k) { return pl->sub_active ? pl->sub_route[k] : RoutePieces{{0u, 0u}, {pl->route_n[k], 0u}}; };
     const bool aligned = ((reinterpret_cast<uintptr_t>(c_colidx) | reinterpret_cast<uintptr_t>(c_vals) | reinterpret_cast<uintptr_t>(pl->dev.jaccard)) & 15u) == 0;
     auto args = [&](int k) {
-        return HeavyArgs{pl->route_list + k * (pl->rows_cap), pieces(k), pl->out_begin, pl->out_end, c_colidx, aligned,
+        return HeavyArgs{pl->route_list + k * (pl->route_cap), pieces(k), pl->out_begin, pl->out_end, c_colidx, aligned,
                          pl->rank_parts, k == ROUTE_RANK_BIG ? pieces(ROUTE_RANK_PARTS) : RoutePieces{}, pl->block_base, pl->blocks_per_row};
     };
     if (const int64_t units = pieces(ROUTE_DIRECT).total()) {
@@ -830,7 +845,7 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
         auto kern = rows_cta_kernel<V, THREADS, true>;
         SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<V, THREADS, true>>()));
         SPSYRK_CUDA_TRY(ch.launch(brief_rows(wide.count[k], pl->sm_count), kern, wide.count[k], THREADS, smem, pl->dev,
-                                  pl->route_list + ROUTE_WIDE * pl->rows_cap + wide.first[k], h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv,
+                                  pl->route_list + ROUTE_WIDE * pl->route_cap + wide.first[k], h.columns, slots, nullptr, pl->out_begin, pl->out_end, c_colidx, cv,
                                   nullptr, 0u));
     }
     SPSYRK_CUDA_TRY(cudaGetLastError());
@@ -1201,7 +1216,7 @@ spsyrk_status_t spsyrk_numeric_rows(spsyrk_plan_t plan, int64_t row_begin, int64
     for (int v = 0; v < 2; ++v) {
         if (!views[v]) continue;
         class_positions_kernel<<<1, 64, 0, st>>>(views[v]->perm, views[v]->class_start_dev, row_begin - pl->dev.r0, row_end - pl->dev.r0, heavy_rows(views[v]) > 0,
-                                                 views[v]->route_list, pl->rows_cap, views[v]->rank_parts, views[v]->route_count,
+                                                 views[v]->route_list, pl->route_cap, views[v]->rank_parts, views[v]->route_count,
                                                  dev_pos + v * POSITION_WORDS);
         note_launches(1);
     }

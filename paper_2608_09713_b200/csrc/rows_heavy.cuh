@@ -26,7 +26,7 @@ namespace spsyrk {
 enum : int { ROUTE_RANK0 = 0, ROUTE_RANK1, ROUTE_RANK2, ROUTE_RANK_MID, ROUTE_RANK_BIG, ROUTE_RANK_PARTS, ROUTE_DIRECT, ROUTE_DENSE8, ROUTE_WIDE, NROUTE };
 
 // A row of the rank kernel is cut into parts of at most slots_big entries; every part but the last has more than
-// slots_big - BASE_BLOCK, so 2^18 columns make at most 22 parts of 20480 doubles.
+// slots_big - BASE_BLOCK (a block more would not have fitted), so 2^18 columns make at most 20 parts of 21504 doubles.
 constexpr int MAX_ROW_PARTS = 24;
 
 // a row or part of one: blocks [first, end) of BASE_BLOCK columns
