@@ -296,7 +296,7 @@ spsyrk_status_t scan_and_total(const RowWs& w, int64_t m, int64_t* d_rowptr_out,
         SPSYRK_CUDA_TRY(scan_launch(ScanArray<uint32_t>{w.cnt}, m, ScanIntoHost{d_rowptr_out, m, w.err, h.dev}, w.partials, w.err, st));
     }
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h.host[1]) return SPSYRK_ERR_BAD_CSR;
+    if (const uint32_t e = h.errors(h.host[1])) return status_of(e);
     *total = h.host[0];
     return SPSYRK_OK;
 }

@@ -35,6 +35,7 @@ cudaError_t HostBlock::acquire() {
         const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&host), HOST_WORDS * sizeof(int64_t), cudaHostAllocMapped | cudaHostAllocPortable);
         if (e != cudaSuccess) { host = nullptr; return e; }
     }
+    host[HOST_GAVE_UP] = 0;
     return cudaHostGetDevicePointer(reinterpret_cast<void**>(&dev), host, 0);
 }
 void HostBlock::release() {
@@ -375,12 +376,6 @@ struct Residency {
     }
 };
 
-spsyrk_status_t status_of(uint32_t e) {
-    if (e & ERRW_BAD_CSR) return SPSYRK_ERR_BAD_CSR;
-    if (e) return SPSYRK_ERR_INTERNAL;
-    return SPSYRK_OK;
-}
-
 [[maybe_unused]] spsyrk_status_t read_err(spsyrk_plan_s* pl, cudaStream_t st) {
     uint32_t e = 0;
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, pl->dev.err, sizeof(e), cudaMemcpyDeviceToHost, st));
@@ -473,13 +468,13 @@ __global__ void plan_facts_kernel(PlanFacts f) { f.publish(0); }
 
 // Work estimate + binning of one view's current row range (dev.desc, dev.mode and diag are set).  The facts the host
 // needs are on their way to `host` when this returns.
-spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, bool analyse, cudaStream_t st) {
+spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, int64_t* gave_up, bool analyse, cudaStream_t st) {
     const int64_t rows = pl->dev.r1 - pl->dev.r0, nb = bin_blocks(rows);
     pl->have_symbolic = false;
     pl->have_onepass = false;
     pl->map_filled = false;
     const PlanDev& P = pl->dev;
-    const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->facts, P.err, host};
+    const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->facts, P.err, host, gave_up};
     if (P.nnz == 0) analyse = false;
     switch (group_width(P.nnz, P.m)) {
         case 4: launch_row_work<4>(pl, analyse, st); break;
@@ -502,12 +497,12 @@ spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, bool analyse, cudaS
 }
 
 // after the synchronisation
-spsyrk_status_t bin_collect(spsyrk_plan_s* pl, const int64_t* host) {
+spsyrk_status_t bin_collect(spsyrk_plan_s* pl, const HostBlock& block, const int64_t* host) {
     std::memcpy(pl->class_start, host + PF_CLASS_START, sizeof(pl->class_start));
     pl->map_items = host[PF_MAP_ITEMS];
     pl->work_total = host[PF_WORK];
     pl->dev.binary = (pl->dev.nnz > 0 && host[PF_OTHER_THAN_ONE] == 0) ? 1 : 0;
-    return status_of((uint32_t)host[PF_ERR]);
+    return status_of(block.errors(host[PF_ERR]));
 }
 
 // Descriptors, work estimate and binning of the plan's current block of output rows and columns; synchronises once.
@@ -537,7 +532,7 @@ spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st)
             }
         }
     }
-    spsyrk_status_t s = bin_launch(pl, pl->host.dev, fresh, st);
+    spsyrk_status_t s = bin_launch(pl, pl->host.dev, pl->host.dev + HOST_GAVE_UP, fresh, st);
     if (s != SPSYRK_OK) return s;
     spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
     if (up) {
@@ -546,7 +541,7 @@ spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st)
         up->dev.desc = pl->desc_hi;
         up->dev.jaccard = pl->dev.jaccard;
         up->diag = false;
-        s = bin_launch(up, pl->host.dev + 16, false, st);
+        s = bin_launch(up, pl->host.dev + 16, pl->host.dev + HOST_GAVE_UP, false, st);
         if (s != SPSYRK_OK) return s;
         if (rows > 0) {
             add_work_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev.work, up->dev.work, rows, pl->work_sum);
@@ -554,8 +549,8 @@ spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st)
         }
     }
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    s = bin_collect(pl, pl->host.host);
-    if (s == SPSYRK_OK && up) s = bin_collect(up, pl->host.host + 16);
+    s = bin_collect(pl, pl->host, pl->host.host);
+    if (s == SPSYRK_OK && up) s = bin_collect(up, pl->host, pl->host.host + 16);
     return s;
 }
 static_assert(PF_WORDS <= 16, "a view's facts take sixteen words of the host block");
@@ -706,9 +701,11 @@ void launch_numeric_warp_all(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
 }
 
 // bounds[p] = r0 + the smallest r in [0, rows] with prefix[r] * parts >= p * prefix[rows]
+// (the prefix sums' error word goes to the host)
 __global__ void partition_kernel(const int64_t* __restrict__ prefix, int64_t rows, int64_t parts, int64_t r0,
-                                 int64_t* __restrict__ bounds) {
+                                 int64_t* __restrict__ bounds, const uint32_t* __restrict__ err, int64_t* __restrict__ host) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p == 0) host[0] = (int64_t)*err;
     if (p > parts) return;
     if (p == parts) { bounds[p] = r0 + rows; return; }
     const int64_t target = p * prefix[rows];
@@ -897,6 +894,7 @@ struct CountsOut {
 #pragma unroll
         for (int k = 0; k < 1 + 2 * NROUTE; ++k) host[1 + k] = (int64_t)w[k];
     }
+    __device__ __forceinline__ void gave_up() const { host[HOST_GAVE_UP] = 1; }
 };
 static_assert(2 + 2 * NROUTE <= 32, "the totals take the first half of the host block");
 
@@ -916,7 +914,7 @@ spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, bool routes, int6
         return SPSYRK_OK;
     }
     const int64_t* h = pl->host.host;
-    const spsyrk_status_t s = status_of((uint32_t)h[1]);
+    const spsyrk_status_t s = status_of(pl->host.errors(h[1]));
     if (s == SPSYRK_OK) *total = h[0];
     for (int k = 0; routes && k < NROUTE; ++k) {
         pl->route_n[k] = heavy_rows(pl) ? (uint32_t)h[2 + k] : 0u;
@@ -1101,12 +1099,12 @@ spsyrk_status_t spsyrk_plan_partition(spsyrk_plan_t plan, int64_t parts, int64_t
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     SPSYRK_CUDA_TRY(exclusive_scan_i64<int64_t>(pl->upper_active ? pl->work_sum : pl->dev.work, rows, pl->work_prefix, pl->partials, pl->dev.err, st));
-    partition_kernel<<<(unsigned)((parts + 1 + 255) / 256), 256, 0, st>>>(pl->work_prefix, rows, parts, pl->dev.r0, pl->part_bounds);
+    partition_kernel<<<(unsigned)((parts + 1 + 255) / 256), 256, 0, st>>>(pl->work_prefix, rows, parts, pl->dev.r0, pl->part_bounds, pl->dev.err, pl->host.dev);
     note_launches(1);
     SPSYRK_CUDA_TRY(cudaGetLastError());
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(bounds, pl->part_bounds, (size_t)(parts + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    return SPSYRK_OK;
+    return status_of((uint32_t)pl->host.host[0]);
 }
 
 spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t* nnz_out, void* cuda_stream) {
@@ -1180,7 +1178,7 @@ namespace {
 // out[(2 * c) + e] = first position of class c's row list (ascending local row ids) whose row is >= bound[e]; behind them the
 // pieces of the heavy rows' lists (route_positions), where there are any
 constexpr int POSITION_WORDS = 2 * NCLASS + 4 * NROUTE;
-static_assert(32 + 2 * POSITION_WORDS <= HOST_WORDS, "the positions of both views in the rest of the host block");
+static_assert(32 + 2 * POSITION_WORDS <= HOST_GAVE_UP, "the positions of both views in the rest of the host block");
 __global__ void class_positions_kernel(const int32_t* __restrict__ perm, const int64_t* __restrict__ class_start_dev, int64_t lo_row,
                                        int64_t hi_row, bool heavy, const int32_t* __restrict__ lists, int64_t cap, const int2* __restrict__ rank_parts,
                                        const uint32_t* __restrict__ lengths, int64_t* __restrict__ out) {

@@ -7,20 +7,11 @@
 #include <type_traits>
 
 #include "../../include/spsyrk.h"
+#include "errors.h"
 
 namespace spsyrk {
 
 constexpr unsigned FULL_MASK = 0xffffffffu;
-
-// bits of the device error word
-enum : uint32_t {
-    ERRW_BAD_ROWPTR = 1u,
-    ERRW_BAD_COL = 2u,
-    ERRW_UNSORTED = 4u,
-    ERRW_INTERNAL = 8u,
-    ERRW_UPPER = 16u,
-    ERRW_BAD_CSR = ERRW_BAD_ROWPTR | ERRW_BAD_COL | ERRW_UNSORTED,
-};
 
 // Bounds-checked build (-DSPSYRK_CHECKED, a second library next to the regular one): every index into a
 // shared-memory accumulator, hash or landing slot and every output offset that the kernels compute is
@@ -41,11 +32,14 @@ void note_launches(int n);
 // one synchronisation and no copy, where a copy into ordinary memory took 3 us of device time and as much again
 // on the host, up to five in a row.  Blocks of HOST_WORDS words come from a pool (defined in api.cu).
 constexpr int HOST_WORDS = 160;
+constexpr int HOST_GAVE_UP = HOST_WORDS - 1;  // set by a wait that ran out while the facts were being published; cleared by acquire
 struct HostBlock {
     int64_t* host = nullptr;
     int64_t* dev = nullptr;  // the same memory as kernels see it
     cudaError_t acquire();
     void release();
+    // the error word that a kernel has sent along; a tile that gave up may have set its bit after that
+    uint32_t errors(int64_t word) const { return (uint32_t)word | (host[HOST_GAVE_UP] ? (uint32_t)ERRW_INTERNAL : 0u); }
 };
 struct ScopedHostBlock : HostBlock {
     ~ScopedHostBlock() { release(); }
@@ -218,7 +212,7 @@ __device__ __forceinline__ uint32_t lower_bound_i32(const int32_t* __restrict__ 
 // ---------------------------------------------------------------------------------------
 // Device-wide exclusive scan in one launch, by decoupled look-back (Merrill & Garland, "Single-pass
 // Parallel Prefix Scan with Decoupled Look-back", 2016):
-//   out(i, sum_{r<i} in(r)) for i in [0, n): out stores the prefix; out.total(sum) once at the end.
+//   out(i, sum_{r<i} in(r)) for i in [0, n): out stores the prefix; out.total(sum) once at the end; out.gave_up() if a wait ran out.
 // A CTA takes its tile's number from a counter, so a tile only ever waits for tiles that running CTAs
 // hold; it publishes its own sum, adds up what the tiles before it have published and publishes its
 // inclusive prefix.  A status word is value << 2 | kind, so value and kind arrive together.
@@ -244,8 +238,11 @@ __device__ __forceinline__ void st_status(unsigned long long* p, unsigned long l
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Called by one whole warp: publishes the tile's sum and returns the sum of all tiles before it.
-__device__ __forceinline__ int64_t scan_look_back(unsigned long long* state, int64_t tile, int64_t sum, uint32_t* err) {
+// Called by one whole warp: publishes the tile's sum and returns the sum of all tiles before it.  A wait that runs out sets
+// ERRW_INTERNAL and calls gave_up(): a call that reads the word back returns SPSYRK_ERR_INTERNAL; after an asynchronous one (the
+// mirror's fill) nobody reads it.  The prefix is too small then, so nothing is indexed out of range.
+template <typename GaveUp>
+__device__ __forceinline__ int64_t scan_look_back(unsigned long long* state, int64_t tile, int64_t sum, uint32_t* err, GaveUp gave_up) {
     const int lane = lane_id();
     if (tile == 0) {
         if (lane == 0) st_status(state, ((unsigned long long)sum << 2) | SCAN_PREFIX);
@@ -268,8 +265,11 @@ __device__ __forceinline__ int64_t scan_look_back(unsigned long long* state, int
             if (done) continue;  // (the same for all lanes)
             const int64_t t = last - 32 * k - lane;
             for (int polls = 0; __any_sync(FULL_MASK, (v[k] & 3u) == 0); ++polls) {
-                if (polls == SPIN_LIMIT) {  // the host sees ERRW_INTERNAL; the prefix is too small, so nothing is indexed out of range
-                    if (lane == 0 && err) atomicOr(err, ERRW_INTERNAL);
+                if (polls == SPIN_LIMIT) {
+                    if (lane == 0) {
+                        if (err) atomicOr(err, ERRW_INTERNAL);
+                        gave_up();
+                    }
                     v[k] |= SCAN_PREFIX;
                     break;
                 }
@@ -324,7 +324,7 @@ static __global__ void __launch_bounds__(SCAN_THREADS, 6) scan_kernel(In in, int
     }
     if (ntiles > 1) {
         if (warp == 0) {
-            const int64_t b = scan_look_back(state, tile, tot, err);
+            const int64_t b = scan_look_back(state, tile, tot, err, [&] { out.gave_up(); });
             if (lane == 0) s_before = b;
         }
         __syncthreads();
@@ -352,6 +352,7 @@ struct ScanInto {
     int64_t n;
     __device__ __forceinline__ void operator()(int64_t i, int64_t ex) const { out[i] = ex; }
     __device__ __forceinline__ void total(int64_t t) const { out[n] = t; }
+    __device__ __forceinline__ void gave_up() const {}
 };
 
 // the same, and the total and the error word go to the host (words 0 and 1)
@@ -367,6 +368,7 @@ struct ScanIntoHost {
         host[0] = t;
         host[1] = e;
     }
+    __device__ __forceinline__ void gave_up() const { host[HOST_GAVE_UP] = 1; }
 };
 
 // n >= 1.  The status words are cleared here unless the caller has done so (`cleared`).

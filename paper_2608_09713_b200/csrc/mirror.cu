@@ -264,6 +264,7 @@ struct MirrorRowStart {
         fstart[r] = ex + (l_rowptr[r + 1] - l_rowptr[r]) - (int64_t)diagf[r];
     }
     __device__ __forceinline__ void total(int64_t t) const { f_rowptr[m] = t; }
+    __device__ __forceinline__ void gave_up() const {}
 };
 
 // Measurement aid: CUDA events around the sorting passes (each with its counts and scan).
@@ -526,7 +527,7 @@ extern "C" spsyrk_status_t spsyrk_mirror(int64_t m, int64_t nnz_l, spsyrk_dtype_
             note_launches(1);
             SPSYRK_CUDA_TRY(cudaGetLastError());
             SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-            if (h.host[1]) return SPSYRK_ERR_BAD_CSR;
+            if (h.host[1]) return status_of((uint32_t)h.host[1]);
             *nnz_full_out = 2 * nnz_l - h.host[0];
         }
         return SPSYRK_OK;
@@ -639,7 +640,7 @@ extern "C" spsyrk_status_t spsyrk_mirror_rowptr_noalloc(int64_t m, const int64_t
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&nnz, d_f_rowptr + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, err, 4, cudaMemcpyDeviceToHost, st));
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    if (e & (ERRW_UPPER | ERRW_BAD_ROWPTR)) return SPSYRK_ERR_BAD_CSR;
+    if (e) return status_of(e);
     *nnz_full_out = nnz;
     return SPSYRK_OK;
 }

@@ -214,8 +214,7 @@ extern "C" spsyrk_status_t spsyrk_permute(int64_t m, int64_t n, int64_t nnz, sps
     uint32_t e = 0;
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, w.err, 4, cudaMemcpyDeviceToHost, st));
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    if (e & ERRW_BAD_ROWPTR) return SPSYRK_ERR_BAD_CSR;
-    if (e) return SPSYRK_ERR_INVALID_ARG;
+    if (e) return status_of(e, SPSYRK_ERR_INVALID_ARG);  // so far a column id out of range is one of the maps'
     if (m == 0 || nnz == 0) return SPSYRK_OK;
 
 #define EXPAND(G)                                                                                                        \
@@ -235,6 +234,6 @@ extern "C" spsyrk_status_t spsyrk_permute(int64_t m, int64_t n, int64_t nnz, sps
     if (s != SPSYRK_OK) return s;
     SPSYRK_CUDA_TRY(cudaMemcpyAsync(&e, w.err, 4, cudaMemcpyDeviceToHost, st));
     SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
-    if (e) return SPSYRK_ERR_BAD_CSR;  // a column id outside [0, n)
+    if (e) return status_of(e);
     return SPSYRK_OK;
 }

@@ -70,7 +70,7 @@ __device__ __forceinline__ int64_t radix_look_back(S* words, int64_t tile, int d
         for (int k = 0; k < W; ++k) {
             if (done) continue;
             for (int polls = 0; (v[k] & 3) == 0; ++polls) {
-                if (polls == SPIN_LIMIT) {  // the host sees ERRW_INTERNAL; the sum is too small, nothing is indexed out of range
+                if (polls == SPIN_LIMIT) {  // as in scan_look_back: the sum is too small, nothing is indexed out of range
                     if (err) atomicOr(err, ERRW_INTERNAL);
                     v[k] = (S)SCAN_PREFIX;
                     break;
@@ -133,7 +133,7 @@ struct RadixSmem {
     }
 };
 
-// `err` is the device error word of the caller (used by the bounds-checked build only).
+// `err` is the device error word of the caller: set by a look-back that gives up (and by the bounds-checked build).
 // Emit(dest, key, pa, pb) is called once per element with its position `dest` in the order sorted
 // by the digits seen so far.  pa == nullptr (pb == nullptr) means "this payload is the element's own
 // index".

@@ -342,6 +342,7 @@ struct BinStarts {
         if (c * nblocks == (uint32_t)i) class_start[c] = ex;
     }
     __device__ __forceinline__ void total(int64_t t) const { class_start[NCLASS] = t; }
+    __device__ __forceinline__ void gave_up() const {}
 };
 
 // Second half of the counting sort: the rows in class order (ascending inside a class), for each of them the header
@@ -402,6 +403,7 @@ struct PlanFacts {
     const uint32_t* facts;
     const uint32_t* err;
     int64_t* host;
+    int64_t* gave_up;
     __device__ __forceinline__ void publish(int64_t map_items) const {
         int64_t w[PF_WORDS];  // all loads before the first store: one round trip, not thirteen
 #pragma unroll
@@ -424,6 +426,7 @@ struct ItemStarts {
         itemoff[n] = t;
         facts.publish(t);
     }
+    __device__ __forceinline__ void gave_up() const { *facts.gave_up = 1; }
 };
 
 }  // namespace spsyrk
