@@ -6,9 +6,10 @@
 //   sizes   : rows are ascending, so a row stores its diagonal iff its last entry is the diagonal and
 //             holds an entry above the diagonal iff its last entry is one:
 //             nnz(F) = 2 nnz(C_L) - #diagonals.
-//   sort    : 4-byte values and small matrices go to buckets of columns and from there to their places
-//             (mirror_sort.cuh); 8-byte values of more than 65536 rows go through radix passes of 16-byte
-//             records, the last of which writes F (mirror_rec.cuh);
+//   sort    : 4-byte values of up to 2^24 rows and small matrices go to buckets of columns and from there to their
+//             places (mirror_sort.cuh); 8-byte values of more than 65536 rows go through radix passes of 16-byte
+//             records, the last of which writes F (mirror_rec.cuh); 4-byte values of more rows through radix passes
+//             of separate arrays (radix.cuh);
 //   rows    : row lengths of F, scan -> f_rowptr (in the bucket sort before the last pass), lower parts copied.
 #include <algorithm>
 #include <mutex>
@@ -29,6 +30,10 @@ constexpr int MIRROR_RADIX_BITS = 8;  // digits of the record passes
 // the launches: it is used where both take two passes.  (Product and mirror of 4096 rows: 465 -> 415 us.)
 constexpr int64_t MIRROR_BUCKET_ROWS_8 = 65536;
 bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCKET_ROWS_8; }
+// 4-byte values: what the first pass of the bucket sort leaves of a column must fit two bytes.  (Taking the columns of wider
+// matrices in rounds of 2^24 reads all entries once per round: 2^26 rows and 2.7e8 entries 25.5 ms, 2^27 rows and
+// 4.0e8 entries 59.1 ms, against 16.6 and 26.9 ms by four radix passes.)
+bool mirror_by_radix(int64_t m, size_t sv) { return sv == 4 && m > (int64_t(1) << MS_COLUMN_BITS); }
 
 struct MirrorWs {
     int64_t* partials;
@@ -43,6 +48,11 @@ struct MirrorWs {
     void* rec;           // the records the place pass reads (nnz_l)
     void* rec_tail;      // three passes: what of the first buffer does not fit F's value array
     uint16_t* high;      // 4-byte values: the rests of the columns beside the records
+    // radix passes: two sets of (column, row, value); the one the last pass does not read keeps columns and values in F
+    uint32_t *key_a, *row_a, *key_b, *row_b;
+    void *val_a, *val_b;
+    RadixState rx;       // all zero at the start
+    size_t rx_bytes;
     // record passes
     uint32_t* diagf32;   // m
     uint32_t* rowtot;    // m
@@ -59,9 +69,9 @@ struct MirrorWs {
 // How the sort is cut (see mirror_sort.cuh)
 struct MirrorSplit {
     int lbits, mbits, hbits, pieces;
-    int64_t rounds, chunk, nchunks;
-    int64_t split_hist() const { return (rounds << lbits) * nchunks; }
-    int64_t mid_hist() const { return mbits ? (rounds << (lbits + mbits)) * pieces : 0; }
+    int64_t chunk, nchunks;
+    int64_t split_hist() const { return nchunks << lbits; }
+    int64_t mid_hist() const { return mbits ? (int64_t)pieces << (lbits + mbits) : 0; }
 };
 
 // Column ids of at most so many bits take two passes: parts of nine bits leave runs of eight entries in a tile.  (Two parts of
@@ -71,8 +81,7 @@ constexpr int MIRROR_TWO_PASS_BITS = 18;
 MirrorSplit mirror_split_for(int64_t m, int64_t nnz_l, size_t sv) {
     MirrorSplit s;
     int bits = 1;
-    while (bits < MS_ROUND_BITS && ((m - 1) >> bits) > 0) ++bits;
-    s.rounds = (std::max<int64_t>(m - 1, 0) >> MS_ROUND_BITS) + 1;
+    while (bits < MS_COLUMN_BITS && ((m - 1) >> bits) > 0) ++bits;
     if (bits <= MIRROR_TWO_PASS_BITS) {
         s.lbits = std::max(8, (bits + 1) / 2);  // at least 256 buckets: a bucket is one CTA of the last pass
         s.mbits = 0;
@@ -91,7 +100,7 @@ MirrorSplit mirror_split_for(int64_t m, int64_t nnz_l, size_t sv) {
     else s.chunk = std::max<int64_t>(nnz_l / (MANY * tile), 1) * tile;
     s.chunk = (s.chunk + 31) / 32 * 32;
     s.nchunks = std::max<int64_t>((nnz_l + s.chunk - 1) / s.chunk, 1);
-    s.pieces = (int)std::min<int64_t>(std::max<int64_t>((nnz_l / s.rounds >> s.lbits) / (4 * tile), 1), 64);
+    s.pieces = (int)std::min<int64_t>(std::max<int64_t>((nnz_l >> s.lbits) / (4 * tile), 1), 64);
     return s;
 }
 
@@ -132,6 +141,25 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
         t.tile_rows = (int32_t*)take(2 * std::max<int64_t>(mirror_tiles(nnz_l), 1) * 4);
         t.hist = (uint32_t*)take(hist_n * 4);
         t.offsets = (int64_t*)take((hist_n + 1) * 8);
+    } else if (mirror_by_radix(m, sv)) {
+        // F's column and value arrays hold 4 (2 nnz_l - D) >= 4 nnz_l bytes each: the columns and values of one set.  Passes write
+        // A, B, A, ...: the last one reads B when their number is odd.
+        const int npass = radix_passes((uint64_t)m);  // columns, and m for the diagonal entries
+        const bool b_kept = npass % 2 == 1;
+        t.rowtot = (uint32_t*)take(items * 4);
+        t.seg_start = (unsigned long long*)take(items * 8);
+        t.seg_end = (unsigned long long*)take(items * 8);
+        t.partials = (int64_t*)take(scan_partials_count(items) * 8);
+        t.row_a = (uint32_t*)take(ne * 4);
+        t.row_b = (uint32_t*)take(ne * 4);
+        uint32_t* const key = (uint32_t*)take(ne * 4);
+        void* const val = take(ne * 4);
+        if (b_kept) { t.key_b = key; t.val_b = val; } else { t.key_a = key; t.val_a = val; }
+        const size_t words = radix_state_words(radix_tiles(nnz_l), radix_wide(nnz_l), npass);
+        t.rx_bytes = (RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES + words) * 8;
+        t.rx.bins = (unsigned long long*)take(t.rx_bytes);
+        t.rx.tickets = (uint32_t*)(t.rx.bins + RX_MAX_PASSES * RX_BINS);
+        t.rx.words = t.rx.bins + RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES;
     } else {
         const MirrorSplit sp = mirror_split_for(m, nnz_l, sv);
         const int64_t hist_n = std::max(sp.split_hist(), sp.mid_hist());
@@ -245,6 +273,22 @@ int group_width(int64_t nnz, int64_t m) {
     return avg <= 4 ? 4 : avg <= 8 ? 8 : avg <= 16 ? 16 : 32;
 }
 
+template <typename V>
+void mirror_copy_lower(int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx, const void* l_vals, const int64_t* f_rowptr, int32_t* f_colidx,
+                       void* f_vals, cudaStream_t st) {
+#define COPY(G)                                                                                                                                       \
+    mirror_copy_lower_kernel<V, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, static_cast<const V*>(l_vals), m, f_rowptr, \
+                                                                                    f_colidx, static_cast<V*>(f_vals))
+    switch (group_width(nnz_l, m)) {
+        case 4: COPY(4); break;
+        case 8: COPY(8); break;
+        case 16: COPY(16); break;
+        default: COPY(32); break;
+    }
+#undef COPY
+    note_launches(1);
+}
+
 // row lengths of F: the row's own entries and those of its column, the diagonal once
 struct MirrorRowLength {
     using Value = int64_t;
@@ -287,7 +331,7 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         return SPSYRK_OK;
     }
     const MirrorSplit sp = mirror_split_for(m, nnz_l, sizeof(VB));
-    const int64_t nbuckets = sp.rounds << (sp.lbits + sp.mbits);  // of the place pass
+    const int64_t nbuckets = int64_t(1) << (sp.lbits + sp.mbits);  // of the place pass
     const bool three = sp.mbits > 0;
     const int g = group_width(nnz_l, m);
     uint16_t* const f_high = reinterpret_cast<uint16_t*>(f_colidx);
@@ -313,20 +357,14 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
 #define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf)
     if (g <= 16) ROWS(4); else ROWS(16);
 #undef ROWS
-    for (int64_t q = 0; q < sp.rounds; ++q) {
-        a.round = (uint32_t)q;
-        mirror_split_count_kernel<<<(unsigned)sp.nchunks, MS_THREADS, 0, st>>>(a, w.hist);
-    }
+    mirror_split_count_kernel<<<(unsigned)sp.nchunks, MS_THREADS, 0, st>>>(a, w.hist);
     SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.split_hist(), w.offsets, w.partials, w.err, st));
-    for (int64_t q = 0; q < sp.rounds; ++q) {
-        a.round = (uint32_t)q;
-        mirror_split_kernel<VB><<<(unsigned)sp.nchunks, MS_THREADS, split_smem, st>>>(a);
-    }
-    note_launches(1 + 2 * (int)sp.rounds);
+    mirror_split_kernel<VB><<<(unsigned)sp.nchunks, MS_THREADS, split_smem, st>>>(a);
+    note_launches(3);
     mirror_mark(1, st);
     int pass = 2;
     if constexpr (sizeof(VB) == 4) if (three) {
-        const unsigned units = (unsigned)((sp.rounds << sp.lbits) * sp.pieces);
+        const unsigned units = (unsigned)(sp.pieces << sp.lbits);
         mirror_mid_count_kernel<<<units, MS_THREADS, 0, st>>>(a, w.hist);
         SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.partials, w.err, st));
         const size_t mid_smem = MirrorMidSmem<VB>::bytes(1 << sp.mbits);
@@ -340,18 +378,8 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     mirror_place_kernel<VB><<<(unsigned)nbuckets, MS_THREADS, place_smem, st>>>(a);
     mirror_mark(pass, st);
     g_mirror_passes = pass;
-    const VB* lv = static_cast<const VB*>(l_vals);
-    VB* fv = static_cast<VB*>(f_vals);
-#define COPY(G) \
-    mirror_copy_lower_kernel<VB, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, lv, m, f_rowptr, f_colidx, fv)
-    switch (g) {
-        case 4: COPY(4); break;
-        case 8: COPY(8); break;
-        case 16: COPY(16); break;
-        default: COPY(32); break;
-    }
-#undef COPY
-    note_launches(3);
+    mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+    note_launches(2);
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
     {
@@ -361,6 +389,62 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         if (e & ERRW_INTERNAL) return SPSYRK_ERR_INTERNAL;
     }
 #endif
+    return SPSYRK_OK;
+}
+
+// row lengths of F: the row's own entries and its column's segment of the sorted order
+__global__ void mirror_rowlen_kernel(const int64_t* __restrict__ l_rowptr, const unsigned long long* __restrict__ seg_start,
+                                     const unsigned long long* __restrict__ seg_end, int64_t m, uint32_t* __restrict__ rowtot) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= m) return;
+    const unsigned long long s = seg_start[r], e = seg_end[r];
+    rowtot[r] = (uint32_t)(l_rowptr[r + 1] - l_rowptr[r]) + (e > s ? (uint32_t)(e - s) : 0u);
+}
+
+// 4-byte values of more than 2^24 rows
+spsyrk_status_t mirror_fill_radix(const MirrorWs& ws, int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx, const void* l_vals,
+                                  int64_t* f_rowptr, int32_t* f_colidx, void* f_vals, cudaStream_t st) {
+    if (nnz_l == 0) {
+        SPSYRK_CUDA_TRY(cudaMemsetAsync(f_rowptr, 0, (size_t)(m + 1) * sizeof(int64_t), st));
+        return SPSYRK_OK;
+    }
+    MirrorWs w = ws;
+    if (!w.key_a) { w.key_a = reinterpret_cast<uint32_t*>(f_colidx); w.val_a = f_vals; }
+    if (!w.key_b) { w.key_b = reinterpret_cast<uint32_t*>(f_colidx); w.val_b = f_vals; }
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(w.seg_start, 0xff, (size_t)m * 8, st));
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(w.seg_end, 0, (size_t)m * 8, st));
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(w.rx.bins, 0, w.rx_bytes, st));
+    mirror_mark(0, st);
+#define EXPAND(G) mirror_expand_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.key_b, w.row_b)
+    switch (group_width(nnz_l, m)) {
+        case 4: EXPAND(4); break;
+        case 8: EXPAND(8); break;
+        case 16: EXPAND(16); break;
+        default: EXPAND(32); break;
+    }
+#undef EXPAND
+    note_launches(1);
+    const int npass = radix_passes((uint64_t)m);
+    const uint32_t *key = w.key_b, *row = w.row_b, *val = static_cast<const uint32_t*>(l_vals);
+    SPSYRK_CUDA_TRY(radix_bins<false>(key, nnz_l, npass, w.rx.bins, st));
+    for (int p = 0; p < npass; ++p) {
+        const bool to_a = p % 2 == 0;
+        if (p == npass - 1) {
+            const EmitMirror emit{l_rowptr, (uint32_t)m, f_colidx, static_cast<uint32_t*>(f_vals), w.seg_start, w.seg_end};
+            SPSYRK_CUDA_TRY((radix_pass<uint32_t, false>(key, row, val, nullptr, nnz_l, p, w.rx, emit, w.err, st)));
+        } else {
+            const EmitArrays<uint32_t> emit{to_a ? w.key_a : w.key_b, to_a ? w.row_a : w.row_b, static_cast<uint32_t*>(to_a ? w.val_a : w.val_b)};
+            SPSYRK_CUDA_TRY((radix_pass<uint32_t, false>(key, row, val, nullptr, nnz_l, p, w.rx, emit, w.err, st)));
+            key = emit.keys; row = emit.pa; val = emit.pb;
+        }
+        mirror_mark(p + 1, st);
+        g_mirror_passes = p + 1;
+    }
+    mirror_rowlen_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, w.seg_start, w.seg_end, m, w.rowtot);
+    note_launches(1);
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.rowtot, m, f_rowptr, w.partials, w.err, st));
+    mirror_copy_lower<uint32_t>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+    SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
 }
 
@@ -470,18 +554,7 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
         note_launches(1);
     }
     SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.rowtot, m, f_rowptr, w.partials, w.err, st));
-    if (m > 0 && nnz_l > 0) {
-#define COPY(G) \
-    mirror_copy_lower_kernel<uint64_t, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, lv, m, f_rowptr, f_colidx, fv)
-        switch (g) {
-            case 4: COPY(4); break;
-            case 8: COPY(8); break;
-            case 16: COPY(16); break;
-            default: COPY(32); break;
-        }
-#undef COPY
-        note_launches(1);
-    }
+    if (m > 0 && nnz_l > 0) mirror_copy_lower<uint64_t>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
     {
@@ -538,7 +611,9 @@ extern "C" spsyrk_status_t spsyrk_mirror(int64_t m, int64_t nnz_l, spsyrk_dtype_
         case SPSYRK_F64:
             if (mirror_by_records(m, sv)) return mirror_fill_rec(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
             return mirror_fill<uint64_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
-        default: return mirror_fill<uint32_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
+        default:
+            if (mirror_by_radix(m, sv)) return mirror_fill_radix(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
+            return mirror_fill<uint32_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
     }
 }
 

@@ -17,8 +17,6 @@
 
 namespace spsyrk {
 
-constexpr uint32_t NO_KEY = 0xffffffffu;
-
 // tile of the record passes: with 16-byte records a run of 8 elements per digit is already a full
 // 128-byte line, so tiles can be half the size of the separate-array passes and four CTAs share an SM
 constexpr int MR_THREADS = 256;

@@ -133,6 +133,11 @@ struct RadixSmem {
     }
 };
 
+// Emits that want to see the keys before and after theirs in the tile's order (NO_KEY at its ends): where a key's run begins and ends
+constexpr uint32_t NO_KEY = 0xffffffffu;
+template <typename Emit, typename = void> struct EmitNeighbours : std::false_type {};
+template <typename Emit> struct EmitNeighbours<Emit, std::void_t<decltype(Emit::NEIGHBOURS)>> : std::true_type {};
+
 // `err` is the device error word of the caller: set by a look-back that gives up (and by the bounds-checked build).
 // Emit(dest, key, pa, pb) is called once per element with its position `dest` in the order sorted
 // by the digits seen so far.  pa == nullptr (pb == nullptr) means "this payload is the element's own
@@ -258,6 +263,8 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
         if (dest < 0 || dest >= n) continue;
         if constexpr (HAS_PC) {
             emit(dest, key, s_pa[q], s_pb[q], s_pc[q]);
+        } else if constexpr (EmitNeighbours<Emit>::value) {
+            emit(dest, key, s_pa[q], s_pb[q], q > 0 ? s_key[q - 1] : NO_KEY, q + 1 < tile_n ? s_key[q + 1] : NO_KEY);
         } else {
             emit(dest, key, s_pa[q], s_pb[q]);
         }

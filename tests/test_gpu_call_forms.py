@@ -175,3 +175,59 @@ def test_one_plan_on_two_streams(B, mode):
     for c, v in outs:
         assert torch.equal(c, ci)
         assert float(((v - cv).abs() / scale).max()) <= 1e-5  # (sums of positive products: any order of additions)
+
+
+# ------------------------------------------------------------------ mirror: where the entries lie, how many rows there are
+def lower_triangle(m, rows, cols, dtype, seed=1):
+    """CSR of the distinct (row, column) pairs, on the GPU; values are distinct small numbers."""
+    code = torch.unique(rows * m + cols)
+    r = torch.div(code, m, rounding_mode="floor")
+    rp = torch.searchsorted(r, torch.arange(m + 1, device="cuda"))
+    vals = (torch.arange(code.numel(), device="cuda") % 1_000_003 + seed).to(dtype)
+    return rp, (code - r * m).to(torch.int32), vals
+
+
+def check_mirror(B, m, c, f=None):
+    """F against the union of C_L and its reflection, sorted."""
+    rp, ci, cv = c
+    f_rp, f_ci, f_cv = B.spsyrk_mirror(m, *c) if f is None else f
+    rows = torch.repeat_interleave(torch.arange(m, device="cuda"), rp[1:] - rp[:-1])
+    below = ci < rows
+    code = torch.cat([rows * m + ci, ci[below].long() * m + rows[below]])
+    order = torch.argsort(code)
+    code = code[order]
+    r = torch.div(code, m, rounding_mode="floor")
+    assert torch.equal(f_rp, torch.searchsorted(r, torch.arange(m + 1, device="cuda")))
+    assert torch.equal(f_ci.long(), code - r * m)
+    assert torch.equal(f_cv, torch.cat([cv, cv[below]])[order])
+
+
+def arange(m):
+    return torch.arange(m, device="cuda")
+
+
+def pattern(name, m, k):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + k)
+    rows = torch.randint(0, m, (k,), generator=g, device="cuda")
+    share = torch.rand(k, generator=g, device="cuda", dtype=torch.float64)
+    if name == "spread":
+        cols = (share * (rows + 1)).long()
+    elif name == "one column":
+        rows, cols = arange(m), torch.zeros_like(arange(m))
+    elif name == "every 512th column":
+        cols = (share * (rows // 512 + 1)).long() * 512
+    elif name == "few rows":
+        rows = rows % 7 * (m // 7)
+        cols = (share * (rows + 1)).long()
+    cols = torch.minimum(cols, rows)
+    return torch.cat([rows, arange(m)[:: 1 if name != "few rows" else m // 5]]), torch.cat([cols, arange(m)[:: 1 if name != "few rows" else m // 5]])
+
+
+@pytest.mark.parametrize("name", ["spread", "one column", "every 512th column", "few rows"])
+@pytest.mark.parametrize("m,k,dtype", [(1 << 18, 1 << 21, torch.float32), ((1 << 19) + 1, 20_000_000, torch.int32), ((1 << 20) - 3, 1_000_000, torch.float32),
+                                       (65536, 1 << 21, torch.float64), ((1 << 24) + 1, 3_000_000, torch.float32)])
+def test_mirror_wherever_the_entries_lie(B, name, m, k, dtype):
+    """Buckets that are cut into pieces and buckets that are not, two passes and three, radix passes for few entries and for
+    more than 2^24 rows, rows that are searched for."""
+    check_mirror(B, m, lower_triangle(m, *pattern(name, m, k), dtype))
