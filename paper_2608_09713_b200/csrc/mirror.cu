@@ -40,6 +40,10 @@ struct MirrorWs {
     uint32_t* err;       // [0] error word, [1] number of diagonal entries, [2] finished CTAs
     uint32_t* hist;      // counts of the passes and their prefix sums
     int64_t *offsets, *mid_off;
+    int32_t *mid_first, *first_piece;  // where the pieces of a bucket begin
+    uint8_t* mid_bucket;
+    uint32_t *pieces, *piece_cnt;
+    int2* piece;
     // bucket sort
     uint8_t* diagf;      // m: 1 where the row stores its diagonal entry
     uint32_t* cnt;       // m: entries of C_L per column
@@ -68,10 +72,13 @@ struct MirrorWs {
 
 // How the sort is cut (see mirror_sort.cuh)
 struct MirrorSplit {
-    int lbits, mbits, hbits, pieces;
-    int64_t chunk, nchunks;
+    int lbits, mbits, hbits;
+    int64_t chunk, nchunks;     // split
+    int64_t mid_cap, mid_units;  // mid: entries per piece, pieces at most
+    int64_t cap, max_pieces;    // place: entries from which on a bucket is cut, pieces at most
     int64_t split_hist() const { return nchunks << lbits; }
-    int64_t mid_hist() const { return mbits ? (int64_t)pieces << (lbits + mbits) : 0; }
+    int64_t mid_hist() const { return mid_units << mbits; }
+    int64_t nbuckets() const { return int64_t(1) << (lbits + mbits); }
 };
 
 // Column ids of at most so many bits take two passes: parts of nine bits leave runs of eight entries in a tile.  (Two parts of
@@ -100,7 +107,13 @@ MirrorSplit mirror_split_for(int64_t m, int64_t nnz_l, size_t sv) {
     else s.chunk = std::max<int64_t>(nnz_l / (MANY * tile), 1) * tile;
     s.chunk = (s.chunk + 31) / 32 * 32;
     s.nchunks = std::max<int64_t>((nnz_l + s.chunk - 1) / s.chunk, 1);
-    s.pieces = (int)std::min<int64_t>(std::max<int64_t>((nnz_l >> s.lbits) / (4 * tile), 1), 64);
+    // Pieces of the mid pass: four tiles or more, at most about 16384.  Every bucket has at least one.
+    s.mid_cap = std::max<int64_t>(4 * tile, nnz_l / 16384);
+    s.mid_units = s.mbits ? (int64_t(1) << s.lbits) + nnz_l / s.mid_cap : 0;
+    // A bucket of `place` is cut above a quarter of what a CTA would get if all were equal; of few entries, above 8 to 16 tiles (gone
+    // in 30 to 50 us), but not where it is less than twice the average.  A cut bucket has less than twice len / cap pieces.
+    s.cap = std::max<int64_t>(nnz_l / (148 * 2 * 4), std::min<int64_t>(16 * tile, std::max<int64_t>(8 * tile, 2 * (nnz_l >> (s.lbits + s.mbits)))));
+    s.max_pieces = 2 * (nnz_l / s.cap);
     return s;
 }
 
@@ -170,6 +183,12 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
         t.hist = (uint32_t*)take(hist_n * 4);
         t.offsets = (int64_t*)take((sp.split_hist() + 1) * 8);
         t.mid_off = (int64_t*)take((sp.mid_hist() + 1) * 8);
+        t.mid_first = (int32_t*)take(257 * 4);
+        t.mid_bucket = (uint8_t*)take(sp.mid_units);
+        t.first_piece = (int32_t*)take(sp.nbuckets() * 4);
+        t.pieces = (uint32_t*)take(4);
+        t.piece = (int2*)take(sp.max_pieces * 8);
+        t.piece_cnt = (uint32_t*)take((sp.max_pieces << sp.hbits) * 4);
         t.step_row = (int32_t*)take((ne + 31) / 32 * 4);
         t.rec = take(ne * 2 * sv);
         t.rec_tail = take(sp.mbits ? (mirror_tail_records(m, nnz_l) + 1) * 2 * sv : 0);
@@ -331,13 +350,15 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         return SPSYRK_OK;
     }
     const MirrorSplit sp = mirror_split_for(m, nnz_l, sizeof(VB));
-    const int64_t nbuckets = int64_t(1) << (sp.lbits + sp.mbits);  // of the place pass
     const bool three = sp.mbits > 0;
     const int g = group_width(nnz_l, m);
     uint16_t* const f_high = reinterpret_cast<uint16_t*>(f_colidx);
     MirrorSortArgs a{};
     a.l_rowptr = l_rowptr; a.l_colidx = l_colidx; a.l_vals = l_vals; a.m = m; a.n = nnz_l; a.chunk = sp.chunk; a.nchunks = sp.nchunks;
-    a.lbits = sp.lbits; a.mbits = sp.mbits; a.hbits = sp.hbits; a.pieces = sp.pieces; a.step_row = w.step_row;
+    a.lbits = sp.lbits; a.mbits = sp.mbits; a.hbits = sp.hbits; a.step_row = w.step_row;
+    a.mid_cap = sp.mid_cap; a.mid_units = (int)sp.mid_units; a.mid_first = w.mid_first; a.mid_bucket = w.mid_bucket;
+    a.nbuckets = sp.nbuckets(); a.cap = sp.cap; a.max_pieces = (uint32_t)sp.max_pieces; a.pieces = w.pieces; a.first_piece = w.first_piece;
+    a.piece = w.piece; a.piece_cnt = w.piece_cnt;
     a.split_off = w.offsets; a.mid_off = w.mid_off;
     a.rec_a = three ? f_vals : w.rec;
     a.rec_a_tail = w.rec_tail;
@@ -347,14 +368,12 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     uint16_t* const last_high = sizeof(VB) == 4 ? w.high : f_high;
     a.high_b = last_high;
     a.high_a = !three ? last_high : sizeof(VB) == 4 ? f_high : f_high + nnz_l;  // (only the last pass's rests are read 16 bytes at a time)
-    a.place_off = three ? w.mid_off : w.offsets;
-    a.place_stride = three ? sp.pieces : sp.nchunks;
     a.cnt = w.cnt; a.fstart = w.fstart; a.f_colidx = f_colidx; a.f_vals = f_vals; a.err = w.err;
     const size_t split_smem = MirrorSplitSmem<VB>::bytes(1 << sp.lbits), place_smem = MirrorPlaceSmem<VB>::bytes(1 << sp.hbits);
     SPSYRK_CUDA_TRY(allow_shared_memory<mirror_split_kernel<VB>>());
     SPSYRK_CUDA_TRY(allow_shared_memory<mirror_place_kernel<VB>>());
     mirror_mark(0, st);
-#define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf)
+#define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf, w.cnt, w.pieces)
     if (g <= 16) ROWS(4); else ROWS(16);
 #undef ROWS
     mirror_split_count_kernel<<<(unsigned)sp.nchunks, MS_THREADS, 0, st>>>(a, w.hist);
@@ -364,7 +383,7 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     mirror_mark(1, st);
     int pass = 2;
     if constexpr (sizeof(VB) == 4) if (three) {
-        const unsigned units = (unsigned)(sp.pieces << sp.lbits);
+        const unsigned units = (unsigned)sp.mid_units;
         mirror_mid_count_kernel<<<units, MS_THREADS, 0, st>>>(a, w.hist);
         SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.partials, w.err, st));
         const size_t mid_smem = MirrorMidSmem<VB>::bytes(1 << sp.mbits);
@@ -373,9 +392,10 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         note_launches(2);
         mirror_mark(pass++, st);
     }
-    mirror_column_count_kernel<<<(unsigned)nbuckets, MS_THREADS, 0, st>>>(a, last_high);
+    const unsigned place_units = (unsigned)(sp.nbuckets() + sp.max_pieces);
+    mirror_column_count_kernel<<<place_units, MS_THREADS, 0, st>>>(a, last_high);
     SPSYRK_CUDA_TRY(scan_launch(MirrorRowLength{l_rowptr, w.cnt, w.diagf}, m, MirrorRowStart{l_rowptr, w.diagf, f_rowptr, w.fstart, m}, w.partials, w.err, st));
-    mirror_place_kernel<VB><<<(unsigned)nbuckets, MS_THREADS, place_smem, st>>>(a);
+    mirror_place_kernel<VB><<<place_units, MS_THREADS, place_smem, st>>>(a);
     mirror_mark(pass, st);
     g_mirror_passes = pass;
     mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);

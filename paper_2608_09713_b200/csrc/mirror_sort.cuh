@@ -6,11 +6,16 @@
 //   mid   : (three passes) every bucket's entries go to one of 2^M buckets each by the next part;
 //   place : a CTA walks a bucket in order, ranks every entry inside its column (the high part) and writes
 //           it to its place in F.  Rows arrive ascending, so rank order is row order.
-// Buckets by low bits are of nearly equal size whatever the matrix (columns of C_L get shorter to the right,
+// Buckets by low bits are of nearly equal size for most matrices (columns of C_L get shorter to the right,
 // hubs sit together before a relabelling), so one CTA per bucket is a fair share of work, and a bucket's
 // CTA needs no per-tile histogram: before `place`, the entries of every column are counted from the high
 // parts that the pass before wrote beside the records (two bytes each), and with the row lengths of C_L that gives
-// F's row pointers by one scan, before F is written.  Diagonal entries travel along: the diagonal entry of
+// F's row pointers by one scan, before F is written.  A bucket that holds more than its share (a column that most rows
+// store, columns a power of two apart, fewer buckets than the GPU has room for) is cut into pieces: each piece counts its columns, and
+// a piece starts behind what the pieces before it hold.  Which buckets are cut is known on the GPU only, so the launches have
+// room for as many pieces as there can be.  (One CTA per bucket whatever its size: 4e6 rows that all store column 0,
+// 12.97 ms against 1.29; 2^18 rows over every 512th column 6.01 ms against 0.26; 2.9e8 entries of a dense triangle of
+// doubles, 256 buckets on 296 places, 8.07 ms against 7.44.)  Diagonal entries travel along: the diagonal entry of
 // column j is the first of its column and its place, one before the reflected entries, is where the row's own
 // diagonal belongs anyway.
 //
@@ -54,18 +59,26 @@ struct MirrorSortArgs {
     int64_t chunk, nchunks;
     const int32_t* step_row;   // row of every 32nd entry
     const int64_t* split_off;  // [part * nchunks + chunk], one more at the end
-    // mid: every bucket of the split in `pieces` equal parts, one CTA each
-    int pieces;
-    const int64_t* mid_off;    // [part * (pieces << L) + (bucket * pieces + piece)], one more at the end
+    // mid: every bucket of the split in pieces of about mid_cap entries, one CTA each, numbered in the order of the entries
+    int64_t mid_cap;
+    int mid_units;             // launched (there are at most so many)
+    int32_t* mid_first;        // [(1 << L) + 1] the first piece of every bucket
+    uint8_t* mid_bucket;       // [mid_units] the bucket of every piece
+    const int64_t* mid_off;    // [part * mid_units + piece], one more at the end
     // records and rests of the split (two pieces: [0, a_split) and the tail) and what `place` reads
     void *rec_a, *rec_a_tail;
     int64_t a_split;
     uint16_t* high_a;
     void* rec_b;
     uint16_t* high_b;
-    const int64_t* place_off;  // bucket b of `place` is [place_off[b * place_stride], place_off[(b + 1) * place_stride])
-    int64_t place_stride;
-    uint32_t* cnt;             // entries per column
+    // place: one CTA per bucket, and one per piece of the buckets of more than `cap` entries
+    int64_t nbuckets, cap;
+    uint32_t max_pieces;       // launched (there are at most so many)
+    uint32_t* pieces;          // pieces of all cut buckets, zero before the last split
+    int32_t* first_piece;      // [nbuckets] -1: not cut
+    int2* piece;               // [max_pieces] (bucket, number inside it)
+    uint32_t* piece_cnt;       // [max_pieces << H] entries per column
+    uint32_t* cnt;             // entries per column; zero before
     const int64_t* fstart;     // where column j's entries go in F
     int32_t* f_colidx;
     void* f_vals;
@@ -105,16 +118,21 @@ __device__ __forceinline__ void ms_count(int64_t e0, int64_t e1, int bits, uint3
 }
 
 // G lanes per row: the row of every 32nd entry; whether the row stores its diagonal entry (rows are ascending: it is
-// the last one)
+// the last one); the counters that later passes add to
 template <int G>
 static __global__ void __launch_bounds__(256) mirror_rows_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx, int64_t m,
-                                                                 int64_t n, int32_t* __restrict__ step_row, uint8_t* __restrict__ diagf) {
+                                                                 int64_t n, int32_t* __restrict__ step_row, uint8_t* __restrict__ diagf,
+                                                                 uint32_t* __restrict__ cnt, uint32_t* __restrict__ pieces) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
     if (r >= m) return;
     const int64_t p0 = max(l_rowptr[r], (int64_t)0), p1 = min(l_rowptr[r + 1], n);
     for (int64_t s = (p0 + 31) / 32 + gl; s * 32 < p1; s += G) step_row[s] = (int32_t)r;
-    if (gl == 0) diagf[r] = (p1 > p0 && (int64_t)l_colidx[p1 - 1] == r) ? 1 : 0;
+    if (gl == 0) {
+        diagf[r] = (p1 > p0 && (int64_t)l_colidx[p1 - 1] == r) ? 1 : 0;
+        cnt[r] = 0;
+        if (r == 0) *pieces = 0;
+    }
 }
 
 // entries per (low part, chunk)
@@ -124,34 +142,97 @@ static __global__ void __launch_bounds__(MS_THREADS) mirror_split_count_kernel(M
     ms_count<8>(e0, e1, A.lbits, hist + blockIdx.x, A.nchunks, [&](int64_t e) { return ms_key(A.l_colidx[e], A.m) & mask; });
 }
 
-// piece of a bucket of the split that a CTA of the mid pass handles
-__device__ __forceinline__ void ms_piece(const MirrorSortArgs& A, int64_t unit, int64_t* e0, int64_t* e1) {
-    const int64_t bucket = unit / A.pieces, piece = unit - bucket * A.pieces;
-    const int64_t b0 = A.split_off[bucket * A.nchunks], len = A.split_off[(bucket + 1) * A.nchunks] - b0;
-    *e0 = b0 + len * piece / A.pieces;
-    *e1 = b0 + len * (piece + 1) / A.pieces;
+// The pieces of the mid pass (one CTA: a thread per bucket, L = 8)
+static __device__ void ms_mid_pieces(const MirrorSortArgs& A, uint32_t* scratch) {
+    __shared__ uint32_t s_first[257];
+    const int t = threadIdx.x;
+    const int64_t len = A.split_off[(int64_t)(t + 1) * A.nchunks] - A.split_off[(int64_t)t * A.nchunks];
+    uint32_t total;
+    const uint32_t ex = block_exclusive_scan<uint32_t, MS_THREADS>((uint32_t)max((len + A.mid_cap - 1) / A.mid_cap, (int64_t)1), scratch, &total);
+    s_first[t] = ex;
+    A.mid_first[t] = (int32_t)ex;
+    if (t == 0) {
+        s_first[256] = total;
+        A.mid_first[256] = (int32_t)total;
+    }
+    __syncthreads();
+    for (uint32_t u = t; u < total && u < (uint32_t)A.mid_units; u += MS_THREADS) {
+        int lo = 0, hi = 256;  // last bucket whose first piece is <= u
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (s_first[mid] <= u) lo = mid; else hi = mid;
+        }
+        A.mid_bucket[u] = (uint8_t)lo;
+    }
+    __syncthreads();
 }
-// row of the mid pass's histogram and offsets for (unit, part)
-__device__ __forceinline__ int64_t ms_mid_index(const MirrorSortArgs& A, int64_t unit, int part) {
-    return (int64_t)part * ((int64_t)A.pieces << A.lbits) + unit;
+// entries of a piece of the mid pass (none behind the last piece)
+__device__ __forceinline__ void ms_mid_piece(const MirrorSortArgs& A, int unit, int64_t* e0, int64_t* e1) {
+    *e0 = *e1 = 0;
+    if (unit >= A.mid_first[256]) return;
+    const int bucket = A.mid_bucket[unit], first = A.mid_first[bucket], count = A.mid_first[bucket + 1] - first;
+    const int64_t b0 = A.split_off[bucket * A.nchunks], len = A.split_off[(bucket + 1) * A.nchunks] - b0;
+    *e0 = b0 + len * (unit - first) / count;
+    *e1 = b0 + len * (unit - first + 1) / count;
 }
 
 static __global__ void __launch_bounds__(MS_THREADS) mirror_mid_count_kernel(MirrorSortArgs A, uint32_t* __restrict__ hist) {
     int64_t e0, e1;
-    ms_piece(A, blockIdx.x, &e0, &e1);
+    ms_mid_piece(A, blockIdx.x, &e0, &e1);
     const uint32_t mask = (1u << A.mbits) - 1u;
-    ms_count<8>(e0, e1, A.mbits, hist + ms_mid_index(A, blockIdx.x, 0), (int64_t)A.pieces << A.lbits,
-                [&](int64_t e) { return (uint32_t)A.high_a[e] & mask; });
+    ms_count<8>(e0, e1, A.mbits, hist + blockIdx.x, A.mid_units, [&](int64_t e) { return (uint32_t)A.high_a[e] & mask; });
 }
 
-// entries per column, one CTA per bucket of the place pass
+// first entry of bucket b of `place` (of the end: b = nbuckets)
+__device__ __forceinline__ int64_t ms_bucket_start(const MirrorSortArgs& A, int64_t b) {
+    if (b >= A.nbuckets) return A.n;
+    if (A.mbits == 0) return A.split_off[b * A.nchunks];
+    return A.mid_off[(b >> A.lbits) * A.mid_units + A.mid_first[b & ((1 << A.lbits) - 1)]];
+}
+
+// The pieces of the buckets that are cut, by all CTAs of the pass before `place`
+static __device__ void ms_place_pieces(const MirrorSortArgs& A) {
+    for (int64_t b = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; b < A.nbuckets; b += (int64_t)MS_THREADS * gridDim.x) {
+        const int64_t len = ms_bucket_start(A, b + 1) - ms_bucket_start(A, b);
+        int32_t first = -1;
+        if (len > A.cap) {
+            const uint32_t count = (uint32_t)((len + A.cap - 1) / A.cap);
+            first = (int32_t)atomicAdd(A.pieces, count);
+            for (uint32_t k = 0; k < count; ++k)
+                if (SPSYRK_IN_RANGE(first + k < A.max_pieces, A.err)) A.piece[first + k] = make_int2((int)b, (int)k);
+        }
+        A.first_piece[b] = first;
+    }
+}
+
+// What a CTA of the column counts and of `place` handles: a piece (the first max_pieces CTAs), or a bucket that is not cut
+struct MirrorUnit {
+    int64_t bucket, e0, e1;
+    int32_t first, number;  // of a piece: the bucket's first piece, its number in the bucket; first = -1: a whole bucket
+};
+__device__ __forceinline__ bool ms_unit(const MirrorSortArgs& A, int64_t u, MirrorUnit* x) {
+    if (u < A.max_pieces) {
+        if (u >= *A.pieces) return false;
+        const int2 p = A.piece[u];
+        const int64_t b0 = ms_bucket_start(A, p.x), len = ms_bucket_start(A, (int64_t)p.x + 1) - b0, count = (len + A.cap - 1) / A.cap;
+        *x = MirrorUnit{p.x, b0 + len * p.y / count, b0 + len * (p.y + 1) / count, (int32_t)u - p.y, p.y};
+        return true;
+    }
+    const int64_t b = u - A.max_pieces;
+    if (A.first_piece[b] >= 0) return false;
+    *x = MirrorUnit{b, ms_bucket_start(A, b), ms_bucket_start(A, b + 1), -1, 0};
+    return true;
+}
+
+// entries per column
 static __global__ void __launch_bounds__(MS_THREADS) mirror_column_count_kernel(MirrorSortArgs A, const uint16_t* __restrict__ high) {
     __shared__ uint32_t h[MS_MAX_BINS];
+    MirrorUnit unit;
+    if (!ms_unit(A, blockIdx.x, &unit)) return;
     const int nb = 1 << A.hbits;
     for (int d = threadIdx.x; d < nb; d += MS_THREADS) h[d] = 0;
     __syncthreads();
-    const int64_t bucket = blockIdx.x;
-    const int64_t b0 = A.place_off[bucket * A.place_stride], b1 = A.place_off[(bucket + 1) * A.place_stride];
+    const int64_t b0 = unit.e0, b1 = unit.e1;
     // eight parts per load where the array is 16-byte aligned
     const int64_t a0 = min((b0 + 7) & ~int64_t(7), b1), a1 = max(a0, b1 & ~int64_t(7));
     auto one = [&](uint32_t x) { atomicAdd(&h[x & (nb - 1)], 1u); };
@@ -164,10 +245,14 @@ static __global__ void __launch_bounds__(MS_THREADS) mirror_column_count_kernel(
     for (int64_t e = a1 + threadIdx.x; e < b1; e += MS_THREADS) one(high[e]);
     __syncthreads();
     const int low = A.lbits + A.mbits;
-    const int64_t col0 = bucket;  // column of bin 0
     for (int d = threadIdx.x; d < nb; d += MS_THREADS) {
-        const int64_t j = col0 + ((int64_t)d << low);
-        if (j < A.m) A.cnt[j] = h[d];
+        const int64_t j = unit.bucket + ((int64_t)d << low);
+        if (unit.first >= 0) {
+            A.piece_cnt[((int64_t)(unit.first + unit.number) << A.hbits) + d] = h[d];
+            if (j < A.m && h[d]) atomicAdd(&A.cnt[j], h[d]);
+        } else if (j < A.m) {
+            A.cnt[j] = h[d];
+        }
     }
 }
 
@@ -196,7 +281,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     using SM = MirrorSplitSmem<VB>;
     constexpr int ITEMS = T::ITEMS, TILE = SM::TILE, CHUNK = 32 * ITEMS;
     extern __shared__ __align__(16) unsigned char ms_smem[];
-    __shared__ uint32_t scratch[32];
+    __shared__ uint32_t scratch[33];
     __shared__ uint32_t s_bits[MS_WARPS][ITEMS];  // a bit where a row starts
     const int nb = 1 << A.lbits;
     typename T::Rec* s_rec = reinterpret_cast<typename T::Rec*>(ms_smem);       // [TILE] the tile in bucket order
@@ -209,6 +294,8 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     uint32_t* rows_of_warp = reinterpret_cast<uint32_t*>(ms_smem) + warp * (CHUNK + 1);
     static_assert((size_t)MS_WARPS * (CHUNK + 1) * 4 <= (size_t)TILE * sizeof(typename T::Rec), "rows fit the tile's space");
     uint32_t* bits = s_bits[warp];
+    if (A.mbits == 0) ms_place_pieces(A);
+    else if (blockIdx.x == 0) ms_mid_pieces(A, scratch);
     const int64_t e0 = (int64_t)blockIdx.x * A.chunk, e1 = min(e0 + A.chunk, A.n);
     const VB* __restrict__ vals = static_cast<const VB*>(A.l_vals);
     int64_t gbase[4];
@@ -316,18 +403,19 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     constexpr bool KEYS = sizeof(VB) == 4;
     constexpr int ITEMS = T::ITEMS, TILE = mirror_tile<VB>();
     extern __shared__ __align__(16) unsigned char ms_smem[];
-    __shared__ uint32_t scratch[32];
+    __shared__ uint32_t scratch[33];
     const int nb = 1 << A.mbits;
     typename T::Rec* s_rec = reinterpret_cast<typename T::Rec*>(ms_smem);       // [TILE]
     int64_t* s_goff = reinterpret_cast<int64_t*>(s_rec + TILE);                 // [nb]
     uint16_t* count = reinterpret_cast<uint16_t*>(s_goff + nb);                 // [WARPS][nb]
     uint16_t* s_rest = count + MS_WARPS * nb;                                   // [TILE] (4-byte values)
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    ms_place_pieces(A);
     int64_t e0, e1;
-    ms_piece(A, blockIdx.x, &e0, &e1);
+    ms_mid_piece(A, blockIdx.x, &e0, &e1);
     int64_t gbase[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) gbase[k] = 4 * tid + k < nb ? A.mid_off[ms_mid_index(A, blockIdx.x, 4 * tid + k)] : 0;
+    for (int k = 0; k < 4; ++k) gbase[k] = 4 * tid + k < nb ? A.mid_off[(int64_t)(4 * tid + k) * A.mid_units + blockIdx.x] : 0;
     bucket_clear_counts<MS_THREADS>(count, nb);
     for (int64_t base = e0; base < e1; base += TILE) {
         const int64_t end = min(base + TILE, e1);
@@ -388,7 +476,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     using T = MirrorSortTraits<VB>;
     constexpr int ITEMS = T::ITEMS, TILE = mirror_tile<VB>();
     extern __shared__ __align__(16) unsigned char ms_smem[];
-    __shared__ uint32_t scratch[32];
+    __shared__ uint32_t scratch[33];
     const int nb = 1 << A.hbits, low = A.lbits + A.mbits;
     VB* s_val = reinterpret_cast<VB*>(ms_smem);                          // [TILE] the tile in column order
     int64_t* s_goff = reinterpret_cast<int64_t*>(s_val + TILE);          // [nb]
@@ -396,14 +484,21 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     uint16_t* count = reinterpret_cast<uint16_t*>(s_row + TILE);         // [WARPS][nb]
     uint16_t* s_bin = count + MS_WARPS * nb;                             // [TILE]
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    const int64_t bucket = blockIdx.x;
-    const int64_t b0 = A.place_off[bucket * A.place_stride], b1 = A.place_off[(bucket + 1) * A.place_stride];
-    const int64_t col0 = bucket;  // column of bin 0
+    MirrorUnit unit;
+    if (!ms_unit(A, blockIdx.x, &unit)) return;
+    const int64_t b0 = unit.e0, b1 = unit.e1, col0 = unit.bucket;  // column of bin 0
     int64_t gbase[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int64_t j = col0 + ((int64_t)(4 * tid + k) << low);
         gbase[k] = 4 * tid + k < nb && j < A.m ? A.fstart[j] : 0;
+    }
+    if (4 * tid < nb) {  // behind what the pieces before hold
+#pragma unroll 4
+        for (int q = 0; q < unit.number; ++q) {
+            const uint4 c = *reinterpret_cast<const uint4*>(A.piece_cnt + ((int64_t)(unit.first + q) << A.hbits) + 4 * tid);
+            gbase[0] += c.x; gbase[1] += c.y; gbase[2] += c.z; gbase[3] += c.w;
+        }
     }
     const typename T::Rec* __restrict__ recs = static_cast<const typename T::Rec*>(A.rec_b);
     VB* __restrict__ f_vals = static_cast<VB*>(A.f_vals);
