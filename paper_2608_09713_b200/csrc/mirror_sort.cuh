@@ -259,6 +259,11 @@ static __global__ void __launch_bounds__(MS_THREADS) mirror_column_count_kernel(
 // Consecutive entries of a tile that one warp owns: whole steps of 32, the same number for every warp
 __device__ __forceinline__ int ms_warp_span(int64_t tile_n) { return (int)((tile_n + MS_THREADS - 1) / MS_THREADS) * 32; }
 
+// row of the first entry of step s (of a step behind the last: the last row)
+__device__ __forceinline__ int64_t ms_step_row(const MirrorSortArgs& A, int64_t s) {
+    return s * 32 < A.n ? (int64_t)min((uint32_t)A.step_row[s], (uint32_t)(A.m - 1)) : A.m - 1;
+}
+
 // Shared memory of the three passes: the tile (records, with the part or rest of the column beside them), offsets, counters
 template <typename VB>
 struct MirrorSplitSmem {
@@ -321,12 +326,27 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
         __syncthreads();  // the last tile has left shared memory, the counters are clear
         if (wn > 0) {
             // rows of the warp's entries: a bit per row start, the ids of the rows in their order
-            if (lane < ITEMS) bits[lane] = 0;
-            const int64_t r0 = min((uint32_t)A.step_row[w0 >> 5], (uint32_t)(A.m - 1));
+            const int64_t r0 = ms_step_row(A, w0 >> 5), r1 = ms_step_row(A, ((w0 + wn - 1) >> 5) + 1);  // the first row, one not before the last
+            const bool walk = r1 - r0 <= 2 * CHUNK;
+            if (lane < ITEMS) bits[lane] = walk ? 0u : 0xffffffffu;
             if (lane == 0) rows_of_warp[0] = (uint32_t)r0;
             __syncwarp();
+            if (!walk) {
+                // Most rows are empty: every entry's row is searched for between the rows of two steps and entered as if it
+                // began there.  (Walking along 1e7 rows, 32 at a time, took 2.4 ms for 4000 entries.)
+#pragma unroll 1
+                for (int i = lane; i < wn; i += 32) {
+                    const int64_t e = w0 + i;
+                    int64_t lo = ms_step_row(A, e >> 5), hi = ms_step_row(A, (e >> 5) + 1);
+                    while (lo < hi) {  // the last row that starts at or before the entry
+                        const int64_t mid = (lo + hi + 1) >> 1;
+                        if (A.l_rowptr[mid] <= e) lo = mid; else hi = mid - 1;
+                    }
+                    rows_of_warp[i + 1] = (uint32_t)lo;
+                }
+            }
             int found = 1;
-            for (int64_t r = r0 + 1 + lane;; r += 32) {
+            for (int64_t r = r0 + 1 + lane; walk; r += 32) {
                 const int64_t s = r < A.m ? A.l_rowptr[r] : INT64_MAX, x = r < A.m ? A.l_rowptr[r + 1] : INT64_MAX;
                 const bool on = s > w0 && s < w0 + wn && x > s;
                 const unsigned votes = __ballot_sync(FULL_MASK, on);

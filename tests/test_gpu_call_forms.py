@@ -231,3 +231,26 @@ def test_mirror_wherever_the_entries_lie(B, name, m, k, dtype):
     """Buckets that are cut into pieces and buckets that are not, two passes and three, radix passes for few entries and for
     more than 2^24 rows, rows that are searched for."""
     check_mirror(B, m, lower_triangle(m, *pattern(name, m, k), dtype))
+
+
+def test_mirror_takes_about_the_same_time_wherever_the_entries_lie(B):
+    """2^18 rows: entries in one column, in every 512th column, or two entries in all, against entries all over."""
+    m = 1 << 18
+
+    def microseconds(c):
+        B.spsyrk_mirror(m, *c)
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            B.spsyrk_mirror(m, *c)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3)
+        return best
+
+    spread = microseconds(lower_triangle(m, *pattern("spread", m, 1 << 22), torch.float32))
+    ends = torch.tensor([3, m - 1], device="cuda")
+    for c in (lower_triangle(m, *pattern("one column", m, 0), torch.float32), lower_triangle(m, *pattern("every 512th column", m, 1 << 22), torch.float32),
+              lower_triangle(m, ends, ends, torch.float32)):
+        assert microseconds(c) < 3 * spread
