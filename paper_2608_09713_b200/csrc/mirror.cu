@@ -8,8 +8,8 @@
 //             nnz(F) = 2 nnz(C_L) - #diagonals.
 //   sort    : 4-byte values of up to 2^24 rows and small matrices go to buckets of columns and from there to their
 //             places (mirror_sort.cuh); 8-byte values of more than 65536 rows go through radix passes of 16-byte
-//             records, the last of which writes F (mirror_rec.cuh); 4-byte values of more rows through radix passes
-//             of separate arrays (radix.cuh);
+//             records, the last of which writes F (mirror_rec.cuh); 4-byte values of more rows, or of few entries for
+//             their rows, through radix passes of separate arrays (radix.cuh);
 //   rows    : row lengths of F, scan -> f_rowptr (in the bucket sort before the last pass), lower parts copied.
 #include <algorithm>
 #include <mutex>
@@ -30,11 +30,6 @@ constexpr int MIRROR_RADIX_BITS = 8;  // digits of the record passes
 // the launches: it is used where both take two passes.  (Product and mirror of 4096 rows: 465 -> 415 us.)
 constexpr int64_t MIRROR_BUCKET_ROWS_8 = 65536;
 bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCKET_ROWS_8; }
-// 4-byte values: what the first pass of the bucket sort leaves of a column must fit two bytes.  (Taking the columns of wider
-// matrices in rounds of 2^24 reads all entries once per round: 2^26 rows and 2.7e8 entries 25.5 ms, 2^27 rows and
-// 4.0e8 entries 59.1 ms, against 16.6 and 26.9 ms by four radix passes.)
-bool mirror_by_radix(int64_t m, size_t sv) { return sv == 4 && m > (int64_t(1) << MS_COLUMN_BITS); }
-
 struct MirrorWs {
     int64_t* partials;
     uint32_t* err;       // [0] error word, [1] number of diagonal entries, [2] finished CTAs
@@ -117,6 +112,19 @@ MirrorSplit mirror_split_for(int64_t m, int64_t nnz_l, size_t sv) {
     return s;
 }
 
+// 4-byte values: what the first pass of the bucket sort leaves of a column must fit two bytes.  (Taking the columns of wider
+// matrices in rounds of 2^24 reads all entries once per round: 2^26 rows and 2.7e8 entries 25.5 ms, 2^27 rows and
+// 4.0e8 entries 59.1 ms, against 16.6 and 26.9 ms by four radix passes.)  Three passes of the bucket sort need entries for their
+// buckets, 2^14 to 2^16 of them; with few per bucket the radix passes are faster, for whose every launch the entries count.
+// Buckets against radix passes: 2^22 rows, 92 entries per bucket 1134 us to 494; 640 per bucket 1706 to 1293; 2176 per bucket
+// 3624 to 4094.  2^20 rows, 1088 per bucket 1143 to 1111.  2^24 rows, 1280 per bucket 5221 to 5564.
+constexpr int64_t MIRROR_BUCKET_FILL = 1024;
+bool mirror_by_radix(int64_t m, int64_t nnz_l, size_t sv) {
+    if (sv == 8) return false;
+    const MirrorSplit s = mirror_split_for(m, nnz_l, sv);
+    return m > (int64_t(1) << MS_COLUMN_BITS) || (s.mbits > 0 && nnz_l < MIRROR_BUCKET_FILL * s.nbuckets());
+}
+
 int64_t mirror_tail_records(int64_t m, int64_t nnz_l) { return (std::min(m, nnz_l) + 1) / 2; }
 
 // Scratch inside the output.  Until the last pass writes it, F's memory is free.  Three passes need two record buffers
@@ -154,7 +162,7 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
         t.tile_rows = (int32_t*)take(2 * std::max<int64_t>(mirror_tiles(nnz_l), 1) * 4);
         t.hist = (uint32_t*)take(hist_n * 4);
         t.offsets = (int64_t*)take((hist_n + 1) * 8);
-    } else if (mirror_by_radix(m, sv)) {
+    } else if (mirror_by_radix(m, nnz_l, sv)) {
         // F's column and value arrays hold 4 (2 nnz_l - D) >= 4 nnz_l bytes each: the columns and values of one set.  Passes write
         // A, B, A, ...: the last one reads B when their number is odd.
         const int npass = radix_passes((uint64_t)m);  // columns, and m for the diagonal entries
@@ -421,7 +429,7 @@ __global__ void mirror_rowlen_kernel(const int64_t* __restrict__ l_rowptr, const
     rowtot[r] = (uint32_t)(l_rowptr[r + 1] - l_rowptr[r]) + (e > s ? (uint32_t)(e - s) : 0u);
 }
 
-// 4-byte values of more than 2^24 rows
+// 4-byte values of more than 2^24 rows, or of few entries per bucket
 spsyrk_status_t mirror_fill_radix(const MirrorWs& ws, int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx, const void* l_vals,
                                   int64_t* f_rowptr, int32_t* f_colidx, void* f_vals, cudaStream_t st) {
     if (nnz_l == 0) {
@@ -632,7 +640,7 @@ extern "C" spsyrk_status_t spsyrk_mirror(int64_t m, int64_t nnz_l, spsyrk_dtype_
             if (mirror_by_records(m, sv)) return mirror_fill_rec(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
             return mirror_fill<uint64_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
         default:
-            if (mirror_by_radix(m, sv)) return mirror_fill_radix(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
+            if (mirror_by_radix(m, nnz_l, sv)) return mirror_fill_radix(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
             return mirror_fill<uint32_t>(w, m, nnz_l, d_l_rowptr, d_l_colidx, d_l_vals, d_f_rowptr, d_f_colidx, d_f_vals, st);
     }
 }

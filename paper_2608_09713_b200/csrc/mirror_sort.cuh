@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
 }
 
 // ---------------------------------------------------------------------------------------------
-// Matrices of more than 2^24 rows: radix passes of (column, row, value) arrays (radix.cuh)
+// Matrices of more than 2^24 rows, or of few entries for their rows: radix passes of (column, row, value) arrays (radix.cuh)
 // ---------------------------------------------------------------------------------------------
 // G lanes per row: the (column, row) pair of every entry; the diagonal entry, and one above the diagonal (rows that are not
 // ascending can hide one from the size step), sorts past the end as column m and takes no part in the reflection
