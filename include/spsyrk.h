@@ -214,8 +214,9 @@ spsyrk_status_t spsyrk_onepass_compact(spsyrk_plan_t plan, const int64_t *d_c_ro
  *      ascending) is left out of the reflection; it never indexes outside the arrays.
  *      Until this step's work on the stream has completed, d_f_colidx and d_f_vals (the sizes step 2
  *      gave: nnz_full entries each) also serve as scratch of the sort, which is why the workspace is about
- *      1.3 (4-byte values) to 1.5 (8-byte values) times the bytes of C_L and not 3 times; both arrays must
- *      be 16-byte aligned and must not overlap each other, the workspace or C_L (INVALID_ARG if misaligned).
+ *      1.3 to 2.6 (4-byte values, the more the fewer entries a row has) and 1.5 (8-byte values) times the bytes
+ *      of C_L and not 3 times.  They must not overlap each other, the workspace or C_L, and with 8-byte values
+ *      both must be 16-byte aligned (INVALID_ARG if not).
  * nnz_l = d_l_rowptr[m].  Errors: INVALID_ARG, WORKSPACE, BAD_CSR (an entry above the diagonal), CUDA.
  */
 spsyrk_status_t spsyrk_mirror(int64_t m, int64_t nnz_l, spsyrk_dtype_t dtype,

@@ -351,8 +351,10 @@ void mirror_mark(int i, cudaStream_t st) {
 template <typename VB>
 spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx,
                             const void* l_vals, int64_t* f_rowptr, int32_t* f_colidx, void* f_vals, cudaStream_t st) {
-    // F's arrays hold records and rests during the sort: both must take 16-byte accesses
-    if (nnz_l > 0 && ((reinterpret_cast<uintptr_t>(f_vals) | reinterpret_cast<uintptr_t>(f_colidx)) & 15u)) return SPSYRK_ERR_INVALID_ARG;
+    // F's arrays hold records and rests during the sort.  8-byte values: both must take 16-byte accesses.  4-byte values: the rests
+    // are moved one by one and the records of 8 bytes begin at the first multiple of 8, one of them fewer.
+    if (sizeof(VB) == 8 && nnz_l > 0 && ((reinterpret_cast<uintptr_t>(f_vals) | reinterpret_cast<uintptr_t>(f_colidx)) & 15u)) return SPSYRK_ERR_INVALID_ARG;
+    const int64_t skipped = (reinterpret_cast<uintptr_t>(f_vals) & 7u) ? 1 : 0;
     if (m == 0 || nnz_l == 0) {
         SPSYRK_CUDA_TRY(cudaMemsetAsync(f_rowptr, 0, (size_t)(m + 1) * sizeof(int64_t), st));
         return SPSYRK_OK;
@@ -368,9 +370,9 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     a.nbuckets = sp.nbuckets(); a.cap = sp.cap; a.max_pieces = (uint32_t)sp.max_pieces; a.pieces = w.pieces; a.first_piece = w.first_piece;
     a.piece = w.piece; a.piece_cnt = w.piece_cnt;
     a.split_off = w.offsets; a.mid_off = w.mid_off;
-    a.rec_a = three ? f_vals : w.rec;
+    a.rec_a = three ? static_cast<void*>(static_cast<char*>(f_vals) + 4 * skipped) : w.rec;
     a.rec_a_tail = w.rec_tail;
-    a.a_split = three ? nnz_l - mirror_tail_records(m, nnz_l) : nnz_l;
+    a.a_split = three ? nnz_l - mirror_tail_records(m, nnz_l) - skipped : nnz_l;  // (the tail has room for one more)
     a.rec_b = w.rec;
     // the rests: the last pass reads them only for 4-byte values, and then not from F's memory
     uint16_t* const last_high = sizeof(VB) == 4 ? w.high : f_high;

@@ -254,3 +254,29 @@ def test_mirror_takes_about_the_same_time_wherever_the_entries_lie(B):
     for c in (lower_triangle(m, *pattern("one column", m, 0), torch.float32), lower_triangle(m, *pattern("every 512th column", m, 1 << 22), torch.float32),
               lower_triangle(m, ends, ends, torch.float32)):
         assert microseconds(c) < 3 * spread
+
+
+@pytest.mark.parametrize("m,k", [(5000, 50_000), ((1 << 19) + 1, 20_000_000), ((1 << 24) + 1, 1_000_000)])
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_mirror_of_4_byte_values_into_unaligned_arrays(B, m, k, shift):
+    """F's arrays may begin at any multiple of four bytes (8-byte values: multiples of sixteen)."""
+    import ctypes
+    c = lower_triangle(m, *pattern("spread", m, k), torch.float32)
+    rp, ci, cv = c
+    nnz_f = 2 * ci.numel() - m
+    lib, code = B._lib, B._DTYPE_CODE[torch.float32]
+    size = ctypes.c_size_t(0)
+    B._check(lib.spsyrk_mirror(m, ci.numel(), code, None, None, None, None, None, None, None, None, ctypes.byref(size), None), "size")
+    ws = torch.empty(size.value, dtype=torch.uint8, device="cuda")
+    f_rp = torch.empty(m + 1, dtype=torch.int64, device="cuda")
+    f_ci = torch.full((nnz_f + 2 * shift,), -9, dtype=torch.int32, device="cuda")
+    f_cv = torch.full((nnz_f + 2 * shift,), -9.0, device="cuda")
+    nnz = ctypes.c_int64(0)
+    args = (m, ci.numel(), code, B._p(rp), B._p(ci), B._p(cv), B._p(f_rp))
+    B._check(lib.spsyrk_mirror(*args, None, None, ctypes.byref(nnz), B._p(ws), ctypes.byref(size), B._stream(None)), "sizes")
+    assert nnz.value == nnz_f
+    ci_out, cv_out = f_ci[shift : shift + nnz_f], f_cv[shift : shift + nnz_f]
+    B._check(lib.spsyrk_mirror(*args, B._p(ci_out), B._p(cv_out), ctypes.byref(nnz), B._p(ws), ctypes.byref(size), B._stream(None)), "fill")
+    check_mirror(B, m, c, (f_rp, ci_out, cv_out))
+    for t in (f_ci, f_cv):
+        assert bool((t[:shift] == -9).all()) and bool((t[shift + nnz_f :] == -9).all())
