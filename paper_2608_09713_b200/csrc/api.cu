@@ -1050,7 +1050,13 @@ spsyrk_status_t spsyrk_plan(spsyrk_plan_t* plan, int64_t m, int64_t n, int64_t n
     carve(pl, up, d_workspace, m, n, nnz, sv, full);
     pl->upper = up;  // (the copy into the upper view happened with a null link)
 
-    auto fail = [&](spsyrk_status_t s) { pl->host.release(); delete up; delete pl; return s; };
+    auto fail = [&](spsyrk_status_t s) {
+        if (s == SPSYRK_ERR_CUDA) cudaStreamSynchronize(st);  // a kernel under way may still write into the host block
+        pl->host.release();
+        delete up;
+        delete pl;
+        return s;
+    };
 #define PLAN_TRY(expr) do { if ((expr) != cudaSuccess) return fail(SPSYRK_ERR_CUDA); } while (0)
     PLAN_TRY(pl->host.acquire());
     PLAN_TRY(cudaMemsetAsync(pl->zero_all, 0, pl->zero_all_bytes, st));
