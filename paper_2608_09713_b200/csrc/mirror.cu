@@ -199,7 +199,7 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
         t.piece_cnt = (uint32_t*)take((sp.max_pieces << sp.hbits) * 4);
         t.step_row = (int32_t*)take((ne + 31) / 32 * 4);
         t.rec = take(ne * 2 * sv);
-        t.rec_tail = take(sp.mbits ? (mirror_tail_records(m, nnz_l) + 1) * 2 * sv : 0);
+        t.rec_tail = take(sp.mbits ? (mirror_tail_records(m, nnz_l) + 1) * sizeof(uint2) : 0);
         t.high = (uint16_t*)take(sv == 8 ? 0 : ne * 2);
     }
     if (w) *w = t;
@@ -360,7 +360,7 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         return SPSYRK_OK;
     }
     const MirrorSplit sp = mirror_split_for(m, nnz_l, sizeof(VB));
-    const bool three = sp.mbits > 0;
+    const bool three = sp.mbits > 0;  // (4-byte values only)
     const int g = group_width(nnz_l, m);
     uint16_t* const f_high = reinterpret_cast<uint16_t*>(f_colidx);
     MirrorSortArgs a{};
@@ -377,7 +377,7 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     // the rests: the last pass reads them only for 4-byte values, and then not from F's memory
     uint16_t* const last_high = sizeof(VB) == 4 ? w.high : f_high;
     a.high_b = last_high;
-    a.high_a = !three ? last_high : sizeof(VB) == 4 ? f_high : f_high + nnz_l;  // (only the last pass's rests are read 16 bytes at a time)
+    a.high_a = three ? f_high : last_high;
     a.cnt = w.cnt; a.fstart = w.fstart; a.f_colidx = f_colidx; a.f_vals = f_vals; a.err = w.err;
     const size_t split_smem = MirrorSplitSmem<VB>::bytes(1 << sp.lbits), place_smem = MirrorPlaceSmem<VB>::bytes(1 << sp.hbits);
     SPSYRK_CUDA_TRY(allow_shared_memory<mirror_split_kernel<VB>>());
@@ -392,13 +392,13 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     note_launches(3);
     mirror_mark(1, st);
     int pass = 2;
-    if constexpr (sizeof(VB) == 4) if (three) {
+    if (three) {
         const unsigned units = (unsigned)sp.mid_units;
         mirror_mid_count_kernel<<<units, MS_THREADS, 0, st>>>(a, w.hist);
         SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.partials, w.err, st));
-        const size_t mid_smem = MirrorMidSmem<VB>::bytes(1 << sp.mbits);
-        SPSYRK_CUDA_TRY(allow_shared_memory<mirror_mid_kernel<VB>>());
-        mirror_mid_kernel<VB><<<units, MS_THREADS, mid_smem, st>>>(a);
+        const size_t mid_smem = MirrorMidSmem::bytes(1 << sp.mbits);
+        SPSYRK_CUDA_TRY(allow_shared_memory<mirror_mid_kernel>());
+        mirror_mid_kernel<<<units, MS_THREADS, mid_smem, st>>>(a);
         note_launches(2);
         mirror_mark(pass++, st);
     }
@@ -523,7 +523,6 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
     constexpr int NB = 1 << BITS;
     const uint64_t* lv = static_cast<const uint64_t*>(l_vals);
     uint64_t* fv = static_cast<uint64_t*>(f_vals);
-    const int g = group_width(nnz_l, m);
     // F's arrays hold records and digit bytes during the sort: both must take 16-byte accesses
     if (nnz_l > 0 && ((reinterpret_cast<uintptr_t>(f_vals) | reinterpret_cast<uintptr_t>(f_colidx)) & 15u)) return SPSYRK_ERR_INVALID_ARG;
     if (m > 0) {

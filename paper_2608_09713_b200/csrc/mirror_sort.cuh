@@ -409,26 +409,21 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     }
 }
 
-template <typename VB>
+// (4-byte values: 8-byte ones have at most 65536 rows here, two passes)
 struct MirrorMidSmem {
-    static constexpr int TILE = mirror_tile<VB>();
-    static size_t bytes(int nb) {
-        return (size_t)TILE * sizeof(typename MirrorSortTraits<VB>::Rec) + (sizeof(VB) == 4 ? (size_t)TILE * 2 : 0) + (size_t)nb * 8 + (size_t)MS_WARPS * nb * 2;
-    }
+    static size_t bytes(int nb) { return (size_t)mirror_tile<uint32_t>() * (sizeof(uint2) + 2) + (size_t)nb * 8 + (size_t)MS_WARPS * nb * 2; }
 };
 
-template <typename VB>
-__global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mirror_mid_kernel(MirrorSortArgs A) {
-    using T = MirrorSortTraits<VB>;
-    constexpr bool KEYS = sizeof(VB) == 4;
-    constexpr int ITEMS = T::ITEMS, TILE = mirror_tile<VB>();
+static __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<uint32_t>::MIN_CTAS) mirror_mid_kernel(MirrorSortArgs A) {
+    using T = MirrorSortTraits<uint32_t>;
+    constexpr int ITEMS = T::ITEMS, TILE = mirror_tile<uint32_t>();
     extern __shared__ __align__(16) unsigned char ms_smem[];
     __shared__ uint32_t scratch[33];
     const int nb = 1 << A.mbits;
     typename T::Rec* s_rec = reinterpret_cast<typename T::Rec*>(ms_smem);       // [TILE]
     int64_t* s_goff = reinterpret_cast<int64_t*>(s_rec + TILE);                 // [nb]
     uint16_t* count = reinterpret_cast<uint16_t*>(s_goff + nb);                 // [WARPS][nb]
-    uint16_t* s_rest = count + MS_WARPS * nb;                                   // [TILE] (4-byte values)
+    uint16_t* s_rest = count + MS_WARPS * nb;                                   // [TILE]
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     ms_place_pieces(A);
     int64_t e0, e1;
@@ -446,16 +441,16 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
         typename T::Rec rec[ITEMS];
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            if constexpr (KEYS) rest[i] = 0;
+            rest[i] = 0;
             rec[i] = typename T::Rec{};
             if (i * 32 + lane < wn) {
                 const int64_t e = w0 + i * 32 + lane;
-                rec[i] = *ms_rec_at<VB>(A.rec_a, A.rec_a_tail, A.a_split, e);
-                if constexpr (KEYS) rest[i] = A.high_a[e];
+                rec[i] = *ms_rec_at<uint32_t>(A.rec_a, A.rec_a_tail, A.a_split, e);
+                rest[i] = A.high_a[e];
                 valid |= 1u << i;
             }
         }
-        const auto bin = [&](int i) { return (KEYS ? rest[i] : rec[i].x >> A.lbits) & (uint32_t)(nb - 1); };
+        const auto bin = [&](int i) { return rest[i] & (uint32_t)(nb - 1); };
         __syncthreads();  // the last tile has left shared memory, the counters are clear
         uint32_t rk[ITEMS];
         uint16_t* mycount = count + warp * nb;
@@ -468,7 +463,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
                 const uint32_t q = mycount[bin(i)] + rk[i];
                 if (!SPSYRK_IN_RANGE(q < (uint32_t)TILE, A.err)) continue;
                 s_rec[q] = rec[i];
-                if constexpr (KEYS) s_rest[q] = (uint16_t)rest[i];
+                s_rest[q] = (uint16_t)rest[i];
             }
         }
         __syncthreads();
@@ -476,8 +471,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
 #pragma unroll 4
         for (int q = tid; q < total; q += MS_THREADS) {
             const typename T::Rec r = s_rec[q];
-            uint32_t k;
-            if constexpr (KEYS) k = s_rest[q]; else k = r.x >> A.lbits;
+            const uint32_t k = s_rest[q];
             const int64_t dest = s_goff[k & (nb - 1)] + q;
             if (!SPSYRK_IN_RANGE(dest >= 0 && dest < A.n, A.err)) continue;
             static_cast<typename T::Rec*>(A.rec_b)[dest] = r;
