@@ -219,9 +219,8 @@ __device__ __forceinline__ bool ms_unit(const MirrorSortArgs& A, int64_t u, Mirr
         return true;
     }
     const int64_t b = u - A.max_pieces;
-    if (A.first_piece[b] >= 0) return false;
     *x = MirrorUnit{b, ms_bucket_start(A, b), ms_bucket_start(A, b + 1), -1, 0};
-    return true;
+    return A.first_piece[b] < 0;
 }
 
 // entries per column
