@@ -103,6 +103,19 @@ def test_nothing_of_a_plan_is_under_way_when_it_returns(B):
         assert np.array_equal(cv.cpu().numpy().astype(np.float64), ref.vals)
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+def test_plan_of_no_rows_then_all(B, mode):
+    """The binary analysis belongs to the plan, not to its row range: a plan of no rows, of one row, then of all."""
+    a = random_csr(700, 5000, 60, np.int32, 9, ones=True)
+    a.colidx[a.rowptr[:-1]] = 0  # a column that every row stores: heavy, and every row of the lower triangle is dense
+    d = dev(a)
+    for r0, r1 in ((0, 0), (350, 351), (700, 700)):
+        plan = B.spsyrk_plan(a.m, a.n, *d, mode=mode, row_begin=r0, row_end=r1)
+        run_and_compare(B, a, mode, r0, r1, plan=plan)
+        B.spsyrk_plan_set_rows(plan, 0, a.m)
+        run_and_compare(B, a, mode, plan=plan)
+
+
 def heavy_matrix(m, dtype, seed):
     """Rows with more than 32 nonzeros over columns of about 40 entries, in every part of the range, among rows with one
     nonzero; a few rows that outgrow the smaller slot counts."""
