@@ -149,8 +149,9 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t *d_c_rowptr, int64_t
  * of rows i and j; Algorithm 2 line 2 restricts it to the lower triangle).  Writes
  * d_c_colidx[nnz] (global column ids, ascending inside a row) and d_c_vals[nnz] of the plan's
  * dtype (F32 input is accumulated in double and rounded once; I32 wraps modulo 2^32).
- * d_c_rowptr must be the array spsyrk_symbolic wrote for this plan.  Asynchronous.
- * Errors: INVALID_ARG, SEQUENCE, CUDA.
+ * d_c_rowptr must be the array spsyrk_symbolic wrote for this plan.  Asynchronous.  Passes of one plan into
+ * different arrays (these and spsyrk_numeric_rows) may be under way on several streams at a time; the host calls
+ * on one plan must not overlap.  Errors: INVALID_ARG, SEQUENCE, CUDA.
  */
 spsyrk_status_t spsyrk_numeric(spsyrk_plan_t plan, const int64_t *d_c_rowptr,
                                int32_t *d_c_colidx, void *d_c_vals, void *cuda_stream);

@@ -309,7 +309,7 @@ def spsyrk_mirror_enable_timing(on: bool = True):
 
 
 def spsyrk_mirror_timings():
-    """Device milliseconds of the sorting passes of the last spsyrk_mirror fill on 8-byte values."""
+    """Device milliseconds of the sorting passes of the last spsyrk_mirror fill."""
     n = _int(0)
     ms = (ctypes.c_float * 4)()
     _check(_lib.spsyrk_mirror_timings(ctypes.byref(n), ms), "spsyrk_mirror_timings")

@@ -218,7 +218,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     const size_t zero_words = cz.off;
     // The two buffer sets of the radix sort (key, row, position, value per nonzero) are reused: the set that
     // the last pass does not read receives the column lists that pass writes (row ids and records), and the
-    // set it does read holds, once the sort is over, the block descriptors and the heavy-row accumulator slices.
+    // set it does read holds, once the sort is over, the block descriptors.
     const size_t set_bytes = (size_t)nnz * (12 + sv) + 4 * ALIGN;
     auto set_a = c.take<char>(set_bytes);
     auto set_b = c.take<char>(set_bytes);

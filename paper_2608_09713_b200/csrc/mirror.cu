@@ -27,7 +27,9 @@ constexpr int MIRROR_RADIX_BITS = 8;  // digits of the record passes
 
 // 8-byte values: the record passes move 16-byte records in runs that the cut into buckets does not reach (three
 // passes over 5.4e8 records: 14.7 ms and 1.6 for histograms and scans, against 15.9 and 1.1), but the bucket sort takes half
-// the launches: it is used where both take two passes.  (Product and mirror of 4096 rows: 465 -> 415 us.)
+// the launches: it is used where both take two passes.  (Product and mirror of 4096 rows: 465 -> 415 us.  65537 rows and 2.0e6
+// entries: 250 us by records, 170 by buckets; 262144 rows and 8.1e6 entries 503 to 432, 2.6e8 entries 8.61 to 8.30 ms: where
+// buckets take two passes and records three, up to 2^18 rows, the line could lie higher.)
 constexpr int64_t MIRROR_BUCKET_ROWS_8 = 65536;
 bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCKET_ROWS_8; }
 struct MirrorWs {

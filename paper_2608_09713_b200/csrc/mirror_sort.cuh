@@ -25,8 +25,8 @@
 // A pass is bound by the load/store pipe and by what a CTA waits for at its barriers, 75 to 100 cycles per 32 entries and
 // SM.  128 registers (two CTAs of 256 threads) hold a tile without spills; three to five CTAs with fewer registers
 // took 1.2 to 2 times as long.  6.4e8 single-precision entries with 18-bit columns (the large power-law workload):
-// split 6.8 ms, place 6.2, counts and scans 1.0, against 15.0 for three passes of 8-bit digits, 2.0 for the
-// (key, row) expansion that `split` does without and 2.8 for histograms and scans before.
+// the whole mirror 15.3 ms; three passes of 8-bit digits took 15.0, the (key, row) expansion that `split` does without 2.0 and
+// their histograms and scans 2.8, beside the lower parts.
 #pragma once
 #include "bucket.cuh"
 

@@ -16,7 +16,7 @@
 // Before, every heavy row went through a bitmap, 32-bit ranks and one size of slots (512 threads up to 32768 products, 1024
 // above), rows with more entries than slots into global slices with L2 atomics, dense rows of binary matrices
 // through a 200 KB tile with one CTA per SM.  Large power-law workload (96 000 heavy rows, 1.46e9 products, single precision):
-// 15.3 ms before, 12.2 now; binary Zipf workload of 50000 rows (1.25e9 counts and similarities): 10.8 ms before, dense8
+// 15.3 ms before, 12.1 now; binary Zipf workload of 50000 rows (1.25e9 counts and similarities): 10.8 ms before, dense8
 // 4.4 ms = 3.4 TB/s of output.
 #pragma once
 #include "transpose.cuh"
@@ -78,9 +78,11 @@ static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDe
         } else if (R.binary && dense && deg <= 255 && U <= R.dense8) {
             route = ROUTE_DENSE8;
         } else if ((R.binary && dense) || (U <= R.chunk && w >= (int64_t)(U / 4))) {
-            // one chunk: a product takes about 25 cycles of an SM per 32 in one walk against 75 in two, a column 1/8 against
-            // 1/40.  (Longer ranges in chunks of 8192 columns: 14 ms per 1e9 products for the searches, barriers and
-            // sweeps of every chunk, against 6.7 in parts of the rank kernel.)
+            // One chunk: direct walks the lists once and sweeps every column, rank walks them twice and sweeps a bitmap.  Measured
+            // on equal rows of doubles, direct against rank: 11000 columns and w = U/8 333 us to 242, U/4 374 to 373, U/2 472 to
+            // 554; 8192 columns 218 to 154, 248 to 234, 302 to 345; 2048 columns 54 to 46, 55 to 50, 57 to 57: the line
+            // lies between U/4 and U/2.  (Longer ranges in chunks of 8192 columns: 14 ms per 1e9 products for the
+            // searches, barriers and sweeps of every chunk, against 6.7 in parts of the rank kernel.)
             route = ROUTE_DIRECT;
         } else if (entries <= R.slots_small) {
             route = U <= R.bits0 ? ROUTE_RANK0 : U <= R.bits1 ? ROUTE_RANK1 : ROUTE_RANK2;
@@ -363,9 +365,9 @@ struct RankSmem {
     }
 };
 
-// Bound by latency and by the shared-memory pipe (adds of doubles are compare-and-swap loops, 21 cycles per 32): what
-// counts is how many rows an SM has under way, so the bitmap has 16-bit ranks per 64 columns (a rank per 32-bit
-// word: twice the shared memory) and the slots come in three sizes.
+// Bound by latency and by the shared-memory pipe (an add of doubles takes 17 cycles of an SM per 32 random slots, of 32-bit
+// integers 2.7): what counts is how many rows an SM has under way, so the bitmap has 16-bit ranks per 64 columns (a rank per
+// 32-bit word: twice the shared memory) and the slots come in three sizes.
 template <typename V, int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS) rows_rank_kernel(PlanDev P, HeavyArgs H, uint32_t columns, uint32_t slots, V* __restrict__ c_vals) {
     using Acc = typename AccOf<V>::type;
