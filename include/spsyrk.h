@@ -404,7 +404,8 @@ spsyrk_status_t spsyrk_plan_buffers(spsyrk_plan_t plan, const int64_t **d_colptr
  * spsyrk_plan_enable_timing : from now on spsyrk_symbolic / spsyrk_numeric record CUDA events on
  *     the caller's stream around the launch of every row class.
  * spsyrk_plan_timings       : device milliseconds of the last symbolic and numeric call per row
- *     class (index = class, 0 unused); waits for those events.  A numeric entry is 0 if numeric
+ *     class (index = class, 0 unused); waits for those events.  The heavy rows (classes 6 and 7) share
+ *     their numeric launches: their time is numeric_ms[7], numeric_ms[6] is 0.  A numeric entry is 0 if numeric
  *     has not run since timing was enabled.
  * spsyrk_launch_count       : kernels launched by this library in this process so far.
  */
