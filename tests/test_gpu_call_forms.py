@@ -190,6 +190,22 @@ def test_one_plan_on_two_streams(B, mode):
         assert float(((v - cv).abs() / scale).max()) <= 1e-5  # (sums of positive products: any order of additions)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.int32])
+def test_heavy_rows_through_the_host_entry(B, dtype):
+    """A power-law product large enough to be computed and downloaded in six row blocks, against the same on the device."""
+    a = W.rmat(15, 16, 7)
+    vals = torch.from_numpy(a.vals).to(dtype) if dtype == torch.float32 else torch.arange(a.vals.size, dtype=torch.int32) % 5
+    d = (torch.from_numpy(a.rowptr), torch.from_numpy(a.colidx), vals)
+    rp, ci, cv, _ = B.tril_syrk(a.m, a.n, *(t.cuda() for t in d))
+    assert ci.numel() > 24 << 20  # a block per 4 << 20 entries
+    h_rp, h_ci, h_cv = B.spsyrk_host_tril(a.m, a.n, *d)
+    assert torch.equal(h_rp, rp.cpu()) and torch.equal(h_ci, ci.cpu())
+    if dtype == torch.int32:
+        assert torch.equal(h_cv, cv.cpu())
+    else:  # (sums of positive products: any order of additions)
+        assert float(((h_cv - cv.cpu()).abs() / cv.cpu()).max()) <= 1e-5
+
+
 # ------------------------------------------------------------------ mirror: where the entries lie, how many rows there are
 def lower_triangle(m, rows, cols, dtype, seed=1):
     """CSR of the distinct (row, column) pairs, on the GPU; values are distinct small numbers."""
