@@ -4,9 +4,8 @@
 //   spsyrk_column_panel : A_s = A(:, [k0, k1)), the operand of one term of the sum;
 //   spsyrk_accumulate   : Z = X + Y on sorted CSR rows, the "+=" itself.
 //
-// The sum works row by row: G lanes per row when rows are short, one warp walking both rows in
-// windows when they are longer (add_merge_kernel).  Both input rows are ascending, so an entry's
-// place in the merged row is
+// The sum works row by row: G lanes per row when rows are short, a warp or a CTA along the merge path when they are
+// longer (merge_row).  In the G-lane kernels, an entry's place in the merged row is
 //     its own index + the number of entries of the other row below it - the matches below it,
 // where a match is a column stored in both rows (it is emitted once, from X's side, with x + y).
 // The other row's count is a binary search; the matches below come from a running count over the
@@ -29,7 +28,8 @@ int group_width(int64_t nnz, int64_t m) {
 struct RowWs {
     uint32_t* cnt;  // m
     int64_t* partials;
-    uint32_t* err;
+    int32_t* list;   // m: long rows of the sum
+    uint32_t *err, *words;
 };
 
 size_t carve(RowWs* w, void* ws, int64_t m) {
@@ -45,7 +45,9 @@ size_t carve(RowWs* w, void* ws, int64_t m) {
     RowWs t;
     t.cnt = (uint32_t*)take(items * 4);
     t.partials = (int64_t*)take(scan_partials_count(items + 1) * 8);
-    t.err = (uint32_t*)take(4);
+    t.list = (int32_t*)take(items * 4);
+    t.err = (uint32_t*)take(16);
+    t.words = t.err + 1;
     if (w) *w = t;
     return (off + ALIGN - 1) / ALIGN * ALIGN;
 }
@@ -117,170 +119,275 @@ __device__ __forceinline__ uint32_t walk_row(const int32_t* __restrict__ self, u
     return matched;
 }
 
-// One warp per row for rows of more than a few entries: the two rows are walked in windows of
-// MERGE_WIN column ids each.  Everything up to the smaller of the two windows' last ids is known
-// completely, so those entries are merged at once: an entry's place is the output position reached
-// so far + its index in its own window + the entries of the other window below it (a search over the
-// window in shared memory) - the matches below it (votes).  All global accesses are coalesced and a
-// step brings in up to 2 x MERGE_WIN ids with one round of loads.
+// Rows of more than a few entries: T threads (a warp, or a CTA for the longest rows) merge a row MERGE_ITEMS * T entries
+// at a time along the merge path (Odeh, Green, Mwassi, Shmueli & Birk, "Merge Path - Parallel Merging Made Simple", 2012).  A
+// tile holds the next ids of both rows in shared memory; a thread finds by a binary search where its MERGE_ITEMS entries of
+// the merged order begin in either row and merges them one after the other, x before y where both store a column;
+// such a pair is emitted once, with x + y, by the thread that has its x.  The emitted entries are put in order in the
+// shared memory of the ids and written out by consecutive threads.
+// What bounds it: instruction issue, and for rows of one or two tiles the latency of a tile's steps.
+// Sum of two panel products of a power-law graph of 2^15 vertices (3.6e7 entries in, 2.9e7 out, f32): 196 us for the size step, 412 for the fill.
+// (Before: one warp per row, whatever its length, in windows of 32 ids with a search and votes per entry: 1402 us.)
 constexpr int MERGE_WARPS = 8;
-constexpr int MERGE_PER_LANE = 1;  // ids per lane and window; 4 was measured: no faster on long rows, slower on short ones
-constexpr int MERGE_WIN = 32 * MERGE_PER_LANE;
+constexpr int MERGE_ITEMS = 8;
+constexpr int MERGE_LONG_THREADS = 256;
+// Rows of more entries (of both inputs together) than this are put on a list and merged by a CTA each: 16 tiles of a warp
+// or two of a CTA.
+constexpr uint32_t MERGE_LONG = 4096;
 
-template <typename V, bool FILL>
-__global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(int64_t m, const int64_t* __restrict__ x_rowptr,
-                                                                     const int32_t* __restrict__ x_colidx, const V* __restrict__ x_vals,
-                                                                     const int64_t* __restrict__ y_rowptr,
-                                                                     const int32_t* __restrict__ y_colidx, const V* __restrict__ y_vals,
-                                                                     uint32_t* __restrict__ cnt, const int64_t* __restrict__ z_rowptr,
-                                                                     int32_t* __restrict__ z_colidx, V* __restrict__ z_vals, uint32_t* err) {
-    constexpr int32_t INF = 0x7fffffff;  // above every column id
-    constexpr int U = MERGE_PER_LANE;
-    constexpr uint32_t WIN = MERGE_WIN;
-    __shared__ int32_t s_x[MERGE_WARPS][MERGE_WIN];
-    __shared__ int32_t s_y[MERGE_WARPS][MERGE_WIN];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
-    const int64_t r = (int64_t)blockIdx.x * MERGE_WARPS + warp;
-    if (r >= m) return;
-    const int64_t x0 = x_rowptr[r], y0 = y_rowptr[r];
-    const int64_t lx64 = x_rowptr[r + 1] - x0, ly64 = y_rowptr[r + 1] - y0;
-    if (lx64 < 0 || ly64 < 0 || lx64 + ly64 > 0x7fffffffLL) {
-        if (lane == 0) {
-            atomicOr(err, ERRW_BAD_ROWPTR);
-            if (!FILL) cnt[r] = 0;
-        }
-        return;
-    }
-    const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
-    const int64_t z0 = FILL ? z_rowptr[r] : 0;
-    const uint32_t lz = FILL ? (uint32_t)(z_rowptr[r + 1] - z0) : 0u;
-    const unsigned lt = (1u << lane) - 1u;
-    int32_t* wx = s_x[warp];
-    int32_t* wy = s_y[warp];
-    // number of ids below key among the first n (ascending) ids of a window
-    auto below = [&](const int32_t* win, uint32_t n, int32_t key) -> uint32_t {
-        uint32_t pos = 0;
-#pragma unroll
-        for (uint32_t step = WIN / 2; step > 0; step >>= 1)
-            if (pos + step <= n && win[pos + step - 1] < key) pos += step;
-        if (pos < n && win[pos] < key) ++pos;  // a full window with every probed id below: the last one
-        return pos;
-    };
-    uint32_t ix = 0, iy = 0, out = 0, matches = 0;
-    int32_t lastx = -1, lasty = -1;
-    while (ix < lx || iy < ly) {  // warp-uniform
-        const uint32_t nx = min(WIN, lx - ix), ny = min(WIN, ly - iy);
-        int32_t xa[U], ya[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t e = u * 32 + lane;
-            xa[u] = e < nx ? x_colidx[x0 + ix + e] : INF;
-            ya[u] = e < ny ? y_colidx[y0 + iy + e] : INF;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            wx[u * 32 + lane] = xa[u];
-            wy[u * 32 + lane] = ya[u];
-        }
-        __syncwarp();
-        const int32_t bx = ix + WIN < lx ? wx[WIN - 1] : INF, by = iy + WIN < ly ? wy[WIN - 1] : INF;
-        const int32_t bound = min(bx, by);
-        uint32_t cx = 0, cy = 0, cmx = 0, cmy = 0;  // taken from x, from y, matches seen from either side so far
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t e = u * 32 + lane;
-            // rows must be strictly ascending (also across windows)
-            const int32_t px = e == 0 ? lastx : wx[e - 1], py = e == 0 ? lasty : wy[e - 1];
-            if ((e < nx && px >= xa[u]) || (e < ny && py >= ya[u])) atomicOr(err, ERRW_UNSORTED);
-            const bool takex = e < nx && xa[u] <= bound, takey = e < ny && ya[u] <= bound;
-            const uint32_t ry = takex ? below(wy, ny, xa[u]) : 0u;
-            const bool mx = takex && ry < ny && wy[ry] == xa[u];
-            const uint32_t rx = takey ? below(wx, nx, ya[u]) : 0u;
-            const bool my = takey && rx < nx && wx[rx] == ya[u];
-            const unsigned vx = __ballot_sync(FULL_MASK, takex), vy = __ballot_sync(FULL_MASK, takey);
-            const unsigned vmx = __ballot_sync(FULL_MASK, mx), vmy = __ballot_sync(FULL_MASK, my);
-            if (FILL) {
-                if (takex) {
-                    const uint32_t pos = out + e + ry - (cmx + __popc(vmx & lt));
-                    if (pos < lz) {
-                        z_colidx[z0 + pos] = xa[u];
-                        const V xv = x_vals[x0 + ix + e];
-                        z_vals[z0 + pos] = mx ? (V)(xv + y_vals[y0 + iy + ry]) : xv;
-                    }
-                }
-                if (takey && !my) {
-                    const uint32_t pos = out + e + rx - (cmy + __popc(vmy & lt));
-                    if (pos < lz) {
-                        z_colidx[z0 + pos] = ya[u];
-                        z_vals[z0 + pos] = y_vals[y0 + iy + e];
-                    }
-                }
-            }
-            cx += __popc(vx);
-            cy += __popc(vy);
-            cmx += __popc(vmx);
-            cmy += __popc(vmy);
-        }
-        if (cx > 0) lastx = wx[cx - 1];
-        if (cy > 0) lasty = wy[cy - 1];
-        out += cx + cy - cmx;
-        matches += cmx;
-        ix += cx;
-        iy += cy;
-        __syncwarp();  // the windows are rewritten
-    }
-    if (!FILL && lane == 0) cnt[r] = lx + ly - matches;
+// rows for which a kernel of the sum leaves the work to add_long_kernel
+struct LongRows {
+    int32_t* list;    // m
+    uint32_t* words;  // [0] rows listed, [1] batches of rows handed out, [2] listed rows handed out; all zero at the start
+    __device__ __forceinline__ void add(int64_t r) const { list[atomicAdd(words, 1u)] = (int32_t)r; }
+};
+
+template <int T>
+__device__ __forceinline__ void merge_sync() {
+    if (T == 32) __syncwarp();
+    else __syncthreads();
 }
 
+// shared memory of a merge: the ids of a tile of either row, one more behind them as a sentinel
+template <int T>
+struct MergeSmem {
+    uint32_t x[T * MERGE_ITEMS + 1], y[T * MERGE_ITEMS + 1];
+    uint32_t scratch[33];
+    uint32_t end;  // entries of x in the tile
+};
+
+// Merges the rows xc[0, lx) and yc[0, ly); thread `t` of T.  FILL: the merged row goes to zc, zv (at most lz entries: always
+// enough with the row pointer of the size step; keeps a stale one from writing outside); otherwise the rows are checked.
+// Returns the number of entries of the merged row.  Rows that are not strictly ascending set the
+// error bit in the size step; their merge is wrong but stays inside the rows.
+template <typename V, bool FILL, int T>
+__device__ __forceinline__ uint32_t merge_row(const int32_t* __restrict__ xc, const V* __restrict__ xv, uint32_t lx, const int32_t* __restrict__ yc,
+                                              const V* __restrict__ yv, uint32_t ly, int32_t* __restrict__ zc, V* __restrict__ zv, uint32_t lz,
+                                              MergeSmem<T>& S, int t, uint32_t* err) {
+    constexpr uint32_t TILE = T * MERGE_ITEMS;
+    constexpr uint32_t NONE = 0xffffu, INF = 0xffffffffu;  // (a negative id fails the check and is merged as 0)
+    static_assert(TILE < NONE, "positions inside a tile are 16 bits");
+    uint32_t ix = 0, iy = 0, out = 0;
+    // A warp brings in consecutive ids, 32 per step, and hands each to the next lane for the check of the order.
+    auto load = [&](const int32_t* __restrict__ ids, uint32_t first, uint32_t n, uint32_t* window) {
+        const uint32_t base = (uint32_t)(t & ~31) * MERGE_ITEMS, lane = t & 31;
+        if (base >= n) return;
+        int32_t before = -1;
+        if (!FILL && lane == 0 && first + base > 0) before = ids[first + base - 1];
+        bool bad = false;
+        int32_t id[MERGE_ITEMS];
+#pragma unroll
+        for (int u = 0; u < MERGE_ITEMS; ++u) id[u] = base + u * 32 + lane < n ? ids[first + base + u * 32 + lane] : 0x7fffffff;
+#pragma unroll
+        for (int u = 0; u < MERGE_ITEMS; ++u) {
+            const uint32_t e = base + u * 32 + lane;
+            if (e < n) window[e] = (uint32_t)max(id[u], 0);
+            if (!FILL) {
+                int32_t left = __shfl_up_sync(FULL_MASK, id[u], 1);
+                if (lane == 0) left = before;
+                bad |= e < n && left >= id[u];
+                before = __shfl_sync(FULL_MASK, id[u], 31);
+            }
+        }
+        if (!FILL && bad) atomicOr(err, ERRW_UNSORTED);
+    };
+    while (ix < lx || iy < ly) {  // the same for all threads
+        const uint32_t nx = min(TILE, lx - ix), ny = min(TILE, ly - iy);
+        load(xc, ix, nx, S.x);
+        load(yc, iy, ny, S.y);
+        if (t == 0) S.x[nx] = S.y[ny] = INF;
+        merge_sync<T>();
+        const uint32_t total = min(TILE, nx + ny);
+        const uint32_t d = min((uint32_t)t * MERGE_ITEMS, total), d_end = min(d + MERGE_ITEMS, total);
+        uint32_t xi = d > ny ? d - ny : 0u, hi = min(d, nx);  // entries of x among the first d of the merged order
+        while (xi < hi) {
+            const uint32_t mid = (xi + hi) >> 1;
+            if (S.x[mid] <= S.y[d - 1 - mid]) xi = mid + 1;
+            else hi = mid;
+        }
+        uint32_t yi = d - xi;
+        uint32_t a = S.x[xi], b = S.y[yi];
+        if (xi > 0 && S.x[xi - 1] == b) b = S.y[++yi];  // the pair went with its x (never the sentinel: ids are at most 2^31 - 1)
+        uint32_t col[MERGE_ITEMS], src[MERGE_ITEMS];  // src: position in x's window | position in y's << 16
+        uint32_t n = 0;
+#pragma unroll
+        for (int i = 0; i < MERGE_ITEMS; ++i) {
+            const bool go = xi + yi < d_end;
+            const bool tx = a <= b, ty = b <= a;
+            if (FILL) {
+                col[i] = tx ? a : b;
+                src[i] = (tx ? xi : NONE) | (ty ? yi : NONE) << 16;
+            }
+            if (go) {
+                ++n;
+                if (tx) a = S.x[min(++xi, nx)];
+                if (ty) b = S.y[min(++yi, ny)];
+            }
+        }
+        if (t == T - 1) S.end = xi << 16 | yi;
+        uint32_t rank, sum;
+        if (T == 32) {
+            const uint32_t incl = warp_inclusive_scan<uint32_t>(n);
+            sum = __shfl_sync(FULL_MASK, incl, 31);
+            rank = incl - n;
+            __syncwarp();  // the windows are read
+        } else {
+            rank = block_exclusive_scan<uint32_t, T == 32 ? 64 : T>(n, S.scratch, &sum);
+        }
+        const uint32_t end = S.end;
+        if (FILL) {
+#pragma unroll
+            for (int i = 0; i < MERGE_ITEMS; ++i) {
+                if (i < n) {
+                    S.x[rank + i] = col[i];
+                    S.y[rank + i] = src[i];
+                }
+            }
+            merge_sync<T>();
+            const uint32_t n_out = out < lz ? min(sum, lz - out) : 0u;
+            for (uint32_t i = t; i < n_out; i += T) {
+                const uint32_t s = S.y[i], sx = s & NONE, sy = s >> 16;
+                V v{}, w{};
+                if (sx != NONE) v = xv[ix + sx];
+                if (sy != NONE) w = yv[iy + sy];
+                zc[out + i] = (int32_t)S.x[i];
+                zv[out + i] = sx == NONE ? w : sy == NONE ? v : (V)(v + w);
+            }
+        }
+        merge_sync<T>();  // the windows are rewritten
+        out += sum;
+        ix += end >> 16;
+        iy += end & 0xffffu;
+    }
+    return out;
+}
+
+// the operands of the sum and, when it is filled, the result
+template <typename V>
+struct SumArgs {
+    int64_t m;
+    const int64_t* x_rowptr;
+    const int32_t* x_colidx;
+    const V* x_vals;
+    const int64_t* y_rowptr;
+    const int32_t* y_colidx;
+    const V* y_vals;
+    uint32_t* cnt;             // size step
+    const int64_t* z_rowptr;   // fill step
+    int32_t* z_colidx;
+    V* z_vals;
+    uint32_t* err;
+};
+
+template <typename V, bool FILL, int T>
+__device__ __forceinline__ void sum_row(const SumArgs<V>& A, int64_t r, int64_t x0, uint32_t lx, int64_t y0, uint32_t ly, MergeSmem<T>& S, int t) {
+    const int64_t z0 = FILL ? A.z_rowptr[r] : 0;
+    const uint32_t lz = FILL ? (uint32_t)(A.z_rowptr[r + 1] - z0) : 0u;
+    const uint32_t n = merge_row<V, FILL, T>(A.x_colidx + x0, FILL ? A.x_vals + x0 : nullptr, lx, A.y_colidx + y0, FILL ? A.y_vals + y0 : nullptr, ly,
+                                             FILL ? A.z_colidx + z0 : nullptr, FILL ? A.z_vals + z0 : nullptr, lz, S, t, A.err);
+    if (!FILL && t == 0) A.cnt[r] = n;
+}
+
+// One warp per row.  The warps draw batches of rows: with eight rows to a CTA the longest of them kept the places of the others
+// (19 % of the warps active on average).
+template <typename V, bool FILL>
+__global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(SumArgs<V> A, LongRows longer, int batch) {
+    __shared__ MergeSmem<32> smem[MERGE_WARPS];
+    const int warp = threadIdx.x >> 5, lane = lane_id();
+    for (;;) {
+        uint32_t ticket = 0;
+        if (lane == 0) ticket = atomicAdd(longer.words + 1, 1u);
+        const int64_t first = (int64_t)__shfl_sync(FULL_MASK, ticket, 0) * batch;
+        if (first >= A.m) return;
+        const int64_t last = min(first + batch, A.m);
+        for (int64_t r = first; r < last; ++r) {
+            const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
+            const int64_t lx = A.x_rowptr[r + 1] - x0, ly = A.y_rowptr[r + 1] - y0;
+            if (lx < 0 || ly < 0 || lx + ly > 0x7fffffffLL) {
+                if (lane == 0) {
+                    atomicOr(A.err, ERRW_BAD_ROWPTR);
+                    if (!FILL) A.cnt[r] = 0;
+                }
+            } else if (lx + ly > MERGE_LONG) {
+                if (lane == 0) longer.add(r);
+            } else {
+                sum_row<V, FILL, 32>(A, r, x0, (uint32_t)lx, y0, (uint32_t)ly, smem[warp], lane);
+            }
+        }
+    }
+}
+
+// one CTA per listed row
+template <typename V, bool FILL>
+__global__ void __launch_bounds__(MERGE_LONG_THREADS) add_long_kernel(SumArgs<V> A, LongRows rows) {
+    __shared__ MergeSmem<MERGE_LONG_THREADS> smem;
+    __shared__ uint32_t s_ticket;
+    const uint32_t n = rows.words[0];
+    for (;;) {
+        if (threadIdx.x == 0) s_ticket = atomicAdd(rows.words + 2, 1u);
+        __syncthreads();
+        const uint32_t i = s_ticket;
+        if (i >= n) return;
+        const int64_t r = rows.list[i];
+        const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
+        // (a row of this length has at least one tile, whose barriers separate this look at the ticket from the next)
+        sum_row<V, FILL, MERGE_LONG_THREADS>(A, r, x0, (uint32_t)(A.x_rowptr[r + 1] - x0), y0, (uint32_t)(A.y_rowptr[r + 1] - y0), smem, (int)threadIdx.x);
+    }
+}
+
+// G lanes per row, where rows are short on average
 template <int G>
-__global__ void __launch_bounds__(256) add_count_kernel(int64_t m, const int64_t* __restrict__ x_rowptr,
-                                                        const int32_t* __restrict__ x_colidx, const int64_t* __restrict__ y_rowptr,
-                                                        const int32_t* __restrict__ y_colidx, uint32_t* __restrict__ cnt,
-                                                        uint32_t* err) {
+__global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A, LongRows longer) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
-    if (r >= m) return;  // whole groups leave together
-    const int64_t x0 = x_rowptr[r], y0 = y_rowptr[r];
-    const int64_t lx64 = x_rowptr[r + 1] - x0, ly64 = y_rowptr[r + 1] - y0;
+    if (r >= A.m) return;  // whole groups leave together
+    const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
+    const int64_t lx64 = A.x_rowptr[r + 1] - x0, ly64 = A.y_rowptr[r + 1] - y0;
     if (lx64 < 0 || ly64 < 0 || lx64 + ly64 > 0x7fffffffLL) {
-        if (gl == 0) { atomicOr(err, ERRW_BAD_ROWPTR); cnt[r] = 0; }
+        if (gl == 0) { atomicOr(A.err, ERRW_BAD_ROWPTR); A.cnt[r] = 0; }
+        return;
+    }
+    if (lx64 + ly64 > MERGE_LONG) {
+        if (gl == 0) longer.add(r);
         return;
     }
     const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
+    const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
     // the sortedness of X is checked here, that of Y inside the walk
     for (uint32_t t = 1 + gl; t < lx; t += G)
-        if (x_colidx[x0 + t - 1] >= x_colidx[x0 + t]) atomicOr(err, ERRW_UNSORTED);
-    const uint32_t matched =
-        walk_row<G>(y_colidx + y0, ly, x_colidx + x0, lx, err, [](uint32_t, uint32_t, bool, uint32_t, int32_t) {});
-    if (gl == 0) cnt[r] = lx + ly - matched;
+        if (xc[t - 1] >= xc[t]) atomicOr(A.err, ERRW_UNSORTED);
+    const uint32_t matched = walk_row<G>(yc, ly, xc, lx, A.err, [](uint32_t, uint32_t, bool, uint32_t, int32_t) {});
+    if (gl == 0) A.cnt[r] = lx + ly - matched;
 }
 
 template <typename V, int G>
-__global__ void __launch_bounds__(256) add_fill_kernel(int64_t m, const int64_t* __restrict__ x_rowptr,
-                                                       const int32_t* __restrict__ x_colidx, const V* __restrict__ x_vals,
-                                                       const int64_t* __restrict__ y_rowptr, const int32_t* __restrict__ y_colidx,
-                                                       const V* __restrict__ y_vals, const int64_t* __restrict__ z_rowptr,
-                                                       int32_t* __restrict__ z_colidx, V* __restrict__ z_vals, uint32_t* err) {
+__global__ void __launch_bounds__(256) add_fill_kernel(SumArgs<V> A, LongRows longer) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    if (r >= m) return;
-    const int64_t x0 = x_rowptr[r], y0 = y_rowptr[r], z0 = z_rowptr[r];
-    const uint32_t lx = (uint32_t)(x_rowptr[r + 1] - x0), ly = (uint32_t)(y_rowptr[r + 1] - y0);
-    const uint32_t lz = (uint32_t)(z_rowptr[r + 1] - z0);
+    if (r >= A.m) return;
+    const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r], z0 = A.z_rowptr[r];
+    const int64_t lx64 = A.x_rowptr[r + 1] - x0, ly64 = A.y_rowptr[r + 1] - y0;
+    if (lx64 + ly64 > MERGE_LONG) {
+        if ((threadIdx.x & (G - 1)) == 0) longer.add(r);
+        return;
+    }
+    const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
+    const uint32_t lz = (uint32_t)(A.z_rowptr[r + 1] - z0);
+    const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
     // entries of X: all are emitted, matched ones with the sum
-    walk_row<G>(x_colidx + x0, lx, y_colidx + y0, ly, err, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
+    walk_row<G>(xc, lx, yc, ly, A.err, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
         const uint32_t pos = t + lb - before;
         if (pos < lz) {  // always true for the row pointer of the size step; keeps a stale one from writing outside
-            z_colidx[z0 + pos] = col;
-            const V xv = x_vals[x0 + t];
-            z_vals[z0 + pos] = match ? (V)(xv + y_vals[y0 + lb]) : xv;
+            A.z_colidx[z0 + pos] = col;
+            const V xv = A.x_vals[x0 + t];
+            A.z_vals[z0 + pos] = match ? (V)(xv + A.y_vals[y0 + lb]) : xv;
         }
     });
     // entries of Y: only the ones X does not store
-    walk_row<G>(y_colidx + y0, ly, x_colidx + x0, lx, err, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
+    walk_row<G>(yc, ly, xc, lx, A.err, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
         const uint32_t pos = t + lb - before;
         if (!match && pos < lz) {
-            z_colidx[z0 + pos] = col;
-            z_vals[z0 + pos] = y_vals[y0 + t];
+            A.z_colidx[z0 + pos] = col;
+            A.z_vals[z0 + pos] = A.y_vals[y0 + t];
         }
     });
 }
@@ -317,24 +424,30 @@ void launch_panel_fill(int g, int64_t m, const int64_t* rowptr, const int32_t* c
     note_launches(1);
 }
 
-template <typename V>
-void launch_add_fill(int g, int64_t m, const int64_t* xr, const int32_t* xc, const void* xv, const int64_t* yr, const int32_t* yc,
-                     const void* yv, const int64_t* zr, int32_t* zc, void* zv, uint32_t* err, cudaStream_t st) {
-#define FILL(G)                                                                                                             \
-    add_fill_kernel<V, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(m, xr, xc, static_cast<const V*>(xv), yr, yc,          \
-                                                                           static_cast<const V*>(yv), zr, zc, static_cast<V*>(zv), \
-                                                                           err)
-    switch (g) {
-        case 4: FILL(4); break;
-        case 8: FILL(8); break;
-        case 16: FILL(16); break;
-        default:
-            add_merge_kernel<V, true><<<(unsigned)((m + MERGE_WARPS - 1) / MERGE_WARPS), MERGE_WARPS * 32, 0, st>>>(
-                m, xr, xc, static_cast<const V*>(xv), yr, yc, static_cast<const V*>(yv), nullptr, zr, zc, static_cast<V*>(zv), err);
-            break;
+// kernels of one step of the sum: the rows, then the long ones among them
+template <typename V, bool FILL>
+spsyrk_status_t launch_sum(int g, const SumArgs<V>& A, const RowWs& w, cudaStream_t st) {
+    const LongRows longer{w.list, w.words};
+    const auto blocks = [&](int lanes) { return (unsigned)((A.m * lanes + 255) / 256); };
+    SPSYRK_CUDA_TRY(cudaMemsetAsync(w.words, 0, 12, st));
+    constexpr unsigned MERGE_CTAS = 148 * 8;
+    if (g > 16) {
+        // about 16 batches per warp, of 32 rows at most: 4e6 draws from one counter would take longer than the sum
+        const int batch = (int)std::min<int64_t>(std::max<int64_t>(A.m / (MERGE_CTAS * MERGE_WARPS * 16), 1), 32);
+        add_merge_kernel<V, FILL><<<std::min(MERGE_CTAS, blocks(32)), MERGE_WARPS * 32, 0, st>>>(A, longer, batch);
+    } else if constexpr (FILL) {
+        if (g == 4) add_fill_kernel<V, 4><<<blocks(4), 256, 0, st>>>(A, longer);
+        else if (g == 8) add_fill_kernel<V, 8><<<blocks(8), 256, 0, st>>>(A, longer);
+        else add_fill_kernel<V, 16><<<blocks(16), 256, 0, st>>>(A, longer);
+    } else {
+        if (g == 4) add_count_kernel<4><<<blocks(4), 256, 0, st>>>(A, longer);
+        else if (g == 8) add_count_kernel<8><<<blocks(8), 256, 0, st>>>(A, longer);
+        else add_count_kernel<16><<<blocks(16), 256, 0, st>>>(A, longer);
     }
-#undef FILL
-    note_launches(1);
+    add_long_kernel<V, FILL><<<148 * 4, MERGE_LONG_THREADS, 0, st>>>(A, longer);
+    note_launches(2);
+    SPSYRK_CUDA_TRY(cudaGetLastError());
+    return SPSYRK_OK;
 }
 
 bool dtype_ok(spsyrk_dtype_t t) { return t == SPSYRK_F64 || t == SPSYRK_F32 || t == SPSYRK_I32; }
@@ -401,39 +514,23 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
         if (!nnz_out) return SPSYRK_ERR_INVALID_ARG;
         SPSYRK_CUDA_TRY(cudaMemsetAsync(w.err, 0, 4, st));
         if (m > 0) {
-#define COUNT(G) \
-    add_count_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(m, d_x_rowptr, d_x_colidx, d_y_rowptr, d_y_colidx, w.cnt, w.err)
-            switch (g) {
-                case 4: COUNT(4); break;
-                case 8: COUNT(8); break;
-                case 16: COUNT(16); break;
-                default:
-                    add_merge_kernel<uint32_t, false><<<(unsigned)((m + MERGE_WARPS - 1) / MERGE_WARPS), MERGE_WARPS * 32, 0, st>>>(
-                        m, d_x_rowptr, d_x_colidx, nullptr, d_y_rowptr, d_y_colidx, nullptr, w.cnt, nullptr, nullptr, nullptr, w.err);
-                    break;
-            }
-#undef COUNT
-            note_launches(1);
+            const spsyrk_status_t s = launch_sum<uint32_t, false>(
+                g, {m, d_x_rowptr, d_x_colidx, nullptr, d_y_rowptr, d_y_colidx, nullptr, w.cnt, nullptr, nullptr, nullptr, w.err}, w, st);
+            if (s != SPSYRK_OK) return s;
         }
         return scan_and_total(w, m, d_z_rowptr, nnz_out, st);
     }
     if (!d_z_vals || (nnz_x > 0 && !d_x_vals) || (nnz_y > 0 && !d_y_vals)) return SPSYRK_ERR_INVALID_ARG;
     if (m == 0) return SPSYRK_OK;
+    const auto fill = [&](auto* z_vals) {
+        using V = std::remove_pointer_t<decltype(z_vals)>;
+        return launch_sum<V, true>(g, {m, d_x_rowptr, d_x_colidx, static_cast<const V*>(d_x_vals), d_y_rowptr, d_y_colidx, static_cast<const V*>(d_y_vals),
+                                       nullptr, d_z_rowptr, d_z_colidx, z_vals, w.err}, w, st);
+    };
     switch (dtype) {
-        case SPSYRK_F64:
-            launch_add_fill<double>(g, m, d_x_rowptr, d_x_colidx, d_x_vals, d_y_rowptr, d_y_colidx, d_y_vals, d_z_rowptr, d_z_colidx,
-                                    d_z_vals, w.err, st);
-            break;
-        case SPSYRK_F32:
-            launch_add_fill<float>(g, m, d_x_rowptr, d_x_colidx, d_x_vals, d_y_rowptr, d_y_colidx, d_y_vals, d_z_rowptr, d_z_colidx,
-                                   d_z_vals, w.err, st);
-            break;
-        default:
-            // unsigned addition wraps modulo 2^32, which is also what two's-complement int32 addition means
-            launch_add_fill<uint32_t>(g, m, d_x_rowptr, d_x_colidx, d_x_vals, d_y_rowptr, d_y_colidx, d_y_vals, d_z_rowptr,
-                                      d_z_colidx, d_z_vals, w.err, st);
-            break;
+        case SPSYRK_F64: return fill(static_cast<double*>(d_z_vals));
+        case SPSYRK_F32: return fill(static_cast<float*>(d_z_vals));
+        // unsigned addition wraps modulo 2^32, which is also what two's-complement int32 addition means
+        default: return fill(static_cast<uint32_t*>(d_z_vals));
     }
-    SPSYRK_CUDA_TRY(cudaGetLastError());
-    return SPSYRK_OK;
 }

@@ -1,0 +1,73 @@
+"""The sparse sum at the edges of its tiles: a warp merges 256 entries of both rows at a time, a CTA 2048; rows of more
+than 4096 entries of both inputs go to a CTA."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2608_09713_b200 import binding
+    return binding
+
+
+def _pair(kind, size, rng):
+    """Ascending ids of one row of X and of Y, `size` entries together (of identical rows: of each)."""
+    if kind == "same":  # every tile ends between the two entries of a pair, or could
+        a = np.sort(rng.choice(3 * size + 1, size, replace=False))
+        return a, a
+    if kind == "shifted":  # one more id in front of Y: the pairs straddle the borders of threads and tiles differently
+        a = np.arange(1, size + 1)
+        return a, np.arange(size)
+    if kind == "blocks":  # long runs of one row between ids of the other
+        ids = np.arange(size)
+        own = (ids // 700) % 2 == 0
+        return ids[own], ids[~own]
+    if kind == "one":  # only X
+        return np.arange(size), np.zeros(0, dtype=np.int64)
+    mask = rng.integers(0, 3, size=size)  # random: X only, Y only, both
+    ids = np.sort(rng.choice(5 * size + 1, size, replace=False))
+    return ids[mask != 1], ids[mask != 0]
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32, torch.int32])
+@pytest.mark.parametrize("empty_rows", [0, 8000], ids=["warp", "group"])  # many empty rows: few lanes per row
+@pytest.mark.parametrize("kind", ["same", "shifted", "blocks", "one", "random"])
+def test_accumulate_at_tile_edges(B, kind, empty_rows, dtype):
+    rng = np.random.default_rng(7)
+    pairs = [_pair(kind, s, rng) for s in (1, 7, 8, 9, 127, 128, 129, 255, 256, 257, 511, 513, 2047, 2048, 2049, 4095, 4096, 4097, 8191, 8192, 8193, 20_011)]
+    pairs += [(np.zeros(0, dtype=np.int64),) * 2] * empty_rows + [pairs[-1], pairs[4]]
+    m = len(pairs)
+    npdt = {torch.float64: np.float64, torch.float32: np.float32, torch.int32: np.int32}[dtype]
+
+    def csr(side):
+        rows = [p[side] for p in pairs]
+        rp = np.concatenate(([0], np.cumsum([r.size for r in rows]))).astype(np.int64)
+        v = rng.integers(-9, 10, size=rp[-1]) if dtype == torch.int32 else rng.standard_normal(rp[-1])
+        return rp, np.concatenate(rows).astype(np.int32), v.astype(npdt)
+
+    x, y = csr(0), csr(1)
+    zr, zc, zv = (t.cpu().numpy() for t in B.spsyrk_accumulate(m, *[torch.from_numpy(t).cuda() for t in x], *[torch.from_numpy(t).cuda() for t in y]))
+    er, ec, ev = oracle.add(m, x[0], x[1], x[2].astype(np.float64), y[0], y[1], y[2].astype(np.float64))
+    assert np.array_equal(zr, er) and np.array_equal(zc, ec)
+    assert np.array_equal(zv, ev.astype(npdt))  # one rounded addition: the double sum of two floats rounds to the float sum
+
+
+@pytest.mark.parametrize("size", [300, 5000])
+@pytest.mark.parametrize("side", [0, 1])
+def test_accumulate_refuses_rows_that_do_not_ascend(B, size, side):
+    """The check across the borders of tiles: one equal pair of neighbours anywhere in the row."""
+    for at in (1, 31, 32, size // 2, 255, 256, 257, size - 1):
+        good = np.arange(size, dtype=np.int32)
+        bad = good.copy()
+        bad[at] = bad[at - 1]
+        cols = [bad, good] if side == 0 else [good, bad]
+        rp = torch.tensor([0, size], dtype=torch.int64, device="cuda")
+        v = torch.ones(size, dtype=torch.float64, device="cuda")
+        with pytest.raises(B.SpsyrkError) as e:
+            B.spsyrk_accumulate(1, rp, torch.from_numpy(cols[0]).cuda(), v, rp, torch.from_numpy(cols[1]).cuda(), v)
+        assert e.value.status == 2
