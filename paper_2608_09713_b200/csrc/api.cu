@@ -169,6 +169,7 @@ struct spsyrk_plan_s {
     // host facts
     int64_t class_start[NCLASS + 1];
     int64_t work_total;
+    uint32_t sparse_heavy[2];  // rows of classes 6 and 7 whose count is not settled by the binning
     bool have_symbolic;
     bool key64;
     bool diag;  // the light-row kernels handle the diagonal apart (lower-triangle mode, whole column range)
@@ -197,14 +198,14 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     const size_t rx_words = radix_state_words(radix_tiles(nnz), radix_wide(nnz), npass);
     // counters in one piece, so that one memset clears them: the binning's, then the plan's, then the column counts
     const int views = full ? 2 : 1;
-    const size_t bin_words = views * (1 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(rows));
+    const size_t bin_words = views * (2 + (size_t)scan_partials_count(NCLASS * nb) + (size_t)scan_partials_count(rows));
     auto zero = c.take<int64_t>(bin_words + 32 + (32 + HEAVY_BINS) / 2 + (size_t)scan_partials_count(std::max<int64_t>(n, 1)) + (size_t)(n + 1) / 2 +
                                 RX_MAX_PASSES * RX_BINS + RX_MAX_PASSES + rx_words);
     Carver cz(zero);
     auto take_words = [&](size_t words) { int64_t* q = zero ? zero + cz.off : nullptr; cz.off += words; return q; };
-    auto work_total_dev = reinterpret_cast<unsigned long long*>(take_words(1));
+    auto work_total_dev = reinterpret_cast<unsigned long long*>(take_words(2));  // and the heavy rows that are not dense
     auto state_bin = take_words(scan_partials_count(NCLASS * nb)), state_items = take_words(scan_partials_count(rows));
-    unsigned long long* u_work_total_dev = full ? reinterpret_cast<unsigned long long*>(take_words(1)) : nullptr;
+    unsigned long long* u_work_total_dev = full ? reinterpret_cast<unsigned long long*>(take_words(2)) : nullptr;
     int64_t* u_state_bin = full ? take_words(scan_partials_count(NCLASS * nb)) : nullptr;
     int64_t* u_state_items = full ? take_words(scan_partials_count(rows)) : nullptr;
     auto err = reinterpret_cast<uint32_t*>(take_words(32));
@@ -414,8 +415,8 @@ void launch_row_work(spsyrk_plan_s* pl, bool analyse, cudaStream_t st) {
     HeavyArrays heavy{pl->colcnt, pl->facts, pl->heavy_id, pl->heavy_mask, 0u};
     if (analyse) heavy.ctas = (unsigned)std::min<int64_t>(2 + std::max<int64_t>(P.n, (int64_t)P.m * G) / BIN_THREADS, (int64_t)pl->sm_count * 8);
     if (nb > 0)
-        row_work_kernel<G><<<(unsigned)nb + heavy.ctas, BIN_THREADS, 0, st>>>(P, pl->cls, BLOCK_CLASS_MAX_WORK, pl->diag, bin_tile(rows), pl->blockhist, nb,
-                                                                             pl->work_total_dev, heavy);
+        row_work_kernel<G><<<(unsigned)nb + heavy.ctas, BIN_THREADS, 0, st>>>(P, pl->cls, BLOCK_CLASS_MAX_WORK, ROW_CHUNK_BITS_MAX_SYMBOLIC, pl->diag, bin_tile(rows), pl->blockhist, nb,
+                                                                             pl->work_total_dev, pl->work_total_dev + 1, heavy);
     else if (analyse) heavy_analysis_kernel<G><<<heavy.ctas, BIN_THREADS, 0, st>>>(P, heavy);
     else return;
     note_launches(1);
@@ -474,7 +475,7 @@ spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, int64_t* gave_up, b
     pl->have_onepass = false;
     pl->map_filled = false;
     const PlanDev& P = pl->dev;
-    const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->facts, P.err, host, gave_up};
+    const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->work_total_dev + 1, pl->facts, P.err, host, gave_up};
     if (P.nnz == 0) analyse = false;
     switch (group_width(P.nnz, P.m)) {
         case 4: launch_row_work<4>(pl, analyse, st); break;
@@ -490,7 +491,7 @@ spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, int64_t* gave_up, b
         return SPSYRK_OK;
     }
     SPSYRK_CUDA_TRY(scan_launch(ScanArray<int32_t>{pl->blockhist}, NCLASS * nb, BinStarts{pl->offsets, (uint32_t)nb, pl->class_start_dev}, pl->state_bin, P.err, st, true));
-    row_scatter_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(P, pl->cls, bin_tile(rows), pl->offsets, nb, pl->diag, pl->perm, pl->hdr, pl->items8, pl->cnt);
+    row_scatter_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(P, pl->cls, bin_tile(rows), pl->offsets, nb, pl->diag, pl->perm, pl->hdr, pl->items8, pl->cnt, pl->block_base, pl->blocks_per_row);
     note_launches(1);
     SPSYRK_CUDA_TRY(scan_launch(ScanArray<uint32_t>{pl->items8}, rows, ItemStarts{pl->itemoff, rows, facts}, pl->state_items, P.err, st, true));
     return SPSYRK_OK;
@@ -501,6 +502,7 @@ spsyrk_status_t bin_collect(spsyrk_plan_s* pl, const HostBlock& block, const int
     std::memcpy(pl->class_start, host + PF_CLASS_START, sizeof(pl->class_start));
     pl->map_items = host[PF_MAP_ITEMS];
     pl->work_total = host[PF_WORK];
+    for (int k = 0; k < 2; ++k) pl->sparse_heavy[k] = (uint32_t)((uint64_t)host[PF_SPARSE_HEAVY] >> (32 * k));
     pl->dev.binary = (pl->dev.nnz > 0 && host[PF_OTHER_THAN_ONE] == 0) ? 1 : 0;
     return status_of(block.errors(host[PF_ERR]));
 }
@@ -725,7 +727,7 @@ uint32_t row_chunk_bits(const spsyrk_plan_s* pl, uint32_t cap) {
 template <int THREADS>
 spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
     const int64_t count = pl->class_start[c + 1] - pl->class_start[c];
-    if (count <= 0) return SPSYRK_OK;
+    if (count <= 0 || pl->sparse_heavy[c - 6] == 0) return SPSYRK_OK;
     const uint32_t cb = row_chunk_bits(pl, ROW_CHUNK_BITS_MAX_SYMBOLIC);
     const size_t smem = CtaRowSmem<int32_t, THREADS, false>::bytes(cb, 0);
     auto kern = rows_cta_kernel<int32_t, THREADS, false>;
@@ -956,7 +958,7 @@ __global__ void onepass_slots_kernel(PlanDev P, const uint8_t* __restrict__ cls,
                                      int32_t* __restrict__ ub) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
-    const int c = cls[r];
+    const int c = cls[r] & (ROW_DENSE - 1);
     const int64_t i = P.r0 + r;
     const int64_t deg = P.rowptr[i + 1] - P.rowptr[i];
     int64_t u = 0;

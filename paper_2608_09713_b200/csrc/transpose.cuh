@@ -179,37 +179,59 @@ template <> struct alignas(16) ColRec<double> { int32_t j; int32_t pad; double v
 template <> struct alignas(8) ColRec<float> { int32_t j; float v; };
 template <> struct alignas(8) ColRec<int32_t> { int32_t j; int32_t v; };
 
+// Rows of more than so many steps of their G lanes are left to the whole CTA at the end: the longest row of a power-law
+// matrix (15 711 nonzeros at 2^18 rows) kept its 16 lanes busy for most of the
+// kernel's 401 us (product and mirror of that matrix 30.63 -> 30.23 ms, of 2^13 rows 352 -> 333 us, row_work_kernel's share included).
+constexpr int LONG_STEPS = 8;
+
 // G lanes per row, one sweep over the nonzeros of A: the checks of the row pointers (a row indexes nothing unless its own
 // two are sane) and of the column ids (in range, strictly ascending inside the row), the column histogram (its scan gives
 // colptr), the explicit row id of every nonzero (the radix sort's first payload), the row lengths, and whether
 // every stored value is one.  Nothing waits for the checks: the kernels up to the plan's one synchronisation test what
-// they index by, or look at the error word first.
+// they index by, or look at the error word first.  Bound by the atomic adds of the histogram (1.4e11 per second on 6.7e7
+// random columns).
 template <int G, typename V>
 static __global__ void __launch_bounds__(256) row_expand_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
                                                                 const V* __restrict__ vals, int32_t m, int32_t n, int64_t nnz,
                                                                 uint32_t* __restrict__ colcnt, uint32_t* __restrict__ rowid,
                                                                 int32_t* __restrict__ adeg, uint32_t* facts, uint32_t* err) {
+    __shared__ int32_t s_long[256 / G];
+    __shared__ int s_nlong;
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
     bool look = __ldca(facts) == 0;  // values are looked at until one differs from one (an old zero only costs a look)
-    bool other = false;
+    bool other = false, is_long = false;
+    auto entry = [&](int64_t p, int64_t p0, int64_t row) {
+        const int32_t k = colidx[p];
+        if (look) {
+            other = !(vals[p] == V(1));
+            look = !other;
+        }
+        if ((uint32_t)k >= (uint32_t)n) atomicOr(err, ERRW_BAD_COL);
+        else atomicAdd(&colcnt[k], 1u);
+        if (p > p0 && colidx[p - 1] >= k) atomicOr(err, ERRW_UNSORTED);
+        rowid[p] = (uint32_t)row;
+    };
     if (gid < m) {
         const int64_t p0 = rowptr[gid], p1 = rowptr[gid + 1];
         if (gl == 0) adeg[gid] = (int32_t)(p1 - p0);
         if (p0 > p1 || p0 < 0 || p1 > nnz) {
             atomicOr(err, ERRW_BAD_ROWPTR);
+        } else if (p1 - p0 > LONG_STEPS * G) {
+            is_long = true;
         } else {
-            for (int64_t p = p0 + gl; p < p1; p += G) {
-                const int32_t k = colidx[p];
-                if (look) {
-                    other = !(vals[p] == V(1));
-                    look = !other;
-                }
-                if ((uint32_t)k >= (uint32_t)n) atomicOr(err, ERRW_BAD_COL);
-                else atomicAdd(&colcnt[k], 1u);
-                if (p > p0 && colidx[p - 1] >= k) atomicOr(err, ERRW_UNSORTED);
-                rowid[p] = (uint32_t)gid;
-            }
+            for (int64_t p = p0 + gl; p < p1; p += G) entry(p, p0, gid);
+        }
+    }
+    if (__syncthreads_or(is_long)) {
+        if (threadIdx.x == 0) s_nlong = 0;
+        __syncthreads();
+        if (is_long && gl == 0) s_long[atomicAdd(&s_nlong, 1)] = (int32_t)gid;
+        __syncthreads();
+        for (int i = 0; i < s_nlong; ++i) {
+            const int64_t row = s_long[i];
+            const int64_t p0 = rowptr[row], p1 = rowptr[row + 1];
+            for (int64_t p = p0 + threadIdx.x; p < p1; p += 256) entry(p, p0, row);
         }
     }
     if (gid == 0 && gl == 0 && (rowptr[0] != 0 || rowptr[m] != nnz)) atomicOr(err, ERRW_BAD_ROWPTR);
@@ -259,10 +281,14 @@ static __global__ void __launch_bounds__(256) block_desc_kernel(PlanDev P, const
     }
 }
 
+constexpr int ROW_DENSE = 8;  // beside the class in cls[]: every column of the row's range is stored
 // Step a2: per-row work w[i] = sum of the descriptor lengths of row i (G lanes per row), the class of the row and
 // the number of rows of every class in every CTA's tile (the first half of a stable counting sort by class).
 //   class 0: no work; 1..5: w <= 32, 64, 128, 256, 512 and at most 32 nonzeros (one warp, register sort)
 //   6: w <= block_max (block class, bitmap accumulator); 7: larger (one 1024-thread CTA)
+//   A heavy row that stores a column of every row of its range (of at most dense_range rows) is dense: it is marked here,
+//   row_scatter_kernel settles its count, and a class with nothing but dense rows needs no counting kernel (50 000 such rows,
+//   a CTA each that only looked at the descriptors: 311 us)
 //   diag: the light-row kernels leave the diagonal products out of their item lists (lower-triangle mode
 //   over the whole column range), so a light row is classed by w minus its number of nonzeros
 // A group takes UNR rows at a time, so that the loads of one row do not wait for those of the row before (one at a time:
@@ -270,28 +296,51 @@ static __global__ void __launch_bounds__(256) block_desc_kernel(PlanDev P, const
 // to itself the compiler serialises the loads of long rows beside the analysis (524288 rows of a power-law matrix, whole
 // plan: 859 us without the bound, 749 with it).
 template <int G>
-static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, bool diag, int64_t tile,
+static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, uint32_t dense_range, bool diag, int64_t tile,
                                                                       int32_t* __restrict__ blockhist, int64_t nblocks,
-                                                                      unsigned long long* __restrict__ work_total, HeavyArrays heavy) {
+                                                                      unsigned long long* __restrict__ work_total, unsigned long long* __restrict__ sparse_heavy, HeavyArrays heavy) {
     if (blockIdx.x >= nblocks) {
         heavy_analysis<G>(P, heavy);
         return;
     }
     constexpr int GROUPS = BIN_THREADS / G;
     constexpr int UNR = 4;
+    constexpr int LONG_CTA = 1024;  // long rows of more nonzeros than this are walked by the whole CTA, not by a warp
     __shared__ int32_t hist[NCLASS];
-    __shared__ unsigned long long cta_sum;
+    __shared__ unsigned long long cta_sum, s_work, s_sparse;
+    __shared__ uint16_t s_long[BIN_MAX_TILE];
+    __shared__ int s_nlong;
     if (threadIdx.x < NCLASS) hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) cta_sum = 0;
+    if (threadIdx.x == 0) {
+        cta_sum = s_work = s_sparse = 0;
+        s_nlong = 0;
+    }
     __syncthreads();
     const int gl = threadIdx.x & (G - 1), group = threadIdx.x / G;
     const int64_t rows = P.r1 - P.r0;
     const int64_t t0 = (int64_t)blockIdx.x * tile, t1 = min(t0 + tile, rows);
     const bool sane = (*P.err & ERRW_BAD_CSR) == 0;  // a matrix that failed its checks has no descriptors
     unsigned long long mine = 0;    // work of the rows this thread owned
+    const bool tril = P.mode == SPSYRK_TRIL;
+    auto range_of = [&](int64_t r) { return tril ? (uint32_t)(P.r0 + (int32_t)r) + 1u : (uint32_t)P.m; };
+    // (the lengths of a row's descriptors add up to less than 2^31)
+    auto settle = [&](int64_t r, int32_t deg, uint32_t w, bool full) {  // one thread per row; full: it stores a column of every row of its range
+        const bool dense = full && range_of(r) <= dense_range;
+        P.work[r] = w;
+        int c;
+        const uint32_t wl = diag ? w - deg : w;  // items of a light row
+        if (w == 0) c = 0;
+        else if (deg <= 32 && wl <= 512) c = wl <= 32 ? 1 : wl <= 64 ? 2 : wl <= 128 ? 3 : wl <= 256 ? 4 : 5;
+        else c = w <= block_max ? 6 : 7;
+        cls[r] = (uint8_t)(c | (dense && c >= 6 ? ROW_DENSE : 0));
+        atomicAdd(&hist[c], 1);
+        if (c >= 6 && !dense) atomicAdd(&s_sparse, c == 6 ? 1ull : 1ull << 32);
+        mine += (unsigned long long)w;
+    };
     for (int64_t base = t0; base < t1; base += GROUPS * UNR) {
-        int64_t p0[UNR], w[UNR];
-        int32_t deg[UNR];
+        int64_t p0[UNR];
+        uint32_t w[UNR], full = 0;  // a bit per row
+        int32_t deg[UNR];  // -1: left for the end
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
             const int64_t r = base + u * GROUPS + group;
@@ -302,32 +351,75 @@ static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev
             }
         }
 #pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            if (deg[u] > LONG_STEPS * G) {
+                if (gl == 0) s_long[atomicAdd(&s_nlong, 1)] = (uint16_t)(base + u * GROUPS + group - t0);
+                deg[u] = -1;
+            }
+        }
+#pragma unroll
         for (int u = 0; u < UNR; ++u) w[u] = gl < deg[u] ? P.desc[p0[u] + gl].y : 0;
 #pragma unroll
-        for (int u = 0; u < UNR; ++u)
-            for (int32_t q = gl + G; q < deg[u]; q += G) w[u] += P.desc[p0[u] + q].y;
+        for (int u = 0; u < UNR; ++u) {
+            const uint32_t range = range_of(base + u * GROUPS + group);
+            bool f = w[u] == range;
+            for (int32_t q = gl + G; q < deg[u]; q += G) {
+                const uint32_t len = P.desc[p0[u] + q].y;
+                w[u] += len;
+                f |= len == range;
+            }
+            full |= (uint32_t)f << u;
+        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) full |= __shfl_xor_sync(FULL_MASK, full, o);
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
             const int64_t r = base + u * GROUPS + group;
 #pragma unroll
             for (int o = G / 2; o > 0; o >>= 1) w[u] += __shfl_xor_sync(FULL_MASK, w[u], o);
-            if (r < t1 && gl == 0) {
-                P.work[r] = w[u];
-                int c;
-                const int64_t wl = diag ? w[u] - deg[u] : w[u];  // items of a light row
-                if (w[u] == 0) c = 0;
-                else if (deg[u] <= 32 && wl <= 512) c = wl <= 32 ? 1 : wl <= 64 ? 2 : wl <= 128 ? 3 : wl <= 256 ? 4 : 5;
-                else c = w[u] <= block_max ? 6 : 7;
-                cls[r] = (uint8_t)c;
-                atomicAdd(&hist[c], 1);
-                mine += (unsigned long long)w[u];
+            if (r < t1 && gl == 0 && deg[u] >= 0) settle(r, deg[u], w[u], (full >> u) & 1u);
+        }
+    }
+    __syncthreads();
+    const int nlong = s_nlong;
+    // the long rows: a warp each, or (of more than LONG_CTA nonzeros) all warps together
+    auto walk = [&](int64_t r, int64_t p0, int32_t deg, int32_t first, int32_t step, bool* full) {
+        const uint32_t range = range_of(r);
+        uint32_t w = 0;
+        bool f = false;
+        for (int32_t q = first; q < deg; q += step) {
+            const uint32_t len = P.desc[p0 + q].y;
+            w += len;
+            f |= len == range;
+        }
+        *full = __any_sync(FULL_MASK, f);
+        return warp_reduce_sum<uint32_t>(w);
+    };
+    for (int whole = 0; whole < 2 && nlong > 0; ++whole) {
+        for (int i = whole ? 0 : threadIdx.x >> 5; i < nlong; i += whole ? 1 : BIN_THREADS / 32) {
+            const int64_t r = t0 + s_long[i], p0 = P.rowptr[P.r0 + r];
+            const int32_t deg = (int32_t)(P.rowptr[P.r0 + r + 1] - p0);
+            if ((deg > LONG_CTA) != (whole == 1)) continue;
+            bool full;
+            const uint32_t w = walk(r, p0, deg, whole ? threadIdx.x : lane_id(), whole ? BIN_THREADS : 32, &full);
+            if (!whole) {
+                if (lane_id() == 0) settle(r, deg, w, full);
+                continue;
             }
+            if (lane_id() == 0) atomicAdd(&s_work, (unsigned long long)w | (unsigned long long)full << 32);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                settle(r, deg, (uint32_t)s_work, (s_work >> 32) != 0);
+                s_work = 0;
+            }
+            __syncthreads();
         }
     }
     const unsigned long long ws = warp_reduce_sum<unsigned long long>(mine);
     if (lane_id() == 0 && ws) atomicAdd(&cta_sum, ws);
     __syncthreads();
     if (threadIdx.x == 0 && cta_sum) atomicAdd(work_total, cta_sum);
+    if (threadIdx.x == 0 && s_sparse) atomicAdd(sparse_heavy, s_sparse);
     if (threadIdx.x < NCLASS) blockhist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = hist[threadIdx.x];
 }
 
@@ -347,11 +439,12 @@ struct BinStarts {
 
 // Second half of the counting sort: the rows in class order (ascending inside a class), for each of them the header
 // (row inside the plan's range, position of its first nonzero in A, number of nonzeros) and the words of the item map
-// it needs (its items rounded up to eight; light rows only).  An empty row's count is settled here.
+// it needs (its items rounded up to eight; light rows only).  The counts of empty and of dense rows are settled here.
 static __global__ void __launch_bounds__(BIN_THREADS) row_scatter_kernel(PlanDev P, const uint8_t* __restrict__ cls, int64_t tile,
                                                                          const int64_t* __restrict__ offsets, int64_t nblocks, bool diag,
                                                                          int32_t* __restrict__ perm, uint4* __restrict__ hdr,
-                                                                         uint32_t* __restrict__ items8, int32_t* __restrict__ cnt) {
+                                                                         uint32_t* __restrict__ items8, int32_t* __restrict__ cnt,
+                                                                         uint32_t* __restrict__ block_base, uint32_t blocks_per_row) {
     constexpr int NW = BIN_THREADS / 32;
     __shared__ int64_t running[NCLASS];
     __shared__ int32_t wcount[NW][NCLASS];
@@ -364,7 +457,12 @@ static __global__ void __launch_bounds__(BIN_THREADS) row_scatter_kernel(PlanDev
         int c = -1;
         int64_t p0 = 0, deg = 0, w = 0;
         if (r < t1) {
-            c = cls[r];
+            c = cls[r] & (ROW_DENSE - 1);
+            if (cls[r] & ROW_DENSE) {  // what the counting kernel would find
+                const uint32_t range = P.mode == SPSYRK_TRIL ? (uint32_t)(P.r0 + r) + 1u : (uint32_t)P.m, blocks = (range + BASE_BLOCK - 1) / BASE_BLOCK;
+                cnt[r] = (int32_t)range;
+                for (uint32_t b = 0; b < blocks && blocks <= blocks_per_row; ++b) block_base[(uint64_t)(P.r0 + r) * blocks_per_row + b] = b * BASE_BLOCK;
+            }
             p0 = P.rowptr[P.r0 + r];
             deg = P.rowptr[P.r0 + r + 1] - p0;
             w = P.work[r];
@@ -396,10 +494,11 @@ static __global__ void __launch_bounds__(BIN_THREADS) row_scatter_kernel(PlanDev
 }
 
 // What the host needs to know about a view of the plan, in the order in which it is written for the host
-enum : int { PF_CLASS_START = 0, PF_MAP_ITEMS = NCLASS + 1, PF_WORK, PF_OTHER_THAN_ONE, PF_ERR, PF_WORDS };
+enum : int { PF_CLASS_START = 0, PF_MAP_ITEMS = NCLASS + 1, PF_WORK, PF_OTHER_THAN_ONE, PF_ERR, PF_SPARSE_HEAVY, PF_WORDS };
 struct PlanFacts {
     const int64_t* class_start;
     const unsigned long long* work_total;
+    const unsigned long long* sparse_heavy;  // rows of class 6, and in the upper half of class 7, that are not dense
     const uint32_t* facts;
     const uint32_t* err;
     int64_t* host;
@@ -412,6 +511,7 @@ struct PlanFacts {
         w[PF_WORK] = (int64_t)*work_total;
         w[PF_OTHER_THAN_ONE] = (int64_t)facts[0];
         w[PF_ERR] = (int64_t)*err;
+        w[PF_SPARSE_HEAVY] = (int64_t)*sparse_heavy;
 #pragma unroll
         for (int c = 0; c < PF_WORDS; ++c) host[c] = w[c];
     }
