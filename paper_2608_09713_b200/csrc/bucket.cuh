@@ -2,9 +2,9 @@
 // of the mirror.
 //
 // A CTA holds a tile of THREADS * ITEMS elements in registers (a warp owns consecutive ones, 32 per step),
-// ranks every element among the equal bins of its warp (one vote per bin bit, counters of 16 bits per
-// warp and bin in shared memory), turns the counters of all warps into slots of the tile in bin order,
-// drops the elements into their slots and writes the tile out in runs of one bin.  Offsets of the bins in
+// ranks every element among the equal bins of its warp (counters of 16 bits per warp and bin in shared memory), turns the
+// counters of all warps into slots of the tile in bin order, drops the elements into their slots, looks whether equal bins
+// kept their order and writes the tile out in runs of one bin.  Offsets of the bins in
 // the output stay in the registers of the thread that owns the bin and are carried from tile to tile, so
 // a CTA that walks a long range of elements needs one offset per bin for all of it.
 #pragma once
@@ -12,39 +12,73 @@
 
 namespace spsyrk {
 
-// Ranks of a warp's elements among the earlier elements of the warp with the same bin.  bin(i) is the bin of step i
-// (counts where bit i of `valid` is set); `count` are the warp's counters, zero on entry, the warp's totals
-// on return.  The votes run bit by bit over all steps, so that the votes of different steps overlap (with all bits of
-// one step after the other a warp waits for each of its votes: 6.6 ms against 4.9 for a pass over 5.4e8 records).
+// What the lanes of a warp may do in any order.  The bounds-checked build takes the odd lanes first, so that what relies on
+// another order is found out.  What follows comes after it.
+template <typename F>
+__device__ __forceinline__ void in_any_order(F f) {
+#ifdef SPSYRK_CHECKED
+    if (lane_id() & 1) f();
+    __syncwarp();
+    if (!(lane_id() & 1)) f();
+#else
+    f();
+#endif
+    __syncwarp();
+}
+
+// Ranks of a warp's elements among the elements of the warp with the same bin: what an atomic add to the warp's counter of
+// the bin returns (two counters per word).  bin(i) is the bin of step i (counts where bit i of `valid` is set); `count` are
+// the warp's counters, zero on entry, the warp's totals on return.  Elements of one bin get different ranks, but which of them
+// comes first is up to the hardware: bucket_in_order looks at the sorted tile.  (One vote per bit of the bin and a step of the
+// lowest lane for its equals before, nine votes of three instructions per 32 elements on 18-bit columns: mirror of 6.4e8
+// single-precision entries 15.2 ms, now 13.9.  The radix and record passes keep their votes: with atomic adds and a look at their
+// tiles they took as long, and longer where many lanes meet in one counter - banded matrix, 7.04 ms against 6.86.)
 template <int ITEMS, typename Bin>
-__device__ __forceinline__ void bucket_rank(Bin bin, uint32_t valid, int bits, uint16_t* count, uint32_t (&rk)[ITEMS]) {
-    const int lane = lane_id();
-#pragma unroll
-    for (int i = 0; i < ITEMS; ++i) rk[i] = __ballot_sync(FULL_MASK, (valid >> i) & 1u);  // lanes with the same bin so far
-#pragma unroll 1
-    for (int bit = 0; bit < bits; ++bit) {
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const bool set = (bin(i) >> bit) & 1u;
-            const unsigned bal = __ballot_sync(FULL_MASK, set);
-            rk[i] &= set ? bal : ~bal;
-        }
-    }
-    // the lowest lane of every group of equal bins moves the warp's counter
-    const uint32_t below = (1u << lane) - 1u;
+__device__ __forceinline__ void bucket_rank(Bin bin, uint32_t valid, uint16_t* count, uint32_t (&rk)[ITEMS]) {
+    uint32_t* words = reinterpret_cast<uint32_t*>(count);
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const bool on = (valid >> i) & 1u;
-        const int leader = on ? __ffs(rk[i]) - 1 : lane;
-        uint32_t prev = 0;
-        if (on && lane == leader) {
-            uint16_t* c = count + bin(i);
-            prev = *c;
-            *c = (uint16_t)(prev + __popc(rk[i]));
-        }
-        rk[i] = __shfl_sync(FULL_MASK, prev, leader) + __popc(rk[i] & below);
-        __syncwarp();
+        const uint32_t d = bin(i), shift = (d & 1u) * 16u;
+        rk[i] = 0;
+        in_any_order([&] {
+            if ((valid >> i) & 1u) rk[i] = (atomicAdd(words + (d >> 1), 1u << shift) >> shift) & 0xffffu;
+        });
     }
+}
+
+// Puts the tile in order where bucket_rank did not: slots [0, total) hold the elements in bin order; wrong(q) tells whether slots
+// q and q + 1 are of one bin and the wrong way round (an element must stand behind those that came before it), exchange(q)
+// exchanges them.  `bad`: the calling thread has seen such a pair.  Every thread calls it; true if the tile was changed.
+// Only elements of one step of a warp can be the wrong way round, 32 neighbours at most, which as many turns put right; what is
+// out of order for another reason (an input that failed its checks) stays so.  (The lanes of a step are served in their
+// order on the hardware this was measured on, so that one look is all it takes.)
+template <int THREADS, typename Wrong, typename Exchange>
+__device__ __forceinline__ bool bucket_in_order(bool bad, int total, Wrong wrong, Exchange exchange) {
+    bool changed = false;
+#pragma unroll 1
+    for (int turn = 0; turn < 32; ++turn) {  // odd-even transposition
+        if (!__syncthreads_or(bad)) return changed;
+        changed = true;
+        bad = false;
+#pragma unroll 1
+        for (int parity = 0; parity < 2; ++parity) {
+            for (int q = 2 * threadIdx.x + parity; q + 1 < total; q += 2 * THREADS) {
+                if (wrong(q)) {
+                    exchange(q);
+                    bad = true;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    return changed;
+}
+
+template <typename T>
+__device__ __forceinline__ void exchange_slots(T* a, int q) {
+    const T t = a[q];
+    a[q] = a[q + 1];
+    a[q + 1] = t;
 }
 
 // Warp counters -> first slot of every (warp, bin) in the tile's bin-major order.  Thread t owns bins 4 t .. 4 t + 3

@@ -25,7 +25,7 @@
 // A pass is bound by the load/store pipe and by what a CTA waits for at its barriers, 75 to 100 cycles per 32 entries and
 // SM.  128 registers (two CTAs of 256 threads) hold a tile without spills; three to five CTAs with fewer registers
 // took 1.2 to 2 times as long.  6.4e8 single-precision entries with 18-bit columns (the large power-law workload):
-// the whole mirror 15.3 ms; three passes of 8-bit digits took 15.0, the (key, row) expansion that `split` does without 2.0 and
+// the whole mirror 13.9 ms (15.2 with ranks by votes); three passes of 8-bit digits took 15.0, the (key, row) expansion that `split` does without 2.0 and
 // their histograms and scans 2.8, beside the lower parts.
 #pragma once
 #include "bucket.cuh"
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
         const auto bin = [&](int i) { return key[i] & (uint32_t)(nb - 1); };
         uint32_t rk[ITEMS];
         uint16_t* mycount = count + warp * nb;
-        bucket_rank<ITEMS>(bin, valid, A.lbits, mycount, rk);
+        bucket_rank<ITEMS>(bin, valid, mycount, rk);
         __syncthreads();
         const int total = bucket_offsets<MS_THREADS>(count, nb, scratch, gbase, s_goff);
 #pragma unroll
@@ -395,6 +395,17 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
         }
         __syncthreads();
         bucket_clear_counts<MS_THREADS>(count, nb);
+        const auto key_at = [&](int q) { if constexpr (SM::KEYS) return s_key[q]; else return s_rec[q].x; };
+        const auto row_at = [&](int q) { if constexpr (SM::KEYS) return s_rec[q].x; else return s_rec[q].y; };
+        // (rows ascend; entries of one row are of different columns, so their order does not matter)
+        const auto wrong = [&](int q) { return ((key_at(q) ^ key_at(q + 1)) & (uint32_t)(nb - 1)) == 0 && row_at(q) > row_at(q + 1); };
+        bool bad = false;
+#pragma unroll 4
+        for (int q = tid; q < total - 1; q += MS_THREADS) bad |= wrong(q);
+        bucket_in_order<MS_THREADS>(bad, total, wrong, [&](int q) {
+            exchange_slots(s_rec, q);
+            if constexpr (SM::KEYS) exchange_slots(s_key, q);
+        });
 #pragma unroll 4
         for (int q = tid; q < total; q += MS_THREADS) {
             const typename T::Rec r = s_rec[q];
@@ -453,7 +464,7 @@ static __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<uint32_t>:
         __syncthreads();  // the last tile has left shared memory, the counters are clear
         uint32_t rk[ITEMS];
         uint16_t* mycount = count + warp * nb;
-        bucket_rank<ITEMS>(bin, valid, A.mbits, mycount, rk);
+        bucket_rank<ITEMS>(bin, valid, mycount, rk);
         __syncthreads();
         const int total = bucket_offsets<MS_THREADS>(count, nb, scratch, gbase, s_goff);
 #pragma unroll
@@ -467,6 +478,14 @@ static __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<uint32_t>:
         }
         __syncthreads();
         bucket_clear_counts<MS_THREADS>(count, nb);
+        const auto wrong = [&](int q) { return ((s_rest[q] ^ s_rest[q + 1]) & (uint32_t)(nb - 1)) == 0 && s_rec[q].x > s_rec[q + 1].x; };
+        bool bad = false;
+#pragma unroll 4
+        for (int q = tid; q < total - 1; q += MS_THREADS) bad |= wrong(q);
+        bucket_in_order<MS_THREADS>(bad, total, wrong, [&](int q) {
+            exchange_slots(s_rec, q);
+            exchange_slots(s_rest, q);
+        });
 #pragma unroll 4
         for (int q = tid; q < total; q += MS_THREADS) {
             const typename T::Rec r = s_rec[q];
@@ -538,7 +557,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
         __syncthreads();  // the last tile has left shared memory, the counters are clear
         uint32_t rk[ITEMS];
         uint16_t* mycount = count + warp * nb;
-        bucket_rank<ITEMS>(bin, valid, A.hbits, mycount, rk);
+        bucket_rank<ITEMS>(bin, valid, mycount, rk);
         __syncthreads();
         const int total = bucket_offsets<MS_THREADS>(count, nb, scratch, gbase, s_goff);
 #pragma unroll
@@ -558,6 +577,14 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
         }
         __syncthreads();
         bucket_clear_counts<MS_THREADS>(count, nb);
+        const auto wrong = [&](int q) { return s_bin[q] == s_bin[q + 1] && s_row[q] > s_row[q + 1]; };
+        bool bad = false;
+#pragma unroll 4
+        for (int q = tid; q < total - 1; q += MS_THREADS) bad |= wrong(q);
+        bucket_in_order<MS_THREADS>(bad, total, wrong, [&](int q) {
+            exchange_slots(s_row, q);
+            exchange_slots(s_val, q);
+        });
 #pragma unroll 4
         for (int q = tid; q < total; q += MS_THREADS) {
             const uint32_t bin = s_bin[q], r = s_row[q];
