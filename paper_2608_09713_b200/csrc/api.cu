@@ -154,7 +154,10 @@ struct spsyrk_plan_s {
     uint32_t* block_base;   // entries of a heavy row before every block of columns, [row][blocks_per_row]
     uint32_t blocks_per_row;
     RoutePieces sub_route[NROUTE];  // with sub_active: the pieces of the heavy rows' lists to compute
-    unsigned long long* route_state;  // both views: [ticket, words of the look-back] each, as many as their heavy rows need
+    // status words of the scan of the counts (the last ones of count_state_words), then for both views [ticket, words of the look-back], as
+    // many as their heavy rows need
+    unsigned long long* count_state;
+    size_t count_state_words;
     uint32_t* facts;       // binary analysis (device): differs-from-one flag, heavy columns, threshold, histogram
     uint8_t* heavy_id;
     uint32_t* heavy_mask;
@@ -246,7 +249,8 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     static_assert(ROUTE_WIDE == NROUTE - 1, "the list that may hold all rows is the last");
     const int64_t route_cap = std::min<int64_t>(rows, ROW_CHUNK_BITS_MAX_NUMERIC);
     auto route_list = c.take<int32_t>(ROUTE_WIDE * route_cap + rows);
-    auto route_state = c.take<unsigned long long>(views * (1 + (size_t)route_tiles(m) * NROUTE));
+    const size_t count_state_words = (size_t)scan_partials_count(rows);
+    auto count_state = c.take<unsigned long long>(count_state_words + views * (1 + (size_t)route_tiles(m) * NROUTE));
     // Rows that the rank kernel takes in parts: their range has at most 2^18 columns and more than the slots hold
     const int64_t ranged = std::min<int64_t>(m, ROW_CHUNK_BITS_MAX_NUMERIC);
     const int64_t slots = rank_slots_big<double>(pow2_at_least((uint64_t)m, 1024u, ROW_CHUNK_BITS_MAX_NUMERIC)), part = slots - BASE_BLOCK;
@@ -293,7 +297,7 @@ size_t carve(spsyrk_plan_s* pl, spsyrk_plan_s* up, void* ws, int64_t m, int64_t 
     }
     if (pl) {
         pl->desc_hi = desc_hi; pl->cnt_tot = cnt_tot; pl->hi_begin = hi_begin; pl->work_sum = work_sum;
-        pl->route_count = route_count; pl->route_list = route_list; pl->route_state = route_state; pl->rank_parts = rank_parts;
+        pl->route_count = route_count; pl->route_list = route_list; pl->count_state = count_state; pl->count_state_words = count_state_words; pl->rank_parts = rank_parts;
         pl->block_base = block_base; pl->blocks_per_row = blocks_per_row;
         pl->dev.mask_stride = mask_stride;
         pl->work_prefix = work_prefix; pl->part_bounds = part_bounds; pl->itemoff = itemoff;
@@ -415,11 +419,12 @@ void launch_row_work(spsyrk_plan_s* pl, bool analyse, cudaStream_t st) {
     HeavyArrays heavy{pl->colcnt, pl->facts, pl->heavy_id, pl->heavy_mask, 0u};
     if (analyse) heavy.ctas = (unsigned)std::min<int64_t>(2 + std::max<int64_t>(P.n, (int64_t)P.m * G) / BIN_THREADS, (int64_t)pl->sm_count * 8);
     if (nb > 0)
-        row_work_kernel<G><<<(unsigned)nb + heavy.ctas, BIN_THREADS, 0, st>>>(P, pl->cls, BLOCK_CLASS_MAX_WORK, ROW_CHUNK_BITS_MAX_SYMBOLIC, pl->diag, bin_tile(rows), pl->blockhist, nb,
-                                                                             pl->work_total_dev, pl->work_total_dev + 1, heavy);
-    else if (analyse) heavy_analysis_kernel<G><<<heavy.ctas, BIN_THREADS, 0, st>>>(P, heavy);
-    else return;
-    note_launches(1);
+        launch_linked(row_work_kernel<G>, (unsigned)nb + heavy.ctas, BIN_THREADS, 0, st, P, pl->cls, BLOCK_CLASS_MAX_WORK, ROW_CHUNK_BITS_MAX_SYMBOLIC, pl->diag,
+                      bin_tile(rows), pl->blockhist, nb, pl->work_total_dev, pl->work_total_dev + 1, heavy);
+    else if (analyse) {
+        heavy_analysis_kernel<G><<<heavy.ctas, BIN_THREADS, 0, st>>>(P, heavy);
+        note_launches(1);
+    }
 }
 
 int group_width(int64_t nnz, int64_t m) {
@@ -491,8 +496,8 @@ spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, int64_t* gave_up, b
         return SPSYRK_OK;
     }
     SPSYRK_CUDA_TRY(scan_launch(ScanArray<int32_t>{pl->blockhist}, NCLASS * nb, BinStarts{pl->offsets, (uint32_t)nb, pl->class_start_dev}, pl->state_bin, P.err, st, true));
-    row_scatter_kernel<<<(unsigned)nb, BIN_THREADS, 0, st>>>(P, pl->cls, bin_tile(rows), pl->offsets, nb, pl->diag, pl->perm, pl->hdr, pl->items8, pl->cnt, pl->block_base, pl->blocks_per_row);
-    note_launches(1);
+    SPSYRK_CUDA_TRY(launch_linked(row_scatter_kernel, (unsigned)nb, BIN_THREADS, 0, st, P, pl->cls, bin_tile(rows), pl->offsets, nb, pl->diag, pl->perm, pl->hdr, pl->items8,
+                                  pl->cnt, pl->block_base, pl->blocks_per_row));
     SPSYRK_CUDA_TRY(scan_launch(ScanArray<uint32_t>{pl->items8}, rows, ItemStarts{pl->itemoff, rows, facts}, pl->state_items, P.err, st, true));
     return SPSYRK_OK;
 }
@@ -774,22 +779,31 @@ spsyrk_status_t route_heavy(spsyrk_plan_s* pl, unsigned long long* state, cudaSt
     const int64_t count = heavy_rows(pl);
     if (count <= 0) return SPSYRK_OK;
     const HeavyShapes h = pl->dtype == SPSYRK_I32 ? heavy_shapes<int32_t>(pl) : heavy_shapes<double>(pl);
-    route_rows_kernel<<<(unsigned)route_tiles(count), ROUTE_THREADS, 0, st>>>(pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt, pl->block_base,
-                                                                              pl->blocks_per_row, pl->route_list, pl->route_cap, pl->rank_parts,
-                                                                              pl->class_start[NCLASS] - pl->class_start[7], pl->route_count, state + 1, state);
-    note_launches(1);
-    SPSYRK_CUDA_TRY(cudaGetLastError());
+    SPSYRK_CUDA_TRY(launch_linked(route_rows_kernel, (unsigned)route_tiles(count), ROUTE_THREADS, 0, st, pl->dev, h.rule, pl->perm + pl->class_start[6], count, pl->cnt,
+                                  pl->block_base, pl->blocks_per_row, pl->route_list, pl->route_cap, pl->rank_parts, pl->class_start[NCLASS] - pl->class_start[7],
+                                  pl->route_count, state + 1, state));
+    return SPSYRK_OK;
+}
+
+// Clears what the counting pass's last steps need zero, in one piece: the status words of the scan of the counts, then the
+// state of the routing (both views).  Before the counting kernels, so that nothing stands between them and those steps.
+spsyrk_status_t clear_count_state(spsyrk_plan_s* pl, int64_t rows, cudaStream_t st) {
+    spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
+    const bool heavy = heavy_rows(pl) || (up && heavy_rows(up));
+    const size_t words = heavy ? 1 + (size_t)route_tiles(heavy_rows(pl)) * NROUTE + (up ? 1 + (size_t)route_tiles(heavy_rows(up)) * NROUTE : 0) : 0;
+    const size_t first = (size_t)(pl->count_state_words - scan_partials_count(rows));  // the scan's words end where the routing's begin
+    if (rows > SCAN_MIN_TILE || heavy)
+        SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->count_state + first, 0, (pl->count_state_words - first + words) * sizeof(unsigned long long), st));
     return SPSYRK_OK;
 }
 
 // the lists of both views; without heavy rows nothing is launched and nobody looks at the list lengths
 spsyrk_status_t route_views(spsyrk_plan_s* pl, cudaStream_t st) {
     spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
-    const size_t words = 1 + (size_t)route_tiles(heavy_rows(pl)) * NROUTE, up_words = up ? 1 + (size_t)route_tiles(heavy_rows(up)) * NROUTE : 0;
     if (!heavy_rows(pl) && !(up && heavy_rows(up))) return SPSYRK_OK;
-    SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->route_state, 0, (words + up_words) * sizeof(unsigned long long), st));
-    const spsyrk_status_t s = route_heavy(pl, pl->route_state, st);
-    return s == SPSYRK_OK && up ? route_heavy(up, pl->route_state + words, st) : s;
+    unsigned long long* const state = pl->count_state + pl->count_state_words;
+    const spsyrk_status_t s = route_heavy(pl, state, st);
+    return s == SPSYRK_OK && up ? route_heavy(up, state + 1 + (size_t)route_tiles(heavy_rows(pl)) * NROUTE, st) : s;
 }
 
 // A launch of one CTA per row or part of one (the CTAs that start take the others over): a brief one if there are few per CTA
@@ -901,9 +915,11 @@ struct CountsOut {
 static_assert(2 + 2 * NROUTE <= 32, "the totals take the first half of the host block");
 
 // prefix sums of per-row counts into out[rows + 1]; what the host needs is on its way
-cudaError_t scan_counts(spsyrk_plan_s* pl, const int32_t* counts, int64_t rows, int64_t* out, cudaStream_t st) {
+// (cleared: clear_count_state has been called for this scan)
+cudaError_t scan_counts(spsyrk_plan_s* pl, const int32_t* counts, int64_t rows, int64_t* out, bool cleared, cudaStream_t st) {
     if (rows == 0) return cudaMemsetAsync(out, 0, sizeof(int64_t), st);
-    return scan_launch(ScanArray<int32_t>{counts}, rows, CountsOut{out, rows, pl->dev.err, pl->route_count, pl->host.dev}, pl->partials, pl->dev.err, st);
+    int64_t* const state = cleared ? reinterpret_cast<int64_t*>(pl->count_state + pl->count_state_words - scan_partials_count(rows)) : pl->partials;
+    return scan_launch(ScanArray<int32_t>{counts}, rows, CountsOut{out, rows, pl->dev.err, pl->route_count, pl->host.dev}, state, pl->dev.err, st, cleared);
 }
 // waits for it
 spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, bool routes, int64_t* total, cudaStream_t st) {
@@ -1122,7 +1138,8 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t
     const int64_t rows = pl->dev.r1 - pl->dev.r0;
     const bool with_map = use_map(pl);
     Chain ch{st, !pl->timing};
-    spsyrk_status_t s = symbolic_view(pl, with_map, ch);
+    spsyrk_status_t s = clear_count_state(pl, rows, st);
+    if (s == SPSYRK_OK) s = symbolic_view(pl, with_map, ch);
     if (s != SPSYRK_OK) return s;
     const int32_t* counts = pl->cnt;
     spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
@@ -1141,7 +1158,7 @@ spsyrk_status_t spsyrk_symbolic(spsyrk_plan_t plan, int64_t* d_c_rowptr, int64_t
         }
         counts = pl->cnt_tot;
     }
-    SPSYRK_CUDA_TRY(scan_counts(pl, counts, rows, d_c_rowptr, st));
+    SPSYRK_CUDA_TRY(scan_counts(pl, counts, rows, d_c_rowptr, true, st));
     if (pl->upper_active && rows > 0) {
         // the upper part of row r starts after its lower part
         upper_begin_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(d_c_rowptr, pl->cnt, rows, pl->hi_begin);
@@ -1258,7 +1275,8 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
     pl->have_onepass = false;
     // heavy rows: their counts come from their own kernels (bitmaps), as in the symbolic pass
     Chain ch{st, !pl->timing};
-    spsyrk_status_t s = launch_symbolic_cta<256>(pl, 6, ch);
+    spsyrk_status_t s = clear_count_state(pl, rows, st);
+    if (s == SPSYRK_OK) s = launch_symbolic_cta<256>(pl, 6, ch);
     if (s != SPSYRK_OK) return s;
     s = launch_symbolic_cta<1024>(pl, 7, ch);
     if (s == SPSYRK_OK) s = route_views(pl, st);
@@ -1267,7 +1285,7 @@ spsyrk_status_t spsyrk_onepass_slots(spsyrk_plan_t plan, int64_t* slot_entries, 
         onepass_slots_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(pl->dev, pl->cls, pl->cnt, pl->diag, rows, pl->ub);
         note_launches(1);
     }
-    SPSYRK_CUDA_TRY(scan_counts(pl, pl->ub, rows, pl->ub_off, st));
+    SPSYRK_CUDA_TRY(scan_counts(pl, pl->ub, rows, pl->ub_off, true, st));
     s = collect_total(pl, rows, true, slot_entries, st);
     if (s != SPSYRK_OK) return s;
     pl->have_onepass = true;
@@ -1299,7 +1317,7 @@ spsyrk_status_t spsyrk_onepass_numeric(spsyrk_plan_t plan, int32_t* d_slot_colid
     pl->cnt_out = nullptr;
     pl->map_filled = map_was;
     if (s != SPSYRK_OK) return s;
-    SPSYRK_CUDA_TRY(scan_counts(pl, pl->cnt, rows, d_c_rowptr, st));
+    SPSYRK_CUDA_TRY(scan_counts(pl, pl->cnt, rows, d_c_rowptr, false, st));
     return collect_total(pl, rows, false, nnz_out, st);
 }
 

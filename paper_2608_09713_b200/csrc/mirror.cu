@@ -34,6 +34,8 @@ constexpr int64_t MIRROR_BUCKET_ROWS_8 = 65536;
 bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCKET_ROWS_8; }
 struct MirrorWs {
     int64_t* partials;
+    int64_t *split_state, *mid_state;  // bucket sort: status words of the scans, in one piece with `partials`, state_words long
+    int64_t state_words;
     uint32_t* err;       // [0] error word, [1] number of diagonal entries, [2] finished CTAs
     uint32_t* hist;      // counts of the passes and their prefix sums
     int64_t *offsets, *mid_off;
@@ -189,7 +191,11 @@ size_t carve(MirrorWs* w, void* ws, int64_t m, int64_t nnz_l, size_t sv) {
         t.diagf = (uint8_t*)take(items);
         t.cnt = (uint32_t*)take(items * 4);
         t.fstart = (int64_t*)take(items * 8);
-        t.partials = (int64_t*)take(scan_partials_count(std::max<int64_t>(items, hist_n)) * 8);
+        const int64_t row_words = scan_partials_count(items), split_words = scan_partials_count(sp.split_hist()), mid_words = sp.mbits ? scan_partials_count(sp.mid_hist()) : 0;
+        t.state_words = row_words + split_words + mid_words;
+        t.partials = (int64_t*)take(t.state_words * 8);
+        t.split_state = t.partials + row_words;
+        t.mid_state = t.split_state + split_words;
         t.hist = (uint32_t*)take(hist_n * 4);
         t.offsets = (int64_t*)take((sp.split_hist() + 1) * 8);
         t.mid_off = (int64_t*)take((sp.mid_hist() + 1) * 8);
@@ -271,6 +277,7 @@ __global__ void __launch_bounds__(256) mirror_copy_lower_kernel(const int64_t* _
                                                                 V* __restrict__ f_vals) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
+    link(f_rowptr);
     if (r >= m) return;
     const int64_t p0 = l_rowptr[r], p1 = l_rowptr[r + 1];
     const int64_t fb = f_rowptr[r] - p0;
@@ -306,8 +313,8 @@ template <typename V>
 void mirror_copy_lower(int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx, const void* l_vals, const int64_t* f_rowptr, int32_t* f_colidx,
                        void* f_vals, cudaStream_t st) {
 #define COPY(G)                                                                                                                                       \
-    mirror_copy_lower_kernel<V, G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, static_cast<const V*>(l_vals), m, f_rowptr, \
-                                                                                    f_colidx, static_cast<V*>(f_vals))
+    launch_linked(mirror_copy_lower_kernel<V, G>, (unsigned)((m * G + 255) / 256), 256, 0, st, l_rowptr, l_colidx, static_cast<const V*>(l_vals), m, f_rowptr, \
+                  f_colidx, static_cast<V*>(f_vals))
     switch (group_width(nnz_l, m)) {
         case 4: COPY(4); break;
         case 8: COPY(8); break;
@@ -315,7 +322,6 @@ void mirror_copy_lower(int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const 
         default: COPY(32); break;
     }
 #undef COPY
-    note_launches(1);
 }
 
 // row lengths of F: the row's own entries and those of its column, the diagonal once
@@ -385,33 +391,31 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     SPSYRK_CUDA_TRY(allow_shared_memory<mirror_split_kernel<VB>>());
     SPSYRK_CUDA_TRY(allow_shared_memory<mirror_place_kernel<VB>>());
     mirror_mark(0, st);
-#define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf, w.cnt, w.pieces)
+#define ROWS(G) mirror_rows_kernel<G><<<(unsigned)((m * G + 255) / 256), 256, 0, st>>>(l_rowptr, l_colidx, m, nnz_l, w.step_row, w.diagf, w.cnt, w.pieces, w.partials, w.state_words)
     if (g <= 16) ROWS(4); else ROWS(16);
 #undef ROWS
-    mirror_split_count_kernel<<<(unsigned)sp.nchunks, MS_THREADS, 0, st>>>(a, w.hist);
-    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.split_hist(), w.offsets, w.partials, w.err, st));
-    mirror_split_kernel<VB><<<(unsigned)sp.nchunks, MS_THREADS, split_smem, st>>>(a);
-    note_launches(3);
+    note_launches(1);
+    SPSYRK_CUDA_TRY(launch_linked(mirror_split_count_kernel, (unsigned)sp.nchunks, MS_THREADS, 0, st, a, w.hist));
+    SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.split_hist(), w.offsets, w.split_state, w.err, st, true));
+    SPSYRK_CUDA_TRY(launch_linked(mirror_split_kernel<VB>, (unsigned)sp.nchunks, MS_THREADS, split_smem, st, a));
     mirror_mark(1, st);
     int pass = 2;
     if (three) {
         const unsigned units = (unsigned)sp.mid_units;
-        mirror_mid_count_kernel<<<units, MS_THREADS, 0, st>>>(a, w.hist);
-        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.partials, w.err, st));
+        SPSYRK_CUDA_TRY(launch_linked(mirror_mid_count_kernel, units, MS_THREADS, 0, st, a, w.hist));
+        SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.hist, sp.mid_hist(), w.mid_off, w.mid_state, w.err, st, true));
         const size_t mid_smem = MirrorMidSmem::bytes(1 << sp.mbits);
         SPSYRK_CUDA_TRY(allow_shared_memory<mirror_mid_kernel>());
-        mirror_mid_kernel<<<units, MS_THREADS, mid_smem, st>>>(a);
-        note_launches(2);
+        SPSYRK_CUDA_TRY(launch_linked(mirror_mid_kernel, units, MS_THREADS, mid_smem, st, a));
         mirror_mark(pass++, st);
     }
     const unsigned place_units = (unsigned)(sp.nbuckets() + sp.max_pieces);
-    mirror_column_count_kernel<<<place_units, MS_THREADS, 0, st>>>(a, last_high);
-    SPSYRK_CUDA_TRY(scan_launch(MirrorRowLength{l_rowptr, w.cnt, w.diagf}, m, MirrorRowStart{l_rowptr, w.diagf, f_rowptr, w.fstart, m}, w.partials, w.err, st));
-    mirror_place_kernel<VB><<<place_units, MS_THREADS, place_smem, st>>>(a);
+    SPSYRK_CUDA_TRY(launch_linked(mirror_column_count_kernel, place_units, MS_THREADS, 0, st, a, (const uint16_t*)last_high));
+    SPSYRK_CUDA_TRY(scan_launch(MirrorRowLength{l_rowptr, w.cnt, w.diagf}, m, MirrorRowStart{l_rowptr, w.diagf, f_rowptr, w.fstart, m}, w.partials, w.err, st, true));
+    SPSYRK_CUDA_TRY(launch_linked(mirror_place_kernel<VB>, place_units, MS_THREADS, place_smem, st, a));
     mirror_mark(pass, st);
     g_mirror_passes = pass;
     mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
-    note_launches(2);
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
     {

@@ -122,7 +122,9 @@ __device__ __forceinline__ void ms_count(int64_t e0, int64_t e1, int bits, uint3
 template <int G>
 static __global__ void __launch_bounds__(256) mirror_rows_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx, int64_t m,
                                                                  int64_t n, int32_t* __restrict__ step_row, uint8_t* __restrict__ diagf,
-                                                                 uint32_t* __restrict__ cnt, uint32_t* __restrict__ pieces) {
+                                                                 uint32_t* __restrict__ cnt, uint32_t* __restrict__ pieces, int64_t* __restrict__ scan_state,
+                                                                 int64_t scan_words) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < scan_words; i += (int64_t)gridDim.x * blockDim.x) scan_state[i] = 0;
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
     if (r >= m) return;
@@ -137,6 +139,7 @@ static __global__ void __launch_bounds__(256) mirror_rows_kernel(const int64_t* 
 
 // entries per (low part, chunk)
 static __global__ void __launch_bounds__(MS_THREADS) mirror_split_count_kernel(MirrorSortArgs A, uint32_t* __restrict__ hist) {
+    link();
     const int64_t e0 = (int64_t)blockIdx.x * A.chunk, e1 = min(e0 + A.chunk, A.n);
     const uint32_t mask = (1u << A.lbits) - 1u;
     ms_count<8>(e0, e1, A.lbits, hist + blockIdx.x, A.nchunks, [&](int64_t e) { return ms_key(A.l_colidx[e], A.m) & mask; });
@@ -177,6 +180,7 @@ __device__ __forceinline__ void ms_mid_piece(const MirrorSortArgs& A, int unit, 
 }
 
 static __global__ void __launch_bounds__(MS_THREADS) mirror_mid_count_kernel(MirrorSortArgs A, uint32_t* __restrict__ hist) {
+    link(A.mid_first, A.mid_bucket, A.split_off, A.high_a);
     int64_t e0, e1;
     ms_mid_piece(A, blockIdx.x, &e0, &e1);
     const uint32_t mask = (1u << A.mbits) - 1u;
@@ -227,6 +231,7 @@ __device__ __forceinline__ bool ms_unit(const MirrorSortArgs& A, int64_t u, Mirr
 static __global__ void __launch_bounds__(MS_THREADS) mirror_column_count_kernel(MirrorSortArgs A, const uint16_t* __restrict__ high) {
     __shared__ uint32_t h[MS_MAX_BINS];
     MirrorUnit unit;
+    link(high);
     if (!ms_unit(A, blockIdx.x, &unit)) return;
     const int nb = 1 << A.hbits;
     for (int d = threadIdx.x; d < nb; d += MS_THREADS) h[d] = 0;
@@ -298,6 +303,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     uint32_t* rows_of_warp = reinterpret_cast<uint32_t*>(ms_smem) + warp * (CHUNK + 1);
     static_assert((size_t)MS_WARPS * (CHUNK + 1) * 4 <= (size_t)TILE * sizeof(typename T::Rec), "rows fit the tile's space");
     uint32_t* bits = s_bits[warp];
+    link(A.split_off, A.step_row);
     if (A.mbits == 0) ms_place_pieces(A);
     else if (blockIdx.x == 0) ms_mid_pieces(A, scratch);
     const int64_t e0 = (int64_t)blockIdx.x * A.chunk, e1 = min(e0 + A.chunk, A.n);
@@ -435,6 +441,7 @@ static __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<uint32_t>:
     uint16_t* count = reinterpret_cast<uint16_t*>(s_goff + nb);                 // [WARPS][nb]
     uint16_t* s_rest = count + MS_WARPS * nb;                                   // [TILE]
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    link(A.mid_off, A.rec_a, A.rec_a_tail, A.high_a);
     ms_place_pieces(A);
     int64_t e0, e1;
     ms_mid_piece(A, blockIdx.x, &e0, &e1);
@@ -517,6 +524,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     uint16_t* s_bin = count + MS_WARPS * nb;                             // [TILE]
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     MirrorUnit unit;
+    link(A.rec_b, A.high_b, A.fstart);
     if (!ms_unit(A, blockIdx.x, &unit)) return;
     const int64_t b0 = unit.e0, b1 = unit.e1, col0 = unit.bucket;  // column of bin 0
     int64_t gbase[4];

@@ -94,6 +94,7 @@ template <bool COUNTED, typename Also>
 static __global__ void __launch_bounds__(RX_THREADS) radix_bins_kernel(const uint32_t* __restrict__ in, int64_t n, int passes, unsigned long long* __restrict__ bins,
                                                                        Also also) {
     __shared__ uint32_t h[RX_MAX_PASSES][RX_BINS];
+    link(in);
     for (int d = threadIdx.x; d < RX_MAX_PASSES * RX_BINS; d += RX_THREADS) (&h[0][0])[d] = 0;
     __syncthreads();
     // a CTA counts fewer than 2^32 elements: the sum of all weights of a matrix is below 2^31, and keys are one each
@@ -119,9 +120,7 @@ template <bool COUNTED, typename Also = RadixBinsOnly>
 inline cudaError_t radix_bins(const uint32_t* in, int64_t n, int passes, unsigned long long* bins, cudaStream_t st, Also also = {}) {
     if (n <= 0) return cudaSuccess;
     const int64_t ctas = std::min<int64_t>((n + RX_THREADS * 4 - 1) / (RX_THREADS * 4), 148 * 4);
-    radix_bins_kernel<COUNTED, Also><<<(unsigned)ctas, RX_THREADS, 0, st>>>(in, n, passes, bins, also);
-    note_launches(1);
-    return cudaGetLastError();
+    return launch_linked(radix_bins_kernel<COUNTED, Also>, (unsigned)ctas, RX_THREADS, 0, st, in, n, passes, bins, also);
 }
 
 template <int BITS, typename PB, bool HAS_PC = false>
@@ -173,6 +172,7 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
 
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     static_assert(NB == RX_BINS && NB <= RX_THREADS, "one thread per digit");
+    link(keys, pa, pb, bins);  // (pc is read behind the barriers of the ranking)
     if (tid == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
     const int64_t tile = s_tile, tile_base = tile * RX_TILE;
@@ -306,10 +306,8 @@ inline cudaError_t radix_pass_launch(const uint32_t* keys, const uint32_t* pa, c
     const size_t smem = RadixSmem<RX_BITS, PB, HAS_PC>::bytes();
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nt, RX_THREADS, smem, st>>>(keys, pa, pb, pc, n, pass * RX_BITS, rs.bins + pass * RX_BINS, static_cast<S*>(rs.words) + (size_t)pass * nt * RX_BINS,
-                                                 rs.tickets + pass, emit, err);
-    note_launches(1);
-    return cudaGetLastError();
+    return launch_linked(kern, (unsigned)nt, RX_THREADS, smem, st, keys, pa, pb, pc, n, pass * RX_BITS, rs.bins + pass * RX_BINS,
+                         static_cast<S*>(rs.words) + (size_t)pass * nt * RX_BINS, rs.tickets + pass, emit, err);
 }
 template <typename PB, bool HAS_PC, typename Emit>
 inline cudaError_t radix_pass(const uint32_t* keys, const uint32_t* pa, const PB* pb, const uint32_t* pc, int64_t n, int pass, const RadixState& rs, Emit emit,

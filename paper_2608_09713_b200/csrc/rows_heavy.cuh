@@ -57,6 +57,7 @@ static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDe
     __shared__ uint32_t s_before[NW][NROUTE];  // rows (parts) of the tile's warps before
     __shared__ int64_t s_base[NROUTE];
     __shared__ uint32_t s_tile;
+    link(rows, cnt, block_base);
     if (threadIdx.x == 0) s_tile = (uint32_t)atomicAdd(ticket, 1ull);
     __syncthreads();
     const int64_t tile = s_tile, n = tile * ROUTE_THREADS + threadIdx.x;

@@ -299,6 +299,7 @@ template <int G>
 static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev P, uint8_t* __restrict__ cls, int64_t block_max, uint32_t dense_range, bool diag, int64_t tile,
                                                                       int32_t* __restrict__ blockhist, int64_t nblocks,
                                                                       unsigned long long* __restrict__ work_total, unsigned long long* __restrict__ sparse_heavy, HeavyArrays heavy) {
+    link();
     if (blockIdx.x >= nblocks) {
         heavy_analysis<G>(P, heavy);
         return;
@@ -449,6 +450,7 @@ static __global__ void __launch_bounds__(BIN_THREADS) row_scatter_kernel(PlanDev
     __shared__ int64_t running[NCLASS];
     __shared__ int32_t wcount[NW][NCLASS];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
+    link(cls, offsets);
     if (threadIdx.x < NCLASS) running[threadIdx.x] = offsets[(int64_t)threadIdx.x * nblocks + blockIdx.x];
     const int64_t rows = P.r1 - P.r0;
     const int64_t t0 = (int64_t)blockIdx.x * tile, t1 = min(t0 + tile, rows);
