@@ -729,17 +729,25 @@ uint32_t row_chunk_bits(const spsyrk_plan_s* pl, uint32_t cap) {
     return pow2_at_least(umax, 1024u, cap);
 }
 
-template <int THREADS>
-spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
+// A row's masks of the heavy columns stand for all its products: not where the columns are a part (a block, or the upper part of
+// the rows in full-output mode)
+bool row_masks(const spsyrk_plan_s* pl) { return pl->dev.binary && pl->diag; }
+
+template <int THREADS, bool MASKS>
+spsyrk_status_t launch_symbolic_cta_m(spsyrk_plan_s* pl, int c, Chain& ch) {
     const int64_t count = pl->class_start[c + 1] - pl->class_start[c];
     if (count <= 0 || pl->sparse_heavy[c - 6] == 0) return SPSYRK_OK;
     const uint32_t cb = row_chunk_bits(pl, ROW_CHUNK_BITS_MAX_SYMBOLIC);
     const size_t smem = CtaRowSmem<int32_t, THREADS, false>::bytes(cb, 0);
-    auto kern = rows_cta_kernel<int32_t, THREADS, false>;
-    SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<int32_t, THREADS, false>>()));
-    SPSYRK_CUDA_TRY(ch.launch(brief_rows(count, (int64_t)pl->sm_count * (2048 / THREADS)), kern, (unsigned)count, THREADS, smem, pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt, nullptr, nullptr, nullptr,
-                              nullptr, pl->block_base, pl->blocks_per_row));
+    auto kern = rows_cta_kernel<int32_t, THREADS, false, MASKS>;
+    SPSYRK_CUDA_TRY((allow_shared_memory<rows_cta_kernel<int32_t, THREADS, false, MASKS>>()));
+    SPSYRK_CUDA_TRY(ch.launch(brief_rows(count, (int64_t)pl->sm_count * (2048 / THREADS)), kern, (unsigned)count, THREADS, smem, pl->dev, pl->perm + pl->class_start[c], cb, 0u, pl->cnt,
+                              nullptr, nullptr, nullptr, nullptr, pl->block_base, pl->blocks_per_row));
     return SPSYRK_OK;
+}
+template <int THREADS>
+spsyrk_status_t launch_symbolic_cta(spsyrk_plan_s* pl, int c, Chain& ch) {
+    return row_masks(pl) ? launch_symbolic_cta_m<THREADS, true>(pl, c, ch) : launch_symbolic_cta_m<THREADS, false>(pl, c, ch);
 }
 
 // Shared-memory shapes of the heavy-row kernels and the rule that goes with them.  The small rank kernel is launched
@@ -769,6 +777,7 @@ HeavyShapes heavy_shapes(const spsyrk_plan_s* pl) {
     h.dense8_columns = (uint32_t)std::min<uint64_t>(umax, (SMEM_PER_CTA - Dense8Smem<DENSE8_THREADS>::bytes(0)) / 16 * 16);
     r.dense8 = h.dense8_columns;
     r.binary = pl->dev.binary;
+    r.masks = row_masks(pl);
     return h;
 }
 

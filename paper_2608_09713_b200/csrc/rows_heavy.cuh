@@ -6,8 +6,8 @@
 //            the row fills, and dense rows of binary matrices that dense8 does not take (chunk by chunk).
 // A row with more entries than slots fit an SM is cut into parts of whole blocks of columns: the symbolic pass has left
 // the number of entries before every block.
-//   dense8 : rows of a binary matrix in which every column occurs: four 8-bit counters per word, the heaviest
-//            columns counted through bit masks.
+//   dense8 : rows of a binary matrix in which every column or many a column occurs: four 8-bit counters per word, the
+//            heaviest columns counted through bit masks.
 // All are launched with a CTA per row or part of one, the longest lists first, so that the GPU hands the rows out as CTAs end.
 // (Persistent CTAs that drew their rows from a counter in the plan lost rows when two passes of one plan overlapped; the
 // same rows dealt out beforehand took 1.14 times as long on the large power-law workload.)  In direct and dense8 a CTA
@@ -40,6 +40,7 @@ struct RouteRule {
     uint32_t chunk;                              // columns per chunk of the direct kernel
     uint32_t dense8;                             // columns the packed counters of one row may have
     int binary;
+    int masks;                                   // the rows' masks of the heavy columns stand for whole rows of the lower triangle
 };
 
 // One thread per heavy row: class 7, then class 6, each with the last rows first (they carry the longest lists).  The lists
@@ -76,7 +77,12 @@ static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDe
         const bool dense = entries == U;
         if (U > R.wide) {
             route = ROUTE_WIDE;
-        } else if (R.binary && dense && deg <= 255 && U <= R.dense8) {
+        } else if (R.binary && deg <= 255 && U <= R.dense8 && (dense || (R.masks && w >= (int64_t)U))) {
+            // Rows that are not dense: rank walks all their products twice, direct has 32-bit counters; dense8 walks each once, fewer with
+            // heavy columns, but looks at every column.  Numeric pass of 30 000 rows of random columns, without and with dense8: w = U 2565
+            // us to 2020, 1.3 U 2999 to 1551, 2 U 3737 to 1839; of 6000 rows 147 to 126, 156 to 120, 175 to 137 (below U the two
+            // are level: rank has the fewer columns to look at).  30 000 sets of 60 of 65 536 columns of Zipf frequencies, of
+            // which some lack the most frequent one: all similarities 12.0 ms to 3.1, counting included.
             route = ROUTE_DENSE8;
         } else if ((R.binary && dense) || (U <= R.chunk && w >= (int64_t)(U / 4))) {
             // One chunk: direct walks the lists once and sweeps every column, rank walks them twice and sweeps a bitmap.  Measured
@@ -487,18 +493,6 @@ struct DirectSmem {
 
 constexpr int DIRECT_THREADS = 512;
 
-// a row's bits of the heavy columns (planes in use: 32 columns each)
-struct HeavyMask {
-    uint32_t w[HEAVY_PLANES];
-};
-__device__ __forceinline__ HeavyMask load_heavy_mask(const PlanDev& P, int64_t i, int planes) {
-    HeavyMask k;
-#pragma unroll
-    for (int p = 0; p < HEAVY_PLANES; ++p) k.w[p] = p < planes ? P.heavy_mask[p * P.mask_stride + i] : 0u;
-    return k;
-}
-__device__ __forceinline__ int heavy_planes(const PlanDev& P) { return (int)((min(*P.nheavy, (uint32_t)HEAVY_MAX) + 31u) / 32u); }
-
 // Bound by the adds in shared memory.  Two CTAs of 512 threads per SM: one searches and sweeps while the other adds.
 // A column that occurs is marked by a plain byte store (a bitmap needs an atomic or a look first; accumulators that
 // start as a special NaN need a compare-and-swap loop of their own, which took five times the built-in add).
@@ -616,14 +610,16 @@ struct Dense8Smem {
     static size_t bytes(uint32_t columns) { return ((size_t)columns + 15) / 16 * 16 + 16 + sizeof(ListBatch<int32_t, THREADS>); }
 };
 
-// A dense row of a binary matrix with at most 255 nonzeros: every count is at most the row's own length, so a word holds
+// A row of a binary matrix with at most 255 nonzeros: every count is at most the row's own length, so a word holds
 // four counters and a row is one tile.  The counters start at the overlap of the rows' heavy-column masks (read as
-// planes of 32 columns, four rows j at a time), the remaining lists, short ones, are walked, and the row leaves four
-// entries per thread: groups of four are aligned in the output, where the row starts at any offset.
+// planes of 32 columns, four rows j at a time), the remaining lists, short ones, are walked, and a dense row leaves four
+// entries per thread: groups of four are aligned in the output, where the row starts at any offset.  Of another row the
+// counters that are not zero leave, 32 columns per step of a warp.
 template <typename V, int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, HeavyArgs H, uint32_t columns, V* __restrict__ c_vals) {
     extern __shared__ __align__(16) unsigned char d8_smem[];
     __shared__ RowQueueShared s_queue;
+    __shared__ uint32_t s_warp[THREADS / 32];
     uint32_t* acc = reinterpret_cast<uint32_t*>(d8_smem);  // four columns per word
     ListBatch<int32_t, THREADS>& B = *reinterpret_cast<ListBatch<int32_t, THREADS>*>(d8_smem + ((size_t)columns + 15) / 16 * 16 + 16);
     const int tid = threadIdx.x;
@@ -669,6 +665,34 @@ __global__ void __launch_bounds__(THREADS, CTAS) rows_dense8_kernel(PlanDev P, H
             if constexpr (std::is_same<V, int32_t>::value)
                 if (P.jaccard) store_jaccard<V>(P, ob + j, (int32_t)j, c, (int32_t)deg);
         };
+        if (H.out_end[rloc] - ob != (int64_t)U) {
+            constexpr uint32_t NW = THREADS / 32;
+            const int lane = lane_id(), warp = tid >> 5;
+            const uint32_t steps = (U + 31u) / 32u, per_warp = (steps + NW - 1) / NW;  // of 32 columns; a warp owns consecutive ones
+            const uint32_t j0 = min((uint32_t)warp * per_warp * 32u, U), j1 = min(j0 + per_warp * 32u, U);
+            uint32_t sum = 0;
+            for (uint32_t j = j0 + 4u * lane; j < j1; j += 128u) {
+                const uint32_t left = j1 - j, q = acc[j >> 2] & (left < 4u ? (1u << (8u * left)) - 1u : 0xffffffffu);
+                sum += __popc(__vcmpne4(q, 0u)) / 8;
+            }
+            sum = warp_reduce_sum<uint32_t>(sum);
+            if (lane == 0) s_warp[warp] = sum;
+            __syncthreads();
+            uint32_t at = warp_reduce_sum<uint32_t>(lane < warp ? s_warp[lane < (int)NW ? lane : 0] : 0u);
+            for (uint32_t j = j0 + lane; j - lane < j1; j += 32u) {
+                const int32_t c = j < j1 ? (int32_t)((acc[j >> 2] >> ((j & 3u) * 8u)) & 0xffu) : 0;
+                const unsigned votes = __ballot_sync(FULL_MASK, c != 0);
+                const int64_t o = ob + at + __popc(votes & ((1u << lane) - 1u));
+                if (c != 0 && SPSYRK_IN_RANGE(o < H.out_end[rloc], P.err)) {
+                    c_vals[o] = (V)c;
+                    H.c_colidx[o] = (int32_t)j;
+                    if constexpr (std::is_same<V, int32_t>::value)
+                        if (P.jaccard) store_jaccard<V>(P, o, (int32_t)j, c, (int32_t)deg);
+                }
+                at += __popc(votes);
+            }
+            continue;
+        }
         if (!H.aligned) {
             for (uint32_t j = tid; j < U; j += THREADS) one(j);
             continue;

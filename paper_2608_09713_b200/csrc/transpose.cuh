@@ -172,6 +172,18 @@ static __device__ void heavy_analysis(const PlanDev& P, const HeavyArrays& H) {
 template <int G>
 static __global__ void __launch_bounds__(BIN_THREADS) heavy_analysis_kernel(PlanDev P, HeavyArrays H) { heavy_analysis<G>(P, H); }
 
+// a row's bits of the heavy columns (planes in use: 32 columns each)
+struct HeavyMask {
+    uint32_t w[HEAVY_PLANES];
+};
+__device__ __forceinline__ HeavyMask load_heavy_mask(const PlanDev& P, int64_t i, int planes) {
+    HeavyMask k;
+#pragma unroll
+    for (int p = 0; p < HEAVY_PLANES; ++p) k.w[p] = p < planes ? P.heavy_mask[p * P.mask_stride + i] : 0u;
+    return k;
+}
+__device__ __forceinline__ int heavy_planes(const PlanDev& P) { return (int)((min(*P.nheavy, (uint32_t)HEAVY_MAX) + 31u) / 32u); }
+
 // One entry of a column list as a record: what the light-row numeric kernel gathers (one aligned
 // asynchronous copy per entry, whatever the list's offset).
 template <typename V> struct ColRec;
