@@ -7,7 +7,7 @@
 //             holds an entry above the diagonal iff its last entry is one:
 //             nnz(F) = 2 nnz(C_L) - #diagonals.
 //   sort    : 4-byte values of up to 2^24 rows and small matrices go to buckets of columns and from there to their
-//             places (mirror_sort.cuh); 8-byte values of more than 65536 rows go through radix passes of 16-byte
+//             places (mirror_sort.cuh); 8-byte values of more than 2^18 rows go through radix passes of 16-byte
 //             records, the last of which writes F (mirror_rec.cuh); 4-byte values of more rows, or of few entries for
 //             their rows, through radix passes of separate arrays (radix.cuh);
 //   rows    : row lengths of F, scan -> f_rowptr (in the bucket sort before the last pass), lower parts copied.
@@ -25,12 +25,12 @@ constexpr size_t ALIGN = 256;
 
 constexpr int MIRROR_RADIX_BITS = 8;  // digits of the record passes
 
-// 8-byte values: the record passes move 16-byte records in runs that the cut into buckets does not reach (three
-// passes over 5.4e8 records: 14.7 ms and 1.6 for histograms and scans, against 15.9 and 1.1), but the bucket sort takes half
-// the launches: it is used where both take two passes.  (Product and mirror of 4096 rows: 465 -> 415 us.  65537 rows and 2.0e6
-// entries: 250 us by records, 170 by buckets; 262144 rows and 8.1e6 entries 503 to 432, 2.6e8 entries 8.61 to 8.30 ms: where
-// buckets take two passes and records three, up to 2^18 rows, the line could lie higher.)
-constexpr int64_t MIRROR_BUCKET_ROWS_8 = 65536;
+// 8-byte values: where buckets take two passes and records three, and below that, where both take two and buckets half the
+// launches, the bucket sort is used (records against buckets, product and mirror: 70 000 rows and 9.0e6 entries 847 us to 724,
+// 200 000 rows 1898 to 1763, 262 000 rows 3839 to 3727, a banded matrix of 250 000 rows 1060 to 946, a power-law one of 2^18 rows
+// 37.2 ms to 35.3).  With a third bucket pass the records move in runs as short and the rests of the columns besides: 2^22 rows 35.06
+// ms by records, 35.37 by three bucket passes, a banded matrix of 2e6 rows 6.85 to 7.21.
+constexpr int64_t MIRROR_BUCKET_ROWS_8 = 262144;
 bool mirror_by_records(int64_t m, size_t sv) { return sv == 8 && m > MIRROR_BUCKET_ROWS_8; }
 struct MirrorWs {
     int64_t* partials;
@@ -304,6 +304,61 @@ __global__ void __launch_bounds__(256) mirror_copy_lower_kernel(const int64_t* _
     }
 }
 
+// The same where rows are long on average, and a few much longer than that: a warp per CHUNK consecutive entries, whose rows
+// it finds from the rows of every 32nd entry.  (A warp per row keeps one warp at the longest row of a power-law matrix while the
+// others are done: 6.4e8 single-precision entries, 2 400 per row, product and mirror 28.83 ms, so 28.28.)
+constexpr int COPY_CHUNK = 512;
+constexpr int64_t COPY_LONG_ROWS = 256;  // entries per row from which on
+template <typename V>
+__global__ void __launch_bounds__(256) mirror_copy_chunks_kernel(const int64_t* __restrict__ l_rowptr, const int32_t* __restrict__ l_colidx,
+                                                                 const V* __restrict__ l_vals, int64_t m, int64_t nnz, const int32_t* __restrict__ step_row,
+                                                                 const int64_t* __restrict__ f_rowptr, int32_t* __restrict__ f_colidx, V* __restrict__ f_vals) {
+    const int lane = lane_id();
+    link(step_row, f_rowptr);
+    const int64_t e0 = ((int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)) * COPY_CHUNK;
+    const int64_t e1 = min(e0 + COPY_CHUNK, nnz);
+    auto row_of_step = [&](int64_t e) { return (int64_t)min((uint32_t)step_row[e >> 5], (uint32_t)(m - 1)); };  // e a multiple of 32
+    int64_t r = e0 < e1 ? row_of_step(e0) : 0;
+    for (int64_t p = e0; p < e1;) {  // entries [p, end) are of row r; uniform in the warp
+        const int64_t end = min(l_rowptr[r + 1], e1);
+        const int64_t shift = f_rowptr[r] - l_rowptr[r];
+        constexpr int UNR = 8;
+        for (int64_t q = p + lane; q < end; q += 32 * UNR) {
+            int32_t j[UNR];
+            V v[UNR];
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                if (q + 32 * u < end) {
+                    j[u] = l_colidx[q + 32 * u];
+                    v[u] = l_vals[q + 32 * u];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                if (q + 32 * u < end) {
+                    f_colidx[shift + q + 32 * u] = j[u];
+                    f_vals[shift + q + 32 * u] = v[u];
+                }
+            }
+        }
+        if (end >= e1) break;
+        // the row that holds entry `end`: one of the next 32, or searched for up to the row of the next step
+        const int64_t next = r + 1 + lane;
+        const unsigned after = __ballot_sync(FULL_MASK, next >= m || l_rowptr[next] > end);
+        if (after) {
+            r += __ffs(after) - 1;
+        } else {
+            int64_t lo = r + 32, hi = ((end >> 5) + 1) * 32 < nnz ? row_of_step(((end >> 5) + 1) * 32) : m - 1;
+            while (lo < hi) {  // the last row that starts at or before the entry
+                const int64_t mid = (lo + hi + 1) >> 1;
+                if (l_rowptr[mid] <= end) lo = mid; else hi = mid - 1;
+            }
+            r = lo;
+        }
+        p = max(end, p + 1);  // (row pointers that do not ascend: still to the end)
+    }
+}
+
 int group_width(int64_t nnz, int64_t m) {
     const double avg = m > 0 ? (double)nnz / (double)m : 0.0;
     return avg <= 4 ? 4 : avg <= 8 ? 8 : avg <= 16 ? 16 : 32;
@@ -415,7 +470,13 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
     SPSYRK_CUDA_TRY(launch_linked(mirror_place_kernel<VB>, place_units, MS_THREADS, place_smem, st, a));
     mirror_mark(pass, st);
     g_mirror_passes = pass;
-    mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+    if (nnz_l / m >= COPY_LONG_ROWS) {
+        constexpr int64_t per_cta = 8 * COPY_CHUNK;
+        SPSYRK_CUDA_TRY(launch_linked(mirror_copy_chunks_kernel<VB>, (unsigned)((nnz_l + per_cta - 1) / per_cta), 256, 0, st, l_rowptr, l_colidx, static_cast<const VB*>(l_vals),
+                                      m, nnz_l, (const int32_t*)w.step_row, (const int64_t*)f_rowptr, f_colidx, static_cast<VB*>(f_vals)));
+    } else {
+        mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+    }
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
     {

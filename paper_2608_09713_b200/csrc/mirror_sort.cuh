@@ -1,5 +1,5 @@
 // The column sort of the mirror for 4-byte values of matrices of at most 2^24 rows, and for 8-byte values of at most
-// 65536: C_L's entries by (column, row) in two passes over memory (up to 2^18 rows) or three.
+// 2^18: C_L's entries by (column, row) in two passes over memory (up to 2^18 rows) or three.
 //
 // A column id is cut into parts, from the low end: L bits, M bits (three passes) and H bits.
 //   split : the entries, read from C_L in row order, go to one of 2^L buckets by their low part;
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(MS_THREADS, MirrorSortTraits<VB>::MIN_CTAS) mi
     }
 }
 
-// (4-byte values: 8-byte ones have at most 65536 rows here, two passes)
+// (4-byte values: 8-byte ones have at most 2^18 rows here, two passes)
 struct MirrorMidSmem {
     static size_t bytes(int nb) { return (size_t)mirror_tile<uint32_t>() * (sizeof(uint2) + 2) + (size_t)nb * 8 + (size_t)MS_WARPS * nb * 2; }
 };
