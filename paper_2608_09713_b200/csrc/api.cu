@@ -62,9 +62,9 @@ constexpr size_t LARGE_SMEM_BUDGET = 200 * 1024;
 constexpr int64_t MAX_PARTS = 65536;
 
 // Shared-memory shapes of the heavy-row kernels (see heavy_shapes)
-constexpr int RANK_SMALL_THREADS = 256, RANK_MID_THREADS = 512, RANK_BIG_THREADS = 1024, DENSE8_THREADS = 512;
+constexpr int RANK_SMALL_THREADS = 256, RANK_MID_THREADS = 512, RANK_BIG_THREADS = 1024, DENSE8_THREADS = 512, DENSE8_SHORT_THREADS = 256;
 template <int T, int C> struct RankShape { static constexpr int THREADS = T, CTAS = C; };
-constexpr size_t SMEM_PER_CTA = 226 * 1024;
+constexpr size_t SMEM_PER_CTA = 226 * 1024, SMEM_PER_SM = 228 * 1024, SMEM_OF_A_CTA = 1024;  // the last: taken by every CTA that is resident
 // slots of the largest rank kernel, one CTA per SM: doubles 21504 beside a bitmap of 2^18 columns, 23552 beside 2^17, 24576 beside 2^16
 template <typename V>
 uint32_t rank_slots_big(uint32_t columns) {
@@ -854,9 +854,16 @@ spsyrk_status_t launch_heavy(spsyrk_plan_s* pl, int32_t* c_colidx, void* c_vals,
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK2, h.columns, h.rule.slots_small));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK1, h.rule.bits1, h.rule.slots_small));
     SPSYRK_CUDA_TRY(rank(RankShape<RANK_SMALL_THREADS, 4>{}, ROUTE_RANK0, h.rule.bits0, h.rule.slots_small));
-    if (const int64_t units = pieces(ROUTE_DENSE8).total())
-        SPSYRK_CUDA_TRY((launch_rows<rows_dense8_kernel<V, DENSE8_THREADS, 3>>(pl, ch, units, DENSE8_THREADS, Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns), pl->dev,
-                                                                               args(ROUTE_DENSE8), h.dense8_columns, cv)));
+    if (const int64_t units = pieces(ROUTE_DENSE8).total()) {
+        // Short rows have little to do for many threads: six CTAs of 256 where so many fit an SM, up to about 32 000 columns, three of 512 beyond
+        // (similarities of 3001 sets 203 us to 191, 8000 373 to 335, 24 000 1487 to 1359; of 40 000, five CTAs, 3405 to 3590)
+        const size_t narrow = Dense8Smem<DENSE8_SHORT_THREADS>::bytes(h.dense8_columns);
+        if (6 * (narrow + SMEM_OF_A_CTA + 256) <= SMEM_PER_SM)
+            SPSYRK_CUDA_TRY((launch_rows<rows_dense8_kernel<V, DENSE8_SHORT_THREADS, 6>>(pl, ch, units, DENSE8_SHORT_THREADS, narrow, pl->dev, args(ROUTE_DENSE8), h.dense8_columns, cv)));
+        else
+            SPSYRK_CUDA_TRY((launch_rows<rows_dense8_kernel<V, DENSE8_THREADS, 3>>(pl, ch, units, DENSE8_THREADS, Dense8Smem<DENSE8_THREADS>::bytes(h.dense8_columns), pl->dev,
+                                                                                   args(ROUTE_DENSE8), h.dense8_columns, cv)));
+    }
     const RoutePieces wide = pieces(ROUTE_WIDE);
     for (int k = 0; k < 2; ++k) {
         if (!wide.count[k]) continue;
