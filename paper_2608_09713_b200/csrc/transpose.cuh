@@ -336,6 +336,7 @@ static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev
     unsigned long long mine = 0;    // work of the rows this thread owned
     const bool tril = P.mode == SPSYRK_TRIL;
     auto range_of = [&](int64_t r) { return tril ? (uint32_t)(P.r0 + (int32_t)r) + 1u : (uint32_t)P.m; };
+    auto is_heavy = [&](int32_t deg, uint32_t w) { return deg > 32 || (diag ? w - deg : w) > 512u; };
     // (the lengths of a row's descriptors add up to less than 2^31)
     auto settle = [&](int64_t r, int32_t deg, uint32_t w, bool full) {  // one thread per row; full: it stores a column of every row of its range
         const bool dense = full && range_of(r) <= dense_range;
@@ -343,7 +344,7 @@ static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev
         int c;
         const uint32_t wl = diag ? w - deg : w;  // items of a light row
         if (w == 0) c = 0;
-        else if (deg <= 32 && wl <= 512) c = wl <= 32 ? 1 : wl <= 64 ? 2 : wl <= 128 ? 3 : wl <= 256 ? 4 : 5;
+        else if (!is_heavy(deg, w)) c = wl <= 32 ? 1 : wl <= 64 ? 2 : wl <= 128 ? 3 : wl <= 256 ? 4 : 5;
         else c = w <= block_max ? 6 : 7;
         cls[r] = (uint8_t)(c | (dense && c >= 6 ? ROW_DENSE : 0));
         atomicAdd(&hist[c], 1);
@@ -373,23 +374,32 @@ static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev
 #pragma unroll
         for (int u = 0; u < UNR; ++u) w[u] = gl < deg[u] ? P.desc[p0[u] + gl].y : 0;
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const uint32_t range = range_of(base + u * GROUPS + group);
-            bool f = w[u] == range;
-            for (int32_t q = gl + G; q < deg[u]; q += G) {
-                const uint32_t len = P.desc[p0[u] + q].y;
-                w[u] += len;
-                f |= len == range;
-            }
-            full |= (uint32_t)f << u;
-        }
+        for (int u = 0; u < UNR; ++u)
+            for (int32_t q = gl + G; q < deg[u]; q += G) w[u] += P.desc[p0[u] + q].y;
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) full |= __shfl_xor_sync(FULL_MASK, full, o);
+        for (int u = 0; u < UNR; ++u) {
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) w[u] += __shfl_xor_sync(FULL_MASK, w[u], o);
+        }
+        // heavy rows: does one of the columns cover the row's range?
+        bool heavy_row = false;
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) heavy_row |= is_heavy(deg[u], w[u]);
+        if (__any_sync(FULL_MASK, heavy_row)) {
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                if (!is_heavy(deg[u], w[u])) continue;
+                const uint32_t range = range_of(base + u * GROUPS + group);
+                bool f = false;
+                for (int32_t q = gl; q < deg[u]; q += G) f |= P.desc[p0[u] + q].y == range;
+                full |= (uint32_t)f << u;
+            }
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) full |= __shfl_xor_sync(FULL_MASK, full, o);
+        }
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
             const int64_t r = base + u * GROUPS + group;
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) w[u] += __shfl_xor_sync(FULL_MASK, w[u], o);
             if (r < t1 && gl == 0 && deg[u] >= 0) settle(r, deg[u], w[u], (full >> u) & 1u);
         }
     }
