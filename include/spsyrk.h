@@ -256,7 +256,8 @@ spsyrk_status_t spsyrk_column_panel(int64_t m, int64_t nnz, spsyrk_dtype_t dtype
  * Three-step use:
  *   1. d_workspace == NULL: *workspace_bytes receives the scratch size for m.
  *   2. d_z_colidx == NULL: writes d_z_rowptr[m + 1] and *nnz_out (synchronises).
- *   3. all pointers set: fills d_z_colidx / d_z_vals using the d_z_rowptr of step 2.  Asynchronous.
+ *   3. all pointers set: fills d_z_colidx / d_z_vals using the d_z_rowptr of step 2.  Asynchronous.  Neither reads nor
+ *      writes the workspace: several fills may be under way with the same one, and another call may use it meanwhile.
  * All pointers are device pointers except nnz_out and workspace_bytes (host).
  * nnz_x = d_x_rowptr[m], nnz_y = d_y_rowptr[m] (they only steer how many lanes share a row).
  * Errors: INVALID_ARG, WORKSPACE, BAD_CSR (a row of X or Y not strictly ascending), CUDA.

@@ -28,8 +28,7 @@ int group_width(int64_t nnz, int64_t m) {
 struct RowWs {
     uint32_t* cnt;  // m
     int64_t* partials;
-    int32_t* list;   // m: long rows of the sum
-    uint32_t *err, *words;
+    uint32_t* err;
 };
 
 size_t carve(RowWs* w, void* ws, int64_t m) {
@@ -45,9 +44,7 @@ size_t carve(RowWs* w, void* ws, int64_t m) {
     RowWs t;
     t.cnt = (uint32_t*)take(items * 4);
     t.partials = (int64_t*)take(scan_partials_count(items + 1) * 8);
-    t.list = (int32_t*)take(items * 4);
     t.err = (uint32_t*)take(16);
-    t.words = t.err + 1;
     if (w) *w = t;
     return (off + ALIGN - 1) / ALIGN * ALIGN;
 }
@@ -94,7 +91,8 @@ __global__ void __launch_bounds__(256) panel_fill_kernel(int64_t m, const int64_
 // Walk row `self` G entries at a time; for each entry report (index, lower bound in `other`, match,
 // matches before it) to `visit`.  Returns the number of matches of the row.  Loop bounds are
 // uniform inside the group, so the votes see all of its lanes.
-template <int G, typename Visit>
+// CHECK: a row that does not ascend sets the error bit.
+template <int G, bool CHECK, typename Visit>
 __device__ __forceinline__ uint32_t walk_row(const int32_t* __restrict__ self, uint32_t ls, const int32_t* __restrict__ other,
                                              uint32_t lo_len, uint32_t* err, Visit visit) {
     const unsigned gmask = group_mask<G>();
@@ -108,7 +106,7 @@ __device__ __forceinline__ uint32_t walk_row(const int32_t* __restrict__ self, u
         int32_t col = 0;
         if (t < ls) {
             col = self[t];
-            if (t > 0 && self[t - 1] >= col) atomicOr(err, ERRW_UNSORTED);
+            if (CHECK && t > 0 && self[t - 1] >= col) atomicOr(err, ERRW_UNSORTED);
             lb = lower_bound_i32(other, lo_len, col);
             match = lb < lo_len && other[lb] == col;
         }
@@ -128,19 +126,12 @@ __device__ __forceinline__ uint32_t walk_row(const int32_t* __restrict__ self, u
 // What bounds it: instruction issue, and for rows of one or two tiles the latency of a tile's steps.
 // Sum of two panel products of a power-law graph of 2^15 vertices (3.6e7 entries in, 2.9e7 out, f32): 196 us for the size step, 412 for the fill.
 // (Before: one warp per row, whatever its length, in windows of 32 ids with a search and votes per entry: 1402 us.)
-constexpr int MERGE_WARPS = 8;
+constexpr int MERGE_WARPS = 2;
 constexpr int MERGE_ITEMS = 8;
 constexpr int MERGE_LONG_THREADS = 256;
-// Rows of more entries (of both inputs together) than this are put on a list and merged by a CTA each: 16 tiles of a warp
+// Rows of more entries (of both inputs together) than this are merged by a CTA each (add_long_kernel): 16 tiles of a warp
 // or two of a CTA.
 constexpr uint32_t MERGE_LONG = 4096;
-
-// rows for which a kernel of the sum leaves the work to add_long_kernel
-struct LongRows {
-    int32_t* list;    // m
-    uint32_t* words;  // [0] rows listed, [1] batches of rows handed out, [2] listed rows handed out; all zero at the start
-    __device__ __forceinline__ void add(int64_t r) const { list[atomicAdd(words, 1u)] = (int32_t)r; }
-};
 
 template <int T>
 __device__ __forceinline__ void merge_sync() {
@@ -276,7 +267,7 @@ struct SumArgs {
     const int64_t* z_rowptr;   // fill step
     int32_t* z_colidx;
     V* z_vals;
-    uint32_t* err;
+    uint32_t* err;             // size step
 };
 
 template <typename V, bool FILL, int T>
@@ -288,56 +279,68 @@ __device__ __forceinline__ void sum_row(const SumArgs<V>& A, int64_t r, int64_t 
     if (!FILL && t == 0) A.cnt[r] = n;
 }
 
-// One warp per row.  The warps draw batches of rows: with eight rows to a CTA the longest of them kept the places of the others
-// (19 % of the warps active on average).
+// One warp per row, `batch` consecutive rows per warp.  The launch hands the rows out, in small CTAs: a CTA keeps its place until its
+// last row is done (CTAs of eight rows: 19 % of the warps active on average).  (Counters in the workspace, from which a
+// fixed number of warps drew their rows, lost rows when two fills shared a workspace.)
 template <typename V, bool FILL>
-__global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(SumArgs<V> A, LongRows longer, int batch) {
+__global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(SumArgs<V> A, int batch) {
     __shared__ MergeSmem<32> smem[MERGE_WARPS];
     const int warp = threadIdx.x >> 5, lane = lane_id();
-    for (;;) {
-        uint32_t ticket = 0;
-        if (lane == 0) ticket = atomicAdd(longer.words + 1, 1u);
-        const int64_t first = (int64_t)__shfl_sync(FULL_MASK, ticket, 0) * batch;
-        if (first >= A.m) return;
-        const int64_t last = min(first + batch, A.m);
-        for (int64_t r = first; r < last; ++r) {
-            const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
-            const int64_t lx = A.x_rowptr[r + 1] - x0, ly = A.y_rowptr[r + 1] - y0;
-            if (lx < 0 || ly < 0 || lx + ly > 0x7fffffffLL) {
-                if (lane == 0) {
-                    atomicOr(A.err, ERRW_BAD_ROWPTR);
-                    if (!FILL) A.cnt[r] = 0;
-                }
-            } else if (lx + ly > MERGE_LONG) {
-                if (lane == 0) longer.add(r);
-            } else {
-                sum_row<V, FILL, 32>(A, r, x0, (uint32_t)lx, y0, (uint32_t)ly, smem[warp], lane);
+    const int64_t first = ((int64_t)blockIdx.x * MERGE_WARPS + warp) * batch, last = min(first + batch, A.m);
+    for (int64_t r = first; r < last; ++r) {
+        const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
+        const int64_t lx = A.x_rowptr[r + 1] - x0, ly = A.y_rowptr[r + 1] - y0;
+        if (lx < 0 || ly < 0 || lx + ly > 0x7fffffffLL) {
+            if (!FILL && lane == 0) {
+                atomicOr(A.err, ERRW_BAD_ROWPTR);
+                A.cnt[r] = 0;
             }
+        } else if (lx + ly <= MERGE_LONG) {
+            sum_row<V, FILL, 32>(A, r, x0, (uint32_t)lx, y0, (uint32_t)ly, smem[warp], lane);
         }
     }
 }
 
-// one CTA per listed row
+// The rows of more than MERGE_LONG entries, a CTA each.  The rows are dealt to the CTAs in units of 1 << unit_bits, a unit of every
+// gridDim.x, so that long rows which stand together go to different CTAs; a CTA has at most one unit per thread.  A unit of few
+// entries has no such row: of it only the ends are looked at.
 template <typename V, bool FILL>
-__global__ void __launch_bounds__(MERGE_LONG_THREADS) add_long_kernel(SumArgs<V> A, LongRows rows) {
+__global__ void __launch_bounds__(MERGE_LONG_THREADS) add_long_kernel(SumArgs<V> A, int unit_bits) {
     __shared__ MergeSmem<MERGE_LONG_THREADS> smem;
-    __shared__ uint32_t s_ticket;
-    const uint32_t n = rows.words[0];
-    for (;;) {
-        if (threadIdx.x == 0) s_ticket = atomicAdd(rows.words + 2, 1u);
+    __shared__ int64_t s_unit[MERGE_LONG_THREADS];  // first rows of the units that are looked at row by row
+    __shared__ int64_t s_row[MERGE_LONG_THREADS];
+    __shared__ int s_units, s_rows;
+    const int t = threadIdx.x;
+    auto entries = [&](int64_t a, int64_t b) { return A.x_rowptr[b] - A.x_rowptr[a] + A.y_rowptr[b] - A.y_rowptr[a]; };
+    if (t == 0) s_units = 0;
+    __syncthreads();
+    const int64_t u0 = ((int64_t)blockIdx.x + (int64_t)t * gridDim.x) << unit_bits;
+    if (u0 < A.m && entries(u0, min(u0 + (1 << unit_bits), A.m)) > MERGE_LONG) s_unit[atomicAdd(&s_units, 1)] = u0;
+    __syncthreads();
+    const int n = s_units << unit_bits;
+    for (int base = 0; base < n; base += MERGE_LONG_THREADS) {
+        if (t == 0) s_rows = 0;
         __syncthreads();
-        const uint32_t i = s_ticket;
-        if (i >= n) return;
-        const int64_t r = rows.list[i];
-        const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
-        // (a row of this length has at least one tile, whose barriers separate this look at the ticket from the next)
-        sum_row<V, FILL, MERGE_LONG_THREADS>(A, r, x0, (uint32_t)(A.x_rowptr[r + 1] - x0), y0, (uint32_t)(A.y_rowptr[r + 1] - y0), smem, (int)threadIdx.x);
+        if (base + t < n) {
+            const int64_t r = s_unit[(base + t) >> unit_bits] + ((base + t) & ((1 << unit_bits) - 1));
+            if (r < A.m) {
+                const int64_t lx = A.x_rowptr[r + 1] - A.x_rowptr[r], ly = A.y_rowptr[r + 1] - A.y_rowptr[r];
+                if (lx >= 0 && ly >= 0 && lx + ly > MERGE_LONG && lx + ly <= 0x7fffffffLL) s_row[atomicAdd(&s_rows, 1)] = r;
+            }
+        }
+        __syncthreads();
+        const int rows = s_rows;
+        for (int i = 0; i < rows; ++i) {
+            const int64_t r = s_row[i], x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
+            sum_row<V, FILL, MERGE_LONG_THREADS>(A, r, x0, (uint32_t)(A.x_rowptr[r + 1] - x0), y0, (uint32_t)(A.y_rowptr[r + 1] - y0), smem, t);
+        }
+        __syncthreads();
     }
 }
 
 // G lanes per row, where rows are short on average
 template <int G>
-__global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A, LongRows longer) {
+__global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
     if (r >= A.m) return;  // whole groups leave together
@@ -347,34 +350,28 @@ __global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A, Lon
         if (gl == 0) { atomicOr(A.err, ERRW_BAD_ROWPTR); A.cnt[r] = 0; }
         return;
     }
-    if (lx64 + ly64 > MERGE_LONG) {
-        if (gl == 0) longer.add(r);
-        return;
-    }
+    if (lx64 + ly64 > MERGE_LONG) return;
     const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
     const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
     // the sortedness of X is checked here, that of Y inside the walk
     for (uint32_t t = 1 + gl; t < lx; t += G)
         if (xc[t - 1] >= xc[t]) atomicOr(A.err, ERRW_UNSORTED);
-    const uint32_t matched = walk_row<G>(yc, ly, xc, lx, A.err, [](uint32_t, uint32_t, bool, uint32_t, int32_t) {});
+    const uint32_t matched = walk_row<G, true>(yc, ly, xc, lx, A.err, [](uint32_t, uint32_t, bool, uint32_t, int32_t) {});
     if (gl == 0) A.cnt[r] = lx + ly - matched;
 }
 
 template <typename V, int G>
-__global__ void __launch_bounds__(256) add_fill_kernel(SumArgs<V> A, LongRows longer) {
+__global__ void __launch_bounds__(256) add_fill_kernel(SumArgs<V> A) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (r >= A.m) return;
     const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r], z0 = A.z_rowptr[r];
     const int64_t lx64 = A.x_rowptr[r + 1] - x0, ly64 = A.y_rowptr[r + 1] - y0;
-    if (lx64 + ly64 > MERGE_LONG) {
-        if ((threadIdx.x & (G - 1)) == 0) longer.add(r);
-        return;
-    }
+    if (lx64 + ly64 > MERGE_LONG) return;
     const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
     const uint32_t lz = (uint32_t)(A.z_rowptr[r + 1] - z0);
     const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
     // entries of X: all are emitted, matched ones with the sum
-    walk_row<G>(xc, lx, yc, ly, A.err, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
+    walk_row<G, false>(xc, lx, yc, ly, nullptr, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
         const uint32_t pos = t + lb - before;
         if (pos < lz) {  // always true for the row pointer of the size step; keeps a stale one from writing outside
             A.z_colidx[z0 + pos] = col;
@@ -383,7 +380,7 @@ __global__ void __launch_bounds__(256) add_fill_kernel(SumArgs<V> A, LongRows lo
         }
     });
     // entries of Y: only the ones X does not store
-    walk_row<G>(yc, ly, xc, lx, A.err, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
+    walk_row<G, false>(yc, ly, xc, lx, nullptr, [&](uint32_t t, uint32_t lb, bool match, uint32_t before, int32_t col) {
         const uint32_t pos = t + lb - before;
         if (!match && pos < lz) {
             A.z_colidx[z0 + pos] = col;
@@ -426,25 +423,26 @@ void launch_panel_fill(int g, int64_t m, const int64_t* rowptr, const int32_t* c
 
 // kernels of one step of the sum: the rows, then the long ones among them
 template <typename V, bool FILL>
-spsyrk_status_t launch_sum(int g, const SumArgs<V>& A, const RowWs& w, cudaStream_t st) {
-    const LongRows longer{w.list, w.words};
-    const auto blocks = [&](int lanes) { return (unsigned)((A.m * lanes + 255) / 256); };
-    SPSYRK_CUDA_TRY(cudaMemsetAsync(w.words, 0, 12, st));
-    constexpr unsigned MERGE_CTAS = 148 * 8;
+spsyrk_status_t launch_sum(int g, const SumArgs<V>& A, cudaStream_t st) {
+    const auto blocks = [&](int64_t threads) { return (unsigned)((threads + 255) / 256); };
     if (g > 16) {
-        // about 16 batches per warp, of 32 rows at most: 4e6 draws from one counter would take longer than the sum
-        const int batch = (int)std::min<int64_t>(std::max<int64_t>(A.m / (MERGE_CTAS * MERGE_WARPS * 16), 1), 32);
-        add_merge_kernel<V, FILL><<<std::min(MERGE_CTAS, blocks(32)), MERGE_WARPS * 32, 0, st>>>(A, longer, batch);
+        // consecutive rows per warp: one while that gives at most 32 warps per SM 16 times over, up to 32
+        const int batch = (int)std::min<int64_t>(std::max<int64_t>(A.m / (148 * 32 * 16), 1), 32);
+        const int64_t rows = (int64_t)batch * MERGE_WARPS;
+        add_merge_kernel<V, FILL><<<(unsigned)((A.m + rows - 1) / rows), MERGE_WARPS * 32, 0, st>>>(A, batch);
     } else if constexpr (FILL) {
-        if (g == 4) add_fill_kernel<V, 4><<<blocks(4), 256, 0, st>>>(A, longer);
-        else if (g == 8) add_fill_kernel<V, 8><<<blocks(8), 256, 0, st>>>(A, longer);
-        else add_fill_kernel<V, 16><<<blocks(16), 256, 0, st>>>(A, longer);
+        if (g == 4) add_fill_kernel<V, 4><<<blocks(A.m * 4), 256, 0, st>>>(A);
+        else if (g == 8) add_fill_kernel<V, 8><<<blocks(A.m * 8), 256, 0, st>>>(A);
+        else add_fill_kernel<V, 16><<<blocks(A.m * 16), 256, 0, st>>>(A);
     } else {
-        if (g == 4) add_count_kernel<4><<<blocks(4), 256, 0, st>>>(A, longer);
-        else if (g == 8) add_count_kernel<8><<<blocks(8), 256, 0, st>>>(A, longer);
-        else add_count_kernel<16><<<blocks(16), 256, 0, st>>>(A, longer);
+        if (g == 4) add_count_kernel<4><<<blocks(A.m * 4), 256, 0, st>>>(A);
+        else if (g == 8) add_count_kernel<8><<<blocks(A.m * 8), 256, 0, st>>>(A);
+        else add_count_kernel<16><<<blocks(A.m * 16), 256, 0, st>>>(A);
     }
-    add_long_kernel<V, FILL><<<148 * 4, MERGE_LONG_THREADS, 0, st>>>(A, longer);
+    const int unit_bits = A.m <= 1 << 16 ? 0 : A.m <= 1 << 20 ? 2 : 5;
+    const int64_t units = (A.m + (1 << unit_bits) - 1) >> unit_bits;
+    const int64_t ctas = std::max<int64_t>(std::min<int64_t>(units, 148 * 16), (units + MERGE_LONG_THREADS - 1) / MERGE_LONG_THREADS);
+    add_long_kernel<V, FILL><<<(unsigned)ctas, MERGE_LONG_THREADS, 0, st>>>(A, unit_bits);
     note_launches(2);
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
@@ -515,7 +513,7 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
         SPSYRK_CUDA_TRY(cudaMemsetAsync(w.err, 0, 4, st));
         if (m > 0) {
             const spsyrk_status_t s = launch_sum<uint32_t, false>(
-                g, {m, d_x_rowptr, d_x_colidx, nullptr, d_y_rowptr, d_y_colidx, nullptr, w.cnt, nullptr, nullptr, nullptr, w.err}, w, st);
+                g, {m, d_x_rowptr, d_x_colidx, nullptr, d_y_rowptr, d_y_colidx, nullptr, w.cnt, nullptr, nullptr, nullptr, w.err}, st);
             if (s != SPSYRK_OK) return s;
         }
         return scan_and_total(w, m, d_z_rowptr, nnz_out, st);
@@ -525,7 +523,7 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
     const auto fill = [&](auto* z_vals) {
         using V = std::remove_pointer_t<decltype(z_vals)>;
         return launch_sum<V, true>(g, {m, d_x_rowptr, d_x_colidx, static_cast<const V*>(d_x_vals), d_y_rowptr, d_y_colidx, static_cast<const V*>(d_y_vals),
-                                       nullptr, d_z_rowptr, d_z_colidx, z_vals, w.err}, w, st);
+                                       nullptr, d_z_rowptr, d_z_colidx, z_vals, nullptr}, st);
     };
     switch (dtype) {
         case SPSYRK_F64: return fill(static_cast<double*>(d_z_vals));

@@ -71,3 +71,91 @@ def test_accumulate_refuses_rows_that_do_not_ascend(B, size, side):
         with pytest.raises(B.SpsyrkError) as e:
             B.spsyrk_accumulate(1, rp, torch.from_numpy(cols[0]).cuda(), v, rp, torch.from_numpy(cols[1]).cuda(), v)
         assert e.value.status == 2
+
+
+def _device_csr(lengths, seed):
+    """Rows of the given lengths, ascending with small random gaps, and their values on the GPU."""
+    rng = np.random.default_rng(seed)
+    rp = np.concatenate(([0], np.cumsum(lengths))).astype(np.int64)
+    gaps = np.cumsum(rng.integers(1, 5, size=rp[-1]))
+    col = gaps - np.repeat(np.concatenate(([0], gaps))[rp[:-1]], lengths)
+    return tuple(torch.from_numpy(t).cuda() for t in (rp, col.astype(np.int32), rng.standard_normal(rp[-1])))
+
+
+class _Sum:
+    """The steps of one sum by the C calls, with a workspace of the caller's."""
+
+    def __init__(self, B, x, y):
+        import ctypes
+        self.B, self.x, self.y, self.m = B, x, y, x[0].numel() - 1
+        self.rowptr, self.bytes, self.nnz = torch.empty_like(x[0]), ctypes.c_size_t(0), ctypes.c_int64(0)
+        assert self._call(None, None, None, None) == 0
+
+    def _call(self, col, val, ws, stream):
+        import ctypes
+        p = self.B._p
+        return self.B._lib.spsyrk_accumulate(self.m, 0, self.x[1].numel(), *map(p, self.x), self.y[1].numel(), *map(p, self.y), p(self.rowptr), p(col),
+                                             p(val), ctypes.byref(self.nnz), p(ws), ctypes.byref(self.bytes), self.B._stream(stream))
+
+    def sizes(self, ws):
+        assert self._call(None, None, ws, None) == 0
+        self.out = (torch.full((self.nnz.value,), -1, dtype=torch.int32, device="cuda"), torch.full((self.nnz.value,), -1.0, dtype=torch.float64, device="cuda"))
+
+    def fill(self, ws, stream=None):
+        assert self._call(*self.out, ws, stream) == 0
+
+    def check(self):
+        expected = self.B.spsyrk_accumulate(self.m, *self.x, *self.y)
+        assert torch.equal(self.rowptr, expected[0]) and torch.equal(self.out[0], expected[1]) and torch.equal(self.out[1], expected[2])
+
+
+def _sum(B, kind, seed):
+    rng = np.random.default_rng(seed)
+    m = 60_000 if kind == "short" else 6000
+    def rows():
+        lengths = rng.integers(0, 9, size=m) if kind == "short" else rng.integers(20, 300, size=m)
+        lengths[rng.integers(0, m, 40)] = rng.integers(2000, 9000, 40)  # some of them long
+        return lengths
+    return _Sum(B, _device_csr(rows(), seed), _device_csr(rows(), seed + 1))
+
+
+@pytest.mark.parametrize("kind", ["short", "wide"])
+def test_fill_leaves_the_workspace_alone(B, kind):
+    """What the size step left there is gone and something else stands in its place: the fill does not read it and does not write it."""
+    s = _sum(B, kind, 11)
+    ws = B._workspace(s.bytes.value, torch.device("cuda"))
+    s.sizes(ws)
+    ws.fill_(0x5a)
+    s.fill(ws)
+    s.check()
+    assert bool((ws == 0x5a).all())
+
+
+@pytest.mark.parametrize("kind", ["short", "wide"])
+def test_two_fills_with_one_workspace(B, kind):
+    sums = [_sum(B, kind, 21), _sum(B, kind, 31)]
+    ws = B._workspace(max(s.bytes.value for s in sums), torch.device("cuda"))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for s in sums:
+        s.sizes(ws)
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for s, st in zip(sums, streams):
+            s.fill(ws, st)
+    torch.cuda.synchronize()
+    for s in sums:
+        s.check()
+
+
+def test_fill_on_another_stream_beside_new_tensors(B):
+    """The workspace that the binding allocates is given up when the call returns, with the fill under way on another stream."""
+    s = _sum(B, "wide", 41)
+    expected = B.spsyrk_accumulate(s.m, *s.x, *s.y)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(5):
+        got = B.spsyrk_accumulate(s.m, *s.x, *s.y, stream=side)
+        others = [torch.full((s.bytes.value,), 0x5a, dtype=torch.uint8, device="cuda") for _ in range(3)]
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, expected))
+        del others, got
