@@ -4,8 +4,8 @@
 //   spsyrk_column_panel : A_s = A(:, [k0, k1)), the operand of one term of the sum;
 //   spsyrk_accumulate   : Z = X + Y on sorted CSR rows, the "+=" itself.
 //
-// The sum works row by row: G lanes per row when rows are short, a warp or a CTA along the merge path when they are
-// longer (merge_row).  In the G-lane kernels, an entry's place in the merged row is
+// The sum works row by row: G lanes per row when rows are short, a warp (merge_windows) when they are longer, a CTA (merge_path)
+// for the longest.  In the G-lane kernels, an entry's place in the merged row is
 //     its own index + the number of entries of the other row below it - the matches below it,
 // where a match is a column stored in both rows (it is emitted once, from X's side, with x + y).
 // The other row's count is a binary search; the matches below come from a running count over the
@@ -117,47 +117,105 @@ __device__ __forceinline__ uint32_t walk_row(const int32_t* __restrict__ self, u
     return matched;
 }
 
-// Rows of more than a few entries: T threads (a warp, or a CTA for the longest rows) merge a row MERGE_ITEMS * T entries
-// at a time along the merge path (Odeh, Green, Mwassi, Shmueli & Birk, "Merge Path - Parallel Merging Made Simple", 2012).  A
-// tile holds the next ids of both rows in shared memory; a thread finds by a binary search where its MERGE_ITEMS entries of
-// the merged order begin in either row and merges them one after the other, x before y where both store a column;
-// such a pair is emitted once, with x + y, by the thread that has its x.  The emitted entries are put in order in the
-// shared memory of the ids and written out by consecutive threads.
-// What bounds it: instruction issue, and for rows of one or two tiles the latency of a tile's steps.
-// Sum of two panel products of a power-law graph of 2^15 vertices (3.6e7 entries in, 2.9e7 out, f32): 196 us for the size step, 412 for the fill.
-// (Before: one warp per row, whatever its length, in windows of 32 ids with a search and votes per entry: 1402 us.)
-constexpr int MERGE_WARPS = 2;
-constexpr int MERGE_ITEMS = 8;
-constexpr int MERGE_LONG_THREADS = 256;
-// Rows of more entries (of both inputs together) than this are merged by a CTA each (add_long_kernel): 16 tiles of a warp
-// or two of a CTA.
-constexpr uint32_t MERGE_LONG = 4096;
-
-template <int T>
-__device__ __forceinline__ void merge_sync() {
-    if (T == 32) __syncwarp();
-    else __syncthreads();
+// Rows of more than a few entries.  A warp walks the two rows in windows of 32 ids each.  Everything up to the smaller of the
+// two windows' last ids is known completely, so those entries are merged at once: an entry's place is the output position
+// reached so far + its index in its own window + the entries of the other window below it (a search over the window in shared
+// memory) - the matches below it (votes).  All global accesses are coalesced and a step brings in up to 64 ids with one
+// round of loads.  Bound by the load/store pipe (the searches' bank conflicts).  Sums of 6e7 entries, single precision, both steps, rows of
+// 33, 131, 513 and 2000 entries of both inputs: 1023, 591, 518 and 554 us.  (The merge path by a warp, eight entries a lane: 2700, 974, 683
+// and 658, because a row pays for a whole tile.)
+// FILL: the merged row goes to zc, zv (at most lz entries: always enough with the row pointer of the size step; keeps a
+// stale one from writing outside); otherwise the rows are checked.  Returns the number of entries of the merged row.
+constexpr int MERGE_WARPS = 8;
+struct WindowSmem {
+    int32_t x[32], y[32];
+};
+template <typename V, bool FILL>
+__device__ __forceinline__ uint32_t merge_windows(const int32_t* __restrict__ xc, const V* __restrict__ xv, uint32_t lx, const int32_t* __restrict__ yc,
+                                                  const V* __restrict__ yv, uint32_t ly, int32_t* __restrict__ zc, V* __restrict__ zv, uint32_t lz,
+                                                  WindowSmem& S, uint32_t* err) {
+    constexpr int32_t INF = 0x7fffffff;  // above every column id
+    const uint32_t lane = lane_id();
+    const unsigned lt = (1u << lane) - 1u;
+    // number of ids below key among the first n (ascending) ids of a window
+    auto below = [&](const int32_t* win, uint32_t n, int32_t key) -> uint32_t {
+        uint32_t pos = 0;
+#pragma unroll
+        for (uint32_t step = 16; step > 0; step >>= 1)
+            if (pos + step <= n && win[pos + step - 1] < key) pos += step;
+        if (pos < n && win[pos] < key) ++pos;  // a full window with every probed id below: the last one
+        return pos;
+    };
+    uint32_t ix = 0, iy = 0, out = 0;
+    int32_t lastx = -1, lasty = -1;
+    while (ix < lx || iy < ly) {  // the same for all lanes
+        const uint32_t nx = min(32u, lx - ix), ny = min(32u, ly - iy);
+        const int32_t xa = lane < nx ? xc[ix + lane] : INF, ya = lane < ny ? yc[iy + lane] : INF;
+        S.x[lane] = xa;
+        S.y[lane] = ya;
+        __syncwarp();
+        const int32_t bound = min(ix + 32 < lx ? S.x[31] : INF, iy + 32 < ly ? S.y[31] : INF);
+        if (!FILL) {  // rows must be strictly ascending (also across windows)
+            const int32_t px = lane == 0 ? lastx : S.x[lane - 1], py = lane == 0 ? lasty : S.y[lane - 1];
+            if ((lane < nx && px >= xa) || (lane < ny && py >= ya)) atomicOr(err, ERRW_UNSORTED);
+        }
+        const bool takex = lane < nx && xa <= bound, takey = lane < ny && ya <= bound;
+        const uint32_t ry = takex ? below(S.y, ny, xa) : 0u;
+        const bool mx = takex && ry < ny && S.y[ry] == xa;
+        const unsigned vmx = __ballot_sync(FULL_MASK, mx);
+        const uint32_t cx = __popc(__ballot_sync(FULL_MASK, takex)), cy = __popc(__ballot_sync(FULL_MASK, takey));
+        if (FILL) {
+            const uint32_t rx = takey ? below(S.x, nx, ya) : 0u;
+            const bool my = takey && rx < nx && S.x[rx] == ya;
+            const unsigned vmy = __ballot_sync(FULL_MASK, my);
+            const uint32_t px = out + lane + ry - __popc(vmx & lt), py = out + lane + rx - __popc(vmy & lt);
+            if (takex && px < lz) {
+                zc[px] = xa;
+                const V v = xv[ix + lane];
+                zv[px] = mx ? (V)(v + yv[iy + ry]) : v;
+            }
+            if (takey && !my && py < lz) {
+                zc[py] = ya;
+                zv[py] = yv[iy + lane];
+            }
+        } else {
+            if (cx > 0) lastx = S.x[cx - 1];
+            if (cy > 0) lasty = S.y[cy - 1];
+        }
+        out += cx + cy - __popc(vmx);
+        ix += cx;
+        iy += cy;
+        __syncwarp();  // the windows are rewritten
+    }
+    return out;
 }
 
-// shared memory of a merge: the ids of a tile of either row, one more behind them as a sentinel
-template <int T>
+// The longest rows: a CTA merges a row MERGE_TILE entries at a time along the merge path (Odeh, Green, Mwassi, Shmueli &
+// Birk, "Merge Path - Parallel Merging Made Simple", 2012).  A tile holds the next ids of both rows in shared memory; a thread
+// finds by a binary search where its MERGE_ITEMS entries of the merged order begin in either row and merges them one
+// after the other, x before y where both store a column; such a pair is emitted once, with x + y, by the thread that has its
+// x.  The emitted entries are put in order in the shared memory of the ids and written out by consecutive threads.
+// Bound by instruction issue.  Rows of 10 000 entries: 630 us for 6e7; the windows of a warp take less time in all for shorter rows,
+// but a row's 32 entries after 32 entries keep one warp long after the others.
+constexpr int MERGE_ITEMS = 8;
+constexpr int MERGE_LONG_THREADS = 256;
+constexpr uint32_t MERGE_TILE = MERGE_LONG_THREADS * MERGE_ITEMS;
 struct MergeSmem {
-    uint32_t x[T * MERGE_ITEMS + 1], y[T * MERGE_ITEMS + 1];
+    uint32_t x[MERGE_TILE + 1], y[MERGE_TILE + 1];  // the ids of a tile of either row, one more behind them as a sentinel
     uint32_t scratch[33];
-    uint32_t end;  // entries of x in the tile
+    uint32_t end;  // entries of x and, in the upper half, of y in the tile
 };
 
-// Merges the rows xc[0, lx) and yc[0, ly); thread `t` of T.  FILL: the merged row goes to zc, zv (at most lz entries: always
-// enough with the row pointer of the size step; keeps a stale one from writing outside); otherwise the rows are checked.
-// Returns the number of entries of the merged row.  Rows that are not strictly ascending set the
-// error bit in the size step; their merge is wrong but stays inside the rows.
-template <typename V, bool FILL, int T>
-__device__ __forceinline__ uint32_t merge_row(const int32_t* __restrict__ xc, const V* __restrict__ xv, uint32_t lx, const int32_t* __restrict__ yc,
-                                              const V* __restrict__ yv, uint32_t ly, int32_t* __restrict__ zc, V* __restrict__ zv, uint32_t lz,
-                                              MergeSmem<T>& S, int t, uint32_t* err) {
-    constexpr uint32_t TILE = T * MERGE_ITEMS;
+// As merge_windows, by all threads of the CTA.  Rows that are not strictly ascending set the error bit in the size step; their
+// merge is wrong but stays inside the rows.
+template <typename V, bool FILL>
+__device__ __forceinline__ uint32_t merge_path(const int32_t* __restrict__ xc, const V* __restrict__ xv, uint32_t lx, const int32_t* __restrict__ yc,
+                                               const V* __restrict__ yv, uint32_t ly, int32_t* __restrict__ zc, V* __restrict__ zv, uint32_t lz,
+                                               MergeSmem& S, uint32_t* err) {
+    constexpr int T = MERGE_LONG_THREADS;
     constexpr uint32_t NONE = 0xffffu, INF = 0xffffffffu;  // (a negative id fails the check and is merged as 0)
-    static_assert(TILE < NONE, "positions inside a tile are 16 bits");
+    static_assert(MERGE_TILE < NONE, "positions inside a tile are 16 bits");
+    const int t = threadIdx.x;
     uint32_t ix = 0, iy = 0, out = 0;
     // A warp brings in consecutive ids, 32 per step, and hands each to the next lane for the check of the order.
     auto load = [&](const int32_t* __restrict__ ids, uint32_t first, uint32_t n, uint32_t* window) {
@@ -183,12 +241,12 @@ __device__ __forceinline__ uint32_t merge_row(const int32_t* __restrict__ xc, co
         if (!FILL && bad) atomicOr(err, ERRW_UNSORTED);
     };
     while (ix < lx || iy < ly) {  // the same for all threads
-        const uint32_t nx = min(TILE, lx - ix), ny = min(TILE, ly - iy);
+        const uint32_t nx = min(MERGE_TILE, lx - ix), ny = min(MERGE_TILE, ly - iy);
         load(xc, ix, nx, S.x);
         load(yc, iy, ny, S.y);
         if (t == 0) S.x[nx] = S.y[ny] = INF;
-        merge_sync<T>();
-        const uint32_t total = min(TILE, nx + ny);
+        __syncthreads();
+        const uint32_t total = min(MERGE_TILE, nx + ny);
         const uint32_t d = min((uint32_t)t * MERGE_ITEMS, total), d_end = min(d + MERGE_ITEMS, total);
         uint32_t xi = d > ny ? d - ny : 0u, hi = min(d, nx);  // entries of x among the first d of the merged order
         while (xi < hi) {
@@ -215,16 +273,9 @@ __device__ __forceinline__ uint32_t merge_row(const int32_t* __restrict__ xc, co
                 if (ty) b = S.y[min(++yi, ny)];
             }
         }
-        if (t == T - 1) S.end = xi << 16 | yi;
-        uint32_t rank, sum;
-        if (T == 32) {
-            const uint32_t incl = warp_inclusive_scan<uint32_t>(n);
-            sum = __shfl_sync(FULL_MASK, incl, 31);
-            rank = incl - n;
-            __syncwarp();  // the windows are read
-        } else {
-            rank = block_exclusive_scan<uint32_t, T == 32 ? 64 : T>(n, S.scratch, &sum);
-        }
+        if (t == T - 1) S.end = xi | yi << 16;
+        uint32_t sum;
+        const uint32_t rank = block_exclusive_scan<uint32_t, T>(n, S.scratch, &sum);  // (behind its barriers the windows are read)
         const uint32_t end = S.end;
         if (FILL) {
 #pragma unroll
@@ -234,7 +285,7 @@ __device__ __forceinline__ uint32_t merge_row(const int32_t* __restrict__ xc, co
                     S.y[rank + i] = src[i];
                 }
             }
-            merge_sync<T>();
+            __syncthreads();
             const uint32_t n_out = out < lz ? min(sum, lz - out) : 0u;
             for (uint32_t i = t; i < n_out; i += T) {
                 const uint32_t s = S.y[i], sx = s & NONE, sy = s >> 16;
@@ -245,10 +296,10 @@ __device__ __forceinline__ uint32_t merge_row(const int32_t* __restrict__ xc, co
                 zv[out + i] = sx == NONE ? w : sy == NONE ? v : (V)(v + w);
             }
         }
-        merge_sync<T>();  // the windows are rewritten
+        __syncthreads();  // the windows are rewritten
         out += sum;
-        ix += end >> 16;
-        iy += end & 0xffffu;
+        ix += end & 0xffffu;
+        iy += end >> 16;
     }
     return out;
 }
@@ -263,6 +314,7 @@ struct SumArgs {
     const int64_t* y_rowptr;
     const int32_t* y_colidx;
     const V* y_vals;
+    int64_t longest;           // rows of more entries (of both inputs together) are merged by a CTA each
     uint32_t* cnt;             // size step
     const int64_t* z_rowptr;   // fill step
     int32_t* z_colidx;
@@ -270,24 +322,38 @@ struct SumArgs {
     uint32_t* err;             // size step
 };
 
-template <typename V, bool FILL, int T>
-__device__ __forceinline__ void sum_row(const SumArgs<V>& A, int64_t r, int64_t x0, uint32_t lx, int64_t y0, uint32_t ly, MergeSmem<T>& S, int t) {
+// row r by the warp (merge_windows) or by the CTA (merge_path), `leader` in one thread of it
+template <typename V, bool FILL, typename Smem>
+__device__ __forceinline__ void sum_row(const SumArgs<V>& A, int64_t r, int64_t x0, uint32_t lx, int64_t y0, uint32_t ly, Smem& S, bool leader) {
     const int64_t z0 = FILL ? A.z_rowptr[r] : 0;
     const uint32_t lz = FILL ? (uint32_t)(A.z_rowptr[r + 1] - z0) : 0u;
-    const uint32_t n = merge_row<V, FILL, T>(A.x_colidx + x0, FILL ? A.x_vals + x0 : nullptr, lx, A.y_colidx + y0, FILL ? A.y_vals + y0 : nullptr, ly,
-                                             FILL ? A.z_colidx + z0 : nullptr, FILL ? A.z_vals + z0 : nullptr, lz, S, t, A.err);
-    if (!FILL && t == 0) A.cnt[r] = n;
+    const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
+    const V *xv = FILL ? A.x_vals + x0 : nullptr, *yv = FILL ? A.y_vals + y0 : nullptr;
+    int32_t* zc = FILL ? A.z_colidx + z0 : nullptr;
+    V* zv = FILL ? A.z_vals + z0 : nullptr;
+    uint32_t n;
+    if constexpr (std::is_same<Smem, WindowSmem>::value) n = merge_windows<V, FILL>(xc, xv, lx, yc, yv, ly, zc, zv, lz, S, A.err);
+    else n = merge_path<V, FILL>(xc, xv, lx, yc, yv, ly, zc, zv, lz, S, A.err);
+    if (!FILL && leader) A.cnt[r] = n;
 }
 
-// One warp per row, `batch` consecutive rows per warp.  The launch hands the rows out, in small CTAs: a CTA keeps its place until its
-// last row is done (CTAs of eight rows: 19 % of the warps active on average).  (Counters in the workspace, from which a
-// fixed number of warps drew their rows, lost rows when two fills shared a workspace.)
+// One warp per row.  A CTA has `share` consecutive rows, which its warps draw one after the other.
 template <typename V, bool FILL>
-__global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(SumArgs<V> A, int batch) {
-    __shared__ MergeSmem<32> smem[MERGE_WARPS];
+__global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(SumArgs<V> A, int share) {
+    __shared__ WindowSmem smem[MERGE_WARPS];
+    __shared__ int s_next;
     const int warp = threadIdx.x >> 5, lane = lane_id();
-    const int64_t first = ((int64_t)blockIdx.x * MERGE_WARPS + warp) * batch, last = min(first + batch, A.m);
-    for (int64_t r = first; r < last; ++r) {
+    chain_begin();
+    if (threadIdx.x == 0) s_next = 0;
+    __syncthreads();
+    const int64_t first = (int64_t)blockIdx.x * share;
+    const int n = (int)min((int64_t)share, A.m - first);
+    for (;;) {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(&s_next, 1);
+        i = __shfl_sync(FULL_MASK, i, 0);
+        if (i >= n) break;
+        const int64_t r = first + i;
         const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
         const int64_t lx = A.x_rowptr[r + 1] - x0, ly = A.y_rowptr[r + 1] - y0;
         if (lx < 0 || ly < 0 || lx + ly > 0x7fffffffLL) {
@@ -295,27 +361,29 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32) add_merge_kernel(SumArgs<V> 
                 atomicOr(A.err, ERRW_BAD_ROWPTR);
                 A.cnt[r] = 0;
             }
-        } else if (lx + ly <= MERGE_LONG) {
-            sum_row<V, FILL, 32>(A, r, x0, (uint32_t)lx, y0, (uint32_t)ly, smem[warp], lane);
+        } else if (lx + ly <= A.longest) {
+            sum_row<V, FILL>(A, r, x0, (uint32_t)lx, y0, (uint32_t)ly, smem[warp], lane == 0);
         }
     }
+    chain_end();
 }
 
-// The rows of more than MERGE_LONG entries, a CTA each.  The rows are dealt to the CTAs in units of 1 << unit_bits, a unit of every
+// The longer rows, a CTA each.  The rows are dealt to the CTAs in units of 1 << unit_bits, a unit of every
 // gridDim.x, so that long rows which stand together go to different CTAs; a CTA has at most one unit per thread.  A unit of few
 // entries has no such row: of it only the ends are looked at.
 template <typename V, bool FILL>
-__global__ void __launch_bounds__(MERGE_LONG_THREADS) add_long_kernel(SumArgs<V> A, int unit_bits) {
-    __shared__ MergeSmem<MERGE_LONG_THREADS> smem;
+__global__ void __launch_bounds__(MERGE_LONG_THREADS, 6) add_long_kernel(SumArgs<V> A, int unit_bits) {
+    __shared__ MergeSmem smem;
     __shared__ int64_t s_unit[MERGE_LONG_THREADS];  // first rows of the units that are looked at row by row
     __shared__ int64_t s_row[MERGE_LONG_THREADS];
     __shared__ int s_units, s_rows;
     const int t = threadIdx.x;
+    chain_begin();
     auto entries = [&](int64_t a, int64_t b) { return A.x_rowptr[b] - A.x_rowptr[a] + A.y_rowptr[b] - A.y_rowptr[a]; };
     if (t == 0) s_units = 0;
     __syncthreads();
     const int64_t u0 = ((int64_t)blockIdx.x + (int64_t)t * gridDim.x) << unit_bits;
-    if (u0 < A.m && entries(u0, min(u0 + (1 << unit_bits), A.m)) > MERGE_LONG) s_unit[atomicAdd(&s_units, 1)] = u0;
+    if (u0 < A.m && entries(u0, min(u0 + (1 << unit_bits), A.m)) > A.longest) s_unit[atomicAdd(&s_units, 1)] = u0;
     __syncthreads();
     const int n = s_units << unit_bits;
     for (int base = 0; base < n; base += MERGE_LONG_THREADS) {
@@ -325,22 +393,24 @@ __global__ void __launch_bounds__(MERGE_LONG_THREADS) add_long_kernel(SumArgs<V>
             const int64_t r = s_unit[(base + t) >> unit_bits] + ((base + t) & ((1 << unit_bits) - 1));
             if (r < A.m) {
                 const int64_t lx = A.x_rowptr[r + 1] - A.x_rowptr[r], ly = A.y_rowptr[r + 1] - A.y_rowptr[r];
-                if (lx >= 0 && ly >= 0 && lx + ly > MERGE_LONG && lx + ly <= 0x7fffffffLL) s_row[atomicAdd(&s_rows, 1)] = r;
+                if (lx >= 0 && ly >= 0 && lx + ly > A.longest && lx + ly <= 0x7fffffffLL) s_row[atomicAdd(&s_rows, 1)] = r;
             }
         }
         __syncthreads();
         const int rows = s_rows;
         for (int i = 0; i < rows; ++i) {
             const int64_t r = s_row[i], x0 = A.x_rowptr[r], y0 = A.y_rowptr[r];
-            sum_row<V, FILL, MERGE_LONG_THREADS>(A, r, x0, (uint32_t)(A.x_rowptr[r + 1] - x0), y0, (uint32_t)(A.y_rowptr[r + 1] - y0), smem, t);
+            sum_row<V, FILL>(A, r, x0, (uint32_t)(A.x_rowptr[r + 1] - x0), y0, (uint32_t)(A.y_rowptr[r + 1] - y0), smem, t == 0);
         }
         __syncthreads();
     }
+    chain_end();
 }
 
 // G lanes per row, where rows are short on average
 template <int G>
 __global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A) {
+    chain_begin();
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int gl = threadIdx.x & (G - 1);
     if (r >= A.m) return;  // whole groups leave together
@@ -350,7 +420,7 @@ __global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A) {
         if (gl == 0) { atomicOr(A.err, ERRW_BAD_ROWPTR); A.cnt[r] = 0; }
         return;
     }
-    if (lx64 + ly64 > MERGE_LONG) return;
+    if (lx64 + ly64 > A.longest) return;
     const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
     const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
     // the sortedness of X is checked here, that of Y inside the walk
@@ -362,11 +432,12 @@ __global__ void __launch_bounds__(256) add_count_kernel(SumArgs<uint32_t> A) {
 
 template <typename V, int G>
 __global__ void __launch_bounds__(256) add_fill_kernel(SumArgs<V> A) {
+    chain_begin();
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (r >= A.m) return;
     const int64_t x0 = A.x_rowptr[r], y0 = A.y_rowptr[r], z0 = A.z_rowptr[r];
     const int64_t lx64 = A.x_rowptr[r + 1] - x0, ly64 = A.y_rowptr[r + 1] - y0;
-    if (lx64 + ly64 > MERGE_LONG) return;
+    if (lx64 + ly64 > A.longest) return;
     const uint32_t lx = (uint32_t)lx64, ly = (uint32_t)ly64;
     const uint32_t lz = (uint32_t)(A.z_rowptr[r + 1] - z0);
     const int32_t *xc = A.x_colidx + x0, *yc = A.y_colidx + y0;
@@ -421,30 +492,32 @@ void launch_panel_fill(int g, int64_t m, const int64_t* rowptr, const int32_t* c
     note_launches(1);
 }
 
-// kernels of one step of the sum: the rows, then the long ones among them
+// Entries of the longest row that a warp merges: about twice its share of all, so that no warp is left with one row when the others are
+// done, not fewer than half a tile of a CTA and at most two.  Power-law panels of 2^13, 2^15 and 2^16 rows, 4.5e6, 3.6e7 and 1.0e8 entries: 160, 609
+// and 1189 us; with 4096 for all of them the first takes 319, with 1024 the last 1519; rows of 2000 entries 554 us, with 1024 786.
+int64_t longest_of_a_warp(int64_t entries) { return std::min<int64_t>(std::max<int64_t>(entries / (148 * 24), 1024), 4096); }
+
+// Kernels of one step of the sum, the second beside the first: lanes of a warp share a row up to a mean of 16 entries, warps take
+// the rows beyond.  The line lies where rows that differ much in length turn: power-law panels of 19 entries per row 224 us by 16 lanes, 147
+// by warps.  Equal rows would turn at 30 (21 entries: 1173 us by 16 lanes, 1591 by warps; 29: 968 to 1189; 33: 1023 either way).
 template <typename V, bool FILL>
 spsyrk_status_t launch_sum(int g, const SumArgs<V>& A, cudaStream_t st) {
-    const auto blocks = [&](int64_t threads) { return (unsigned)((threads + 255) / 256); };
-    if (g > 16) {
-        // consecutive rows per warp: one while that gives at most 32 warps per SM 16 times over, up to 32
-        const int batch = (int)std::min<int64_t>(std::max<int64_t>(A.m / (148 * 32 * 16), 1), 32);
-        const int64_t rows = (int64_t)batch * MERGE_WARPS;
-        add_merge_kernel<V, FILL><<<(unsigned)((A.m + rows - 1) / rows), MERGE_WARPS * 32, 0, st>>>(A, batch);
-    } else if constexpr (FILL) {
-        if (g == 4) add_fill_kernel<V, 4><<<blocks(A.m * 4), 256, 0, st>>>(A);
-        else if (g == 8) add_fill_kernel<V, 8><<<blocks(A.m * 8), 256, 0, st>>>(A);
-        else add_fill_kernel<V, 16><<<blocks(A.m * 16), 256, 0, st>>>(A);
-    } else {
-        if (g == 4) add_count_kernel<4><<<blocks(A.m * 4), 256, 0, st>>>(A);
-        else if (g == 8) add_count_kernel<8><<<blocks(A.m * 8), 256, 0, st>>>(A);
-        else add_count_kernel<16><<<blocks(A.m * 16), 256, 0, st>>>(A);
+    Chain ch{st, true};
+    const auto lanes = [&](void (*kern)(SumArgs<V>), int width) { return ch.launch(true, kern, (unsigned)((A.m * width + 255) / 256), 256, 0, A); };
+    if (g <= 16) {
+        if constexpr (FILL) SPSYRK_CUDA_TRY(g == 4 ? lanes(add_fill_kernel<V, 4>, 4) : g == 8 ? lanes(add_fill_kernel<V, 8>, 8) : lanes(add_fill_kernel<V, 16>, 16));
+        else SPSYRK_CUDA_TRY(g == 4 ? lanes(add_count_kernel<4>, 4) : g == 8 ? lanes(add_count_kernel<8>, 8) : lanes(add_count_kernel<16>, 16));
     }
     const int unit_bits = A.m <= 1 << 16 ? 0 : A.m <= 1 << 20 ? 2 : 5;
     const int64_t units = (A.m + (1 << unit_bits) - 1) >> unit_bits;
-    const int64_t ctas = std::max<int64_t>(std::min<int64_t>(units, 148 * 16), (units + MERGE_LONG_THREADS - 1) / MERGE_LONG_THREADS);
-    add_long_kernel<V, FILL><<<(unsigned)ctas, MERGE_LONG_THREADS, 0, st>>>(A, unit_bits);
-    note_launches(2);
-    SPSYRK_CUDA_TRY(cudaGetLastError());
+    const int64_t ctas = std::max<int64_t>(std::min<int64_t>(units, 148 * 12), (units + MERGE_LONG_THREADS - 1) / MERGE_LONG_THREADS);
+    SPSYRK_CUDA_TRY(ch.launch(true, add_long_kernel<V, FILL>, (unsigned)ctas, MERGE_LONG_THREADS, 0, A, unit_bits));
+    if (g > 16) {
+        // the other rows beside the long ones; rows per CTA: one for each warp as long as all of them are at most 16 times what the
+        // GPU holds, up to 32 then
+        const int64_t share = std::min<int64_t>(std::max<int64_t>(A.m / (148 * 32 * 16), 1), 32) * MERGE_WARPS;
+        SPSYRK_CUDA_TRY(ch.launch(true, add_merge_kernel<V, FILL>, (unsigned)((A.m + share - 1) / share), MERGE_WARPS * 32, 0, A, (int)share));
+    }
     return SPSYRK_OK;
 }
 
@@ -508,12 +581,13 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
     RowWs w;
     carve(&w, d_workspace, m);
     const int g = group_width(nnz_x + nnz_y, m);
+    const int64_t longest = longest_of_a_warp(nnz_x + nnz_y);
     if (!d_z_colidx) {  // step 2: sizes
         if (!nnz_out) return SPSYRK_ERR_INVALID_ARG;
         SPSYRK_CUDA_TRY(cudaMemsetAsync(w.err, 0, 4, st));
         if (m > 0) {
             const spsyrk_status_t s = launch_sum<uint32_t, false>(
-                g, {m, d_x_rowptr, d_x_colidx, nullptr, d_y_rowptr, d_y_colidx, nullptr, w.cnt, nullptr, nullptr, nullptr, w.err}, st);
+                g, {m, d_x_rowptr, d_x_colidx, nullptr, d_y_rowptr, d_y_colidx, nullptr, longest, w.cnt, nullptr, nullptr, nullptr, w.err}, st);
             if (s != SPSYRK_OK) return s;
         }
         return scan_and_total(w, m, d_z_rowptr, nnz_out, st);
@@ -523,7 +597,7 @@ extern "C" spsyrk_status_t spsyrk_accumulate(int64_t m, spsyrk_dtype_t dtype, in
     const auto fill = [&](auto* z_vals) {
         using V = std::remove_pointer_t<decltype(z_vals)>;
         return launch_sum<V, true>(g, {m, d_x_rowptr, d_x_colidx, static_cast<const V*>(d_x_vals), d_y_rowptr, d_y_colidx, static_cast<const V*>(d_y_vals),
-                                       nullptr, d_z_rowptr, d_z_colidx, z_vals, nullptr}, st);
+                                       longest, nullptr, d_z_rowptr, d_z_colidx, z_vals, nullptr}, st);
     };
     switch (dtype) {
         case SPSYRK_F64: return fill(static_cast<double*>(d_z_vals));

@@ -1,5 +1,5 @@
-"""The sparse sum at the edges of its tiles: a warp merges 256 entries of both rows at a time, a CTA 2048; rows of more
-than 4096 entries of both inputs go to a CTA."""
+"""The sparse sum at the edges of its windows and tiles: a warp merges 32 entries of either row at a time, a CTA 2048 of both; rows
+of more than 1024 entries of both inputs go to a CTA, where there are many entries those of more than 4096."""
 import numpy as np
 import pytest
 import torch
@@ -39,7 +39,7 @@ def _pair(kind, size, rng):
 @pytest.mark.parametrize("kind", ["same", "shifted", "blocks", "one", "random"])
 def test_accumulate_at_tile_edges(B, kind, empty_rows, dtype):
     rng = np.random.default_rng(7)
-    pairs = [_pair(kind, s, rng) for s in (1, 7, 8, 9, 127, 128, 129, 255, 256, 257, 511, 513, 2047, 2048, 2049, 4095, 4096, 4097, 8191, 8192, 8193, 20_011)]
+    pairs = [_pair(kind, s, rng) for s in (1, 7, 8, 9, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2047, 2048, 2049, 4095, 4096, 4097, 8191, 8192, 8193, 20_011)]
     pairs += [(np.zeros(0, dtype=np.int64),) * 2] * empty_rows + [pairs[-1], pairs[4]]
     m = len(pairs)
     npdt = {torch.float64: np.float64, torch.float32: np.float32, torch.int32: np.int32}[dtype]
@@ -55,6 +55,17 @@ def test_accumulate_at_tile_edges(B, kind, empty_rows, dtype):
     er, ec, ev = oracle.add(m, x[0], x[1], x[2].astype(np.float64), y[0], y[1], y[2].astype(np.float64))
     assert np.array_equal(zr, er) and np.array_equal(zc, ec)
     assert np.array_equal(zv, ev.astype(npdt))  # one rounded addition: the double sum of two floats rounds to the float sum
+
+
+def test_accumulate_of_many_entries(B):
+    """So many entries that a warp merges rows of up to 4096: rows on both sides of that, among rows of 2000."""
+    rng = np.random.default_rng(17)
+    lengths = [np.where(np.arange(7400) % 100 == 0, rng.integers(2040, 2056, 7400), rng.integers(900, 1100, 7400)) for _ in range(2)]
+    x, y = (_device_csr(ln, 51 + i) for i, ln in enumerate(lengths))
+    assert (x[1].numel() + y[1].numel()) // (148 * 24) >= 4096
+    got = [t.cpu().numpy() for t in B.spsyrk_accumulate(7400, *x, *y)]
+    ref = oracle.add(7400, *(t.cpu().numpy() for t in x), *(t.cpu().numpy() for t in y))
+    assert all(np.array_equal(a, b) for a, b in zip(got, ref))
 
 
 @pytest.mark.parametrize("size", [300, 5000])
