@@ -128,6 +128,15 @@ def _workspace(nbytes: int, device) -> torch.Tensor:
     return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
 
 
+def _in_use_on(stream, *tensors):
+    """Memory of the binding's own that a call leaves in use on `stream`: torch's allocator, which knows a tensor by the stream
+    it was allocated for, must not give it to anyone else before the work there has ended."""
+    if stream is not None:
+        for t in tensors:
+            if t is not None:
+                t.record_stream(stream)
+
+
 class Plan:
     """Owner of a spsyrk_plan_t and of the tensors it borrows (A and the workspace)."""
 
@@ -225,6 +234,7 @@ def spsyrk_numeric(plan: Plan, c_rowptr, c_colidx, c_vals, stream=None):
     _dev_check(c_rowptr, c_colidx, c_vals)
     assert c_colidx.dtype == torch.int32 and c_vals.dtype == plan.dtype
     _check(_lib.spsyrk_numeric(plan._h, _p(c_rowptr), _p(c_colidx), _p(c_vals), _stream(stream)), "spsyrk_numeric")
+    _in_use_on(stream, plan._keep["ws"], plan._keep.get("map"))
 
 
 def spsyrk_numeric_rows(plan: Plan, row_begin: int, row_end: int, c_rowptr, c_colidx, c_vals, stream=None):
@@ -232,6 +242,7 @@ def spsyrk_numeric_rows(plan: Plan, row_begin: int, row_end: int, c_rowptr, c_co
     assert c_colidx.dtype == torch.int32 and c_vals.dtype == plan.dtype
     _check(_lib.spsyrk_numeric_rows(plan._h, int(row_begin), int(row_end), _p(c_rowptr), _p(c_colidx), _p(c_vals), _stream(stream)),
            "spsyrk_numeric_rows")
+    _in_use_on(stream, plan._keep["ws"], plan._keep.get("map"))
 
 
 def spsyrk_onepass_slots(plan: Plan, stream=None) -> int:
@@ -260,6 +271,7 @@ def spsyrk_onepass_compact(plan: Plan, c_rowptr, nnz, slot_colidx, slot_vals, c_
     _dev_check(c_rowptr, slot_colidx, slot_vals, c_colidx, c_vals)
     _check(_lib.spsyrk_onepass_compact(plan._h, _p(c_rowptr), int(nnz), _p(slot_colidx), _p(slot_vals), _p(c_colidx), _p(c_vals),
                                        _stream(stream)), "spsyrk_onepass_compact")
+    _in_use_on(stream, plan._keep["ws"])
 
 
 def onepass_syrk(plan: Plan, stream=None, compact=True):
@@ -278,6 +290,7 @@ def onepass_syrk(plan: Plan, stream=None, compact=True):
     c_colidx = torch.empty(max(nnz, 1), dtype=torch.int32, device=dev)
     c_vals = torch.empty(max(nnz, 1), dtype=plan.dtype, device=dev)
     spsyrk_onepass_compact(plan, c_rowptr, nnz, s_col, s_val, c_colidx, c_vals, stream)
+    _in_use_on(stream, s_col, s_val)
     return c_rowptr, c_colidx[:nnz], c_vals[:nnz]
 
 
@@ -379,6 +392,7 @@ def spsyrk_mirror(m, l_rowptr, l_colidx, l_vals, stream=None, workspace=None, ou
         f_vals = torch.empty(max(nnz.value, 1), dtype=l_vals.dtype, device=l_rowptr.device)
     _check(_lib.spsyrk_mirror(m, nnz_l, code, _p(l_rowptr), _p(l_colidx), _p(l_vals), _p(f_rowptr), _p(f_colidx),
                               _p(f_vals), ctypes.byref(nnz), _p(ws), ctypes.byref(sz), st), "spsyrk_mirror(fill)")
+    _in_use_on(stream, ws)
     return f_rowptr, f_colidx[:nnz.value], f_vals[:nnz.value]
 
 

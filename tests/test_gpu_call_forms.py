@@ -24,6 +24,33 @@ def random_csr(m, n, per_row, dtype, seed, ones=False):
     return W.CSR(m, n, rowptr, np.concatenate(rows).astype(np.int32), vals.astype(dtype))
 
 
+# ------------------------------------------------------------------ streams and torch's allocator
+@pytest.mark.parametrize("call", ["product", "one pass", "mirror"])
+def test_memory_of_the_binding_while_another_stream_uses_it(B, call):
+    """A call on another stream than the current one leaves its workspace in use when it returns, and the plan is dropped: new tensors
+    of the current stream must not get that memory yet."""
+    a = random_csr(30_000, 30_000, 12, np.float64, 5)
+    d = dev(a)
+    c = B.tril_syrk(a.m, a.n, *d)[:3]
+
+    def run(stream):
+        if call == "product":
+            return B.tril_syrk(a.m, a.n, *d, stream=stream)[:3]
+        if call == "mirror":
+            return B.spsyrk_mirror(a.m, *c, stream=stream)
+        return B.onepass_syrk(B.spsyrk_plan(a.m, a.n, *d, stream=stream), stream)
+
+    expected = run(None)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(5):
+        got = run(side)
+        others = [torch.full((1 << k,), 0x5a, dtype=torch.uint8, device="cuda") for k in range(12, 29)]
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(got, expected))
+        del others, got
+
+
 # ------------------------------------------------------------------ matrices that fail their checks
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("fault", ["column ids", "one column id", "row pointers", "duplicate"])
