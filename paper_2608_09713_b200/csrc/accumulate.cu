@@ -467,10 +467,11 @@ spsyrk_status_t scan_and_total(const RowWs& w, int64_t m, int64_t* d_rowptr_out,
     if (m == 0) {
         SPSYRK_CUDA_TRY(cudaMemsetAsync(d_rowptr_out, 0, sizeof(int64_t), st));
         h.host[0] = h.host[1] = 0;
-    } else {
-        SPSYRK_CUDA_TRY(scan_launch(ScanArray<uint32_t>{w.cnt}, m, ScanIntoHost{d_rowptr_out, m, w.err, h.dev}, w.partials, w.err, st));
+    } else if (scan_launch(ScanArray<uint32_t>{w.cnt}, m, ScanIntoHost{d_rowptr_out, m, w.err, h.dev}, w.partials, w.err, st) != cudaSuccess) {
+        cudaStreamSynchronize(st);  // the error may be an earlier launch's: the scan is under way then and writes into the host block
+        return SPSYRK_ERR_CUDA;
     }
-    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+    SPSYRK_CUDA_TRY(wait_for(st));
     if (const uint32_t e = h.errors(h.host[1])) return status_of(e);
     *total = h.host[0];
     return SPSYRK_OK;

@@ -386,18 +386,19 @@ void launch_block_desc(spsyrk_plan_s* pl, cudaStream_t st) {
 
 // analyse: the binary analysis is due (a new plan's first view); at least two CTAs, at most what the GPU holds beside others
 template <int G>
-void launch_row_work(spsyrk_plan_s* pl, bool analyse, cudaStream_t st) {
+cudaError_t launch_row_work(spsyrk_plan_s* pl, bool analyse, cudaStream_t st) {
     const PlanDev& P = pl->dev;
     const int64_t rows = P.r1 - P.r0, nb = bin_blocks(rows);
     HeavyArrays heavy{pl->colcnt, pl->facts, pl->heavy_id, pl->heavy_mask, 0u};
     if (analyse) heavy.ctas = (unsigned)std::min<int64_t>(2 + std::max<int64_t>(P.n, (int64_t)P.m * G) / BIN_THREADS, (int64_t)pl->sm_count * 8);
     if (nb > 0)
-        launch_linked(row_work_kernel<G>, (unsigned)nb + heavy.ctas, BIN_THREADS, 0, st, P, pl->cls, BLOCK_CLASS_MAX_WORK, ROW_CHUNK_BITS_MAX_SYMBOLIC, pl->diag,
-                      bin_tile(rows), pl->blockhist, nb, pl->work_total_dev, pl->work_total_dev + 1, heavy);
-    else if (analyse) {
+        return launch_linked(row_work_kernel<G>, (unsigned)nb + heavy.ctas, BIN_THREADS, 0, st, P, pl->cls, BLOCK_CLASS_MAX_WORK, ROW_CHUNK_BITS_MAX_SYMBOLIC, pl->diag,
+                             bin_tile(rows), pl->blockhist, nb, pl->work_total_dev, pl->work_total_dev + 1, heavy);
+    if (analyse) {
         heavy_analysis_kernel<G><<<heavy.ctas, BIN_THREADS, 0, st>>>(P, heavy);
         note_launches(1);
     }
+    return cudaGetLastError();
 }
 
 int group_width(int64_t nnz, int64_t m) {
@@ -456,10 +457,10 @@ spsyrk_status_t bin_launch(spsyrk_plan_s* pl, int64_t* host, int64_t* gave_up, b
     const PlanFacts facts{pl->class_start_dev, pl->work_total_dev, pl->work_total_dev + 1, pl->facts, P.err, host, gave_up};
     if (P.nnz == 0) analyse = false;
     switch (group_width(P.nnz, P.m)) {
-        case 4: launch_row_work<4>(pl, analyse, st); break;
-        case 8: launch_row_work<8>(pl, analyse, st); break;
-        case 16: launch_row_work<16>(pl, analyse, st); break;
-        default: launch_row_work<32>(pl, analyse, st); break;
+        case 4: SPSYRK_CUDA_TRY(launch_row_work<4>(pl, analyse, st)); break;
+        case 8: SPSYRK_CUDA_TRY(launch_row_work<8>(pl, analyse, st)); break;
+        case 16: SPSYRK_CUDA_TRY(launch_row_work<16>(pl, analyse, st)); break;
+        default: SPSYRK_CUDA_TRY(launch_row_work<32>(pl, analyse, st)); break;
     }
     if (rows == 0) {
         SPSYRK_CUDA_TRY(cudaMemsetAsync(pl->class_start_dev, 0, (NCLASS + 1) * sizeof(int64_t), st));
@@ -528,7 +529,7 @@ spsyrk_status_t estimate_and_bin(spsyrk_plan_s* pl, bool fresh, cudaStream_t st)
             note_launches(1);
         }
     }
-    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+    SPSYRK_CUDA_TRY(wait_for(st));
     s = bin_collect(pl, pl->host, pl->host.host);
     if (s == SPSYRK_OK && up) s = bin_collect(up, pl->host, pl->host.host + 16);
     return s;
@@ -912,7 +913,7 @@ cudaError_t scan_counts(spsyrk_plan_s* pl, const int32_t* counts, int64_t rows, 
 }
 // waits for it
 spsyrk_status_t collect_total(spsyrk_plan_s* pl, int64_t rows, bool routes, int64_t* total, cudaStream_t st) {
-    SPSYRK_CUDA_TRY(cudaStreamSynchronize(st));
+    SPSYRK_CUDA_TRY(wait_for(st));
     spsyrk_plan_s* up = pl->upper_active ? pl->upper : nullptr;
     if (rows == 0) {
         *total = 0;

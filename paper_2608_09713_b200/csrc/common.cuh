@@ -80,6 +80,20 @@ __device__ __forceinline__ void chain_end(bool this_cta) {  // true in one CTA
 }
 __device__ __forceinline__ void chain_end() { chain_end(blockIdx.x == 0); }
 
+// Launches, and returns the first error that has not been reported: an earlier launch by <<< >>> of the same call says nothing by itself.
+template <typename... Params>
+[[nodiscard]] inline cudaError_t launch_kernel(const cudaLaunchConfig_t& cfg, void (*kern)(Params...), Params... params) {
+    note_launches(1);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, params...), earlier = cudaGetLastError();
+    return e != cudaSuccess ? e : earlier;
+}
+
+// Waits for the stream, and returns the error of a launch that has not been reported.
+inline cudaError_t wait_for(cudaStream_t st) {
+    const cudaError_t launched = cudaGetLastError(), e = cudaStreamSynchronize(st);
+    return launched != cudaSuccess ? launched : e;
+}
+
 // A chain of kernels that do not depend on one another (see chain_begin).  With `overlap` off every launch is an ordinary one,
 // and so is that of a kernel that fills the GPU for long (`brief` false): its CTAs would start one by one as those of the
 // kernel before end, and a persistent grid that shares its rows out beforehand ends with the last of them.  (All launches
@@ -90,7 +104,7 @@ struct Chain {
     bool overlap;
     bool first = true;
     template <typename... Params, typename... Args>
-    cudaError_t launch(bool brief, void (*kern)(Params...), unsigned grid, int threads, size_t smem, Args... args) {
+    [[nodiscard]] cudaError_t launch(bool brief, void (*kern)(Params...), unsigned grid, int threads, size_t smem, Args... args) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(grid);
         cfg.blockDim = dim3((unsigned)threads);
@@ -102,8 +116,7 @@ struct Chain {
         cfg.attrs = &attr;
         cfg.numAttrs = overlap && brief && !first ? 1 : 0;
         first = false;
-        note_launches(1);
-        return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+        return launch_kernel(cfg, kern, static_cast<Params>(args)...);
     }
 };
 
@@ -120,7 +133,7 @@ __device__ __forceinline__ void link(P&... p) {
     (..., [&] { asm volatile("" : "+l"(p)::"memory"); }());
 }
 template <typename... Params, typename... Args>
-inline cudaError_t launch_linked(void (*kern)(Params...), unsigned grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+[[nodiscard]] inline cudaError_t launch_linked(void (*kern)(Params...), unsigned grid, int threads, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3((unsigned)threads);
@@ -131,8 +144,7 @@ inline cudaError_t launch_linked(void (*kern)(Params...), unsigned grid, int thr
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    note_launches(1);
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    return launch_kernel(cfg, kern, static_cast<Params>(args)...);
 }
 
 __host__ __device__ constexpr int ilog2_ce(int v) { return v <= 1 ? 0 : 1 + ilog2_ce(v >> 1); }

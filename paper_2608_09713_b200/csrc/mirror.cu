@@ -365,16 +365,16 @@ int group_width(int64_t nnz, int64_t m) {
 }
 
 template <typename V>
-void mirror_copy_lower(int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx, const void* l_vals, const int64_t* f_rowptr, int32_t* f_colidx,
-                       void* f_vals, cudaStream_t st) {
+cudaError_t mirror_copy_lower(int64_t m, int64_t nnz_l, const int64_t* l_rowptr, const int32_t* l_colidx, const void* l_vals, const int64_t* f_rowptr, int32_t* f_colidx,
+                              void* f_vals, cudaStream_t st) {
 #define COPY(G)                                                                                                                                       \
-    launch_linked(mirror_copy_lower_kernel<V, G>, (unsigned)((m * G + 255) / 256), 256, 0, st, l_rowptr, l_colidx, static_cast<const V*>(l_vals), m, f_rowptr, \
-                  f_colidx, static_cast<V*>(f_vals))
+    return launch_linked(mirror_copy_lower_kernel<V, G>, (unsigned)((m * G + 255) / 256), 256, 0, st, l_rowptr, l_colidx, static_cast<const V*>(l_vals), m, f_rowptr, \
+                         f_colidx, static_cast<V*>(f_vals))
     switch (group_width(nnz_l, m)) {
-        case 4: COPY(4); break;
-        case 8: COPY(8); break;
-        case 16: COPY(16); break;
-        default: COPY(32); break;
+        case 4: COPY(4);
+        case 8: COPY(8);
+        case 16: COPY(16);
+        default: COPY(32);
     }
 #undef COPY
 }
@@ -475,7 +475,7 @@ spsyrk_status_t mirror_fill(const MirrorWs& w, int64_t m, int64_t nnz_l, const i
         SPSYRK_CUDA_TRY(launch_linked(mirror_copy_chunks_kernel<VB>, (unsigned)((nnz_l + per_cta - 1) / per_cta), 256, 0, st, l_rowptr, l_colidx, static_cast<const VB*>(l_vals),
                                       m, nnz_l, (const int32_t*)w.step_row, (const int64_t*)f_rowptr, f_colidx, static_cast<VB*>(f_vals)));
     } else {
-        mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+        SPSYRK_CUDA_TRY(mirror_copy_lower<VB>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st));
     }
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
@@ -540,7 +540,7 @@ spsyrk_status_t mirror_fill_radix(const MirrorWs& ws, int64_t m, int64_t nnz_l, 
     mirror_rowlen_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l_rowptr, w.seg_start, w.seg_end, m, w.rowtot);
     note_launches(1);
     SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.rowtot, m, f_rowptr, w.partials, w.err, st));
-    mirror_copy_lower<uint32_t>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+    SPSYRK_CUDA_TRY(mirror_copy_lower<uint32_t>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st));
     SPSYRK_CUDA_TRY(cudaGetLastError());
     return SPSYRK_OK;
 }
@@ -650,7 +650,7 @@ spsyrk_status_t mirror_fill_rec(const MirrorWs& w, int64_t m, int64_t nnz_l, con
         note_launches(1);
     }
     SPSYRK_CUDA_TRY(exclusive_scan_i64<uint32_t>(w.rowtot, m, f_rowptr, w.partials, w.err, st));
-    if (m > 0 && nnz_l > 0) mirror_copy_lower<uint64_t>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st);
+    if (m > 0 && nnz_l > 0) SPSYRK_CUDA_TRY(mirror_copy_lower<uint64_t>(m, nnz_l, l_rowptr, l_colidx, l_vals, f_rowptr, f_colidx, f_vals, st));
     SPSYRK_CUDA_TRY(cudaGetLastError());
 #ifdef SPSYRK_CHECKED
     {
