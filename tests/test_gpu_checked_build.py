@@ -1,7 +1,8 @@
 """The bounds-checked build of the library (libspsyrk_checked.so: every shared-memory slot and output
 offset the kernels compute is tested before it is used; a violation is reported as an internal
-error instead of touching memory) must run the reduced workloads, the mirror and the random-matrix
-sweep clean: every call returns SPSYRK_OK and every result still matches the oracle.  The selected
+error instead of touching memory; lanes that may do something in any order do it in another one) must run the reduced
+workloads, the mirror by every sort and at its lines, the rows that have a path of their own, the sparse sum and the
+random-matrix sweep clean: every call returns SPSYRK_OK and every result still matches the oracle.  The selected
 tests are run once more in a child process that loads that build."""
 import os
 import subprocess
@@ -26,7 +27,9 @@ def test_checked_build_runs_clean():
            "tests/test_gpu_parity.py::test_rows_at_every_class_boundary", "tests/test_gpu_parity.py::test_blocks",
            "tests/test_gpu_parity.py::test_symm", "tests/test_gpu_parity.py::test_one_pass_mode",
            "tests/test_gpu_parity.py::test_numeric_by_row_blocks", "tests/test_gpu_parity.py::test_mirror_general_lower_triangles",
-           "tests/test_gpu_random.py"]
+           "tests/test_gpu_parity.py::test_mirror_few_entries_many_rows", "tests/test_gpu_call_forms.py::test_mirror_wherever_the_entries_lie",
+           "tests/test_gpu_mirror_lines.py", "tests/test_gpu_accumulate.py", "tests/test_gpu_binary_rows.py", "tests/test_gpu_light_rows.py",
+           "tests/test_gpu_plan_rows.py", "tests/test_gpu_random.py"]
     run = subprocess.run([sys.executable, "-m", "pytest", *sel, "-m", "gpu", "-x", "-q", "-p", "no:cacheprovider"],
                          cwd=ROOT, env=env, capture_output=True, text=True, timeout=3000)
     assert run.returncode == 0, run.stdout[-4000:] + run.stderr[-2000:]

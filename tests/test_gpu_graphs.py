@@ -39,9 +39,9 @@ def _replays(call, outputs, expected):
             assert torch.equal(t, e)
 
 
-# by buckets in two passes, by records, by radix passes, by buckets in three passes; small and of several tiles
+# by buckets in two passes (small and of several tiles), by records, by radix passes, by buckets in three passes
 @pytest.mark.parametrize("m,d,dtype", [(500, 4, torch.float64), (9000, 8, torch.float64), (9000, 8, torch.float32), (70_000, 6, torch.float64),
-                                       (300_000, 4, torch.float32), (300_000, 12, torch.float32)])
+                                       (300_000, 4, torch.float64), (300_000, 4, torch.float32), (300_000, 12, torch.float32)])
 def test_mirror_fill_replays(B, m, d, dtype):
     c = _product(B, m, d, dtype)
     expected = B.spsyrk_mirror(m, *c)

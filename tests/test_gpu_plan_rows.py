@@ -1,5 +1,5 @@
-"""Rows that the plan treats apart: long ones (left to a warp or the whole CTA; only so many of a CTA's rows) and dense
-ones (their counts are settled without a counting kernel)."""
+"""Rows that the plan treats apart: long ones (left to a warp or the whole CTA) and dense ones (their counts are settled without
+a counting kernel)."""
 import numpy as np
 import pytest
 import torch
@@ -39,7 +39,7 @@ def _check(a, ref, out):
 def test_long_rows_among_short_ones(B, average, mode):
     g = 4 if average <= 4 else 8 if average <= 8 else 16 if average <= 16 else 32
     edges = [8 * g - 1, 8 * g, 8 * g + 1, 1023, 1024, 1025, 4000]
-    crowd = [8 * g + 5] * 300  # more long rows next to each other than a CTA keeps for the end
+    crowd = [8 * g + 5] * 300  # long rows only: a CTA's whole tile of them
     short = (sum(edges) + sum(crowd)) * 2 // average
     lengths = [average // 2] * (short // 2) + edges + [average // 2] * (short // 2) + crowd
     a = _matrix(lengths, 60_000, average)
