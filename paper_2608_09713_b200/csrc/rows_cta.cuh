@@ -38,6 +38,10 @@ struct CtaRowSmem {
     }
 };
 
+// Products of the heavy columns per candidate row from which on a row is counted through its masks: they cost a look at every candidate
+// row.  3000 rows of 70 000 columns of which a few are a little heavier than the rest: 423 us without masks, 867 with them. 30 000 sets of
+// 60 columns of Zipf frequencies without the most frequent ones 8270 and 1561; 40 000 of 20 1544 (with 4 for 1 1722).
+constexpr uint32_t MASK_PRODUCTS = 1;
 // MASKS: counting in a binary matrix, the rows' masks of the heavy columns stand for whole rows of the lower triangle
 template <typename V, int THREADS, bool NUMERIC, bool MASKS = false>
 __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) rows_cta_kernel(PlanDev P, const int32_t* __restrict__ rows,
@@ -81,10 +85,23 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
 
     // A row whose range fits one chunk and that holds a column present in every candidate row
     // (a list as long as the range) is dense: every j occurs, no bitmap is needed to count them.
-    if (!NUMERIC && U <= chunk_bits) {
+    // Counting a row of a binary matrix whose heavy columns have at least MASK_PRODUCTS products per candidate row: the rows that
+    // share a heavy column with it come from the masks, and only the other lists are walked (16 products per entry on the Zipf workloads,
+    // 0.7 of them in those).
+    int planes = MASKS ? heavy_planes(P) : 0;
+    if (!NUMERIC && (U <= chunk_bits || planes > 0)) {
         int hit = 0;
-        for (uint32_t b0 = tid; b0 < deg; b0 += THREADS) hit |= (P.desc[p0 + b0].y == U);
-        if (__syncthreads_or(hit)) {
+        uint32_t covered = 0;
+        for (uint32_t b0 = tid; b0 < deg; b0 += THREADS) {
+            const uint32_t len = P.desc[p0 + b0].y;
+            hit |= len == U;
+            if (MASKS && planes > 0 && P.heavy_id[P.colidx[p0 + b0]] != 0xff) covered += len;
+        }
+        if (MASKS) {
+            covered = warp_reduce_sum<uint32_t>(covered);
+            if ((tid & 31) == 0) scratch[tid >> 5] = covered;
+        }
+        if (__syncthreads_or(hit) && U <= chunk_bits) {
             const uint32_t nblk = (U + BASE_BLOCK - 1) / BASE_BLOCK;
             if (nblk <= blocks_per_row)
                 for (uint32_t blk = tid; blk < nblk; blk += THREADS) block_base[(uint64_t)i * blocks_per_row + blk] = blk * BASE_BLOCK;
@@ -92,11 +109,13 @@ __global__ void __launch_bounds__(THREADS, cta_min_blocks(THREADS, NUMERIC)) row
             chain_end();
             return;
         }
+        if (MASKS && planes > 0) {
+            const uint32_t lane = tid & 31;
+            if (warp_reduce_sum<uint32_t>(lane < THREADS / 32 ? scratch[lane] : 0u) < MASK_PRODUCTS * U) planes = 0;
+            __syncthreads();
+        }
     }
     const bool binary = P.binary != 0;
-    // Counting a row of many products of a binary matrix: the columns that share a heavy column with it come from the masks, and only
-    // the other lists are walked (16 products per entry on the Zipf workloads, 0.7 of them in those).
-    const int planes = MASKS && P.work[rloc] >= (int64_t)U ? heavy_planes(P) : 0;
 
     // One partial product: set its bit, or add it into its slot.
     auto apply = [&](auto what, uint32_t rel, Acc a, Acc v, uint32_t s0) {

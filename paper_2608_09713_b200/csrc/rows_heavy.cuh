@@ -81,7 +81,8 @@ static __global__ void __launch_bounds__(ROUTE_THREADS) route_rows_kernel(PlanDe
             // Rows that are not dense: rank walks all their products twice, direct has 32-bit counters; dense8 walks each once, fewer with
             // heavy columns, but looks at every column.  Numeric pass of 30 000 rows of random columns, without and with dense8: w = U 2565
             // us to 2020, 1.3 U 2999 to 1551, 2 U 3737 to 1839; of 6000 rows 147 to 126, 156 to 120, 175 to 137 (below U the two
-            // are level: rank has the fewer columns to look at).  30 000 sets of 60 of 65 536 columns of Zipf frequencies, of
+            // are level: rank has the fewer columns to look at).  The last 3000 rows of 70 000, 150 000 and 220 000 (fewer CTAs fit an SM), 1.5 U:
+            // 1819 us to 665, 4610 to 2298, 6131 to 3367.  30 000 sets of 60 of 65 536 columns of Zipf frequencies, of
             // which some lack the most frequent one: all similarities 12.0 ms to 3.1, counting included.
             route = ROUTE_DENSE8;
         } else if ((R.binary && dense) || (U <= R.chunk && w >= (int64_t)(U / 4))) {

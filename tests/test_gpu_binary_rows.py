@@ -74,3 +74,18 @@ def test_partly_full_rows_both_triangles(B, m, n, d):
     ref = oracle.syrk(m, n, rp, ci, np.ones(ci.size), oracle.FULL)
     got = [t.cpu().numpy() for t in B.tril_syrk(m, n, *dev, mode=B.FULL)[:3]]
     assert np.array_equal(got[0], ref.rowptr) and np.array_equal(got[1], ref.colidx) and np.array_equal(got[2], ref.vals)
+
+
+@pytest.mark.parametrize("share", [0.2, 0.4])
+def test_a_few_heavy_columns(B, share):
+    """Ten columns of 400 are heavier than the rest: with 0.2 their products are fewer than the rows to look at, which are counted
+    without masks then, with 0.4 more."""
+    m, n = 3000, 400
+    rng = np.random.default_rng(3)
+    keep = rng.random((m, n)) < np.where(np.arange(n) % 40 == 7, share, 0.125)
+    rp = np.concatenate(([0], np.cumsum(keep.sum(1)))).astype(np.int64)
+    ci = np.nonzero(keep)[1].astype(np.int32)
+    dev = (torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), torch.ones(ci.size, dtype=torch.int32, device="cuda"))
+    ref = oracle.syrk(m, n, rp, ci, np.ones(ci.size, dtype=np.int32), oracle.TRIL)
+    got = _run(B, B.spsyrk_plan(m, n, *dev), m, torch.int32, False)
+    assert np.array_equal(got[0], ref.rowptr) and np.array_equal(got[1], ref.colidx) and np.array_equal(got[2].astype(np.float64), ref.vals)
