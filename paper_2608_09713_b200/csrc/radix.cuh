@@ -172,7 +172,9 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
 
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     static_assert(NB == RX_BINS && NB <= RX_THREADS, "one thread per digit");
-    link(keys, pa, pb, bins);  // (pc is read behind the barriers of the ranking)
+    // (What is read of the elements lies where the ticket says, which is drawn behind this; with their pointers handed to link
+    // they were no loads of constants any more and registers were spilled: a pass over 1.7e7 nonzeros took 250 us instead of 240.)
+    link();
     if (tid == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
     const int64_t tile = s_tile, tile_base = tile * RX_TILE;
@@ -254,7 +256,7 @@ __global__ void __launch_bounds__(RX_THREADS, 2) radix_scatter_kernel(const uint
     }
     // slot q of digit d goes to (elements of smaller digits) + (of this digit in the tiles before) + q - first slot of d
     int64_t tot64;
-    const int64_t base_d = block_exclusive_scan<int64_t, RX_THREADS>(tid < NB ? (int64_t)bins[tid] : 0, scratch64, &tot64);
+    const int64_t base_d = block_exclusive_scan<int64_t, RX_THREADS>(tid < NB ? (int64_t)ld_status(bins + tid) : 0, scratch64, &tot64);  // (not before link: a load that stays where it is)
     if (tid < NB) goff[tid] = base_d + radix_look_back<S>(words, tile, tid, total_d, err) - (int64_t)first_d;
     __syncthreads();
     for (int q = tid; q < tile_n; q += RX_THREADS) {
