@@ -35,6 +35,8 @@ UNIT = "MAC/s"
 # DRAM bytes per launch of the dominant kernel from the ncu capture summarised under profiles/
 # (bytes per useful multiply-add, multiplied by the launch's multiply-adds); None = not captured.
 NCU_TRAFFIC_BYTES_PER_MAC = 32.8
+# rows above which the mirror of 8-byte values goes by record passes (MIRROR_BUCKET_ROWS_8 in csrc/mirror.cu), by buckets below
+MIRROR_RECORD_ROWS = 1 << 18
 
 
 def measured_peaks():
@@ -462,7 +464,7 @@ def roofline_and_variants(a, args, line, ctx, headline):
         if pms:
             pm = np.mean(np.array(pms), axis=0)
             line["mirror_pass"]["sort_passes_ms"] = [float(x) for x in pm]
-            if sv == 8 and a.m > 65536:
+            if sv == 8 and a.m > MIRROR_RECORD_ROWS:
                 # a record pass moves a 16-byte record in and out plus the digit byte it writes and the next histogram reads
                 pass_bytes = nnz_c * (16 + 16 + 2)
                 mid = int(np.argmax(pm))

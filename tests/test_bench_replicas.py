@@ -45,3 +45,12 @@ def test_single_process_needs_no_process_group():
     # lower-triangle mode classes a light row by its products without the d_i diagonal ones
     w = bench.class_of_rows(work - deg, deg, work)
     assert list(w) == [0, 1, 2, 6, 7, 1]
+
+
+def test_the_bench_knows_which_mirrors_go_by_records():
+    """The roofline of a record pass is reported where the library makes record passes."""
+    import re
+    sys.path.insert(0, ROOT)
+    import bench
+    source = open(os.path.join(ROOT, "paper_2608_09713_b200", "csrc", "mirror.cu")).read()
+    assert bench.MIRROR_RECORD_ROWS == int(re.search(r"MIRROR_BUCKET_ROWS_8 = (\d+);", source).group(1))
