@@ -68,6 +68,22 @@ def test_accumulate_of_many_entries(B):
     assert all(np.array_equal(a, b) for a, b in zip(got, ref))
 
 
+@pytest.mark.parametrize("m", [65_536, 65_537, 1 << 20, (1 << 20) + 3])  # long rows are looked for row by row, by units of 4 rows, of 32
+@pytest.mark.parametrize("mean", [2, 20], ids=["lanes", "warps"])
+def test_long_rows_wherever_they_stand(B, m, mean):
+    """The first, the last, neighbours, rows at the ends of a unit, and a unit that is long in all but not in any row."""
+    rng = np.random.default_rng(m)
+    csr = []
+    for side in range(2):
+        lengths = rng.integers(0, mean + 1, size=m)
+        lengths[[0, 1, 31, 32, 127, 128, m // 2, m // 2 + 1, m - 4, m - 1]] = rng.integers(600, 5000, size=10)
+        lengths[4096:4096 + 32] = 60
+        csr.append(_device_csr(lengths, m + side))
+    got = [t.cpu().numpy() for t in B.spsyrk_accumulate(m, *csr[0], *csr[1])]
+    ref = oracle.add(m, *(t.cpu().numpy() for t in csr[0] + csr[1]))
+    assert all(np.array_equal(a, b) for a, b in zip(got, ref))
+
+
 @pytest.mark.parametrize("size", [300, 5000])
 @pytest.mark.parametrize("side", [0, 1])
 def test_accumulate_refuses_rows_that_do_not_ascend(B, size, side):
