@@ -121,7 +121,8 @@ __device__ __forceinline__ uint32_t walk_row(const int32_t* __restrict__ self, u
 // two windows' last ids is known completely, so those entries are merged at once: an entry's place is the output position
 // reached so far + its index in its own window + the entries of the other window below it (a search over the window in shared
 // memory) - the matches below it (votes).  All global accesses are coalesced and a step brings in up to 64 ids with one
-// round of loads.  Bound by the load/store pipe (the searches' bank conflicts).  Sums of 6e7 entries, single precision, both steps, rows of
+// round of loads.  Bound by instruction issue (rows of 131 entries: 86 % of the slots in the size step, 77 in the fill; load/store pipe 54
+// and 50 %, DRAM 16 and 32).  Sums of 6e7 entries, single precision, both steps, rows of
 // 33, 131, 513 and 2000 entries of both inputs: 1023, 591, 518 and 554 us.  (The merge path by a warp, eight entries a lane: 2700, 974, 683
 // and 658, because a row pays for a whole tile.)
 // FILL: the merged row goes to zc, zv (at most lz entries: always enough with the row pointer of the size step; keeps a
@@ -195,8 +196,9 @@ __device__ __forceinline__ uint32_t merge_windows(const int32_t* __restrict__ xc
 // finds by a binary search where its MERGE_ITEMS entries of the merged order begin in either row and merges them one
 // after the other, x before y where both store a column; such a pair is emitted once, with x + y, by the thread that has its
 // x.  The emitted entries are put in order in the shared memory of the ids and written out by consecutive threads.
-// Bound by instruction issue.  Rows of 10 000 entries: 630 us for 6e7; the windows of a warp take less time in all for shorter rows,
-// but a row's 32 entries after 32 entries keep one warp long after the others.
+// Bound by the steps of a tile, one behind the other (size step: issue slots and load/store pipe 68 % each; fill 56 and 55, waits for the
+// values and at the barriers).  Rows of 10 000 entries: 630 us for 6e7; the windows of a warp take less time in all for
+// shorter rows, but a row's 32 entries after 32 entries keep one warp long after the others.
 constexpr int MERGE_ITEMS = 8;
 constexpr int MERGE_LONG_THREADS = 256;
 constexpr uint32_t MERGE_TILE = MERGE_LONG_THREADS * MERGE_ITEMS;
