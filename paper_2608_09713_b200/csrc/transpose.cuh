@@ -364,11 +364,15 @@ static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev
                 deg[u] = (int32_t)(P.rowptr[P.r0 + r + 1] - p0[u]);
             }
         }
+        const int32_t longest = max(max(deg[0], deg[1]), max(deg[2], deg[3]));
+        static_assert(UNR == 4, "the longest of a group's rows");
+        if (longest > LONG_STEPS * G) {
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (deg[u] > LONG_STEPS * G) {
-                if (gl == 0) s_long[atomicAdd(&s_nlong, 1)] = (uint16_t)(base + u * GROUPS + group - t0);
-                deg[u] = -1;
+            for (int u = 0; u < UNR; ++u) {
+                if (deg[u] > LONG_STEPS * G) {
+                    if (gl == 0) s_long[atomicAdd(&s_nlong, 1)] = (uint16_t)(base + u * GROUPS + group - t0);
+                    deg[u] = -1;
+                }
             }
         }
 #pragma unroll
@@ -381,11 +385,8 @@ static __global__ void __launch_bounds__(BIN_THREADS, 6) row_work_kernel(PlanDev
 #pragma unroll
             for (int o = G / 2; o > 0; o >>= 1) w[u] += __shfl_xor_sync(FULL_MASK, w[u], o);
         }
-        // heavy rows: does one of the columns cover the row's range?
-        bool heavy_row = false;
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) heavy_row |= is_heavy(deg[u], w[u]);
-        if (__any_sync(FULL_MASK, heavy_row)) {
+        // heavy rows: does one of the columns cover the row's range?  (a look at the largest first: light rows have little else to do here)
+        if (__any_sync(FULL_MASK, longest > 32 || max(max(w[0], w[1]), max(w[2], w[3])) > 512u)) {
 #pragma unroll
             for (int u = 0; u < UNR; ++u) {
                 if (!is_heavy(deg[u], w[u])) continue;
